@@ -134,6 +134,84 @@ __device__ __forceinline__ float apply_act(float x, int act) {
   }
 }
 
+// 2^x and 1/x by the special-function unit.
+__device__ __forceinline__ float sfu_ex2(float x) { float y; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
+__device__ __forceinline__ float sfu_rcp(float x) { float y; asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
+
+// log(1 + exp(x)) = max(x, 0) + log1p(e), e = exp(-|x|) in (0, 1]: log1p(e) / e as a polynomial fitted to the minimax
+// relative error on (0, 1] (2e-7), so that small results keep their relative accuracy.
+__device__ __forceinline__ float softplus_fast(float x) {
+  const float e = sfu_ex2(-1.4426950408889634f * fabsf(x));
+  float p = -0.0085390963f;
+  p = fmaf(p, e, 0.044089238f); p = fmaf(p, e, -0.10768117f); p = fmaf(p, e, 0.17745204f);
+  p = fmaf(p, e, -0.2449545f); p = fmaf(p, e, 0.33275478f); p = fmaf(p, e, -0.49997405f); p = fmaf(p, e, 0.9999998f);
+  return fmaf(p, e, fmaxf(x, 0.f));
+}
+// x Phi(x) = max(x, 0) - |x| Q(|x|) with the normal tail Q(a) = exp(-a^2 / 2) g(t), t = 1 / (1 + a / 4); g as a
+// polynomial fitted to the minimax relative error for 0 <= a <= 9.5 (1.2e-7); beyond that exp(-a^2 / 2) < 3e-20.
+__device__ __forceinline__ float gelu_fast(float x) {
+  const float a = fabsf(x) > 64.f ? 64.f : fabsf(x), t = sfu_rcp(fmaf(0.25f, a, 1.f)), e = sfu_ex2(-0.72134752044448170f * a * a);
+  float p = -0.098380317f;
+  p = fmaf(p, t, 0.37461082f); p = fmaf(p, t, -0.33402116f); p = fmaf(p, t, 0.35451113f); p = fmaf(p, t, -0.02167429f);
+  p = fmaf(p, t, 0.12915299f); p = fmaf(p, t, 0.095545365f); p = fmaf(p, t, 0.00025551728f);
+  return fmaf(-a * e, p, fmaxf(x, 0.f));
+}
+// The activation of a block of values, for the kernels that round it to bf16 (2^-9): within 5e-7 of apply_act.
+// The selection is outside the loop over the block, and the library functions (log1pf, expf, erff: tens of
+// instructions and branches each, inlined once per column) are not used: see the epilogues of the phi kernels.
+template <int N>
+__device__ __forceinline__ void act_block(float (&y)[N], int act) {
+  switch (act) {
+    case ACT_RELU:
+#pragma unroll
+      for (int e = 0; e < N; ++e) y[e] = fmaxf(y[e], 0.f);
+      break;
+    case ACT_IDENTITY: break;
+    case ACT_SOFTPLUS:
+#pragma unroll
+      for (int e = 0; e < N; ++e) y[e] = softplus_fast(y[e]);
+      break;
+    case ACT_ELU1:
+#pragma unroll
+      for (int e = 0; e < N; ++e) y[e] = y[e] > 0.f ? y[e] + 1.f : sfu_ex2(1.4426950408889634f * y[e]);
+      break;
+    default:
+#pragma unroll
+      for (int e = 0; e < N; ++e) y[e] = gelu_fast(y[e]);
+      break;
+  }
+}
+// The power part + 1 of a block of values of one polynomial part (part <= 3).
+template <int N>
+__device__ __forceinline__ void power_block(float (&y)[N], int part) {
+  if (part == 0) return;
+#pragma unroll
+  for (int e = 0; e < N; ++e) {
+    const float u = y[e], u2 = u * u;
+    y[e] = part == 1 ? u2 : part == 2 ? u2 * u : u2 * u2;
+  }
+}
+
+// What the epilogues of the phi kernels do to a block of accumulator columns [col0, col0 + N) of a non-ReLU layer
+// (bias already added): the activation, for the last layer (is_u) the power of the columns' polynomial parts and zero
+// beyond D'.  D' is a multiple of 32 and P at most 4, so a part is a whole number of eight columns
+// and D' ends on a block.
+template <int N>
+__device__ __forceinline__ void act_power_block(float (&y)[N], int act, bool is_u, int col0, int part_w, int Dp) {
+  static_assert(N % 8 == 0 && N <= 32, "blocks of whole parts");
+  act_block(y, act);
+  if (!is_u) return;
+#pragma unroll
+  for (int g = 0; g < N; g += 8) {
+    float z[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) z[e] = y[g + e];
+    if (part_w < Dp) power_block(z, (col0 + g) / part_w);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) y[g + e] = col0 < Dp ? z[e] : 0.f;
+  }
+}
+
 // Element-wise power of the polynomial expansion: output feature j of D' belongs to part
 // j / (D'/P) (0-based) and is raised to that index plus one.
 __device__ __forceinline__ float poly_power(float u, int part) {

@@ -307,25 +307,12 @@ readout_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUt
           }
         }
       } else {
-        const int act = is_u ? a.act_out : a.act_hidden;
-        if (GEN && is_u) {                                          // parts end anywhere; features beyond D' are zero
+        float y[NC];
 #pragma unroll
-          for (int e = 0; e < NC; e += 2) {
-            const int f0 = col0 + e;
-            const float y0 = apply_act(__uint_as_float(x[e]) + bias[e], act);
-            const float y1 = apply_act(__uint_as_float(x[e + 1]) + bias[e + 1], act);
-            w[e >> 1] = pack_bf16(f0 < Dp ? poly_power(y0, f0 / part_w) : 0.f,
-                                  f0 + 1 < Dp ? poly_power(y1, (f0 + 1) / part_w) : 0.f);
-          }
-        } else {
-          const int part = is_u ? col0 / part_w : 0;
+        for (int e = 0; e < NC; ++e) y[e] = __uint_as_float(x[e]) + bias[e];
+        act_power_block(y, is_u ? a.act_out : a.act_hidden, is_u, col0, part_w, Dp);
 #pragma unroll
-          for (int e = 0; e < NC; e += 2) {
-            const float y0 = apply_act(__uint_as_float(x[e]) + bias[e], act);
-            const float y1 = apply_act(__uint_as_float(x[e + 1]) + bias[e + 1], act);
-            w[e >> 1] = pack_bf16(poly_power(y0, part), poly_power(y1, part));
-          }
-        }
+        for (int e = 0; e < NC; e += 2) w[e >> 1] = pack_bf16(y[e], y[e + 1]);
       }
     };
     auto readout_store = [&](int jt) {                              // fp32 read-out of tile jt leaves TMEM

@@ -1,0 +1,58 @@
+"""Single kernels and dispatch branches at the sizes and values where they can go wrong (edges of tiles, remainders,
+the ends of their ranges), against the fp64 oracle.  Gates as in test_gpu_parity.py."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import rehyat_oracle as orc
+from paper_2601_04342_b200 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_2601_04342_b200 import build
+    build.build()
+
+
+def _forward(wl, x, layout="bhnd", **kw):
+    from paper_2601_04342_b200 import binding
+    op = binding.for_workload(wl, **kw)
+    q, k, v = (x[n].cuda() for n in ("q", "k", "v"))
+    if layout == "bnhd":
+        q, k, v = (t.transpose(1, 2).contiguous() for t in (q, k, v))
+    pq, pk = ({n: t.cuda() for n, t in x[m].items()} for m in ("phi_q", "phi_k"))
+    y = op.forward(q, k, v, pq, pk, wl.T, wl.H, wl.W, wl.Tc, wl.To, layout=layout)
+    assert op.status() == 0
+    op.close()
+    return (y.transpose(1, 2) if layout == "bnhd" else y).double().cpu().numpy()
+
+
+def _oracle(wl, x, **kw):
+    f = synth.to_f64(x)
+    return orc.hybrid_direct(f["q"], f["k"], f["v"], f["phi_q"], f["phi_k"], wl.T, wl.HW, wl.Tc, wl.To, P=wl.P, **kw)
+
+
+def _gate(y, ref, dtype):
+    err = np.abs(y - ref)
+    if dtype == "fp32":
+        assert err.max() <= 1e-4, f"max-abs {err.max():.3e}"
+        return
+    assert err.max() <= 2e-2, f"max-abs {err.max():.3e}"
+    worst = (err / (3e-3 + 2.0 ** -7 * np.abs(ref))).max()
+    assert worst <= 1.0, f"internal gate exceeded x{worst:.2f}, max-abs {err.max():.3e}"
+    assert np.sqrt((err ** 2).mean() / (ref ** 2).mean()) <= 1e-2
+
+
+@pytest.mark.parametrize("act_hidden,act_out,P,Dp", [("gelu", "softplus", 1, 256), ("softplus", "elu1", 4, 96),
+                                                     ("elu1", "relu", 3, 192), ("gelu", "relu", 2, 96)])
+def test_activations_over_their_whole_range(act_hidden, act_out, P, Dp):
+    """The activations of the tensor-core phi kernels with arguments from deep in the tails to well above zero
+    (first layer of standard deviation 4 here, 0.2 in the other tests), parts that end inside 16 columns."""
+    wl = synth.Workload("acts", 1, 2, 128, 5, 10, 20, 2, 1, "bf16", True, P=P, seed=synth.BASE_SEED + 401, phi_dim=Dp)
+    x = synth.make_inputs(wl, v_frame_offsets=True)
+    for m in ("phi_q", "phi_k"):
+        x[m]["W1"] = (x[m]["W1"].float() * 18).to(torch.bfloat16)
+    y = _forward(wl, x, act_hidden=act_hidden, act_out=act_out)
+    _gate(y, _oracle(wl, x, act_hidden=act_hidden, act_out=act_out), "bf16")
