@@ -16,6 +16,7 @@
 #include <cstring>
 #include <mutex>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/rehyat.h"
@@ -139,12 +140,11 @@ int check_config(const rehyat_config* c) {
 // cannot lower it under a live one.
 template <typename T, int D>
 int set_simt_attributes() {
-  const int smem_state = (SIMT_TM * (2 * D + 256) + phi_hidden_floats(256, 1)) * (int)sizeof(float);
-  const int smem_rd = (SIMT_TM * (D + 256) + phi_hidden_floats(256, 1)) * (int)sizeof(float);
-  const int smem_win = (WIN_BM * (D + 4) + WIN_BN * (D + 4) + WIN_BN * D + WIN_BM * (WIN_BN + 4)) * (int)sizeof(float);
-  if (cudaFuncSetAttribute(state_partial_simt<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_state) != cudaSuccess ||
-      cudaFuncSetAttribute(readout_simt<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_rd) != cudaSuccess ||
-      cudaFuncSetAttribute(window_simt<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_win) != cudaSuccess)
+  const auto smem = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  if (cudaFuncSetAttribute(state_partial_simt<T, D>, smem, simt_phi_smem(D, 256, 256, true)) != cudaSuccess ||
+      cudaFuncSetAttribute(readout_simt<T, D>, smem, simt_phi_smem(D, 256, 256, false)) != cudaSuccess ||
+      cudaFuncSetAttribute(window_simt<T, D, 1>, smem, WinSimt<T, D, 1>::SMEM) != cudaSuccess ||
+      cudaFuncSetAttribute(window_simt<T, D, 4>, smem, WinSimt<T, D, 4>::SMEM) != cudaSuccess)
     return REHYAT_ERR_CUDA;
   return REHYAT_OK;
 }
@@ -168,6 +168,24 @@ ptx::WaitArgs next_wait(rehyat_ctx* ctx) {
 // Which steps of a chunk group to enqueue.
 enum Parts : int { PART_STATE = 1 /* increments + scan */, PART_READOUT = 2, PART_WINDOW = 4 };
 
+// Into how many CTAs to cut a (chunk, batch*head) unit of `tiles` tiles when `units` of them run at one CTA per SM: the
+// number up to `most` that costs the fewest tile-times over all waves.
+int pick_parts(long long tiles, long long units, int most, int n_sm) {
+  long long best = -1;
+  int best_s = 1;
+  for (int s = 1; s <= most; ++s) {
+    const long long cost = ((units * s + n_sm - 1) / n_sm) * ((tiles + s - 1) / s);
+    if (best < 0 || cost < best) { best = cost; best_s = s; }
+  }
+  return best_s;
+}
+// Chunks of the group whose linear set is not empty (at least 1).
+int busy_readout(const Geo& g) {
+  int busy = 0;
+  for (int t = g.t0; t < g.t0 + g.G; ++t) busy += geo_linear(g, t);
+  return busy > 0 ? busy : 1;
+}
+
 template <typename T, int D>
 int launch_group_simt(rehyat_ctx* ctx, const T* q, const T* k, const T* v, T* out, const rehyat_phi_params* phi,
                       const Geo& g, int n_split, int carry_slot, int parts, cudaStream_t st) {
@@ -175,13 +193,11 @@ int launch_group_simt(rehyat_ctx* ctx, const T* q, const T* k, const T* v, T* ou
   const int rd_half = ctx->tensor_ok ? 1 : 0;     // the tensor-core window kernels read the bf16 form of the read-out
   PhiDims pd = {D, c.phi_hidden, c.phi_dim, c.poly_degree, c.act_hidden, c.act_out, c.phi_layers > 2 ? c.phi_layers - 2 : 0};
   constexpr int SD = D + 4;
-  const int tiles = (g.Np + SIMT_TM - 1) / SIMT_TM;
   if (parts & PART_STATE) {
     PhiPtrs<T> wk = {(const T*)phi->k_W1, (const T*)phi->k_b1, (const T*)phi->k_W2, (const T*)phi->k_b2,
                      (const T*)phi->k_Wmid, (const T*)phi->k_bmid};
-    const size_t smem_state = ((size_t)SIMT_TM * (2 * D + pd.Dp) + phi_hidden_floats(pd.Dh, pd.n_mid)) * sizeof(float);
     ctx->prof.begin(REHYAT_PROF_STATE, st);
-    state_partial_simt<T, D><<<dim3(n_split, g.G, g.BH), SIMT_PHI_THREADS, smem_state, st>>>(
+    state_partial_simt<T, D><<<dim3(n_split, g.G, g.BH), SIMT_THREADS, simt_phi_smem(D, pd.Dh, pd.Dp, true), st>>>(
         k, v, wk, pd, g, n_split, ctx->partial);
     ctx->prof.end(REHYAT_PROF_STATE, st);
     const size_t per_slot = (size_t)g.BH * pd.Dp * SD;
@@ -194,46 +210,43 @@ int launch_group_simt(rehyat_ctx* ctx, const T* q, const T* k, const T* v, T* ou
   if (parts & PART_READOUT) {
     PhiPtrs<T> wq = {(const T*)phi->q_W1, (const T*)phi->q_b1, (const T*)phi->q_W2, (const T*)phi->q_b2,
                      (const T*)phi->q_Wmid, (const T*)phi->q_bmid};
-    const size_t smem_rd = ((size_t)SIMT_TM * (D + pd.Dp) + phi_hidden_floats(pd.Dh, pd.n_mid)) * sizeof(float);
+    const int tiles = (g.Np + SIMT_TM - 1) / SIMT_TM;
+    const int parts_rd = pick_parts(tiles, (long long)busy_readout(g) * g.BH, tiles < 64 ? tiles : 64, ctx->tc.n_sm);
+    const int per_cta = (tiles + parts_rd - 1) / parts_rd;
     ctx->prof.begin(REHYAT_PROF_READOUT, st);
-    readout_simt<T, D><<<dim3(tiles, g.G, g.BH), SIMT_PHI_THREADS, smem_rd, st>>>(q, wq, pd, g, ctx->state,
-                                                                                 ctx->readout, ctx->rd_cap, rd_half);
+    readout_simt<T, D><<<dim3((tiles + per_cta - 1) / per_cta, g.G, g.BH), SIMT_THREADS, simt_phi_smem(D, pd.Dh, pd.Dp, false), st>>>(
+        q, wq, pd, g, ctx->state, ctx->readout, ctx->rd_cap, rd_half, per_cta);
     ctx->prof.end(REHYAT_PROF_READOUT, st);
     ctx->last_launches += 1;
   }
   if (parts & PART_WINDOW) {
-    const size_t smem_win = (size_t)(WIN_BM * (D + 4) + WIN_BN * (D + 4) + WIN_BN * D + WIN_BM * (WIN_BN + 4)) * sizeof(float);
-    const int wtiles = (g.Np + WIN_BM - 1) / WIN_BM;
     ctx->prof.begin(REHYAT_PROF_WINDOW, st);
-    window_simt<T, D><<<dim3(wtiles, g.G, g.BH), WIN_THREADS, smem_win, st>>>(
-        q, k, v, out, g, ctx->readout, ctx->rd_cap, 1.0f / sqrtf((float)D), c.c_mode, ctx->share_now);
+    const auto launch = [&](auto split) {
+      constexpr int WK = decltype(split)::value;
+      using S = WinSimt<T, D, WK>;
+      window_simt<T, D, WK><<<dim3((g.Np + S::BM - 1) / S::BM, g.G, g.BH), SIMT_THREADS, S::SMEM, st>>>(
+          q, k, v, out, g, ctx->readout, ctx->rd_cap, 1.0f / sqrtf((float)D), c.c_mode, ctx->share_now);
+    };
+    // Tiles of 128 rows need the fewest loads per multiply-add; below two waves of them the SMs are better filled by
+    // tiles of 32 rows whose keys are shared among four warps (2 heads x 1,071 tokens of 64 channels: 12 tiles of the one,
+    // 90 of the other, for 148 SMs).
+    if ((long long)((g.Np + 127) / 128) * g.G * g.BH >= 2LL * ctx->tc.n_sm) launch(std::integral_constant<int, 1>());
+    else launch(std::integral_constant<int, 4>());
     ctx->prof.end(REHYAT_PROF_WINDOW, st);
     ctx->last_launches += 1;
   }
   return cudaGetLastError() == cudaSuccess ? REHYAT_OK : REHYAT_ERR_CUDA;
 }
 
-// Split of a chunk's state increment over CTAs.  Tensor-core kernels: one CTA per (split, chunk, head)
-// and one CTA per SM, so pick the split that needs the fewest token tiles per SM over all waves.
+// Split of a chunk's state increment over CTAs: one CTA per (split, chunk, head) and one CTA per SM.
 int pick_state_split(const rehyat_ctx* ctx, const Geo& g, int n_chunks_in_group, int tokens_per_increment) {
-  int n_split = ctx->partial_units / (n_chunks_in_group > 0 ? n_chunks_in_group : 1);
-  const int most = ctx->tensor_ok && ctx->tc.phi_ok ? 16 : 8;   // a lone chunk (a chunk-by-chunk step) over all SMs
-  if (n_split > most) n_split = most;
-  if (n_split < 1) n_split = 1;
-  if (ctx->tensor_ok && ctx->tc.phi_ok) {
-    const int n_sm = ctx->tc.n_sm;
-    int busy = 0;                                   // chunks of the group that admit keys into the state
-    for (int t = g.t0 > 1 ? g.t0 : 1; t < g.t0 + n_chunks_in_group; ++t) busy += geo_lo(g, t) > geo_lo(g, t - 1);
-    const long long units = (long long)(busy > 0 ? busy : 1) * g.BH, tiles = (tokens_per_increment + 127) / 128;
-    long long best = -1;
-    int best_s = 1;
-    for (int s = 1; s <= n_split; ++s) {
-      const long long cost = ((units * s + n_sm - 1) / n_sm) * ((tiles + s - 1) / s);
-      if (best < 0 || cost < best) { best = cost; best_s = s; }
-    }
-    n_split = best_s;
-  }
-  return n_split;
+  int most = ctx->partial_units / (n_chunks_in_group > 0 ? n_chunks_in_group : 1);
+  if (most > 16) most = 16;                         // a lone chunk (a chunk-by-chunk step) over all SMs
+  if (most < 1) most = 1;
+  const int tile = ctx->tensor_ok && ctx->tc.phi_ok ? 128 : SIMT_TM;
+  int busy = 0;                                     // chunks of the group that admit keys into the state
+  for (int t = g.t0 > 1 ? g.t0 : 1; t < g.t0 + n_chunks_in_group; ++t) busy += geo_lo(g, t) > geo_lo(g, t - 1);
+  return pick_parts((tokens_per_increment + tile - 1) / tile, (long long)(busy > 0 ? busy : 1) * g.BH, most, ctx->tc.n_sm);
 }
 
 // Enqueues the requested steps for the chunks [g.t0, g.t0 + g.G) with whichever kernel family the context uses.
@@ -1054,9 +1067,13 @@ int rehyat_forward_static(const rehyat_config* cfg, const void* q, const void* k
   tmp.cfg.max_chunk_frames = chunk_eff;
   tmp.state = base;
   tmp.partial = base + n_chunks * slot;
-  tmp.readout = base + 2 * n_chunks * slot;
+  // what the states and the read-out leave of the array is for the partial sums: at least one per chunk (`need`), and a
+  // chunk's increment is split over as many CTAs as there are (up to 16)
+  const long long units = ((long long)kStaticScratchFloats - n_chunks * slot - BH * rd_cap * SD) / slot;
+  tmp.partial_units = (int)(units < 16 * n_chunks ? units : 16 * n_chunks);
+  tmp.readout = base + n_chunks * slot + tmp.partial_units * slot;
   tmp.Gmax = (int)n_chunks;
-  tmp.partial_units = (int)n_chunks;
+  cudaDeviceGetAttribute(&tmp.tc.n_sm, cudaDevAttrMultiProcessorCount, cfg->device);
   tmp.rd_rows = (int)rd_rows;
   tmp.rd_cap = (int)rd_cap;
   tmp.bh_max = (int)BH;

@@ -5,14 +5,28 @@
 //   scan_states         exclusive running sum of the chunk increments along the chunk axis
 //   readout_simt        phi_q on a query tile and phi_q(Q) s_t, phi_q(Q) z_t (Eq. 7, 9, 16)
 //   window_simt         softmax window with an online maximum (Eq. 6, 8) + joint normaliser (Eq. 5)
+//
+// All of them are matrix products on the FMA pipe.  They use the packed fma.rn.f32x2 throughout: it does two
+// multiply-adds per lane and issue, 101 - 108 per cycle and SM here against 60 - 72 of the scalar form.  Where the
+// reduction index is the contiguous one in both operands (Q K^T, the MLP layers) a pair holds the partial sums over even
+// and odd terms; where the output columns are contiguous (P V, phi^T V, phi s) it holds two columns.  A lane owns 4 - 8
+// rows x 4 - 16 columns, lanes of a warp 4 row groups x 8 column groups, so that an operand load of a warp touches 4 or
+// 8 different 16-byte pieces in different banks and feeds at least five packed instructions.
 #pragma once
 
 #include "rehyat_common.cuh"
+#include "rehyat_ptx.cuh"
 
 namespace rehyat {
 
 constexpr int SIMT_TM = 32;         // tokens per phi tile
-constexpr int SIMT_PHI_THREADS = 512;
+constexpr int SIMT_THREADS = 256;
+// Weights of the phi layers and the state reach the FMA pipe through slabs of 32 rows x 64 bytes, private to a warp
+// (a warp owns 32 output columns): no barrier but the warp's own between a slab's copy and its use.
+constexpr int SIMT_SLAB_ROW = 80;                      // bytes; the pad keeps eight consecutive rows in different banks
+constexpr int SIMT_SLAB = 32 * SIMT_SLAB_ROW;
+constexpr int SIMT_STAGES = 6;
+constexpr int SIMT_SLAB_BYTES = SIMT_THREADS / 32 * SIMT_STAGES * SIMT_SLAB;
 
 struct PhiDims {
   int d, Dh, Dp, P, act_hidden, act_out;
@@ -25,123 +39,227 @@ struct PhiPtrs {
   const T* Wm; const T* bm;                             // [n_mid][Dh][Dh], [n_mid][Dh] of the head (n_mid > 0)
 };
 
-// Shared memory (floats) of the hidden activations: one [TM][Dh] buffer, two when there are hidden layers in
-// between (they alternate as input and output).
-__host__ __device__ inline int phi_hidden_floats(int Dh, int n_mid) { return SIMT_TM * Dh * (n_mid > 0 ? 2 : 1); }
+// Row stride (floats) of the two buffers of activations, and the bytes of shared memory of the phi kernels:
+// X [TM][d + 4], two activation buffers, optionally V [TM][d], the slabs, TM floats.
+__host__ __device__ inline int simt_act_ld(int Dh, int Dp) { return (Dh > Dp ? Dh : Dp) + 4; }
+__host__ __device__ inline int simt_phi_smem(int d, int Dh, int Dp, bool with_v) {
+  return 4 * (SIMT_TM * (d + 4) + 2 * SIMT_TM * simt_act_ld(Dh, Dp) + (with_v ? SIMT_TM * d : 0) + SIMT_TM) + SIMT_SLAB_BYTES;
+}
 
-// phi of SIMT_TM tokens held in Xs [TM][d] -> Fs [TM][Dp].  Hs (phi_hidden_floats) is scratch.
-// `valid` rows carry tokens; the rest of Fs is forced to zero.
+// 16 bytes global -> shared, zeros if !valid (the address must be readable memory or is not touched then).
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool valid) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(valid ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// Four consecutive elements in shared memory as two pairs of floats.
+__device__ __forceinline__ void ld_pairs(const float* p, uint64_t& a, uint64_t& b) {
+  const ulonglong2 u = *reinterpret_cast<const ulonglong2*>(p);
+  a = u.x; b = u.y;
+}
+__device__ __forceinline__ void ld_pairs(const __nv_bfloat16* p, uint64_t& a, uint64_t& b) {
+  const uint2 u = *reinterpret_cast<const uint2*>(p);
+  a = ptx::pk2u(u.x << 16, u.x & 0xffff0000u);
+  b = ptx::pk2u(u.y << 16, u.y & 0xffff0000u);
+}
+__device__ __forceinline__ float pair_sum(uint64_t v) {
+  float lo, hi;
+  ptx::upk2(v, lo, hi);
+  return lo + hi;
+}
+
+// What one warp computes of a layer y = x W^T, W [N][K] row-major: the 32 columns from cb*32 on and RT*4 rows from
+// row0 on (lane: rows row0 + lane/8 + 4 i, columns cb*32 + lane%8 + 8 jj).
 template <typename T>
-__device__ void phi_tile_simt(const float* Xs, float* Hs, float* Fs, const PhiPtrs<T>& w,
-                              const PhiDims& pd, int valid) {
-  const int tid = threadIdx.x, NT = blockDim.x;
-  constexpr int RG = 4, RPG = SIMT_TM / RG;   // row groups of 8 rows
-  // layer 1
-  for (int idx = tid; idx < pd.Dh * RG; idx += NT) {
-    const int j = idx % pd.Dh, r0 = (idx / pd.Dh) * RPG;
-    float acc[RPG];
+struct SimtUnit {
+  static constexpr int KS = 64 / (int)sizeof(T);       // K extent of a slab
+  const T* W;
+  int N, K, cb;
+  bool active;
+  uint32_t slab;                                       // shared address of the warp's slabs
+  const uint8_t* slab_ptr;
+  __device__ __forceinline__ int slabs() const { return (K + KS - 1) / KS; }
+  // one commit group per call, also when there is nothing to copy
+  __device__ __forceinline__ void issue(int s, int lane) const {
+    if (active && s < slabs()) {
+      const uint32_t dst = slab + (s % SIMT_STAGES) * SIMT_SLAB;
 #pragma unroll
-    for (int r = 0; r < RPG; ++r) acc[r] = 0.f;
-    const T* wrow = w.W1 + (size_t)j * pd.d;
-    for (int k = 0; k < pd.d; k += 4) {
-      float4 wv = ld4(wrow + k);
-#pragma unroll
-      for (int r = 0; r < RPG; ++r) {
-        float4 x = *reinterpret_cast<const float4*>(Xs + (r0 + r) * pd.d + k);
-        acc[r] = fmaf(x.x, wv.x, acc[r]); acc[r] = fmaf(x.y, wv.y, acc[r]);
-        acc[r] = fmaf(x.z, wv.z, acc[r]); acc[r] = fmaf(x.w, wv.w, acc[r]);
+      for (int u = 0; u < 4; ++u) {
+        const int c = lane + 32 * u, r = c >> 2, ch = c & 3;
+        const int row = min(cb * 32 + r, N - 1), k = s * KS + ch * (KS / 4);
+        cp_async16(dst + r * SIMT_SLAB_ROW + ch * 16, W + (size_t)row * K + (k < K ? k : 0), k < K);
       }
     }
-    const float b = ldf(w.b1 + j);
-#pragma unroll
-    for (int r = 0; r < RPG; ++r) Hs[(r0 + r) * pd.Dh + j] = apply_act(acc[r] + b, pd.act_hidden);
+    cp_async_commit();
   }
-  __syncthreads();
-  // hidden layers in between: h <- act_hidden(Wm h + bm), the two buffers alternating
-  for (int m = 0; m < pd.n_mid; ++m) {
-    float* Hn = Hs + ((m & 1) ? 0 : SIMT_TM * pd.Dh);
-    const float* Hp = Hs + ((m & 1) ? SIMT_TM * pd.Dh : 0);
-    for (int idx = tid; idx < pd.Dh * RG; idx += NT) {
-      const int j = idx % pd.Dh, r0 = (idx / pd.Dh) * RPG;
-      float acc[RPG];
+};
+
+template <typename T, int RT>
+__device__ __forceinline__ void simt_unit_gemm(const SimtUnit<T>& un, const float* x, int ldx, int lane, uint64_t (&acc)[RT][4]) {
+  const int cg = lane & 7;
 #pragma unroll
-      for (int r = 0; r < RPG; ++r) acc[r] = 0.f;
-      const T* wrow = w.Wm + ((size_t)m * pd.Dh + j) * pd.Dh;
-      for (int k = 0; k < pd.Dh; k += 4) {
-        float4 wv = ld4(wrow + k);
+  for (int i = 0; i < RT; ++i)
 #pragma unroll
-        for (int r = 0; r < RPG; ++r) {
-          float4 x = *reinterpret_cast<const float4*>(Hp + (r0 + r) * pd.Dh + k);
-          acc[r] = fmaf(x.x, wv.x, acc[r]); acc[r] = fmaf(x.y, wv.y, acc[r]);
-          acc[r] = fmaf(x.z, wv.z, acc[r]); acc[r] = fmaf(x.w, wv.w, acc[r]);
+    for (int jj = 0; jj < 4; ++jj) acc[i][jj] = 0ull;
+  const int n = un.slabs();
+#pragma unroll 1
+  for (int s = 0; s < n; ++s) {
+    cp_async_wait<SIMT_STAGES - 2>();
+    __syncwarp();                                      // the slab is there for all lanes; they are done with the one before
+    un.issue(s + SIMT_STAGES - 1, lane);
+    const T* w = reinterpret_cast<const T*>(un.slab_ptr + (s % SIMT_STAGES) * SIMT_SLAB + cg * SIMT_SLAB_ROW);
+    const float* xs = x + s * SimtUnit<T>::KS;
+    const auto four = [&](int k) {                     // four terms of the sums
+      uint64_t wa[4], wb[4];
+#pragma unroll
+      for (int jj = 0; jj < 4; ++jj)
+        ld_pairs(reinterpret_cast<const T*>(reinterpret_cast<const uint8_t*>(w) + jj * 8 * SIMT_SLAB_ROW) + k, wa[jj], wb[jj]);
+#pragma unroll
+      for (int i = 0; i < RT; ++i) {
+        uint64_t xa, xb;
+        ld_pairs(xs + i * 4 * ldx + k, xa, xb);
+#pragma unroll
+        for (int jj = 0; jj < 4; ++jj) {
+          acc[i][jj] = ptx::fma2(xa, wa[jj], acc[i][jj]);
+          acc[i][jj] = ptx::fma2(xb, wb[jj], acc[i][jj]);
         }
       }
-      const float b = ldf(w.bm + (size_t)m * pd.Dh + j);
+    };
+    if ((s + 1) * SimtUnit<T>::KS <= un.K) {
 #pragma unroll
-      for (int r = 0; r < RPG; ++r) Hn[(r0 + r) * pd.Dh + j] = apply_act(acc[r] + b, pd.act_hidden);
+      for (int k = 0; k < SimtUnit<T>::KS; k += 4) four(k);
+    } else {
+#pragma unroll 1
+      for (int k = 0; s * SimtUnit<T>::KS + k < un.K; k += 4) four(k);
     }
-    __syncthreads();
   }
-  Hs += (pd.n_mid & 1) ? SIMT_TM * pd.Dh : 0;          // where the last hidden activations are
-  // last layer + polynomial expansion
+}
+
+// Bias, activation and, for the last layer, power and the mask of valid rows; into out [TM][ldo].
+template <typename T, int RT>
+__device__ __forceinline__ void simt_unit_finish(const SimtUnit<T>& un, const T* bias, int act, bool last, int part_w, int row0,
+                                                 int valid, float* out, int ldo, int lane, const uint64_t (&acc)[RT][4]) {
+  const int rg = lane >> 3, cg = lane & 7;
+#pragma unroll
+  for (int jj = 0; jj < 4; ++jj) {
+    const int j = un.cb * 32 + cg + 8 * jj;
+    if (j >= un.N) continue;
+    const float b = ldf(bias + j);
+#pragma unroll
+    for (int i = 0; i < RT; ++i) {
+      const float y = pair_sum(acc[i][jj]) + b;
+      out[(row0 + rg + 4 * i) * ldo + j] = act == ACT_RELU ? fmaxf(y, 0.f) : y;
+    }
+  }
+  if (act == ACT_RELU && !(last && (part_w < un.N || valid < SIMT_TM))) return;
+  // rolled: the library's log1pf, expf and erff inlined once, not once per accumulator.  A lane reads back its own values.
+#pragma unroll 1
+  for (int e = 0; e < RT * 4; ++e) {
+    const int j = un.cb * 32 + cg + 8 * (e & 3), r = row0 + rg + 4 * (e >> 2);
+    if (j >= un.N) continue;
+    float* o = out + r * ldo + j;
+    float y = *o;
+    if (act != ACT_RELU) y = apply_act(y, act);
+    if (last) y = r < valid ? poly_power(y, j / part_w) : 0.f;
+    *o = y;
+  }
+}
+
+// phi of SIMT_TM tokens held in Xs [TM][d + 4]; h0, h1 are the two activation buffers [TM][ldh].  Returns the one that
+// holds the features [TM][D'], rows from `valid` on forced to zero.  `x_free` runs once Xs has been read by all warps
+// (after a barrier).  Ends without a barrier.
+template <typename T, typename XFree>
+__device__ __forceinline__ float* phi_tile_simt(const float* Xs, float* h0, float* h1, int ldh, uint8_t* slabs,
+                                                const PhiPtrs<T>& w, const PhiDims& pd, int valid, XFree&& x_free) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, rg = lane >> 3;
   const int part_w = pd.Dp / pd.P;
-  for (int idx = tid; idx < pd.Dp * RG; idx += NT) {
-    const int j = idx % pd.Dp, r0 = (idx / pd.Dp) * RPG;
-    float acc[RPG];
+  SimtUnit<T> un;
+  un.slab_ptr = slabs + warp * SIMT_STAGES * SIMT_SLAB;
+  un.slab = ptx::smem_u32(un.slab_ptr);
+  const float* in = Xs;
+  int ldi = pd.d + 4;
+  float* out = h0;
+#pragma unroll 1
+  for (int l = 0; l < pd.n_mid + 2; ++l) {
+    const bool first = l == 0, last = l == pd.n_mid + 1;
+    un.W = first ? w.W1 : last ? w.W2 : w.Wm + (size_t)(l - 1) * pd.Dh * pd.Dh;
+    un.N = last ? pd.Dp : pd.Dh;
+    un.K = first ? pd.d : pd.Dh;
+    const T* bias = first ? w.b1 : last ? w.b2 : w.bm + (size_t)(l - 1) * pd.Dh;
+    const int act = last ? pd.act_out : pd.act_hidden;
+    // a warp per 32 columns and all 32 rows; widths up to 128 give it 16 rows, so that up to eight warps have work
+    const int n_cb = (un.N + 31) >> 5, row_units = n_cb > 4 ? 1 : 2;
+    un.cb = warp % n_cb;
+    un.active = warp / n_cb < row_units;
+    __syncwarp();                                      // all lanes are done with the slabs of the layer before
 #pragma unroll
-    for (int r = 0; r < RPG; ++r) acc[r] = 0.f;
-    const T* wrow = w.W2 + (size_t)j * pd.Dh;
-    for (int k = 0; k < pd.Dh; k += 4) {
-      float4 wv = ld4(wrow + k);
-#pragma unroll
-      for (int r = 0; r < RPG; ++r) {
-        float4 x = *reinterpret_cast<const float4*>(Hs + (r0 + r) * pd.Dh + k);
-        acc[r] = fmaf(x.x, wv.x, acc[r]); acc[r] = fmaf(x.y, wv.y, acc[r]);
-        acc[r] = fmaf(x.z, wv.z, acc[r]); acc[r] = fmaf(x.w, wv.w, acc[r]);
+    for (int s = 0; s < SIMT_STAGES - 1; ++s) un.issue(s, lane);
+    cp_async_wait<SIMT_STAGES - 1>();                  // copies into Xs, if any, are older than the slabs
+    __syncthreads();                                   // the layer's input is complete
+    if (l == 1) x_free();
+    if (un.active) {
+      if (row_units == 1) {
+        uint64_t acc[8][4];
+        simt_unit_gemm<T, 8>(un, in + rg * ldi, ldi, lane, acc);
+        simt_unit_finish<T, 8>(un, bias, act, last, part_w, 0, valid, out, ldh, lane, acc);
+      } else {
+        const int row0 = warp / n_cb * 16;
+        uint64_t acc[4][4];
+        simt_unit_gemm<T, 4>(un, in + (row0 + rg) * ldi, ldi, lane, acc);
+        simt_unit_finish<T, 4>(un, bias, act, last, part_w, row0, valid, out, ldh, lane, acc);
       }
     }
-    const float b = ldf(w.b2 + j);
-    const int part = j / part_w;
-#pragma unroll
-    for (int r = 0; r < RPG; ++r) {
-      float u = apply_act(acc[r] + b, pd.act_out);
-      Fs[(r0 + r) * pd.Dp + j] = (r0 + r) < valid ? poly_power(u, part) : 0.f;
-    }
+    in = out;
+    ldi = ldh;
+    out = out == h0 ? h1 : h0;
   }
-  __syncthreads();
+  return const_cast<float*>(in);
 }
 
-// Loads rows [tok0, tok0+TM) x [0, ncol) of one head into smem as floats (zero beyond tok_end).
-template <typename T>
-__device__ void load_rows_simt(float* dst, const T* base, long long stride_n, int tok0, int tok_end,
-                               int ncol) {
-  const int per_row = ncol / 4;
-  for (int idx = threadIdx.x; idx < SIMT_TM * per_row; idx += blockDim.x) {
-    const int r = idx / per_row, c = (idx % per_row) * 4;
+// Loads rows [tok0, tok0+TM) x [0, D) of one head into shared memory as floats (row stride ld), zero beyond tok_end:
+// fp32 by cp.async (complete after the caller's next wait), bf16 converted on the way.
+template <int D>
+__device__ __forceinline__ void load_rows_simt(float* dst, int ld, const float* base, long long stride_n, int tok0, int tok_end) {
+#pragma unroll
+  for (int idx = threadIdx.x; idx < SIMT_TM * (D / 4); idx += SIMT_THREADS) {
+    const int r = idx / (D / 4), c = (idx % (D / 4)) * 4;
+    const bool ok = tok0 + r < tok_end;
+    cp_async16(ptx::smem_u32(dst + r * ld + c), base + (ok ? (long long)(tok0 + r) * stride_n + c : 0), ok);
+  }
+}
+template <int D>
+__device__ __forceinline__ void load_rows_simt(float* dst, int ld, const __nv_bfloat16* base, long long stride_n, int tok0, int tok_end) {
+#pragma unroll
+  for (int idx = threadIdx.x; idx < SIMT_TM * (D / 4); idx += SIMT_THREADS) {
+    const int r = idx / (D / 4), c = (idx % (D / 4)) * 4;
     float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
     if (tok0 + r < tok_end) x = ld4(base + (long long)(tok0 + r) * stride_n + c);
-    *reinterpret_cast<float4*>(dst + r * ncol + c) = x;
+    *reinterpret_cast<float4*>(dst + r * ld + c) = x;
   }
 }
 
-// grid (n_split, G, BH), SIMT_PHI_THREADS threads, dynamic smem TM*(2d + Dp) + phi_hidden_floats floats.
+// grid (n_split, G, BH), SIMT_THREADS threads, dynamic smem simt_phi_smem(.., true).
 // Chunk t = t0 + blockIdx.y admits the keys [lo_{t-1}, lo_t) into the state (Eq. 17-18: only the
 // newly admitted tokens).  Split s takes a contiguous share of them and writes
 // partial[blockIdx.y][s][bh] = sum_j phi_k(k_j) [v_j | 1]  as [Dp][SD] floats, SD = d + 4,
 // column d holding the z part.
 template <typename T, int D>
-__global__ void __launch_bounds__(SIMT_PHI_THREADS)
+__global__ void __launch_bounds__(SIMT_THREADS)
 state_partial_simt(const T* __restrict__ k, const T* __restrict__ v, PhiPtrs<T> wk, PhiDims pd, Geo g,
                    int n_split, float* __restrict__ partial) {
   extern __shared__ __align__(16) float smem[];
   constexpr int SD = D + 4;
+  const int ldh = simt_act_ld(pd.Dh, pd.Dp);
   float* Xs = smem;
-  float* Vs = Xs + SIMT_TM * D;
-  float* Hs = Vs + SIMT_TM * D;
-  float* Fs = Hs + phi_hidden_floats(pd.Dh, pd.n_mid);
+  float* Vs = Xs + SIMT_TM * (D + 4);
+  float* h0 = Vs + SIMT_TM * D;
+  float* h1 = h0 + SIMT_TM * ldh;
+  uint8_t* slabs = reinterpret_cast<uint8_t*>(h1 + SIMT_TM * ldh);
 
   const int s = blockIdx.x, ci = blockIdx.y, bh = blockIdx.z, t = g.t0 + ci;
-  const int head = bh % g.n_heads;
+  const int head = bh % g.n_heads, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int lo_prev = t > 0 ? geo_lo(g, t - 1) : 0, lo = geo_lo(g, t);
   const int len = lo - lo_prev;
   int per = (len + n_split - 1) / n_split;
@@ -154,41 +272,71 @@ state_partial_simt(const T* __restrict__ k, const T* __restrict__ v, PhiPtrs<T> 
                   pd.n_mid ? wk.bm + (size_t)head * pd.n_mid * pd.Dh : nullptr};
   const long long hoff = head_offset(g, bh);
 
-  // thread -> (feature f, half of the value columns)
-  const int f = threadIdx.x % 256, half = threadIdx.x / 256;
-  constexpr int HC = D / 2;
-  float acc[HC];
+  // The sums stay in registers over the CTA's tokens.  A warp owns blocks of FT*4 features, a lane FT features of each
+  // (consecutive) and the columns (lane%8)*4 + 32 q: 128 sums a lane, whatever D.
+  constexpr int FT = D / 16, NB = 128 / D, NQ = D / 32;
+  const int fg = lane >> 3, cg = lane & 7;
+  uint64_t acc[NB][FT][NQ * 2];
   float zacc = 0.f;
 #pragma unroll
-  for (int c = 0; c < HC; ++c) acc[c] = 0.f;
-
-  for (int tok0 = a; tok0 < b; tok0 += SIMT_TM) {
-    load_rows_simt(Xs, k + hoff, g.stride_n, tok0, b, D);
-    load_rows_simt(Vs, v + hoff, g.stride_n, tok0, b, D);
-    __syncthreads();
-    phi_tile_simt(Xs, Hs, Fs, w, pd, b - tok0);
-    if (f < pd.Dp) {
-      for (int r = 0; r < SIMT_TM; ++r) {
-        const float fv = Fs[r * pd.Dp + f];
-        zacc += fv;
-        const float* vr = Vs + r * D + half * HC;
+  for (int n = 0; n < NB; ++n)
 #pragma unroll
-        for (int c = 0; c < HC; c += 4) {
-          float4 x = *reinterpret_cast<const float4*>(vr + c);
-          acc[c] = fmaf(fv, x.x, acc[c]); acc[c + 1] = fmaf(fv, x.y, acc[c + 1]);
-          acc[c + 2] = fmaf(fv, x.z, acc[c + 2]); acc[c + 3] = fmaf(fv, x.w, acc[c + 3]);
+    for (int u = 0; u < FT; ++u)
+#pragma unroll
+      for (int q = 0; q < NQ * 2; ++q) acc[n][u][q] = 0ull;
+
+  if (a < b) {
+    load_rows_simt<D>(Xs, D + 4, k + hoff, g.stride_n, a, b);
+    load_rows_simt<D>(Vs, D, v + hoff, g.stride_n, a, b);
+    cp_async_commit();
+  }
+#pragma unroll 1
+  for (int tok0 = a; tok0 < b; tok0 += SIMT_TM) {
+    const float* F = phi_tile_simt<T>(Xs, h0, h1, ldh, slabs, w, pd, b - tok0, [&]() {
+      if (tok0 + SIMT_TM < b) load_rows_simt<D>(Xs, D + 4, k + hoff, g.stride_n, tok0 + SIMT_TM, b);
+    });
+    __syncthreads();
+    if (threadIdx.x < pd.Dp)
+#pragma unroll 8
+      for (int r = 0; r < SIMT_TM; ++r) zacc += F[r * ldh + threadIdx.x];
+#pragma unroll
+    for (int n = 0; n < NB; ++n) {
+      const int f0 = (warp + 8 * n) * (FT * 4);
+      if (f0 >= pd.Dp) continue;                       // the same for the whole warp
+      const float* fp = F + f0 + fg * FT;
+#pragma unroll 2
+      for (int r = 0; r < SIMT_TM; ++r) {
+        uint64_t vv[NQ * 2], ff[FT];
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) ld_pairs(Vs + r * D + cg * 4 + 32 * q, vv[2 * q], vv[2 * q + 1]);
+#pragma unroll
+        for (int u = 0; u < FT; u += 4) {
+          const float4 f4 = *reinterpret_cast<const float4*>(fp + r * ldh + u);
+          ff[u] = ptx::pk2(f4.x, f4.x); ff[u + 1] = ptx::pk2(f4.y, f4.y);
+          ff[u + 2] = ptx::pk2(f4.z, f4.z); ff[u + 3] = ptx::pk2(f4.w, f4.w);
         }
+#pragma unroll
+        for (int u = 0; u < FT; ++u)
+#pragma unroll
+          for (int q = 0; q < NQ * 2; ++q) acc[n][u][q] = ptx::fma2(ff[u], vv[q], acc[n][u][q]);
       }
     }
     __syncthreads();
+    if (tok0 + SIMT_TM < b) load_rows_simt<D>(Vs, D, v + hoff, g.stride_n, tok0 + SIMT_TM, b);
+    cp_async_commit();
   }
-  if (f < pd.Dp) {
-    float* dst = partial + (((size_t)ci * n_split + s) * g.BH + bh) * pd.Dp * SD + (size_t)f * SD;
+  float* dst = partial + (((size_t)ci * n_split + s) * g.BH + bh) * pd.Dp * SD;
 #pragma unroll
-    for (int c = 0; c < HC; c += 4)
-      *reinterpret_cast<float4*>(dst + half * HC + c) = make_float4(acc[c], acc[c + 1], acc[c + 2], acc[c + 3]);
-    if (half == 1) *reinterpret_cast<float4*>(dst + D) = make_float4(zacc, 0.f, 0.f, 0.f);
-  }
+  for (int n = 0; n < NB; ++n)
+#pragma unroll
+    for (int u = 0; u < FT; ++u) {
+      const int f = (warp + 8 * n) * (FT * 4) + fg * FT + u;
+      if (f >= pd.Dp) continue;
+#pragma unroll
+      for (int q = 0; q < NQ; ++q)
+        *reinterpret_cast<ulonglong2*>(dst + (size_t)f * SD + cg * 4 + 32 * q) = make_ulonglong2(acc[n][u][2 * q], acc[n][u][2 * q + 1]);
+    }
+  if (threadIdx.x < pd.Dp) *reinterpret_cast<float4*>(dst + (size_t)threadIdx.x * SD + D) = make_float4(zacc, 0.f, 0.f, 0.f);
 }
 
 // state[i] = carry + sum_{u<=i} sum_s partial[u][s]   for the G chunks of the group, where carry
@@ -232,69 +380,138 @@ __global__ void combine_bidirectional(const float* __restrict__ cum, float* __re
   }
 }
 
-// grid (tiles per chunk, G, BH), SIMT_PHI_THREADS threads.  Linear read-out of one tile of
-// SIMT_TM queries of chunk t: rd[bh][row in group][0..d) = phi_q(q_i) s_t, [d] = phi_q(q_i) z_t, in the fp32
-// layout of rd_index or (rd_half, for the tensor-core window kernels) as fp16 ratios in the layout of rdh_index.
+// grid (CTAs per chunk, G, BH), SIMT_THREADS threads, dynamic smem simt_phi_smem(.., false).  Linear read-out of
+// `tiles_per_cta` tiles of SIMT_TM queries of chunk t: rd[bh][row in group][0..d) = phi_q(q_i) s_t,
+// [d] = phi_q(q_i) z_t, in the fp32 layout of rd_index or (rd_half, for the tensor-core window kernels) as fp16 ratios
+// in the layout of rdh_index.
 template <typename T, int D>
-__global__ void __launch_bounds__(SIMT_PHI_THREADS)
+__global__ void __launch_bounds__(SIMT_THREADS)
 readout_simt(const T* __restrict__ q, PhiPtrs<T> wq, PhiDims pd, Geo g, const float* __restrict__ state,
-             float* __restrict__ rd, int rd_rows, int rd_half) {
+             float* __restrict__ rd, int rd_rows, int rd_half, int tiles_per_cta) {
   extern __shared__ __align__(16) float smem[];
   constexpr int SD = D + 4;
+  const int ldh = simt_act_ld(pd.Dh, pd.Dp);
   float* Xs = smem;
-  float* Hs = Xs + SIMT_TM * D;
-  float* Fs = Hs + phi_hidden_floats(pd.Dh, pd.n_mid);
+  float* h0 = Xs + SIMT_TM * (D + 4);
+  float* h1 = h0 + SIMT_TM * ldh;
+  float* nl_s = h1 + SIMT_TM * ldh;                    // phi_q(q_i) z_t of the tile's rows
+  uint8_t* slabs = reinterpret_cast<uint8_t*>(nl_s + SIMT_TM);
 
-  const int ci = blockIdx.y, bh = blockIdx.z, t = g.t0 + ci;
+  const int ci = blockIdx.y, bh = blockIdx.z, t = g.t0 + ci, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (!geo_linear(g, t)) return;                       // empty linear set: nothing to read out
   const int q0 = geo_q0(g, t), q1 = geo_q1(g, t);
-  const int tok0 = q0 + blockIdx.x * SIMT_TM;
-  if (tok0 >= q1) return;
+  const int a = q0 + (int)blockIdx.x * tiles_per_cta * SIMT_TM, b = min(a + tiles_per_cta * SIMT_TM, q1);
+  if (a >= b) return;
   const int head = bh % g.n_heads;
   PhiPtrs<T> w = {wq.W1 + (size_t)head * pd.Dh * D, wq.b1 + (size_t)head * pd.Dh,
                   wq.W2 + (size_t)head * pd.Dp * pd.Dh, wq.b2 + (size_t)head * pd.Dp,
                   pd.n_mid ? wq.Wm + (size_t)head * pd.n_mid * pd.Dh * pd.Dh : nullptr,
                   pd.n_mid ? wq.bm + (size_t)head * pd.n_mid * pd.Dh : nullptr};
-  load_rows_simt(Xs, q + q_row_offset(g, bh, 0), g.qstride_n, tok0, q1, D);
-  __syncthreads();
-  phi_tile_simt(Xs, Hs, Fs, w, pd, q1 - tok0);
-
+  const T* qh = q + q_row_offset(g, bh, 0);
   const float* S = state + ((size_t)ci * g.BH + bh) * pd.Dp * SD;
-  constexpr int RG = 4, RPG = SIMT_TM / RG;
-  float* nl_s = Xs;                                    // phi_q(q_i) z_t of the tile's rows (Xs is no longer needed)
-  if (rd_half) {
-    // the tensor-core window kernels read the ratio aL / nL (see rdh_index): the denominators come first
-    for (int r = threadIdx.x; r < SIMT_TM; r += blockDim.x) {
-      float acc = 0.f;
-      for (int ff = 0; ff < pd.Dp; ++ff) acc = fmaf(Fs[r * pd.Dp + ff], S[(size_t)ff * SD + D], acc);
-      nl_s[r] = acc;
-      if (tok0 + r < q1) rd[rdh_index(g, rd_rows, D, bh, ci, tok0 + r - q0, rdh_pieces(D) - 1) * 4] = acc;
+
+  // phi s_t: a warp has 32 columns and TM * (D/32) / 8 rows, a lane four consecutive columns of RR rows
+  constexpr int NCB = D / 32, RR = D / 32;
+  const int rg = lane >> 3, cg = lane & 7, cb = warp % NCB, row0 = warp / NCB * (4 * RR);
+  uint8_t* const slab_ptr = slabs + warp * SIMT_STAGES * SIMT_SLAB;
+  const uint32_t slab = ptx::smem_u32(slab_ptr);
+  auto issue_state = [&](int s) {                      // features [16 s, 16 s + 16) x 32 columns, rows of 128 bytes
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int c = lane + 32 * u, f = s * 16 + (c >> 3);
+      cp_async16(slab + (s % SIMT_STAGES) * SIMT_SLAB + c * 16, S + (size_t)(f < pd.Dp ? f : 0) * SD + cb * 32 + (c & 7) * 4, f < pd.Dp);
     }
+    cp_async_commit();
+  };
+
+  load_rows_simt<D>(Xs, D + 4, qh, g.qstride_n, a, b);
+  cp_async_commit();
+#pragma unroll 1
+  for (int tok0 = a; tok0 < b; tok0 += SIMT_TM) {
+    const float* F = phi_tile_simt<T>(Xs, h0, h1, ldh, slabs, w, pd, b - tok0, [&]() {
+      if (tok0 + SIMT_TM < b) load_rows_simt<D>(Xs, D + 4, qh, g.qstride_n, tok0 + SIMT_TM, b);
+    });
+    __syncwarp();                                      // the warp's slabs are free
+#pragma unroll
+    for (int s = 0; s < SIMT_STAGES - 1; ++s) issue_state(s);
     __syncthreads();
-  }
-  const int ncol = rd_half ? D : D + 1;
-  for (int idx = threadIdx.x; idx < ncol * RG; idx += blockDim.x) {
-    const int c = idx % ncol, r0 = (idx / ncol) * RPG;
-    float acc[RPG];
+    // nL of the warp's four rows, the lanes sharing the features
+    {
+      constexpr int RW = SIMT_TM / (SIMT_THREADS / 32);
+      float nl[RW] = {};
+      for (int f = lane; f < pd.Dp; f += 32) {
+        const float z = S[(size_t)f * SD + D];
 #pragma unroll
-    for (int r = 0; r < RPG; ++r) acc[r] = 0.f;
-    for (int ff = 0; ff < pd.Dp; ++ff) {
-      const float sv = S[(size_t)ff * SD + c];
+        for (int r = 0; r < RW; ++r) nl[r] = fmaf(F[(warp * RW + r) * ldh + f], z, nl[r]);
+      }
 #pragma unroll
-      for (int r = 0; r < RPG; ++r) acc[r] = fmaf(Fs[(r0 + r) * pd.Dp + ff], sv, acc[r]);
-    }
+      for (int r = 0; r < RW; ++r) {
 #pragma unroll
-    for (int r = 0; r < RPG; ++r) {
-      const int tok = tok0 + r0 + r;
-      if (tok >= q1) continue;
-      if (!rd_half) {
-        rd[rd_index(g, rd_rows, D, bh, ci, tok - q0, c >> 2) + (c & 3)] = acc[r];
-      } else {
-        const float nl = nl_s[r0 + r], ratio = nl != 0.f ? acc[r] / nl : 0.f;
-        reinterpret_cast<__half*>(rd)[rdh_index(g, rd_rows, D, bh, ci, tok - q0, c >> 3) * 8 + (c & 7)] =
-            __float2half_rn(fminf(fmaxf(ratio, -65504.f), 65504.f));
+        for (int o = 16; o; o >>= 1) nl[r] += __shfl_xor_sync(0xffffffffu, nl[r], o);
+        if (lane == r) {
+          const int tok = tok0 + warp * RW + r;
+          nl_s[warp * RW + r] = nl[r];
+          if (tok < b) {
+            if (rd_half) rd[rdh_index(g, rd_rows, D, bh, ci, tok - q0, rdh_pieces(D) - 1) * 4] = nl[r];
+            else rd[rd_index(g, rd_rows, D, bh, ci, tok - q0, D / 4)] = nl[r];
+          }
+        }
       }
     }
+    uint64_t acc[RR][2];
+#pragma unroll
+    for (int i = 0; i < RR; ++i) acc[i][0] = acc[i][1] = 0ull;
+    const float* fr = F + (row0 + rg) * ldh;
+    const int n_slab = (pd.Dp + 15) / 16;
+#pragma unroll 1
+    for (int s = 0; s < n_slab; ++s) {
+      cp_async_wait<SIMT_STAGES - 2>();
+      __syncwarp();
+      issue_state(s + SIMT_STAGES - 1);
+      const float* sp = reinterpret_cast<const float*>(slab_ptr + (s % SIMT_STAGES) * SIMT_SLAB) + cg * 4;
+#pragma unroll 1
+      for (int k0 = 0; k0 < 16 && s * 16 + k0 < pd.Dp; k0 += 8) {
+#pragma unroll
+        for (int h = 0; h < 8; h += 4) {
+          float4 f4[RR];
+#pragma unroll
+          for (int i = 0; i < RR; ++i) f4[i] = *reinterpret_cast<const float4*>(fr + i * 4 * ldh + s * 16 + k0 + h);
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            uint64_t s0, s1;
+            ld_pairs(sp + (k0 + h + e) * 32, s0, s1);
+#pragma unroll
+            for (int i = 0; i < RR; ++i) {
+              const float x = e == 0 ? f4[i].x : e == 1 ? f4[i].y : e == 2 ? f4[i].z : f4[i].w;
+              acc[i][0] = ptx::fma2(ptx::pk2(x, x), s0, acc[i][0]);
+              acc[i][1] = ptx::fma2(ptx::pk2(x, x), s1, acc[i][1]);
+            }
+          }
+        }
+      }
+    }
+    if (rd_half) __syncthreads();                      // nl_s
+    const int c0 = cb * 32 + cg * 4;
+#pragma unroll
+    for (int i = 0; i < RR; ++i) {
+      const int r = row0 + rg + 4 * i, tok = tok0 + r;
+      if (tok >= b) continue;
+      float y[4];
+      ptx::upk2(acc[i][0], y[0], y[1]);
+      ptx::upk2(acc[i][1], y[2], y[3]);
+      if (!rd_half) {
+        *reinterpret_cast<float4*>(rd + rd_index(g, rd_rows, D, bh, ci, tok - q0, c0 >> 2)) = make_float4(y[0], y[1], y[2], y[3]);
+      } else {
+        // the tensor-core window kernels read the ratio aL / nL (see rdh_index)
+        const float nl = nl_s[r];
+        uint2 h2;
+        __half* h = reinterpret_cast<__half*>(&h2);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) h[e] = __float2half_rn(fminf(fmaxf(nl != 0.f ? y[e] / nl : 0.f, -65504.f), 65504.f));
+        *reinterpret_cast<uint2*>(reinterpret_cast<__half*>(rd) + rdh_index(g, rd_rows, D, bh, ci, tok - q0, c0 >> 3) * 8 + (c0 & 7)) = h2;
+      }
+    }
+    __syncwarp();                                      // the slabs may be refilled; buffers: barriers of the next phi_tile
   }
 }
 
@@ -390,117 +607,198 @@ qk_prepare(const T* __restrict__ q, const T* __restrict__ k, T* __restrict__ qo,
   }
 }
 
-// grid (tiles per chunk of WIN_BM rows, G, BH), 128 threads.  Softmax window of Eq. 6 and 8 with a
-// running row maximum, then the joint normalisation of Eq. 5 with the linear read-out `rd`.
-constexpr int WIN_BM = 32, WIN_BN = 64, WIN_THREADS = 128;
+// Softmax window of Eq. 6 and 8 with a running row maximum, then the joint normalisation of Eq. 5 with the linear
+// read-out `rd`.  grid (tiles per chunk of BM rows, G, BH), SIMT_THREADS threads.
+// A warp has 16 query rows and 1/WK of the keys of every key tile (BM = 128 / WK rows per CTA); the WK warps of the same
+// rows keep maxima and sums of their own and are merged at the end.  WK = 1 needs the fewest loads per multiply-add,
+// WK = 4 gives a short sequence four times as many CTAs (window_simt_split chooses).  Per key tile two barriers: V is
+// copied in while Q K^T runs, the next K while P V runs.
+template <typename T, int D, int WK>
+struct WinSimt {
+  static constexpr int BM = 128 / WK, BN = WK == 1 ? 64 : 128, KJ = BN / WK / 8;     // KJ: keys per lane and tile
+  static constexpr int LDQ = D + 4, LDK = D + 16 / (int)sizeof(T), LDP = BN / WK + 4;
+  static constexpr int Q_BYTES = BM * LDQ * 4, K_BYTES = BN * LDK * (int)sizeof(T), V_BYTES = BN * D * (int)sizeof(T);
+  static constexpr int P_BYTES = SIMT_THREADS / 32 * 16 * LDP * 4;
+  static constexpr int KV_BYTES = K_BYTES + V_BYTES;
+  // merging: (WK - 1) * 2 warps leave D/2 sums and 8 statistics per lane where K and V were
+  static constexpr int M_BYTES = WK == 1 ? 0 : (WK - 1) * (8 / WK) * 32 * (D / 2 + 8) * 4;
+  static constexpr int SMEM = Q_BYTES + P_BYTES + (KV_BYTES > M_BYTES ? KV_BYTES : M_BYTES);
+};
 
-template <typename T, int D>
-__global__ void __launch_bounds__(WIN_THREADS)
+template <typename T, int D, int WK>
+__global__ void __launch_bounds__(SIMT_THREADS)
 window_simt(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v, T* __restrict__ out,
             Geo g, const float* __restrict__ rd, int rd_rows, float scale, int c_mode, float* __restrict__ share) {
+  using S = WinSimt<T, D, WK>;
   extern __shared__ __align__(16) float smem[];
-  constexpr int LDK = D + 4, LDP = WIN_BN + 4;
-  constexpr int DC = D / 16;                 // output columns per thread
-  float* Qs = smem;                          // [BM][LDK]
-  float* Ks = Qs + WIN_BM * LDK;             // [BN][LDK]
-  float* Vs = Ks + WIN_BN * LDK;             // [BN][D]
-  float* Ps = Vs + WIN_BN * D;               // [BM][LDP]
+  constexpr int KJ = S::KJ, NQ = D / 32, RGS = 8 / WK;          // RGS: row groups of 16 per CTA
+  float* Qs = smem;                                             // [BM][LDQ]
+  float* Ps = Qs + S::BM * S::LDQ;                              // [8 warps][16][LDP]
+  T* Ks = reinterpret_cast<T*>(Ps + S::P_BYTES / 4);            // [BN][LDK]
+  T* Vs = Ks + S::BN * S::LDK;                                  // [BN][D]
 
   const int ci = blockIdx.y, bh = blockIdx.z, t = g.t0 + ci;
   const int q0 = geo_q0(g, t), q1 = geo_q1(g, t), lo = geo_lo(g, t), hi = q1;
   const bool linear = geo_linear(g, t);
-  const int row0 = q0 + blockIdx.x * WIN_BM;
+  const int row0 = q0 + blockIdx.x * S::BM;
   if (row0 >= q1) return;
   const long long hoff = head_offset(g, bh);
-  const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, rg = lane >> 3, cg = lane & 7;
+  const int wr = warp % RGS, wk = warp / RGS;                   // row group, key group
 
-  for (int idx = tid; idx < WIN_BM * (D / 4); idx += WIN_THREADS) {
+  auto load_tile = [&](T* dst, int ld, const T* base, int j0) { // BN keys from j0 on, zeros beyond the window
+    constexpr int PER = 16 / (int)sizeof(T), CH = D / PER;
+#pragma unroll 4
+    for (int idx = tid; idx < S::BN * CH; idx += SIMT_THREADS) {
+      const int r = idx / CH, c = (idx % CH) * PER;
+      const bool ok = j0 + r < hi;
+      cp_async16(ptx::smem_u32(dst + r * ld + c), base + hoff + (ok ? (long long)(j0 + r) * g.stride_n + c : 0), ok);
+    }
+    cp_async_commit();
+  };
+  load_tile(Ks, S::LDK, k, lo);
+  for (int idx = tid; idx < S::BM * (D / 4); idx += SIMT_THREADS) {
     const int r = idx / (D / 4), c = (idx % (D / 4)) * 4;
     float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
     if (row0 + r < q1) x = ld4(q + q_row_offset(g, bh, row0 + r) + c);
-    *reinterpret_cast<float4*>(Qs + r * LDK + c) = x;
+    *reinterpret_cast<float4*>(Qs + r * S::LDQ + c) = x;
   }
 
-  float m[4], l[4], acc[4][DC];
+  // lane: rows wr*16 + rg + 4 i; keys cg + 8 jj of the warp's share of a tile; output columns cg*4 + 32 n
+  float m[4], l[4];
+  uint64_t acc[4][NQ * 2];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     m[i] = -INFINITY; l[i] = 0.f;
 #pragma unroll
-    for (int c = 0; c < DC; ++c) acc[i][c] = 0.f;
+    for (int c = 0; c < NQ * 2; ++c) acc[i][c] = 0ull;
   }
+  const float* qp = Qs + (wr * 16 + rg) * S::LDQ;
+  const T* kp = Ks + (wk * (S::BN / WK) + cg) * S::LDK;
+  const T* vp = Vs + wk * (S::BN / WK) * D + cg * 4;
+  float* pw = Ps + (warp * 16 + rg) * S::LDP;
 
-  for (int j0 = lo; j0 < hi; j0 += WIN_BN) {
-    __syncthreads();
-    for (int idx = tid; idx < WIN_BN * (D / 4); idx += WIN_THREADS) {
-      const int r = idx / (D / 4), c = (idx % (D / 4)) * 4;
-      float4 kk = make_float4(0.f, 0.f, 0.f, 0.f), vv = kk;
-      if (j0 + r < hi) {
-        kk = ld4(k + hoff + (long long)(j0 + r) * g.stride_n + c);
-        vv = ld4(v + hoff + (long long)(j0 + r) * g.stride_n + c);
-      }
-      *reinterpret_cast<float4*>(Ks + r * LDK + c) = kk;
-      *reinterpret_cast<float4*>(Vs + r * D + c) = vv;
-    }
-    __syncthreads();
-    // scaled logits of rows ty*4+i, columns tx + 16*jj
-    float sv[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int jj = 0; jj < 4; ++jj) sv[i][jj] = 0.f;
-    for (int kk = 0; kk < D; kk += 4) {
-      float4 qa[4], kb[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) qa[i] = *reinterpret_cast<const float4*>(Qs + (ty * 4 + i) * LDK + kk);
-#pragma unroll
-      for (int jj = 0; jj < 4; ++jj) kb[jj] = *reinterpret_cast<const float4*>(Ks + (tx + 16 * jj) * LDK + kk);
+#pragma unroll 1
+  for (int j0 = lo; j0 < hi; j0 += S::BN) {
+    cp_async_wait<0>();
+    __syncthreads();                                            // K is there; V of the tile before has been read
+    load_tile(Vs, D, v, j0);
+    const int n_here = hi - (j0 + wk * (S::BN / WK));           // keys of the window in this warp's share (<= 0: none)
+    if (n_here > 0) {
+      uint64_t s2[4][KJ];
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int jj = 0; jj < 4; ++jj) {
-          sv[i][jj] = fmaf(qa[i].x, kb[jj].x, sv[i][jj]); sv[i][jj] = fmaf(qa[i].y, kb[jj].y, sv[i][jj]);
-          sv[i][jj] = fmaf(qa[i].z, kb[jj].z, sv[i][jj]); sv[i][jj] = fmaf(qa[i].w, kb[jj].w, sv[i][jj]);
+        for (int jj = 0; jj < KJ; ++jj) s2[i][jj] = 0ull;
+#pragma unroll 2
+      for (int kk = 0; kk < D; kk += 4) {
+        uint64_t qa[4], qb[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) ld_pairs(qp + i * 4 * S::LDQ + kk, qa[i], qb[i]);
+#pragma unroll
+        for (int jj = 0; jj < KJ; ++jj) {
+          uint64_t ka, kb;
+          ld_pairs(kp + jj * 8 * S::LDK + kk, ka, kb);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            s2[i][jj] = ptx::fma2(qa[i], ka, s2[i][jj]);
+            s2[i][jj] = ptx::fma2(qb[i], kb, s2[i][jj]);
+          }
         }
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      float tmax = -INFINITY;
-#pragma unroll
-      for (int jj = 0; jj < 4; ++jj) {
-        sv[i][jj] = (j0 + tx + 16 * jj < hi) ? sv[i][jj] * scale : -INFINITY;
-        tmax = fmaxf(tmax, sv[i][jj]);
-      }
-#pragma unroll
-      for (int o = 1; o < 16; o <<= 1) tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, o));
-      const float m_new = fmaxf(m[i], tmax);          // finite: every tile has a valid column
-      const float alpha = expf(m[i] - m_new);         // exp(-inf) = 0 on the first tile
-      float psum = 0.f;
-#pragma unroll
-      for (int jj = 0; jj < 4; ++jj) {
-        const float p = expf(sv[i][jj] - m_new);
-        psum += p;
-        Ps[(ty * 4 + i) * LDP + tx + 16 * jj] = p;
-      }
-#pragma unroll
-      for (int o = 1; o < 16; o <<= 1) psum += __shfl_xor_sync(0xffffffffu, psum, o);
-      l[i] = l[i] * alpha + psum;
-      m[i] = m_new;
-#pragma unroll
-      for (int c = 0; c < DC; ++c) acc[i][c] *= alpha;
-    }
-    __syncthreads();
-    for (int j = 0; j < WIN_BN; ++j) {
-      float vv[DC];
-#pragma unroll
-      for (int c = 0; c < DC; c += 4) {
-        float4 x = *reinterpret_cast<const float4*>(Vs + j * D + tx * DC + c);
-        vv[c] = x.x; vv[c + 1] = x.y; vv[c + 2] = x.z; vv[c + 3] = x.w;
       }
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const float p = Ps[(ty * 4 + i) * LDP + j];
+        float sv[KJ], tmax = -INFINITY;
 #pragma unroll
-        for (int c = 0; c < DC; ++c) acc[i][c] = fmaf(p, vv[c], acc[i][c]);
+        for (int jj = 0; jj < KJ; ++jj) {
+          sv[jj] = cg + 8 * jj < n_here ? pair_sum(s2[i][jj]) * scale : -INFINITY;
+          tmax = fmaxf(tmax, sv[jj]);
+        }
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, o));
+        const float m_new = fmaxf(m[i], tmax);                  // finite: the share has a valid key
+        const float alpha = expf(m[i] - m_new);                 // exp(-inf) = 0 on the first tile
+        float psum = 0.f;
+#pragma unroll
+        for (int jj = 0; jj < KJ; ++jj) {
+          const float p = expf(sv[jj] - m_new);
+          psum += p;
+          pw[i * 4 * S::LDP + cg + 8 * jj] = p;
+        }
+        l[i] = l[i] * alpha + psum;                             // of this lane's keys; added over the lanes at the end
+        m[i] = m_new;
+        const uint64_t a2 = ptx::pk2(alpha, alpha);
+#pragma unroll
+        for (int c = 0; c < NQ * 2; ++c) acc[i][c] = ptx::mul2(acc[i][c], a2);
+      }
+    }
+    cp_async_wait<0>();
+    __syncthreads();                                            // V is there, P of the warp too; K has been read
+    if (j0 + S::BN < hi) load_tile(Ks, S::LDK, k, j0 + S::BN);
+    if (n_here > 0) {
+#pragma unroll 1
+      for (int j = 0; j < S::BN / WK; j += 4) {
+        float4 p4[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) p4[i] = *reinterpret_cast<const float4*>(pw + i * 4 * S::LDP + j);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          uint64_t pp[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float x = e == 0 ? p4[i].x : e == 1 ? p4[i].y : e == 2 ? p4[i].z : p4[i].w;
+            pp[i] = ptx::pk2(x, x);
+          }
+#pragma unroll
+          for (int n = 0; n < NQ; ++n) {
+            uint64_t va, vb;
+            ld_pairs(vp + (j + e) * D + 32 * n, va, vb);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              acc[i][2 * n] = ptx::fma2(pp[i], va, acc[i][2 * n]);
+              acc[i][2 * n + 1] = ptx::fma2(pp[i], vb, acc[i][2 * n + 1]);
+            }
+          }
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) l[i] += __shfl_xor_sync(0xffffffffu, l[i], o);
+
+  if constexpr (WK > 1) {
+    // warps of key group 0 merge the others' sums; a group whose share of every tile was empty has m = -inf, l = 0
+    uint64_t* mo = reinterpret_cast<uint64_t*>(Ks);             // [(WK-1) * RGS][D/4][32]
+    float* ms = reinterpret_cast<float*>(mo + (WK - 1) * RGS * (D / 4) * 32);   // [(WK-1) * RGS][8][32]
+    __syncthreads();
+    if (wk > 0) {
+      const int w = (wk - 1) * RGS + wr;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        ms[(w * 8 + i) * 32 + lane] = m[i];
+        ms[(w * 8 + 4 + i) * 32 + lane] = l[i];
+#pragma unroll
+        for (int c = 0; c < NQ * 2; ++c) mo[(w * (D / 4) + i * NQ * 2 + c) * 32 + lane] = acc[i][c];
+      }
+    }
+    __syncthreads();
+    if (wk > 0) return;
+#pragma unroll 1
+    for (int o = 0; o < WK - 1; ++o) {
+      const int w = o * RGS + wr;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float mo_i = ms[(w * 8 + i) * 32 + lane], lo_i = ms[(w * 8 + 4 + i) * 32 + lane];
+        const float m_new = fmaxf(m[i], mo_i);                  // finite: key group 0 starts with a valid key
+        const float fa = expf(m[i] - m_new), fb = mo_i == -INFINITY && lo_i == 0.f ? 0.f : expf(mo_i - m_new);
+        l[i] = l[i] * fa + lo_i * fb;
+        m[i] = m_new;
+        const uint64_t fa2 = ptx::pk2(fa, fa), fb2 = ptx::pk2(fb, fb);
+#pragma unroll
+        for (int c = 0; c < NQ * 2; ++c)
+          acc[i][c] = ptx::fma2(mo[(w * (D / 4) + i * NQ * 2 + c) * 32 + lane], fb2, ptx::mul2(acc[i][c], fa2));
       }
     }
   }
@@ -510,7 +808,7 @@ window_simt(const T* __restrict__ q, const T* __restrict__ k, const T* __restric
   // branches against r = max(m_i, 0): window * exp(m_i - r), linear * exp(-r).
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const int row = row0 + ty * 4 + i;
+    const int row = row0 + wr * 16 + rg + 4 * i;
     if (row >= q1) continue;
     float ws = 1.f, lam = 0.f, nL = 0.f;
     if (linear) {
@@ -523,12 +821,17 @@ window_simt(const T* __restrict__ q, const T* __restrict__ k, const T* __restric
       nL = rd[rd_index(g, rd_rows, D, bh, ci, row - q0, D / 4)];
     }
     const float inv = 1.f / (l[i] * ws + lam * nL);
-    if (share != nullptr && tx == 0) share[(size_t)bh * g.N + row] = lam * nL * inv;   // part of the normaliser that is linear
-    T* orow = out + out_row_offset(g, bh, row) + tx * DC;
+    if (share != nullptr && cg == 0) share[(size_t)bh * g.N + row] = lam * nL * inv;   // part of the normaliser that is linear
+    T* orow = out + out_row_offset(g, bh, row) + cg * 4;
 #pragma unroll
-    for (int c = 0; c < DC; ++c) {
-      const float aL = linear ? rd[rd_index(g, rd_rows, D, bh, ci, row - q0, (tx * DC + c) >> 2) + ((tx * DC + c) & 3)] : 0.f;
-      stf(orow + c, (acc[i][c] * ws + lam * aL) * inv);
+    for (int n = 0; n < NQ; ++n) {
+      float4 aL = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (linear) aL = *reinterpret_cast<const float4*>(rd + rd_index(g, rd_rows, D, bh, ci, row - q0, cg + 8 * n));
+      float y[4];
+      ptx::upk2(acc[i][2 * n], y[0], y[1]);
+      ptx::upk2(acc[i][2 * n + 1], y[2], y[3]);
+      st4(orow + 32 * n, (y[0] * ws + lam * aL.x) * inv, (y[1] * ws + lam * aL.y) * inv, (y[2] * ws + lam * aL.z) * inv,
+          (y[3] * ws + lam * aL.w) * inv);
     }
   }
 }

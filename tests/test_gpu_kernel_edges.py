@@ -56,3 +56,18 @@ def test_activations_over_their_whole_range(act_hidden, act_out, P, Dp):
         x[m]["W1"] = (x[m]["W1"].float() * 18).to(torch.bfloat16)
     y = _forward(wl, x, act_hidden=act_hidden, act_out=act_out)
     _gate(y, _oracle(wl, x, act_hidden=act_hidden, act_out=act_out), "bf16")
+
+
+# (dtype, d, heads, T, H, W, Tc, To, D_h, D', P, layers): the CUDA-core kernels.  Chunks that end inside tiles of 32, 64
+# and 128 rows and keys, window shares of a key group that are empty, phi widths that end inside blocks of 8 to 32
+# columns and slabs of 16 or 32, one and both shapes of the window kernel (336 tiles of 128 rows take the wide one).
+@pytest.mark.parametrize("dtype,d,nh,T,H,W,Tc,To,Dh,Dp,P,layers", [
+    ("fp32", 64, 2, 5, 1, 3, 1, 1, 8, 8, 1, 2), ("fp32", 128, 3, 4, 3, 11, 1, 2, 24, 40, 2, 3),
+    ("fp32", 64, 24, 7, 10, 13, 1, 1, 128, 128, 2, 2), ("fp32", 128, 24, 7, 3, 43, 1, 0, 136, 200, 2, 2),
+    ("fp32", 128, 2, 3, 8, 16, 1, 1, 256, 256, 4, 4), ("bf16", 64, 24, 7, 10, 13, 1, 1, 72, 104, 1, 2),
+    ("bf16", 128, 2, 6, 5, 13, 2, 1, 40, 136, 2, 3), ("bf16", 64, 2, 4, 9, 17, 2, 1, 256, 8, 1, 2)])
+def test_cuda_core_kernels(dtype, d, nh, T, H, W, Tc, To, Dh, Dp, P, layers):
+    wl = synth.Workload("simt", 1, nh, d, T, H, W, Tc, To, dtype, dtype == "bf16", P=P, seed=synth.BASE_SEED + 402, phi_hidden=Dh,
+                        phi_dim=Dp, phi_layers=layers)
+    x = synth.make_inputs(wl, v_frame_offsets=True)
+    _gate(_forward(wl, x, impl="simt"), _oracle(wl, x), dtype)
