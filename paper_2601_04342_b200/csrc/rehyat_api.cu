@@ -186,9 +186,11 @@ int busy_readout(const Geo& g) {
   return busy > 0 ? busy : 1;
 }
 
+unsigned scan_blocks(size_t per_slot) { return (unsigned)((per_slot / 4 + SCAN_THREADS - 1) / SCAN_THREADS); }
+
 template <typename T, int D>
 int launch_group_simt(rehyat_ctx* ctx, const T* q, const T* k, const T* v, T* out, const rehyat_phi_params* phi,
-                      const Geo& g, int n_split, int carry_slot, int parts, cudaStream_t st) {
+                      const Geo& g, int n_split, float* state_out, const float* carry, int parts, cudaStream_t st) {
   const rehyat_config& c = ctx->cfg;
   const int rd_half = ctx->tensor_ok ? 1 : 0;     // the tensor-core window kernels read the bf16 form of the read-out
   PhiDims pd = {D, c.phi_hidden, c.phi_dim, c.poly_degree, c.act_hidden, c.act_out, c.phi_layers > 2 ? c.phi_layers - 2 : 0};
@@ -202,8 +204,7 @@ int launch_group_simt(rehyat_ctx* ctx, const T* q, const T* k, const T* v, T* ou
     ctx->prof.end(REHYAT_PROF_STATE, st);
     const size_t per_slot = (size_t)g.BH * pd.Dp * SD;
     ctx->prof.begin(REHYAT_PROF_SCAN, st);
-    scan_states<<<(unsigned)((per_slot + 255) / 256), 256, 0, st>>>(ctx->partial, ctx->state, per_slot, g.G,
-                                                                     n_split, carry_slot);
+    scan_states<<<scan_blocks(per_slot), SCAN_THREADS, 0, st>>>(ctx->partial, state_out, per_slot, g.G, n_split, carry, nullptr, D);
     ctx->prof.end(REHYAT_PROF_SCAN, st);
     ctx->last_launches += 2;
   }
@@ -240,7 +241,10 @@ int launch_group_simt(rehyat_ctx* ctx, const T* q, const T* k, const T* v, T* ou
 
 // Split of a chunk's state increment over CTAs: one CTA per (split, chunk, head) and one CTA per SM.
 int pick_state_split(const rehyat_ctx* ctx, const Geo& g, int n_chunks_in_group, int tokens_per_increment) {
-  int most = ctx->partial_units / (n_chunks_in_group > 0 ? n_chunks_in_group : 1);
+  // the buffer holds partial_units increments of bh_max problems; a call with fewer of them (one head of
+  // rehyat_forward_host) has room for more splits
+  const long long units = (long long)ctx->partial_units * ctx->bh_max / g.BH;
+  int most = (int)(units / (n_chunks_in_group > 0 ? n_chunks_in_group : 1));
   if (most > 16) most = 16;                         // a lone chunk (a chunk-by-chunk step) over all SMs
   if (most < 1) most = 1;
   const int tile = ctx->tensor_ok && ctx->tc.phi_ok ? 128 : SIMT_TM;
@@ -250,17 +254,19 @@ int pick_state_split(const rehyat_ctx* ctx, const Geo& g, int n_chunks_in_group,
 }
 
 // Enqueues the requested steps for the chunks [g.t0, g.t0 + g.G) with whichever kernel family the context uses.
+// PART_STATE writes the states of the chunks to `state_out` (the context's state slots, or slots of `cum`), starting
+// from `carry` (null: zero).
 int run_parts(rehyat_ctx* ctx, const void* q, const void* k, const void* v, void* out, const rehyat_phi_params* phi,
-              const Geo& g, int batch, int n_split, int carry_slot, int parts, cudaStream_t st) {
+              const Geo& g, int batch, int n_split, float* state_out, const float* carry, int parts, cudaStream_t st) {
   const rehyat_config& c = ctx->cfg;
   int rc = REHYAT_OK;
   if (ctx->tensor_ok) {
     using B = __nv_bfloat16;
     if (!ctx->tc.phi_ok) {
       rc = c.head_dim == 64
-               ? launch_group_simt<B, 64>(ctx, (const B*)q, (const B*)k, (const B*)v, (B*)out, phi, g, n_split, carry_slot,
+               ? launch_group_simt<B, 64>(ctx, (const B*)q, (const B*)k, (const B*)v, (B*)out, phi, g, n_split, state_out, carry,
                                           parts & (PART_STATE | PART_READOUT), st)
-               : launch_group_simt<B, 128>(ctx, (const B*)q, (const B*)k, (const B*)v, (B*)out, phi, g, n_split, carry_slot,
+               : launch_group_simt<B, 128>(ctx, (const B*)q, (const B*)k, (const B*)v, (B*)out, phi, g, n_split, state_out, carry,
                                            parts & (PART_STATE | PART_READOUT), st);
     } else {
       if (parts & PART_STATE) {
@@ -271,8 +277,8 @@ int run_parts(rehyat_ctx* ctx, const void* q, const void* k, const void* v, void
         ctx->prof.end(REHYAT_PROF_STATE, st);
         const size_t per_slot = (size_t)g.BH * c.phi_dim * (c.head_dim + 4);
         ctx->prof.begin(REHYAT_PROF_SCAN, st);
-        scan_states<<<(unsigned)((per_slot + 255) / 256), 256, 0, st>>>(ctx->partial, ctx->state, per_slot, g.G, n_split,
-                                                                         carry_slot, ctx->tc.state_bf16, c.head_dim);
+        scan_states<<<scan_blocks(per_slot), SCAN_THREADS, 0, st>>>(ctx->partial, state_out, per_slot, g.G, n_split, carry,
+                                                                    state_out == ctx->state ? ctx->tc.state_bf16 : nullptr, c.head_dim);
         ctx->prof.end(REHYAT_PROF_SCAN, st);
         ctx->last_launches += 2;
       }
@@ -293,13 +299,13 @@ int run_parts(rehyat_ctx* ctx, const void* q, const void* k, const void* v, void
     }
   } else if (c.dtype == REHYAT_DTYPE_FP32) {
     rc = c.head_dim == 64
-             ? launch_group_simt<float, 64>(ctx, (const float*)q, (const float*)k, (const float*)v, (float*)out, phi, g, n_split, carry_slot, parts, st)
-             : launch_group_simt<float, 128>(ctx, (const float*)q, (const float*)k, (const float*)v, (float*)out, phi, g, n_split, carry_slot, parts, st);
+             ? launch_group_simt<float, 64>(ctx, (const float*)q, (const float*)k, (const float*)v, (float*)out, phi, g, n_split, state_out, carry, parts, st)
+             : launch_group_simt<float, 128>(ctx, (const float*)q, (const float*)k, (const float*)v, (float*)out, phi, g, n_split, state_out, carry, parts, st);
   } else {
     using B = __nv_bfloat16;
     rc = c.head_dim == 64
-             ? launch_group_simt<B, 64>(ctx, (const B*)q, (const B*)k, (const B*)v, (B*)out, phi, g, n_split, carry_slot, parts, st)
-             : launch_group_simt<B, 128>(ctx, (const B*)q, (const B*)k, (const B*)v, (B*)out, phi, g, n_split, carry_slot, parts, st);
+             ? launch_group_simt<B, 64>(ctx, (const B*)q, (const B*)k, (const B*)v, (B*)out, phi, g, n_split, state_out, carry, parts, st)
+             : launch_group_simt<B, 128>(ctx, (const B*)q, (const B*)k, (const B*)v, (B*)out, phi, g, n_split, state_out, carry, parts, st);
   }
   return rc;
 }
@@ -625,44 +631,40 @@ int rehyat_forward(rehyat_ctx* ctx, const void* q, const void* k, const void* v,
   if (c.bidirectional && n_chunks > 1) {
     // Eq. 10-12: the linear set of a chunk is everything outside its window.  Pass 1 sums the state frame by
     // frame (running sums cum[0..frames]); pass 2 forms each chunk's state from three of those sums.
-    const size_t per_slot = (size_t)g.BH * c.phi_dim * (c.head_dim + 4), slot_bytes = per_slot * sizeof(float);
-    if (cudaMemsetAsync(ctx->cum, 0, slot_bytes, st) != cudaSuccess) return REHYAT_ERR_CUDA;
+    const size_t per_slot = (size_t)g.BH * c.phi_dim * (c.head_dim + 4);
     Geo gs = g;
     gs.Np = (int)HW; gs.ToHW = 0;
-    int carry = -1;
     for (int f0 = 1; f0 <= frames; f0 += ctx->Gmax) {
       gs.t0 = f0;                                // "chunk" f admits frame f-1: [lo_{f-1}, lo_f) = [(f-1) HW, f HW)
       gs.G = frames + 1 - f0 < ctx->Gmax ? frames + 1 - f0 : ctx->Gmax;
       const int ns = pick_state_split(ctx, gs, gs.G, (int)HW);
-      const int rc = run_parts(ctx, nullptr, k, v, nullptr, phi, gs, batch, ns, carry, PART_STATE, st);
+      float* cum = ctx->cum + (size_t)f0 * per_slot;
+      const int rc = run_parts(ctx, nullptr, k, v, nullptr, phi, gs, batch, ns, cum, f0 > 1 ? cum - per_slot : nullptr, PART_STATE, st);
       if (rc != REHYAT_OK) return rc;
-      if (cudaMemcpyAsync((uint8_t*)ctx->cum + (size_t)f0 * slot_bytes, ctx->state, (size_t)gs.G * slot_bytes,
-                          cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-        return REHYAT_ERR_CUDA;
-      carry = gs.G - 1;
     }
     g.prefix = 1;                                // every chunk reads its state, whatever lo_t is
     for (int t0 = 0; t0 < n_chunks; t0 += G) {
       g.t0 = t0;
       g.G = (n_chunks - t0) < G ? (n_chunks - t0) : G;
-      combine_bidirectional<<<(unsigned)((per_slot + 255) / 256), 256, 0, st>>>(
+      combine_bidirectional<<<scan_blocks(per_slot), SCAN_THREADS, 0, st>>>(
           ctx->cum, ctx->state, per_slot, g, (int)HW, frames,
           (ctx->tensor_ok && ctx->tc.phi_ok) ? ctx->tc.state_bf16 : nullptr, c.head_dim);
       ctx->last_launches += 1;
-      const int rc = run_parts(ctx, q, k, v, out, phi, g, batch, 1, -1, PART_READOUT | PART_WINDOW, st);
+      const int rc = run_parts(ctx, q, k, v, out, phi, g, batch, 1, nullptr, nullptr, PART_READOUT | PART_WINDOW, st);
       if (rc != REHYAT_OK) return rc;
     }
     return REHYAT_OK;
   }
-  int carry_slot = -1;
+  const size_t per_slot = (size_t)g.BH * c.phi_dim * (c.head_dim + 4);
+  const float* carry = nullptr;
   for (int t0 = 0; t0 < n_chunks; t0 += G) {
     g.t0 = t0;
     g.G = (n_chunks - t0) < G ? (n_chunks - t0) : G;
     const bool any_linear = geo_lo(g, t0 + g.G - 1) > 0;
-    const int rc = run_parts(ctx, q, k, v, out, phi, g, batch, n_split, carry_slot,
+    const int rc = run_parts(ctx, q, k, v, out, phi, g, batch, n_split, ctx->state, carry,
                              (any_linear ? PART_STATE | PART_READOUT : 0) | PART_WINDOW, st);
     if (rc != REHYAT_OK) return rc;
-    if (any_linear) carry_slot = g.G - 1;
+    if (any_linear) carry = ctx->state + (size_t)(g.G - 1) * per_slot;
   }
   return REHYAT_OK;
 }
@@ -890,7 +892,7 @@ int rehyat_stream_step(rehyat_ctx* ctx, const void* q_chunk, const void* k_chunk
   g.q_off = h; g.Nq = Np;
   ctx->share_now = nullptr;
   ctx->last_impl = ctx->tensor_ok ? (ctx->tc.phi_ok ? 2 : 1) : 0;
-  int rc = run_parts(ctx, q_used, kwin, vwin, out_chunk, phi, g, s.batch, 1, -1, (s.has_state ? PART_READOUT : 0) | PART_WINDOW, st);
+  int rc = run_parts(ctx, q_used, kwin, vwin, out_chunk, phi, g, s.batch, 1, nullptr, nullptr, (s.has_state ? PART_READOUT : 0) | PART_WINDOW, st);
   if (rc != REHYAT_OK) return rc;
   // 3. Eq. 17-18: the tokens that leave the window before the next chunk enter the running state
   const int keep = (long long)s.overlap * HW < (long long)h + Np ? s.overlap * HW : h + Np;
@@ -899,7 +901,8 @@ int rehyat_stream_step(rehyat_ctx* ctx, const void* q_chunk, const void* k_chunk
     Geo gs = g;
     gs.Np = leave; gs.ToHW = 0; gs.q_shift = 0; gs.prefix = 0; gs.t0 = 1; gs.G = 1;   // increment of "chunk 1" = [0, leave)
     const int n_split = pick_state_split(ctx, gs, 1, leave);
-    rc = run_parts(ctx, nullptr, kwin, vwin, nullptr, phi, gs, s.batch, n_split, s.has_state ? 0 : -1, PART_STATE, st);
+    rc = run_parts(ctx, nullptr, kwin, vwin, nullptr, phi, gs, s.batch, n_split, ctx->state, s.has_state ? ctx->state : nullptr,
+                   PART_STATE, st);
     if (rc != REHYAT_OK) return rc;
     s.has_state = 1;
   }
@@ -973,8 +976,8 @@ int rehyat_stream_import(rehyat_ctx* ctx, const void* host_buf, size_t bytes, vo
   if (s.has_state && ctx->tensor_ok && ctx->tc.phi_ok) {
     // the bf16 copy of the state that the tensor-core read-out multiplies with: a scan over zero increments
     const size_t per_slot = stream_state_floats(ctx);
-    scan_states<<<(unsigned)((per_slot + 255) / 256), 256, 0, st>>>(ctx->partial, ctx->state, per_slot, 1, 0, 0,
-                                                                     ctx->tc.state_bf16, c.head_dim);
+    scan_states<<<scan_blocks(per_slot), SCAN_THREADS, 0, st>>>(ctx->partial, ctx->state, per_slot, 1, 0, ctx->state,
+                                                                ctx->tc.state_bf16, c.head_dim);
   }
   const size_t es = elem_size(c.dtype), width = (size_t)s.halo * c.head_dim * es, pitch = (size_t)s.cap_tokens * c.head_dim * es;
   const int BH = s.batch * c.n_heads;

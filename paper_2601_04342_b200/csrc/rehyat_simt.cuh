@@ -12,6 +12,9 @@
 // and odd terms; where the output columns are contiguous (P V, phi^T V, phi s) it holds two columns.  A lane owns 4 - 8
 // rows x 4 - 16 columns, lanes of a warp 4 row groups x 8 column groups, so that an operand load of a warp touches 4 or
 // 8 different 16-byte pieces in different banks and feeds at least five packed instructions.
+// What bounds them: shared-memory loads and the FMA pipe together (window: 67 % and 59 % busy).  12 heads x 12,600 tokens
+// of 128 channels in fp32: window 6.55 -> 4.78 ms, state 2.74 -> 1.31 ms, read-out 2.77 -> 1.28 ms against one column and
+// eight rows a thread with weights read from global memory.
 #pragma once
 
 #include "rehyat_common.cuh"
@@ -339,44 +342,75 @@ state_partial_simt(const T* __restrict__ k, const T* __restrict__ v, PhiPtrs<T> 
   if (threadIdx.x < pd.Dp) *reinterpret_cast<float4*>(dst + (size_t)threadIdx.x * SD + D) = make_float4(zacc, 0.f, 0.f, 0.f);
 }
 
-// state[i] = carry + sum_{u<=i} sum_s partial[u][s]   for the G chunks of the group, where carry
-// is the state of the chunk before the group (slot `carry_slot`, or zero: s_0 = z_0 = 0, Eq. 14-15).
-// One thread per state element; the chunk axis is walked in order, splits in fixed order, so the
-// result does not depend on scheduling.
-__global__ void scan_states(const float* __restrict__ partial, float* __restrict__ state,
-                            size_t per_slot, int G, int n_split, int carry_slot,
-                            __nv_bfloat16* __restrict__ state_bf16 = nullptr, int D = 0) {
-  const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= per_slot) return;
-  float run = carry_slot >= 0 ? state[(size_t)carry_slot * per_slot + e] : 0.f;
-  // optional bf16 copy of the s part, [slot][bh][feature][D], the B operand of the tensor-core read-out
+// Four consecutive state elements, stored as fp32 and, for the s part (column < D), as bf16 in the copy
+// [slot][bh][feature][D] that the tensor-core read-out multiplies with.
+__device__ __forceinline__ void store_state4(float* state, __nv_bfloat16* state_bf16, size_t per_slot, int D, int slot, size_t e, float4 x) {
+  *reinterpret_cast<float4*>(state + (size_t)slot * per_slot + e) = x;
   const size_t row = e / (D + 4), col = e % (D + 4);
-  const size_t per_slot_b = per_slot / (D + 4) * D;
-  for (int i = 0; i < G; ++i) {
-    float inc = 0.f;
-    for (int s = 0; s < n_split; ++s) inc += partial[((size_t)i * n_split + s) * per_slot + e];
-    run += inc;
-    state[(size_t)i * per_slot + e] = run;
-    if (state_bf16 != nullptr && col < (size_t)D) state_bf16[(size_t)i * per_slot_b + row * D + col] = __float2bfloat16_rn(run);
+  if (state_bf16 != nullptr && col < (size_t)D)
+    st4(state_bf16 + (size_t)slot * (per_slot / (D + 4) * D) + row * D + col, x.x, x.y, x.z, x.w);
+}
+__device__ __forceinline__ float4 add4(float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
+
+// state[i] = carry + sum_{u<=i} sum_s partial[u][s]   for the G chunks of the group, where `carry` is the state of the
+// chunk before the group (or null: s_0 = z_0 = 0, Eq. 14-15; it may be a slot of `state`).
+// One thread per four state elements; the chunk axis is walked in order, splits in fixed order, so the
+// result does not depend on scheduling.  Bound by the latency of the partial sums' loads: eight are in flight per thread
+// (one at a time, as the sums need them, the 28 loads of the 480 x 832 layer took 18.9 us between two events, this 12.5;
+// an empty kernel takes 8).
+constexpr int SCAN_THREADS = 128;
+__global__ void __launch_bounds__(SCAN_THREADS)
+scan_states(const float* __restrict__ partial, float* state, size_t per_slot, int G, int n_split, const float* carry,
+            __nv_bfloat16* __restrict__ state_bf16, int D) {
+  const size_t e = ((size_t)blockIdx.x * SCAN_THREADS + threadIdx.x) * 4;
+  if (e >= per_slot) return;
+  float4 run = make_float4(0.f, 0.f, 0.f, 0.f), inc = run;
+  if (carry != nullptr) run = *reinterpret_cast<const float4*>(carry + e);
+  if (n_split == 0) {
+    for (int i = 0; i < G; ++i) store_state4(state, state_bf16, per_slot, D, i, e, run);
+    return;
+  }
+  const int total = G * n_split;
+  int i = 0, s = 0;
+#pragma unroll 1
+  for (int l0 = 0; l0 < total; l0 += 8) {
+    float4 x[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (l0 + u < total) x[u] = *reinterpret_cast<const float4*>(partial + (size_t)(l0 + u) * per_slot + e);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      if (l0 + u >= total) break;
+      inc = add4(inc, x[u]);
+      if (++s == n_split) {
+        run = add4(run, inc);
+        store_state4(state, state_bf16, per_slot, D, i++, e, run);
+        inc = make_float4(0.f, 0.f, 0.f, 0.f);
+        s = 0;
+      }
+    }
   }
 }
 
 // Bidirectional linear sets (Eq. 10-12): TL_t = [0, lo_t) + [hi_t, N).  `cum[f]` is the state summed over the
-// frames before frame f (cum[0] = 0, cum[T] = all tokens), so the state of chunk t is
-// cum[lo_t / HW] + (cum[T] - cum[hi_t / HW]).  One thread per state element, written into the slots the
+// frames before frame f (cum[T] = all tokens; cum[0] = 0 is not read), so the state of chunk t is
+// cum[lo_t / HW] + (cum[T] - cum[hi_t / HW]).  One thread per four state elements, written into the slots the
 // read-out uses (plus the bf16 copy of the s part for the tensor-core read-out).
-__global__ void combine_bidirectional(const float* __restrict__ cum, float* __restrict__ state, size_t per_slot, Geo g,
-                                      int HW, int T, __nv_bfloat16* __restrict__ state_bf16 = nullptr, int D = 0) {
-  const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(SCAN_THREADS)
+combine_bidirectional(const float* __restrict__ cum, float* __restrict__ state, size_t per_slot, Geo g,
+                      int HW, int T, __nv_bfloat16* __restrict__ state_bf16, int D) {
+  const size_t e = ((size_t)blockIdx.x * SCAN_THREADS + threadIdx.x) * 4;
   if (e >= per_slot) return;
-  const size_t row = e / (D + 4), col = e % (D + 4);
-  const size_t per_slot_b = per_slot / (D + 4) * D;
-  const float total = cum[(size_t)T * per_slot + e];
+  const auto at = [&](int f) {
+    return f > 0 ? *reinterpret_cast<const float4*>(cum + (size_t)f * per_slot + e) : make_float4(0.f, 0.f, 0.f, 0.f);
+  };
+  const float4 total = at(T);
+#pragma unroll 4
   for (int i = 0; i < g.G; ++i) {
-    const int t = g.t0 + i, lo_f = geo_lo(g, t) / HW, hi_f = geo_q1(g, t) / HW;
-    const float sv = cum[(size_t)lo_f * per_slot + e] + (total - cum[(size_t)hi_f * per_slot + e]);
-    state[(size_t)i * per_slot + e] = sv;
-    if (state_bf16 != nullptr && col < (size_t)D) state_bf16[(size_t)i * per_slot_b + row * D + col] = __float2bfloat16_rn(sv);
+    const int t = g.t0 + i;
+    const float4 lo = at(geo_lo(g, t) / HW), hi = at(geo_q1(g, t) / HW);
+    store_state4(state, state_bf16, per_slot, D, i, e,
+                 make_float4(lo.x + (total.x - hi.x), lo.y + (total.y - hi.y), lo.z + (total.z - hi.z), lo.w + (total.w - hi.w)));
   }
 }
 
