@@ -199,12 +199,12 @@ int launch_group_simt(rehyat_ctx* ctx, const T* q, const T* k, const T* v, T* ou
     PhiPtrs<T> wk = {(const T*)phi->k_W1, (const T*)phi->k_b1, (const T*)phi->k_W2, (const T*)phi->k_b2,
                      (const T*)phi->k_Wmid, (const T*)phi->k_bmid};
     ctx->prof.begin(REHYAT_PROF_STATE, st);
-    state_partial_simt<T, D><<<dim3(n_split, g.G, g.BH), SIMT_THREADS, simt_phi_smem(D, pd.Dh, pd.Dp, true), st>>>(
-        k, v, wk, pd, g, n_split, ctx->partial);
+    launch_kernel(state_partial_simt<T, D>, dim3(n_split, g.G, g.BH), SIMT_THREADS, simt_phi_smem(D, pd.Dh, pd.Dp, true), st,
+                  k, v, wk, pd, g, n_split, ctx->partial);
     ctx->prof.end(REHYAT_PROF_STATE, st);
     const size_t per_slot = (size_t)g.BH * pd.Dp * SD;
     ctx->prof.begin(REHYAT_PROF_SCAN, st);
-    scan_states<<<scan_blocks(per_slot), SCAN_THREADS, 0, st>>>(ctx->partial, state_out, per_slot, g.G, n_split, carry, nullptr, D);
+    launch_kernel(scan_states, dim3(scan_blocks(per_slot)), SCAN_THREADS, 0, st, ctx->partial, state_out, per_slot, g.G, n_split, carry, nullptr, D);
     ctx->prof.end(REHYAT_PROF_SCAN, st);
     ctx->last_launches += 2;
   }
@@ -215,18 +215,19 @@ int launch_group_simt(rehyat_ctx* ctx, const T* q, const T* k, const T* v, T* ou
     const int parts_rd = pick_parts(tiles, (long long)busy_readout(g) * g.BH, tiles < 64 ? tiles : 64, ctx->tc.n_sm);
     const int per_cta = (tiles + parts_rd - 1) / parts_rd;
     ctx->prof.begin(REHYAT_PROF_READOUT, st);
-    readout_simt<T, D><<<dim3((tiles + per_cta - 1) / per_cta, g.G, g.BH), SIMT_THREADS, simt_phi_smem(D, pd.Dh, pd.Dp, false), st>>>(
-        q, wq, pd, g, ctx->state, ctx->readout, ctx->rd_cap, rd_half, per_cta);
+    launch_kernel(readout_simt<T, D>, dim3((tiles + per_cta - 1) / per_cta, g.G, g.BH), SIMT_THREADS, simt_phi_smem(D, pd.Dh, pd.Dp, false), st,
+                  q, wq, pd, g, ctx->state, ctx->readout, ctx->rd_cap, rd_half, per_cta);
     ctx->prof.end(REHYAT_PROF_READOUT, st);
     ctx->last_launches += 1;
   }
   if (parts & PART_WINDOW) {
     ctx->prof.begin(REHYAT_PROF_WINDOW, st);
+    const int wait_first = !(parts & PART_READOUT);
     const auto launch = [&](auto split) {
       constexpr int WK = decltype(split)::value;
       using S = WinSimt<T, D, WK>;
-      window_simt<T, D, WK><<<dim3((g.Np + S::BM - 1) / S::BM, g.G, g.BH), SIMT_THREADS, S::SMEM, st>>>(
-          q, k, v, out, g, ctx->readout, ctx->rd_cap, 1.0f / sqrtf((float)D), c.c_mode, ctx->share_now);
+      launch_kernel(window_simt<T, D, WK>, dim3((g.Np + S::BM - 1) / S::BM, g.G, g.BH), SIMT_THREADS, S::SMEM, st,
+                    q, k, v, out, g, ctx->readout, ctx->rd_cap, 1.0f / sqrtf((float)D), c.c_mode, ctx->share_now, wait_first);
     };
     // Tiles of 128 rows need the fewest loads per multiply-add; below two waves of them the SMs are better filled by
     // tiles of 32 rows whose keys are shared among four warps (2 heads x 1,071 tokens of 64 channels: 12 tiles of the one,
@@ -277,7 +278,7 @@ int run_parts(rehyat_ctx* ctx, const void* q, const void* k, const void* v, void
         ctx->prof.end(REHYAT_PROF_STATE, st);
         const size_t per_slot = (size_t)g.BH * c.phi_dim * (c.head_dim + 4);
         ctx->prof.begin(REHYAT_PROF_SCAN, st);
-        scan_states<<<scan_blocks(per_slot), SCAN_THREADS, 0, st>>>(ctx->partial, state_out, per_slot, g.G, n_split, carry,
+        launch_kernel(scan_states, dim3(scan_blocks(per_slot)), SCAN_THREADS, 0, st, ctx->partial, state_out, per_slot, g.G, n_split, carry,
                                                                     state_out == ctx->state ? ctx->tc.state_bf16 : nullptr, c.head_dim);
         ctx->prof.end(REHYAT_PROF_SCAN, st);
         ctx->last_launches += 2;
@@ -293,7 +294,8 @@ int run_parts(rehyat_ctx* ctx, const void* q, const void* k, const void* v, void
     }
     if (rc == REHYAT_OK && (parts & PART_WINDOW)) {
       ctx->prof.begin(REHYAT_PROF_WINDOW, st);
-      rc = tc_launch_window(&ctx->tc, q, k, v, out, g, batch, ctx->readout, ctx->rd_cap, c.c_mode, next_wait(ctx), ctx->share_now, st);
+      rc = tc_launch_window(&ctx->tc, q, k, v, out, g, batch, ctx->readout, ctx->rd_cap, c.c_mode, next_wait(ctx), ctx->share_now,
+                            !(parts & PART_READOUT), st);
       ctx->prof.end(REHYAT_PROF_WINDOW, st);
       ctx->last_launches += 1;
     }
@@ -351,12 +353,12 @@ void launch_qk_prepare(rehyat_ctx* ctx, const void* q, const void* k, void* qo, 
   const dim3 grid(blocks, BH, 2);
   ctx->prof.begin(REHYAT_PROF_QKPREP, st);
   if (c.dtype == REHYAT_DTYPE_FP32) {
-    if (c.head_dim == 64) qk_prepare<float, 64><<<grid, 256, 0, st>>>((const float*)q, (const float*)k, (float*)qo, (float*)ko, pa);
-    else qk_prepare<float, 128><<<grid, 256, 0, st>>>((const float*)q, (const float*)k, (float*)qo, (float*)ko, pa);
+    if (c.head_dim == 64) launch_kernel(qk_prepare<float, 64>, grid, 256, 0, st, (const float*)q, (const float*)k, (float*)qo, (float*)ko, pa);
+    else launch_kernel(qk_prepare<float, 128>, grid, 256, 0, st, (const float*)q, (const float*)k, (float*)qo, (float*)ko, pa);
   } else {
     using B = __nv_bfloat16;
-    if (c.head_dim == 64) qk_prepare<B, 64><<<grid, 256, 0, st>>>((const B*)q, (const B*)k, (B*)qo, (B*)ko, pa);
-    else qk_prepare<B, 128><<<grid, 256, 0, st>>>((const B*)q, (const B*)k, (B*)qo, (B*)ko, pa);
+    if (c.head_dim == 64) launch_kernel(qk_prepare<B, 64>, grid, 256, 0, st, (const B*)q, (const B*)k, (B*)qo, (B*)ko, pa);
+    else launch_kernel(qk_prepare<B, 128>, grid, 256, 0, st, (const B*)q, (const B*)k, (B*)qo, (B*)ko, pa);
   }
   ctx->prof.end(REHYAT_PROF_QKPREP, st);
   ctx->last_launches += 1;
@@ -364,12 +366,14 @@ void launch_qk_prepare(rehyat_ctx* ctx, const void* q, const void* k, void* qo, 
 
 // Copies `rows` token rows of `row_bytes` bytes for each of BH (batch, head) problems between two strided
 // layouts (byte strides; rows are contiguous and 16-byte aligned).  grid (row tiles, BH), 256 threads.
-__global__ void copy_rows(uint8_t* __restrict__ dst0, uint8_t* __restrict__ dst1, long long dst_b, long long dst_h, long long dst_n,
-                          const uint8_t* __restrict__ src0, const uint8_t* __restrict__ src1, long long src_b, long long src_h,
-                          long long src_n, int rows, int row_bytes, int n_heads) {
+__global__ void copy_rows(uint8_t* dst0, uint8_t* dst1, long long dst_b, long long dst_h, long long dst_n, const uint8_t* src0,
+                          const uint8_t* src1, long long src_b, long long src_h, long long src_n, int rows, int row_bytes,
+                          int n_heads) {
+  ptx::grid_dep_wait();
+  ptx::grid_dep_launch();
   // blockIdx.z picks one of two tensor pairs that share their layouts (k and v)
-  uint8_t* __restrict__ dst = blockIdx.z ? dst1 : dst0;
-  const uint8_t* __restrict__ src = blockIdx.z ? src1 : src0;
+  uint8_t* dst = blockIdx.z ? dst1 : dst0;
+  const uint8_t* src = blockIdx.z ? src1 : src0;
   const int bh = blockIdx.y, b = bh / n_heads, h = bh % n_heads;
   const int per_row = row_bytes / 16;
   const long long total = (long long)rows * per_row;
@@ -646,7 +650,7 @@ int rehyat_forward(rehyat_ctx* ctx, const void* q, const void* k, const void* v,
     for (int t0 = 0; t0 < n_chunks; t0 += G) {
       g.t0 = t0;
       g.G = (n_chunks - t0) < G ? (n_chunks - t0) : G;
-      combine_bidirectional<<<scan_blocks(per_slot), SCAN_THREADS, 0, st>>>(
+      launch_kernel(combine_bidirectional, dim3(scan_blocks(per_slot)), SCAN_THREADS, 0, st,
           ctx->cum, ctx->state, per_slot, g, (int)HW, frames,
           (ctx->tensor_ok && ctx->tc.phi_ok) ? ctx->tc.state_bf16 : nullptr, c.head_dim);
       ctx->last_launches += 1;
@@ -781,8 +785,8 @@ void launch_copy_rows2(void* dst0, void* dst1, long long dst_b, long long dst_h,
   if (rows <= 0) return;
   const long long total = (long long)rows * (row_bytes / 16);
   const unsigned blocks = (unsigned)((total + 255) / 256 < 256 ? (total + 255) / 256 : 256);
-  copy_rows<<<dim3(blocks, BH, dst1 ? 2 : 1), 256, 0, st>>>((uint8_t*)dst0, (uint8_t*)dst1, dst_b, dst_h, dst_n, (const uint8_t*)src0,
-                                                 (const uint8_t*)src1, src_b, src_h, src_n, rows, row_bytes, n_heads);
+  launch_kernel(copy_rows, dim3(blocks, BH, dst1 ? 2 : 1), 256, 0, st, (uint8_t*)dst0, (uint8_t*)dst1, dst_b, dst_h, dst_n,
+                (const uint8_t*)src0, (const uint8_t*)src1, src_b, src_h, src_n, rows, row_bytes, n_heads);
 }
 
 }  // namespace
@@ -976,7 +980,7 @@ int rehyat_stream_import(rehyat_ctx* ctx, const void* host_buf, size_t bytes, vo
   if (s.has_state && ctx->tensor_ok && ctx->tc.phi_ok) {
     // the bf16 copy of the state that the tensor-core read-out multiplies with: a scan over zero increments
     const size_t per_slot = stream_state_floats(ctx);
-    scan_states<<<scan_blocks(per_slot), SCAN_THREADS, 0, st>>>(ctx->partial, ctx->state, per_slot, 1, 0, ctx->state,
+    launch_kernel(scan_states, dim3(scan_blocks(per_slot)), SCAN_THREADS, 0, st, ctx->partial, ctx->state, per_slot, 1, 0, ctx->state,
                                                                 ctx->tc.state_bf16, c.head_dim);
   }
   const size_t es = elem_size(c.dtype), width = (size_t)s.halo * c.head_dim * es, pitch = (size_t)s.cap_tokens * c.head_dim * es;

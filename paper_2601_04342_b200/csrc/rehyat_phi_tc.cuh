@@ -121,6 +121,8 @@ phi_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtenso
   const int n_tiles = (tok_b - tok_a + 127) / 128;
 
   if (n_tiles == 0) {                          // nothing admitted: the partial is zero
+    grid_dep_wait();
+    grid_dep_launch();
     float* dst = a.partial + (((size_t)ci * a.n_split + blockIdx.x) * g.BH + bh) * Dp * SD;
     for (int i = threadIdx.x; i < Dp * SD / 4; i += PH_THREADS)
       reinterpret_cast<float4*>(dst)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -139,6 +141,12 @@ phi_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtenso
     wait_ctx_init(&bars->wctx, a.wa);
     fence_mbar_init();
   }
+  if (warp == 9) {
+    tmem_alloc(smem_u32(&bars->tmem_base), 512);
+    tmem_relinquish();
+  }
+  grid_dep_wait();
+  grid_dep_launch();
   // biases as fp32; the ones tile: row 0 of both 64-column sub-tiles is 1, the rest 0
   for (int i = threadIdx.x; i < 256; i += PH_THREADS) {          // zero beyond the widths
     s_b1[i] = i < ex.Dh ? __bfloat162float(a.b1[(size_t)h_idx * ex.Dh + i]) : 0.f;
@@ -153,10 +161,6 @@ phi_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtenso
       ones[i] = (within < 128 && sub < 2) ? 0x3F803F80u : 0u;       // two bf16 ones
     }
     fence_proxy_async_smem();
-  }
-  if (warp == 9) {
-    tmem_alloc(smem_u32(&bars->tmem_base), 512);
-    tmem_relinquish();
   }
   tc_fence_before();
   __syncthreads();

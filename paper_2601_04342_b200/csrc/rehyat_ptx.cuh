@@ -150,6 +150,20 @@ __device__ __forceinline__ bool mbar_wait_drain(uint32_t bar, uint32_t parity, u
 }
 
 // ----------------------------------------------------------------------------- TMA
+// Programmatic dependent launch.  Every kernel of the library is launched as one that may start before its predecessor
+// on the stream has ended (launch_kernel in rehyat_api.cu).  grid_dep_wait returns when that predecessor is complete and
+// its writes are visible; grid_dep_launch lets the next kernel start once all CTAs of this grid have called it or ended.
+// The rule that makes early work safe: a CTA calls grid_dep_launch only after its grid_dep_wait, so that a kernel that
+// has started may use everything but the results of its direct predecessor, and no kernel ends before its predecessor.
+// (Loads of a predecessor's results must not go through pointers the compiler may take for read-only.)
+__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ uint4 ld_global_v4(const void* p) {
+  uint4 v;
+  asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+  return v;
+}
+
 __device__ __forceinline__ void prefetch_tensormap(const void* tmap) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(tmap)) : "memory");
 }

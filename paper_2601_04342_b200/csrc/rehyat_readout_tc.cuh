@@ -88,10 +88,9 @@ readout_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUt
     wait_ctx_init(&bars->wctx, a.wa);
     fence_mbar_init();
   }
-  for (int i = threadIdx.x; i < 256; i += PH_THREADS) {             // biases and z_t as fp32, zero beyond the widths
+  for (int i = threadIdx.x; i < 256; i += PH_THREADS) {             // biases as fp32, zero beyond the widths
     s_b1[i] = i < ex.Dh ? __bfloat162float(a.b1[(size_t)h_idx * ex.Dh + i]) : 0.f;
     s_b2[i] = i < Dp ? __bfloat162float(a.b2[(size_t)h_idx * Dp + i]) : 0.f;
-    s_z[i] = i < Dp ? a.state[(((size_t)ci * g.BH + bh) * Dp + i) * SD + d] : 0.f;
     for (int m = 0; m < n_mid; ++m)
       s_bm[m * 256 + i] = i < ex.Dh ? __bfloat162float(a.bm[((size_t)h_idx * n_mid + m) * ex.Dh + i]) : 0.f;
   }
@@ -134,6 +133,7 @@ readout_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUt
           for (int ks = 0; ks < ks1; ++ks) tma_load_3d(dst + ks * 8192, &tm_s, full, ks * 64, f * 64, ci * g.BH + bh);
       };
       auto state_half = [&](int c) {                                // the blocks of features [128 c, 128 c + 128)
+        grid_dep_wait();                                            // the states are the predecessor's results
         for (int f = 2 * c; f < 2 * c + 2 && f < nf; ++f) state_load(f);
       };
       for (int j = 0; j < n_tiles && alive; ++j) {
@@ -283,6 +283,11 @@ readout_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUt
     // at the head of the next tile, where the whole warp looks at the flag together.
     auto aborted = [&]() -> bool { return __any_sync(0xffffffffu, wait_ctx_aborted(wc) != 0); };
     auto wait = [&](uint64_t* bar, uint32_t parity) { mbar_wait(smem_u32(bar), parity, wc, PH_ERR_EPI); };
+    // z_t: the first result of the predecessor that is needed; the loads and GEMMs of the first tile's H run meanwhile
+    grid_dep_wait();
+    grid_dep_launch();
+    s_z[threadIdx.x] = (int)threadIdx.x < Dp ? a.state[(((size_t)ci * g.BH + bh) * Dp + threadIdx.x) * SD + d] : 0.f;
+    asm volatile("bar.sync 1, 256;" ::: "memory");                  // the eight epilogue warps
     // bias + activation (+ power) of 32 accumulator columns -> 16 bf16 pairs
     auto activate = [&](const auto& x, const float* bias, bool is_u, int col0, auto& w) {
       constexpr int NC = sizeof(x) / sizeof(x[0]);                 // columns of this block

@@ -250,9 +250,10 @@ __device__ __forceinline__ void load_rows_simt(float* dst, int ld, const __nv_bf
 // column d holding the z part.
 template <typename T, int D>
 __global__ void __launch_bounds__(SIMT_THREADS)
-state_partial_simt(const T* __restrict__ k, const T* __restrict__ v, PhiPtrs<T> wk, PhiDims pd, Geo g,
-                   int n_split, float* __restrict__ partial) {
+state_partial_simt(const T* k, const T* v, PhiPtrs<T> wk, PhiDims pd, Geo g, int n_split, float* partial) {
   extern __shared__ __align__(16) float smem[];
+  ptx::grid_dep_wait();
+  ptx::grid_dep_launch();
   constexpr int SD = D + 4;
   const int ldh = simt_act_ld(pd.Dh, pd.Dp);
   float* Xs = smem;
@@ -360,8 +361,10 @@ __device__ __forceinline__ float4 add4(float4 a, float4 b) { return make_float4(
 // an empty kernel takes 8).
 constexpr int SCAN_THREADS = 128;
 __global__ void __launch_bounds__(SCAN_THREADS)
-scan_states(const float* __restrict__ partial, float* state, size_t per_slot, int G, int n_split, const float* carry,
-            __nv_bfloat16* __restrict__ state_bf16, int D) {
+scan_states(const float* partial, float* state, size_t per_slot, int G, int n_split, const float* carry,
+            __nv_bfloat16* state_bf16, int D) {
+  ptx::grid_dep_wait();
+  ptx::grid_dep_launch();
   const size_t e = ((size_t)blockIdx.x * SCAN_THREADS + threadIdx.x) * 4;
   if (e >= per_slot) return;
   float4 run = make_float4(0.f, 0.f, 0.f, 0.f), inc = run;
@@ -397,20 +400,30 @@ scan_states(const float* __restrict__ partial, float* state, size_t per_slot, in
 // cum[lo_t / HW] + (cum[T] - cum[hi_t / HW]).  One thread per four state elements, written into the slots the
 // read-out uses (plus the bf16 copy of the s part for the tensor-core read-out).
 __global__ void __launch_bounds__(SCAN_THREADS)
-combine_bidirectional(const float* __restrict__ cum, float* __restrict__ state, size_t per_slot, Geo g,
-                      int HW, int T, __nv_bfloat16* __restrict__ state_bf16, int D) {
+combine_bidirectional(const float* cum, float* state, size_t per_slot, Geo g, int HW, int T, __nv_bfloat16* state_bf16, int D) {
+  ptx::grid_dep_wait();
+  ptx::grid_dep_launch();
   const size_t e = ((size_t)blockIdx.x * SCAN_THREADS + threadIdx.x) * 4;
   if (e >= per_slot) return;
   const auto at = [&](int f) {
     return f > 0 ? *reinterpret_cast<const float4*>(cum + (size_t)f * per_slot + e) : make_float4(0.f, 0.f, 0.f, 0.f);
   };
   const float4 total = at(T);
-#pragma unroll 4
-  for (int i = 0; i < g.G; ++i) {
-    const int t = g.t0 + i;
-    const float4 lo = at(geo_lo(g, t) / HW), hi = at(geo_q1(g, t) / HW);
-    store_state4(state, state_bf16, per_slot, D, i, e,
-                 make_float4(lo.x + (total.x - hi.x), lo.y + (total.y - hi.y), lo.z + (total.z - hi.z), lo.w + (total.w - hi.w)));
+#pragma unroll 1
+  for (int i0 = 0; i0 < g.G; i0 += 4) {                // eight loads in flight, then four states
+    float4 lo[4], hi[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int t = g.t0 + min(i0 + u, g.G - 1);
+      lo[u] = at(geo_lo(g, t) / HW);
+      hi[u] = at(geo_q1(g, t) / HW);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (i0 + u < g.G)
+        store_state4(state, state_bf16, per_slot, D, i0 + u, e,
+                     make_float4(lo[u].x + (total.x - hi[u].x), lo[u].y + (total.y - hi[u].y), lo[u].z + (total.z - hi[u].z),
+                                 lo[u].w + (total.w - hi[u].w)));
   }
 }
 
@@ -420,8 +433,8 @@ combine_bidirectional(const float* __restrict__ cum, float* __restrict__ state, 
 // in the layout of rdh_index.
 template <typename T, int D>
 __global__ void __launch_bounds__(SIMT_THREADS)
-readout_simt(const T* __restrict__ q, PhiPtrs<T> wq, PhiDims pd, Geo g, const float* __restrict__ state,
-             float* __restrict__ rd, int rd_rows, int rd_half, int tiles_per_cta) {
+readout_simt(const T* q, PhiPtrs<T> wq, PhiDims pd, Geo g, const float* state, float* rd, int rd_rows, int rd_half,
+             int tiles_per_cta) {
   extern __shared__ __align__(16) float smem[];
   constexpr int SD = D + 4;
   const int ldh = simt_act_ld(pd.Dh, pd.Dp);
@@ -466,6 +479,10 @@ readout_simt(const T* __restrict__ q, PhiPtrs<T> wq, PhiDims pd, Geo g, const fl
       if (tok0 + SIMT_TM < b) load_rows_simt<D>(Xs, D + 4, qh, g.qstride_n, tok0 + SIMT_TM, b);
     });
     __syncwarp();                                      // the warp's slabs are free
+    if (tok0 == a) {                                   // phi of the first tile runs while the states are still being summed
+      ptx::grid_dep_wait();
+      ptx::grid_dep_launch();
+    }
 #pragma unroll
     for (int s = 0; s < SIMT_STAGES - 1; ++s) issue_state(s);
     __syncthreads();
@@ -567,11 +584,13 @@ struct QkPrepArgs {
 };
 template <typename T, int D>
 __global__ void __launch_bounds__(256)
-qk_prepare(const T* __restrict__ q, const T* __restrict__ k, T* __restrict__ qo, T* __restrict__ ko, QkPrepArgs a) {
+qk_prepare(const T* q, const T* k, T* qo, T* ko, QkPrepArgs a) {
+  ptx::grid_dep_wait();
+  ptx::grid_dep_launch();
   constexpr int LPR = D / 8;                                        // lanes per row
-  const T* __restrict__ src = blockIdx.z ? k : q;
-  T* __restrict__ dst = blockIdx.z ? ko : qo;
-  const T* __restrict__ wgt = static_cast<const T*>(blockIdx.z ? a.wk : a.wq);
+  const T* src = blockIdx.z ? k : q;
+  T* dst = blockIdx.z ? ko : qo;
+  const T* wgt = static_cast<const T*>(blockIdx.z ? a.wk : a.wq);
   const int bh = blockIdx.y, head = bh % a.n_heads, bat = bh / a.n_heads;
   const long long hoff = (long long)bat * a.sb + (long long)head * a.sh;
   const long long doff = blockIdx.z ? (long long)bat * a.kb + (long long)head * a.kh : (long long)bat * a.qb + (long long)head * a.qh;
@@ -661,8 +680,9 @@ struct WinSimt {
 
 template <typename T, int D, int WK>
 __global__ void __launch_bounds__(SIMT_THREADS)
-window_simt(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v, T* __restrict__ out,
-            Geo g, const float* __restrict__ rd, int rd_rows, float scale, int c_mode, float* __restrict__ share) {
+window_simt(const T* q, const T* k, const T* v, T* out, Geo g, const float* rd, int rd_rows, float scale, int c_mode,
+            float* share, int wait_first) {
+  if (wait_first) ptx::grid_dep_wait();                        // q, k, v may come from the direct predecessor
   using S = WinSimt<T, D, WK>;
   extern __shared__ __align__(16) float smem[];
   constexpr int KJ = S::KJ, NQ = D / 32, RGS = 8 / WK;          // RGS: row groups of 16 per CTA
@@ -837,6 +857,8 @@ window_simt(const T* __restrict__ q, const T* __restrict__ k, const T* __restric
     }
   }
 
+  ptx::grid_dep_wait();                                         // the read-out
+  ptx::grid_dep_launch();
   // Eq. 5: the window sums are relative to c_i = final row maximum m_i.  ROWMAX: the linear terms
   // enter unscaled.  ZERO (c = 0): window terms carry exp(m_i), evaluated stably by measuring both
   // branches against r = max(m_i, 0): window * exp(m_i - r), linear * exp(-r).

@@ -225,8 +225,8 @@ template <int EMU, int D>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 window_tc(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
           const __grid_constant__ CUtensorMap tm_v, __nv_bfloat16* __restrict__ out, Geo g,
-          const float* __restrict__ rd, int rd_rows, float scale, int c_mode, ptx::WaitArgs wa,
-          int n_items, int pairs, float* __restrict__ share) {
+          const float* rd, int rd_rows, float scale, int c_mode, ptx::WaitArgs wa,
+          int n_items, int pairs, float* __restrict__ share, int wait_first) {
   using namespace ptx;
   using SH = WinShape<D>;
   constexpr int TC_TILE_BYTES = SH::TILE_BYTES, TC_SUB_BYTES = SH::SUB_BYTES;
@@ -271,6 +271,10 @@ window_tc(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = bars->tmem_base;
+  if (wait_first) {                                                  // q, k, v may come from the direct predecessor
+    grid_dep_wait();
+    grid_dep_launch();
+  }
 
   if (warp < 4) setmaxnreg_dec<TC_REGS_OTHER>();
   if (warp == 0) {
@@ -420,11 +424,13 @@ window_tc(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
       uint4 rdv[D / 8];                                              // fp16 pairs of aL / nL
       float nL = 0.f;
       if (w.linear) {
+        grid_dep_wait();                                             // the read-out is the predecessor's result
+        grid_dep_launch();
         const int ric = (valid ? row : w.q0) - w.q0, ci = w.ci;      // row inside the chunk: consecutive threads, consecutive pieces
         const uint4* rdh = reinterpret_cast<const uint4*>(rd);
 #pragma unroll
-        for (int u = 0; u < D / 8; ++u) rdv[u] = __ldg(rdh + rdh_index(g, rd_rows, D, w.bh, ci, ric, u));
-        nL = __ldg(reinterpret_cast<const float*>(rdh + rdh_index(g, rd_rows, D, w.bh, ci, ric, rdh_pieces(D) - 1)));
+        for (int u = 0; u < D / 8; ++u) rdv[u] = ld_global_v4(rdh + rdh_index(g, rd_rows, D, w.bh, ci, ric, u));
+        nL = __uint_as_float(ld_global_v4(rdh + rdh_index(g, rd_rows, D, w.bh, ci, ric, rdh_pieces(D) - 1)).x);
       } else {
 #pragma unroll
         for (int u = 0; u < D / 8; ++u) rdv[u] = make_uint4(0u, 0u, 0u, 0u);
@@ -545,10 +551,26 @@ inline bool tc_workspace_create(TcWorkspace* w, int bh_max, int Gmax, int d, int
 }
 inline void tc_workspace_destroy(TcWorkspace* w) { cudaFree(w->state_bf16); w->state_bf16 = nullptr; }
 
+// Launches a kernel that may start before the kernel before it on the stream has ended (see ptx::grid_dep_wait).
+template <typename... P, typename... A>
+inline void launch_kernel(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);        // a failure is left for cudaGetLastError
+}
+
 // window_tc1 (one query tile per item) and its launcher live in rehyat_tc_single.cuh
 inline int tc_launch_window1(int head_dim, int exp_poly, int n_sm, const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
                              __nv_bfloat16* o, const Geo& g, const float* rd, int rd_rows, float scale, int c_mode,
-                             const ptx::WaitArgs& wa, float* share, cudaStream_t st);
+                             const ptx::WaitArgs& wa, float* share, int wait_first, cudaStream_t st);
 inline bool tc_set_attributes1();
 
 inline int tc_set_attributes() {
@@ -610,7 +632,7 @@ inline bool tc_make_tmap_3d(const TcWorkspace* w, CUtensorMap* tm, const void* b
 // Launches window_tc for the chunks of one group.  `rd` is the linear read-out of the group's queries.
 inline int tc_launch_window(TcWorkspace* w, const void* q, const void* k, const void* v, void* out, const Geo& g,
                             int batch, const float* rd, int rd_rows, int c_mode, const ptx::WaitArgs& wa, float* share,
-                            cudaStream_t st) {
+                            int wait_first, cudaStream_t st) {
   CUtensorMap tq, tk, tv;
   if (!tc_make_tmap_q(w, &tq, q, g, batch) || !tc_make_tmap(w, &tk, k, g, batch) || !tc_make_tmap(w, &tv, v, g, batch))
     return REHYAT_ERR_CUDA;
@@ -626,11 +648,11 @@ inline int tc_launch_window(TcWorkspace* w, const void* q, const void* k, const 
   const double cost2 = 2.0 * (double)((n_items + w->n_sm - 1) / w->n_sm), cost1 = 1.08 * (double)((n1 + w->n_sm - 1) / w->n_sm);
   if (w->item_tiles == 1 || (w->item_tiles == 0 && cost1 < 0.93 * cost2)) {
     w->last_item_tiles = 1;
-    return tc_launch_window1(w->head_dim, w->exp_poly, w->n_sm, tq, tk, tv, o, g, rd, rd_rows, scale, c_mode, wa, share, st);
+    return tc_launch_window1(w->head_dim, w->exp_poly, w->n_sm, tq, tk, tv, o, g, rd, rd_rows, scale, c_mode, wa, share, wait_first, st);
   }
   w->last_item_tiles = 2;
 #define REHYAT_LAUNCH_WINDOW(E, D) \
-  window_tc<E, D><<<grid, TC_THREADS, WinShape<D>::SMEM, st>>>(tq, tk, tv, o, g, rd, rd_rows, scale, c_mode, wa, n_items, pairs, share)
+  launch_kernel(window_tc<E, D>, grid, TC_THREADS, WinShape<D>::SMEM, st, tq, tk, tv, o, g, rd, rd_rows, scale, c_mode, wa, n_items, pairs, share, wait_first)
 #define REHYAT_LAUNCH_WINDOW_D(D)                \
   switch (w->exp_poly) {                         \
     case 0: REHYAT_LAUNCH_WINDOW(0, D); break;   \
@@ -663,7 +685,7 @@ inline int tc_launch_state(const TcWorkspace* w, const void* k, const void* v, c
   a.n_split = n_split; a.partial = partial; a.wa = wa;
   const PhiKernelChoice ch = tc_phi_choice(d, Dh, Dp, P, n_mid, act_hidden, act_out);
   const dim3 grid(n_split, g.G, g.BH);
-#define REHYAT_LAUNCH_PHI(R, PC, GEN) phi_tc<R, PC, GEN><<<grid, PH_THREADS, PH_SMEM, st>>>(tk, tv, tw1, tw2, twm, g, a)
+#define REHYAT_LAUNCH_PHI(R, PC, GEN) launch_kernel(phi_tc<R, PC, GEN>, grid, PH_THREADS, PH_SMEM, st, tk, tv, tw1, tw2, twm, g, a)
   if (ch.gen) { if (ch.relu) REHYAT_LAUNCH_PHI(true, 0, true); else REHYAT_LAUNCH_PHI(false, 0, true); }
   else if (ch.pc == 2) REHYAT_LAUNCH_PHI(true, 2, false);
   else if (ch.relu) REHYAT_LAUNCH_PHI(true, 0, false);
@@ -704,7 +726,7 @@ inline int tc_launch_readout(const TcWorkspace* w, const void* q, const rehyat_p
   const int ctas = (tiles + a.tiles_per_cta - 1) / a.tiles_per_cta;
   const PhiKernelChoice ch = tc_phi_choice(d, Dh, Dp, P, n_mid, act_hidden, act_out);
   const dim3 grid(ctas, g.G, g.BH);
-#define REHYAT_LAUNCH_RD(R, PC, GEN) readout_tc<R, PC, GEN><<<grid, PH_THREADS, RD_SMEM, st>>>(tq, tw1, tw2, twm, ts, g, a)
+#define REHYAT_LAUNCH_RD(R, PC, GEN) launch_kernel(readout_tc<R, PC, GEN>, grid, PH_THREADS, RD_SMEM, st, tq, tw1, tw2, twm, ts, g, a)
   if (ch.gen) { if (ch.relu) REHYAT_LAUNCH_RD(true, 0, true); else REHYAT_LAUNCH_RD(false, 0, true); }
   else if (ch.pc == 2) REHYAT_LAUNCH_RD(true, 2, false);
   else if (ch.relu) REHYAT_LAUNCH_RD(true, 0, false);

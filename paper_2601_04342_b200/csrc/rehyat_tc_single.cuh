@@ -51,8 +51,8 @@ template <int EMU, int D>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 window_tc1(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
            const __grid_constant__ CUtensorMap tm_v, __nv_bfloat16* __restrict__ out, Geo g,
-           const float* __restrict__ rd, int rd_rows, float scale, int c_mode, ptx::WaitArgs wa,
-           int n_items, int tiles, float* __restrict__ share) {
+           const float* rd, int rd_rows, float scale, int c_mode, ptx::WaitArgs wa,
+           int n_items, int tiles, float* __restrict__ share, int wait_first) {
   using namespace ptx;
   using SH = WinShape<D>;
   constexpr int TC_TILE_BYTES = SH::TILE_BYTES, TC_SUB_BYTES = SH::SUB_BYTES;
@@ -93,6 +93,10 @@ window_tc1(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = bars->tmem_base;
+  if (wait_first) {                                                  // q, k, v may come from the direct predecessor
+    grid_dep_wait();
+    grid_dep_launch();
+  }
 
   if (warp < 4) setmaxnreg_dec<TC_REGS_OTHER>();
   if (warp == 0) {
@@ -257,11 +261,13 @@ window_tc1(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
       uint4 rdv[D / 16];                                             // fp16 pairs of aL / nL
       float nL = 0.f;
       if (w.linear) {
+        grid_dep_wait();                                             // the read-out is the predecessor's result
+        grid_dep_launch();
         const int ric = (valid ? row : w.q0) - w.q0, ci = w.ci;
         const uint4* rdh = reinterpret_cast<const uint4*>(rd);
 #pragma unroll
-        for (int u = 0; u < D / 16; ++u) rdv[u] = __ldg(rdh + rdh_index(g, rd_rows, D, w.bh, ci, ric, i * (D / 16) + u));
-        nL = __ldg(reinterpret_cast<const float*>(rdh + rdh_index(g, rd_rows, D, w.bh, ci, ric, rdh_pieces(D) - 1)));
+        for (int u = 0; u < D / 16; ++u) rdv[u] = ld_global_v4(rdh + rdh_index(g, rd_rows, D, w.bh, ci, ric, i * (D / 16) + u));
+        nL = __uint_as_float(ld_global_v4(rdh + rdh_index(g, rd_rows, D, w.bh, ci, ric, rdh_pieces(D) - 1)).x);
       } else {
 #pragma unroll
         for (int u = 0; u < D / 16; ++u) rdv[u] = make_uint4(0u, 0u, 0u, 0u);
@@ -337,12 +343,12 @@ window_tc1(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
 // Launches window_tc1 with the tensor maps and arguments tc_launch_window has prepared.
 inline int tc_launch_window1(int head_dim, int exp_poly, int n_sm, const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
                              __nv_bfloat16* o, const Geo& g, const float* rd, int rd_rows, float scale, int c_mode,
-                             const ptx::WaitArgs& wa, float* share, cudaStream_t st) {
+                             const ptx::WaitArgs& wa, float* share, int wait_first, cudaStream_t st) {
   const int tiles = (g.Np + TC_BM - 1) / TC_BM;
   const int n_items = tiles * g.G * g.BH;
   const dim3 grid(n_items < n_sm ? n_items : n_sm);
 #define REHYAT_LAUNCH_WINDOW1(E, D) \
-  window_tc1<E, D><<<grid, TC_THREADS, WinShape<D>::SMEM1, st>>>(tq, tk, tv, o, g, rd, rd_rows, scale, c_mode, wa, n_items, tiles, share)
+  launch_kernel(window_tc1<E, D>, grid, TC_THREADS, WinShape<D>::SMEM1, st, tq, tk, tv, o, g, rd, rd_rows, scale, c_mode, wa, n_items, tiles, share, wait_first)
 #define REHYAT_LAUNCH_WINDOW1_D(D)               \
   switch (exp_poly) {                            \
     case 0: REHYAT_LAUNCH_WINDOW1(0, D); break;  \
