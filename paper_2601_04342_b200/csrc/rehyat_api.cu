@@ -24,6 +24,7 @@
 #include "rehyat_simt.cuh"
 #include "rehyat_tc.cuh"
 #include "rehyat_tc_single.cuh"
+#include "rehyat_f32_tc.cuh"
 
 using namespace rehyat;
 
@@ -146,6 +147,7 @@ int set_simt_attributes() {
       cudaFuncSetAttribute(window_simt<T, D, 1>, smem, WinSimt<T, D, 1>::SMEM) != cudaSuccess ||
       cudaFuncSetAttribute(window_simt<T, D, 4>, smem, WinSimt<T, D, 4>::SMEM) != cudaSuccess)
     return REHYAT_ERR_CUDA;
+  if (sizeof(T) == 4 && cudaFuncSetAttribute(window_f32_tc<D>, smem, F32Shape<D>::SMEM) != cudaSuccess) return REHYAT_ERR_CUDA;
   return REHYAT_OK;
 }
 
@@ -186,6 +188,14 @@ int busy_readout(const Geo& g) {
   return busy > 0 ? busy : 1;
 }
 
+// Does the softmax window of an fp32 call run on the tensor cores (window_f32_tc)?  The two kernels cross between windows
+// of 128 and 256 keys: 1 head of 64, windows of 128 keys 45.3 us a call on the CUDA cores, 48.8 on the tensor cores;
+// of 256 keys 50.8 and 49.1; 24 heads of 128 with windows of 1,200 keys 1,708 and 1,155.
+bool use_f32_tc(const rehyat_ctx* ctx, const Geo& g) {
+  const long long keys = (long long)g.Np + g.ToHW;
+  return ctx->status_dev != nullptr && ctx->cfg.impl != REHYAT_IMPL_SIMT && (keys < g.N ? keys : g.N) > 128;
+}
+
 unsigned scan_blocks(size_t per_slot) { return (unsigned)((per_slot / 4 + SCAN_THREADS - 1) / SCAN_THREADS); }
 
 template <typename T, int D>
@@ -222,12 +232,27 @@ int launch_group_simt(rehyat_ctx* ctx, const T* q, const T* k, const T* v, T* ou
   }
   if (parts & PART_WINDOW) {
     ctx->prof.begin(REHYAT_PROF_WINDOW, st);
-    const int wait_first = !(parts & PART_READOUT);
+    int wait_first = !(parts & PART_READOUT), epoch = 0;
+    int* unsafe = nullptr;
+    if constexpr (sizeof(T) == 4) {
+      if (use_f32_tc(ctx, g)) {
+        const int q_tiles = (g.Np + TC_BM - 1) / TC_BM, n_items = q_tiles * g.G * g.BH;
+        const ptx::WaitArgs wa = next_wait(ctx);
+        unsafe = ctx->status_dev + 2;
+        epoch = wa.epoch;
+        launch_kernel(window_f32_tc<D>, dim3(n_items < ctx->tc.n_sm ? n_items : ctx->tc.n_sm), F32_THREADS, F32Shape<D>::SMEM, st, q, k, v,
+                      out, g, ctx->readout, ctx->rd_cap, 1.0f / sqrtf((float)D), c.c_mode, wa, n_items, q_tiles, ctx->share_now,
+                      wait_first, unsafe);
+        ctx->last_launches += 1;
+        wait_first = 1;
+      }
+    }
     const auto launch = [&](auto split) {
       constexpr int WK = decltype(split)::value;
       using S = WinSimt<T, D, WK>;
       launch_kernel(window_simt<T, D, WK>, dim3((g.Np + S::BM - 1) / S::BM, g.G, g.BH), SIMT_THREADS, S::SMEM, st,
-                    q, k, v, out, g, ctx->readout, ctx->rd_cap, 1.0f / sqrtf((float)D), c.c_mode, ctx->share_now, wait_first);
+                    q, k, v, out, g, ctx->readout, ctx->rd_cap, 1.0f / sqrtf((float)D), c.c_mode, ctx->share_now, wait_first,
+                    unsafe, epoch);
     };
     // Tiles of 128 rows need the fewest loads per multiply-add; below two waves of them the SMs are better filled by
     // tiles of 32 rows whose keys are shared among four warps (2 heads x 1,071 tokens of 64 channels: 12 tiles of the one,

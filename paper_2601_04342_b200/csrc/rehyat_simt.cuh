@@ -681,8 +681,9 @@ struct WinSimt {
 template <typename T, int D, int WK>
 __global__ void __launch_bounds__(SIMT_THREADS)
 window_simt(const T* q, const T* k, const T* v, T* out, Geo g, const float* rd, int rd_rows, float scale, int c_mode,
-            float* share, int wait_first) {
+            float* share, int wait_first, const int* unsafe, int epoch) {
   if (wait_first) ptx::grid_dep_wait();                        // q, k, v may come from the direct predecessor
+  if (unsafe != nullptr && *unsafe != epoch) return;           // behind window_f32_tc, which could do all of it
   using S = WinSimt<T, D, WK>;
   extern __shared__ __align__(16) float smem[];
   constexpr int KJ = S::KJ, NQ = D / 32, RGS = 8 / WK;          // RGS: row groups of 16 per CTA

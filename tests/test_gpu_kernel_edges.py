@@ -71,3 +71,24 @@ def test_cuda_core_kernels(dtype, d, nh, T, H, W, Tc, To, Dh, Dp, P, layers):
                         phi_dim=Dp, phi_layers=layers)
     x = synth.make_inputs(wl, v_frame_offsets=True)
     _gate(_forward(wl, x, impl="simt"), _oracle(wl, x), dtype)
+
+
+# fp32 windows on the tensor cores: one to seven key tiles of 64 with remainders, several items of a CTA one after the
+# other with odd and even numbers of tiles, moving row maxima, both conventions for c.
+@pytest.mark.parametrize("d,nh,T,HW,Tc,To,c_mode", [(64, 3, 4, 129, 1, 0, "rowmax"), (128, 2, 5, 65, 1, 1, "zero"), (64, 160, 3, 65, 1, 1, "rowmax"),
+                                                    (128, 100, 6, 100, 3, 1, "rowmax"), (64, 61, 9, 43, 3, 2, "zero"), (64, 2, 3, 43, 1, 1, "rowmax"), (128, 7, 3, 150, 1, 2, "rowmax")])
+def test_fp32_window_on_the_tensor_cores(d, nh, T, HW, Tc, To, c_mode):
+    wl = synth.Workload("f32tc", 1, nh, d, T, 1, HW, Tc, To, "fp32", False, seed=synth.BASE_SEED + 404)
+    x = synth.make_inputs(wl, v_frame_offsets=True)
+    x["q"] = x["q"] * (2 if c_mode == "rowmax" else 0.5)
+    _gate(_forward(wl, x, impl="auto", c_mode=c_mode), _oracle(wl, x, c_mode=c_mode), "fp32")
+
+
+@pytest.mark.parametrize("where,value", [("k", -3.4e38), ("k", float("-inf")), ("v", float("inf")), ("q", float("nan")), ("v", 1e30),
+                                         ("q", 2.0 ** 41)])
+def test_fp32_values_that_cannot_be_split(where, value):
+    """Values beyond what the split into bf16 parts carries are computed by the CUDA-core kernel, as if it were alone."""
+    wl = synth.Workload("f32big", 1, 3, 128, 4, 10, 20, 1, 1, "fp32", False, seed=synth.BASE_SEED + 405)
+    x = synth.make_inputs(wl)
+    x[where][0, 1, 333, 5] = value
+    np.testing.assert_array_equal(_forward(wl, x, impl="auto"), _forward(wl, x, impl="simt"))
