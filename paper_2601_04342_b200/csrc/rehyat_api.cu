@@ -147,7 +147,10 @@ int set_simt_attributes() {
       cudaFuncSetAttribute(window_simt<T, D, 1>, smem, WinSimt<T, D, 1>::SMEM) != cudaSuccess ||
       cudaFuncSetAttribute(window_simt<T, D, 4>, smem, WinSimt<T, D, 4>::SMEM) != cudaSuccess)
     return REHYAT_ERR_CUDA;
-  if (sizeof(T) == 4 && cudaFuncSetAttribute(window_f32_tc<D>, smem, F32Shape<D>::SMEM) != cudaSuccess) return REHYAT_ERR_CUDA;
+  if (sizeof(T) == 4 && (cudaFuncSetAttribute(window_f32_tc<D>, smem, F32Shape<D>::SMEM) != cudaSuccess ||
+                         cudaFuncSetAttribute(phi_f32_tc<D, true>, smem, PF_SMEM) != cudaSuccess ||
+                         cudaFuncSetAttribute(phi_f32_tc<D, false>, smem, PF_SMEM) != cudaSuccess))
+    return REHYAT_ERR_CUDA;
   return REHYAT_OK;
 }
 
@@ -172,13 +175,14 @@ enum Parts : int { PART_STATE = 1 /* increments + scan */, PART_READOUT = 2, PAR
 
 // Into how many CTAs to cut a (chunk, batch*head) unit of `tiles` tiles when `units` of them run at one CTA per SM: the
 // number up to `most` that costs the fewest tile-times over all waves.
-int pick_parts(long long tiles, long long units, int most, int n_sm) {
+int pick_parts(long long tiles, long long units, int most, int n_sm, long long* cost_out = nullptr) {
   long long best = -1;
   int best_s = 1;
   for (int s = 1; s <= most; ++s) {
     const long long cost = ((units * s + n_sm - 1) / n_sm) * ((tiles + s - 1) / s);
     if (best < 0 || cost < best) { best = cost; best_s = s; }
   }
+  if (cost_out) *cost_out = best;
   return best_s;
 }
 // Chunks of the group whose linear set is not empty (at least 1).
@@ -196,12 +200,39 @@ bool use_f32_tc(const rehyat_ctx* ctx, const Geo& g) {
   return ctx->status_dev != nullptr && ctx->cfg.impl != REHYAT_IMPL_SIMT && (keys < g.N ? keys : g.N) > 128;
 }
 
+// How phi and what follows it are cut into CTAs: `parts` per (chunk, batch*head) unit, for fp32 on the tensor cores
+// (phi_f32_tc, tiles of 128 tokens) or not (tiles of 32).
+struct PhiPlan { int parts; bool f32_tc; };
+// A tile of phi_f32_tc takes about 1.2 times as long as a tile of the CUDA-core kernels (12 heads x 12,600 tokens of 128
+// channels, state: 55 us for each of 8 rounds of tiles on the SMs against 47 us for each of 28), so it is taken where it
+// needs fewer rounds: 24 heads of 64, chunks of 192 tokens 93 -> 66 us a call; one chunk of 64 tokens stays (54 us, not 65).
+PhiPlan plan_phi(const rehyat_ctx* ctx, long long tokens, long long units, int most) {
+  const int n_sm = ctx->tc.n_sm;
+  if (ctx->tensor_ok && ctx->tc.phi_ok) return {pick_parts((tokens + 127) / 128, units, most, n_sm), false};
+  long long simt = 0, tc = 0;
+  const int simt_parts = pick_parts((tokens + SIMT_TM - 1) / SIMT_TM, units, most, n_sm, &simt);
+  if (ctx->status_dev == nullptr || ctx->cfg.impl == REHYAT_IMPL_SIMT || ctx->cfg.dtype != REHYAT_DTYPE_FP32 || ctx->cfg.phi_layers > 2)
+    return {simt_parts, false};
+  const int tc_parts = pick_parts((tokens + 127) / 128, units, most, n_sm, &tc);
+  if (6 * tc < 5 * simt) return {tc_parts, true};
+  return {simt_parts, false};
+}
+PhiF32Args f32_args(rehyat_ctx* ctx, const PhiPtrs<float>& w, const PhiDims& pd, const float* x) {
+  PhiF32Args a = {};
+  a.x = x; a.W1 = w.W1; a.b1 = w.b1; a.W2 = w.W2; a.b2 = w.b2;
+  a.P = pd.P; a.act_hidden = pd.act_hidden; a.act_out = pd.act_out; a.Dh = pd.Dh; a.Dp = pd.Dp;
+  a.wa = next_wait(ctx);
+  a.unsafe = ctx->status_dev + 3;
+  return a;
+}
+
 unsigned scan_blocks(size_t per_slot) { return (unsigned)((per_slot / 4 + SCAN_THREADS - 1) / SCAN_THREADS); }
 
 template <typename T, int D>
 int launch_group_simt(rehyat_ctx* ctx, const T* q, const T* k, const T* v, T* out, const rehyat_phi_params* phi,
-                      const Geo& g, int n_split, float* state_out, const float* carry, int parts, cudaStream_t st) {
+                      const Geo& g, PhiPlan split, float* state_out, const float* carry, int parts, cudaStream_t st) {
   const rehyat_config& c = ctx->cfg;
+  const int n_split = split.parts;
   const int rd_half = ctx->tensor_ok ? 1 : 0;     // the tensor-core window kernels read the bf16 form of the read-out
   PhiDims pd = {D, c.phi_hidden, c.phi_dim, c.poly_degree, c.act_hidden, c.act_out, c.phi_layers > 2 ? c.phi_layers - 2 : 0};
   constexpr int SD = D + 4;
@@ -209,8 +240,20 @@ int launch_group_simt(rehyat_ctx* ctx, const T* q, const T* k, const T* v, T* ou
     PhiPtrs<T> wk = {(const T*)phi->k_W1, (const T*)phi->k_b1, (const T*)phi->k_W2, (const T*)phi->k_b2,
                      (const T*)phi->k_Wmid, (const T*)phi->k_bmid};
     ctx->prof.begin(REHYAT_PROF_STATE, st);
+    const int* unsafe = nullptr;
+    int epoch = 0;
+    if constexpr (sizeof(T) == 4) {
+      if (split.f32_tc) {
+        PhiF32Args a = f32_args(ctx, wk, pd, k);
+        a.v = v; a.partial = ctx->partial; a.n_split = n_split;
+        launch_kernel(phi_f32_tc<D, false>, dim3(n_split, g.G, g.BH), F32_THREADS, PF_SMEM, st, g, a);
+        ctx->last_launches += 1;
+        unsafe = a.unsafe;
+        epoch = a.wa.epoch;
+      }
+    }
     launch_kernel(state_partial_simt<T, D>, dim3(n_split, g.G, g.BH), SIMT_THREADS, simt_phi_smem(D, pd.Dh, pd.Dp, true), st,
-                  k, v, wk, pd, g, n_split, ctx->partial);
+                  k, v, wk, pd, g, n_split, ctx->partial, unsafe, epoch);
     ctx->prof.end(REHYAT_PROF_STATE, st);
     const size_t per_slot = (size_t)g.BH * pd.Dp * SD;
     ctx->prof.begin(REHYAT_PROF_SCAN, st);
@@ -221,12 +264,25 @@ int launch_group_simt(rehyat_ctx* ctx, const T* q, const T* k, const T* v, T* ou
   if (parts & PART_READOUT) {
     PhiPtrs<T> wq = {(const T*)phi->q_W1, (const T*)phi->q_b1, (const T*)phi->q_W2, (const T*)phi->q_b2,
                      (const T*)phi->q_Wmid, (const T*)phi->q_bmid};
-    const int tiles = (g.Np + SIMT_TM - 1) / SIMT_TM;
-    const int parts_rd = pick_parts(tiles, (long long)busy_readout(g) * g.BH, tiles < 64 ? tiles : 64, ctx->tc.n_sm);
-    const int per_cta = (tiles + parts_rd - 1) / parts_rd;
+    const int tiles = (g.Np + SIMT_TM - 1) / SIMT_TM, tc_tiles = (g.Np + 127) / 128;
+    const PhiPlan plan = plan_phi(ctx, g.Np, (long long)busy_readout(g) * g.BH, 64);
+    const int per_cta = (tiles + plan.parts - 1) / plan.parts;
     ctx->prof.begin(REHYAT_PROF_READOUT, st);
+    const int* unsafe = nullptr;
+    int epoch = 0;
+    if constexpr (sizeof(T) == 4) {
+      if (plan.f32_tc) {
+        PhiF32Args a = f32_args(ctx, wq, pd, q);
+        a.state = ctx->state; a.rd = ctx->readout; a.rd_rows = ctx->rd_cap;
+        a.tiles_per_cta = (tc_tiles + plan.parts - 1) / plan.parts;
+        launch_kernel(phi_f32_tc<D, true>, dim3((tc_tiles + a.tiles_per_cta - 1) / a.tiles_per_cta, g.G, g.BH), F32_THREADS, PF_SMEM, st, g, a);
+        ctx->last_launches += 1;
+        unsafe = a.unsafe;
+        epoch = a.wa.epoch;
+      }
+    }
     launch_kernel(readout_simt<T, D>, dim3((tiles + per_cta - 1) / per_cta, g.G, g.BH), SIMT_THREADS, simt_phi_smem(D, pd.Dh, pd.Dp, false), st,
-                  q, wq, pd, g, ctx->state, ctx->readout, ctx->rd_cap, rd_half, per_cta);
+                  q, wq, pd, g, ctx->state, ctx->readout, ctx->rd_cap, rd_half, per_cta, unsafe, epoch);
     ctx->prof.end(REHYAT_PROF_READOUT, st);
     ctx->last_launches += 1;
   }
@@ -266,33 +322,33 @@ int launch_group_simt(rehyat_ctx* ctx, const T* q, const T* k, const T* v, T* ou
 }
 
 // Split of a chunk's state increment over CTAs: one CTA per (split, chunk, head) and one CTA per SM.
-int pick_state_split(const rehyat_ctx* ctx, const Geo& g, int n_chunks_in_group, int tokens_per_increment) {
+PhiPlan pick_state_split(const rehyat_ctx* ctx, const Geo& g, int n_chunks_in_group, int tokens_per_increment) {
   // the buffer holds partial_units increments of bh_max problems; a call with fewer of them (one head of
   // rehyat_forward_host) has room for more splits
   const long long units = (long long)ctx->partial_units * ctx->bh_max / g.BH;
   int most = (int)(units / (n_chunks_in_group > 0 ? n_chunks_in_group : 1));
   if (most > 16) most = 16;                         // a lone chunk (a chunk-by-chunk step) over all SMs
   if (most < 1) most = 1;
-  const int tile = ctx->tensor_ok && ctx->tc.phi_ok ? 128 : SIMT_TM;
   int busy = 0;                                     // chunks of the group that admit keys into the state
   for (int t = g.t0 > 1 ? g.t0 : 1; t < g.t0 + n_chunks_in_group; ++t) busy += geo_lo(g, t) > geo_lo(g, t - 1);
-  return pick_parts((tokens_per_increment + tile - 1) / tile, (long long)(busy > 0 ? busy : 1) * g.BH, most, ctx->tc.n_sm);
+  return plan_phi(ctx, tokens_per_increment, (long long)(busy > 0 ? busy : 1) * g.BH, most);
 }
 
 // Enqueues the requested steps for the chunks [g.t0, g.t0 + g.G) with whichever kernel family the context uses.
 // PART_STATE writes the states of the chunks to `state_out` (the context's state slots, or slots of `cum`), starting
 // from `carry` (null: zero).
 int run_parts(rehyat_ctx* ctx, const void* q, const void* k, const void* v, void* out, const rehyat_phi_params* phi,
-              const Geo& g, int batch, int n_split, float* state_out, const float* carry, int parts, cudaStream_t st) {
+              const Geo& g, int batch, PhiPlan split, float* state_out, const float* carry, int parts, cudaStream_t st) {
   const rehyat_config& c = ctx->cfg;
+  const int n_split = split.parts;
   int rc = REHYAT_OK;
   if (ctx->tensor_ok) {
     using B = __nv_bfloat16;
     if (!ctx->tc.phi_ok) {
       rc = c.head_dim == 64
-               ? launch_group_simt<B, 64>(ctx, (const B*)q, (const B*)k, (const B*)v, (B*)out, phi, g, n_split, state_out, carry,
+               ? launch_group_simt<B, 64>(ctx, (const B*)q, (const B*)k, (const B*)v, (B*)out, phi, g, split, state_out, carry,
                                           parts & (PART_STATE | PART_READOUT), st)
-               : launch_group_simt<B, 128>(ctx, (const B*)q, (const B*)k, (const B*)v, (B*)out, phi, g, n_split, state_out, carry,
+               : launch_group_simt<B, 128>(ctx, (const B*)q, (const B*)k, (const B*)v, (B*)out, phi, g, split, state_out, carry,
                                            parts & (PART_STATE | PART_READOUT), st);
     } else {
       if (parts & PART_STATE) {
@@ -326,13 +382,13 @@ int run_parts(rehyat_ctx* ctx, const void* q, const void* k, const void* v, void
     }
   } else if (c.dtype == REHYAT_DTYPE_FP32) {
     rc = c.head_dim == 64
-             ? launch_group_simt<float, 64>(ctx, (const float*)q, (const float*)k, (const float*)v, (float*)out, phi, g, n_split, state_out, carry, parts, st)
-             : launch_group_simt<float, 128>(ctx, (const float*)q, (const float*)k, (const float*)v, (float*)out, phi, g, n_split, state_out, carry, parts, st);
+             ? launch_group_simt<float, 64>(ctx, (const float*)q, (const float*)k, (const float*)v, (float*)out, phi, g, split, state_out, carry, parts, st)
+             : launch_group_simt<float, 128>(ctx, (const float*)q, (const float*)k, (const float*)v, (float*)out, phi, g, split, state_out, carry, parts, st);
   } else {
     using B = __nv_bfloat16;
     rc = c.head_dim == 64
-             ? launch_group_simt<B, 64>(ctx, (const B*)q, (const B*)k, (const B*)v, (B*)out, phi, g, n_split, state_out, carry, parts, st)
-             : launch_group_simt<B, 128>(ctx, (const B*)q, (const B*)k, (const B*)v, (B*)out, phi, g, n_split, state_out, carry, parts, st);
+             ? launch_group_simt<B, 64>(ctx, (const B*)q, (const B*)k, (const B*)v, (B*)out, phi, g, split, state_out, carry, parts, st)
+             : launch_group_simt<B, 128>(ctx, (const B*)q, (const B*)k, (const B*)v, (B*)out, phi, g, split, state_out, carry, parts, st);
   }
   return rc;
 }
@@ -640,7 +696,7 @@ int rehyat_forward(rehyat_ctx* ctx, const void* q, const void* k, const void* v,
   if (G < 1) return REHYAT_ERR_INVALID_ARG;   // cannot happen: rd_rows >= max chunk size
   if (G > ctx->Gmax) G = ctx->Gmax;
   g.t0 = 0;
-  const int n_split = pick_state_split(ctx, g, G < n_chunks ? G : n_chunks, g.Np);
+  const PhiPlan split = pick_state_split(ctx, g, G < n_chunks ? G : n_chunks, g.Np);
 
   ctx->last_launches = 0;
   ctx->last_impl = ctx->tensor_ok ? (ctx->tc.phi_ok ? 2 : 1) : 0;
@@ -666,7 +722,7 @@ int rehyat_forward(rehyat_ctx* ctx, const void* q, const void* k, const void* v,
     for (int f0 = 1; f0 <= frames; f0 += ctx->Gmax) {
       gs.t0 = f0;                                // "chunk" f admits frame f-1: [lo_{f-1}, lo_f) = [(f-1) HW, f HW)
       gs.G = frames + 1 - f0 < ctx->Gmax ? frames + 1 - f0 : ctx->Gmax;
-      const int ns = pick_state_split(ctx, gs, gs.G, (int)HW);
+      const PhiPlan ns = pick_state_split(ctx, gs, gs.G, (int)HW);
       float* cum = ctx->cum + (size_t)f0 * per_slot;
       const int rc = run_parts(ctx, nullptr, k, v, nullptr, phi, gs, batch, ns, cum, f0 > 1 ? cum - per_slot : nullptr, PART_STATE, st);
       if (rc != REHYAT_OK) return rc;
@@ -679,7 +735,7 @@ int rehyat_forward(rehyat_ctx* ctx, const void* q, const void* k, const void* v,
           ctx->cum, ctx->state, per_slot, g, (int)HW, frames,
           (ctx->tensor_ok && ctx->tc.phi_ok) ? ctx->tc.state_bf16 : nullptr, c.head_dim);
       ctx->last_launches += 1;
-      const int rc = run_parts(ctx, q, k, v, out, phi, g, batch, 1, nullptr, nullptr, PART_READOUT | PART_WINDOW, st);
+      const int rc = run_parts(ctx, q, k, v, out, phi, g, batch, {1, false}, nullptr, nullptr, PART_READOUT | PART_WINDOW, st);
       if (rc != REHYAT_OK) return rc;
     }
     return REHYAT_OK;
@@ -690,7 +746,7 @@ int rehyat_forward(rehyat_ctx* ctx, const void* q, const void* k, const void* v,
     g.t0 = t0;
     g.G = (n_chunks - t0) < G ? (n_chunks - t0) : G;
     const bool any_linear = geo_lo(g, t0 + g.G - 1) > 0;
-    const int rc = run_parts(ctx, q, k, v, out, phi, g, batch, n_split, ctx->state, carry,
+    const int rc = run_parts(ctx, q, k, v, out, phi, g, batch, split, ctx->state, carry,
                              (any_linear ? PART_STATE | PART_READOUT : 0) | PART_WINDOW, st);
     if (rc != REHYAT_OK) return rc;
     if (any_linear) carry = ctx->state + (size_t)(g.G - 1) * per_slot;
@@ -921,7 +977,7 @@ int rehyat_stream_step(rehyat_ctx* ctx, const void* q_chunk, const void* k_chunk
   g.q_off = h; g.Nq = Np;
   ctx->share_now = nullptr;
   ctx->last_impl = ctx->tensor_ok ? (ctx->tc.phi_ok ? 2 : 1) : 0;
-  int rc = run_parts(ctx, q_used, kwin, vwin, out_chunk, phi, g, s.batch, 1, nullptr, nullptr, (s.has_state ? PART_READOUT : 0) | PART_WINDOW, st);
+  int rc = run_parts(ctx, q_used, kwin, vwin, out_chunk, phi, g, s.batch, {1, false}, nullptr, nullptr, (s.has_state ? PART_READOUT : 0) | PART_WINDOW, st);
   if (rc != REHYAT_OK) return rc;
   // 3. Eq. 17-18: the tokens that leave the window before the next chunk enter the running state
   const int keep = (long long)s.overlap * HW < (long long)h + Np ? s.overlap * HW : h + Np;
@@ -929,8 +985,8 @@ int rehyat_stream_step(rehyat_ctx* ctx, const void* q_chunk, const void* k_chunk
   if (leave > 0) {
     Geo gs = g;
     gs.Np = leave; gs.ToHW = 0; gs.q_shift = 0; gs.prefix = 0; gs.t0 = 1; gs.G = 1;   // increment of "chunk 1" = [0, leave)
-    const int n_split = pick_state_split(ctx, gs, 1, leave);
-    rc = run_parts(ctx, nullptr, kwin, vwin, nullptr, phi, gs, s.batch, n_split, ctx->state, s.has_state ? ctx->state : nullptr,
+    const PhiPlan split = pick_state_split(ctx, gs, 1, leave);
+    rc = run_parts(ctx, nullptr, kwin, vwin, nullptr, phi, gs, s.batch, split, ctx->state, s.has_state ? ctx->state : nullptr,
                    PART_STATE, st);
     if (rc != REHYAT_OK) return rc;
     s.has_state = 1;

@@ -348,4 +348,440 @@ window_f32_tc(const float* q, const float* k, const float* v, float* out, Geo g,
   }
 }
 
+// ---------------------------------------------------------------------------------------------
+// phi_f32_tc: the feature map of the fp32 operator on the tensor cores, with the contraction that consumes it:
+// the state increment phi_k(K)^T [V | 1] (READOUT = false, Eq. 17-18) or the read-out phi_q(Q) s_t, phi_q(Q) z_t (true,
+// Eq. 7, 9, 16).  Two-layer maps, widths up to 256 in steps of 8.  Operands are split as in window_f32_tc.
+//
+//   A tile of 128 tokens is a chain of passes of 64 output columns through one pair of accumulators, the small terms of
+//   the split products in one, h h in the other, so that a sum rounds in no more than K / 16 large steps:
+//     H quarters   X W1^T          -> bias, activation, split -> H planes in TMEM (A operand of the next)
+//     U quarters   H W2^T          -> bias, activation, power, split -> phi planes in the space of X, 128 features at a time
+//     consumer     phi s_t         -> added to the read-out in registers            (READOUT)
+//                  phi^T V         -> added to the CTA's partial state in global memory (L2), fp32
+//   warps 0-7   epilogues, two threads per token (TMEM lane) with 32 columns each
+//   warps 8-11  loaders: X, and weights, states or V through a ring of two stages of three planes, split on the way
+//   warp 12     UMMA issuer
+//   TMEM: accumulators [0, 128), H planes [128, 512).
+// A pass waits for the epilogue of the one before: the chain is what bounds a tile (37,000 cycles of MMAs at the default
+// widths, about as long again in hand-overs and epilogues).  12 heads x 12,600 tokens of 128 channels against the
+// CUDA-core kernels: state 1,319 -> 445 us, read-out 1,284 -> 402 us.
+// ---------------------------------------------------------------------------------------------
+struct PhiF32Args {
+  const float *x, *v, *W1, *b1, *W2, *b2, *state;
+  float *rd, *partial;
+  int P, act_hidden, act_out, Dh, Dp, n_split, tiles_per_cta, rd_rows;
+  ptx::WaitArgs wa;
+  int* unsafe;
+};
+struct PhiF32Bars {
+  uint64_t x_full, x_empty, ring_full[2], ring_empty[2], acc_ready, epi_done, drained;
+  uint32_t tmem_base;
+  ptx::WaitCtx wctx;
+  float b1[256], b2[256], z[256];
+  float sums[4][256];          // READOUT: [half][token] shares of phi z_t; else [TMEM quadrant][feature] sums of phi
+};
+constexpr int PF_XPLANE = 128 * 128 * 2, PF_SPLANE = 16384, PF_STAGE = 3 * PF_SPLANE;
+constexpr int PF_SMEM = 3 * PF_XPLANE + 2 * PF_STAGE + (int)sizeof(PhiF32Bars) + 16 + 1024;
+
+template <int D, bool READOUT>
+__global__ void __launch_bounds__(F32_THREADS, 1)
+phi_f32_tc(Geo g, PhiF32Args a) {
+  using namespace ptx;
+  constexpr int SD = D + 4, ND = D / 64;
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t sb = (smem_u32(smem_raw) + 1023u) & ~1023u, s_ring = sb + 3 * PF_XPLANE;
+  uint8_t* smem = smem_raw + (sb - smem_u32(smem_raw));
+  PhiF32Bars* bars = reinterpret_cast<PhiF32Bars*>(smem + 3 * PF_XPLANE + 2 * PF_STAGE);
+  const uint32_t wc = smem_u32(&bars->wctx);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int ci = blockIdx.y, bh = blockIdx.z, t = g.t0 + ci, head = bh % g.n_heads;
+  const int Dh = a.Dh, Dp = a.Dp, nqh = (Dh + 63) >> 6, nqu = (Dp + 63) >> 6, n_half = (nqu + 1) >> 1, ksu = (nqh + 1) >> 1;
+
+  // the tokens [tok_a, tok_b) of this CTA
+  int tok_a, tok_b;
+  float* part = nullptr;
+  if (READOUT) {
+    if (!geo_linear(g, t)) return;
+    const int q0 = geo_q0(g, t), q1 = geo_q1(g, t);
+    tok_a = min(q0 + (int)blockIdx.x * a.tiles_per_cta * 128, q1);
+    tok_b = min(tok_a + a.tiles_per_cta * 128, q1);
+    if (tok_a >= tok_b) return;
+  } else {
+    const int lo_prev = t > 0 ? geo_lo(g, t - 1) : 0, lo = geo_lo(g, t);
+    int per = (lo - lo_prev + a.n_split - 1) / a.n_split;
+    per = (per + 127) / 128 * 128;
+    tok_a = min(lo_prev + (int)blockIdx.x * per, lo);
+    tok_b = min(tok_a + per, lo);
+    part = a.partial + (((size_t)ci * a.n_split + blockIdx.x) * g.BH + bh) * Dp * SD;
+    if (tok_a >= tok_b) {                                            // nothing admitted: the partial is zero
+      grid_dep_wait();
+      grid_dep_launch();
+      for (int i = threadIdx.x; i < Dp * SD / 4; i += F32_THREADS) reinterpret_cast<float4*>(part)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      return;
+    }
+  }
+  const int n_tiles = (tok_b - tok_a + 127) / 128;
+
+  if (threadIdx.x == 0) {
+    mbar_init(smem_u32(&bars->x_full), F32_LOAD_WARPS); mbar_init(smem_u32(&bars->x_empty), 1);
+    for (int s = 0; s < 2; ++s) { mbar_init(smem_u32(&bars->ring_full[s]), F32_LOAD_WARPS); mbar_init(smem_u32(&bars->ring_empty[s]), 1); }
+    mbar_init(smem_u32(&bars->acc_ready), 1); mbar_init(smem_u32(&bars->epi_done), F32_SOFTMAX_WARPS);
+    mbar_init(smem_u32(&bars->drained), 1);
+    wait_ctx_init(&bars->wctx, a.wa);
+    fence_mbar_init();
+  }
+  if (warp == 12) {
+    tmem_alloc(smem_u32(&bars->tmem_base), 512);
+    tmem_relinquish();
+  }
+  if (!READOUT) {                                                    // k may come from the direct predecessor
+    grid_dep_wait();
+    grid_dep_launch();
+  }
+  for (int i = threadIdx.x; i < 256; i += F32_THREADS) {             // zero beyond the widths
+    bars->b1[i] = i < Dh ? a.b1[(size_t)head * Dh + i] : 0.f;
+    bars->b2[i] = i < Dp ? a.b2[(size_t)head * Dp + i] : 0.f;
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = bars->tmem_base;
+  constexpr uint32_t T_H = 128, H_PLANE = 128;
+
+  if (warp >= 8 && warp < 12) {
+    // ------------------------------------------------------------------ loaders
+    const int tl = threadIdx.x - 256;
+    uint32_t big = 0, n_st = 0;
+    bool alive = !a.wa.withhold_loads;
+    float4 x[8][2];
+    // 1,024 chunks of eight columns, of 64 rows x 128 columns (wide) or 128 rows x 64; zeros beyond rows and cols
+    auto fetch = [&](const float* src, long long stride, int rows, int cols, bool wide) {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int c = tl + 128 * u, r = wide ? c >> 4 : c >> 3, col = (wide ? c & 15 : c & 7) * 8;
+        x[u][0] = x[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (r < rows && col < cols) {
+          const float* p = src + (long long)r * stride + col;
+          x[u][0] = ld4(p); x[u][1] = ld4(p + 4);
+        }
+      }
+    };
+    auto put = [&](uint32_t dst, uint32_t plane, uint32_t sub, int row0, bool wide) {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int c = tl + 128 * u, r = row0 + (wide ? c >> 4 : c >> 3), col = (wide ? c & 15 : c & 7) * 8;
+        big = max_bits(max_bits(big, x[u][0]), x[u][1]);
+        uint4 h, m, l;
+        split3(x[u][0].x, x[u][0].y, h.x, m.x, l.x); split3(x[u][0].z, x[u][0].w, h.y, m.y, l.y);
+        split3(x[u][1].x, x[u][1].y, h.z, m.z, l.z); split3(x[u][1].z, x[u][1].w, h.w, m.w, l.w);
+        st_tile_chunk_sw128(dst, sub, r, col, h);
+        st_tile_chunk_sw128(dst + plane, sub, r, col, m);
+        st_tile_chunk_sw128(dst + 2 * plane, sub, r, col, l);
+      }
+    };
+    auto wait = [&](uint64_t* bar, uint32_t parity) {
+      alive = alive && __all_sync(0xffffffffu, mbar_wait(smem_u32(bar), parity, wc, PH_ERR_LOAD));
+      return alive;
+    };
+    auto stage = [&](const float* src, long long stride, int rows, int cols, bool wide) {
+      if (!alive) return;
+      fetch(src, stride, rows, cols, wide);
+      const uint32_t s = n_st & 1;
+      if (!wait(&bars->ring_empty[s], ((n_st >> 1) & 1) ^ 1)) return;
+      put(s_ring + s * PF_STAGE, PF_SPLANE, 8192, 0, wide);
+      fence_proxy_async_smem();
+      mbar_arrive_warp(smem_u32(&bars->ring_full[s]), lane);
+      ++n_st;
+    };
+    const float* xh = READOUT ? a.x + q_row_offset(g, bh, 0) : a.x + head_offset(g, bh);
+    const long long xs = READOUT ? g.qstride_n : g.stride_n;
+    const float* W1 = a.W1 + (size_t)head * Dh * D;
+    const float* W2 = a.W2 + (size_t)head * Dp * Dh;
+    const float* S = READOUT ? a.state + ((size_t)ci * g.BH + bh) * Dp * SD : nullptr;
+    const float* V = READOUT ? nullptr : a.v + head_offset(g, bh);
+    for (int j = 0; j < n_tiles && alive; ++j) {
+      const int tok0 = tok_a + j * 128, rows = min(128, tok_b - tok0);
+      constexpr int PIECES = D / 64;                                 // of 64 rows x 128 columns, or one of 128 x 64
+      if (!wait(&bars->x_empty, (j & 1) ^ 1)) break;
+#pragma unroll 1
+      for (int p = 0; p < PIECES; ++p) {
+        fetch(xh + (long long)(tok0 + p * 64) * xs, xs, rows - p * 64, D, D == 128);
+        put(sb, PF_XPLANE, 16384, p * 64, D == 128);
+      }
+      fence_proxy_async_smem();
+      mbar_arrive_warp(smem_u32(&bars->x_full), lane);
+#pragma unroll 1
+      for (int q = 0; q < nqh; ++q) stage(W1 + (size_t)q * 64 * D, D, Dh - q * 64, D, true);
+#pragma unroll 1
+      for (int hf = 0; hf < n_half; ++hf) {
+#pragma unroll 1
+        for (int q = 2 * hf; q < min(2 * hf + 2, nqu); ++q)
+#pragma unroll 1
+          for (int s = 0; s < ksu; ++s) stage(W2 + (size_t)q * 64 * Dh + s * 128, Dh, Dp - q * 64, Dh - s * 128, true);
+#pragma unroll 1
+        for (int dh = 0; dh < ND; ++dh) {
+          if (READOUT) {
+            grid_dep_wait();                                         // the states are the predecessor's results
+            stage(S + (size_t)hf * 128 * SD + dh * 64, SD, Dp - hf * 128, 64, false);
+          } else {
+            stage(V + (long long)tok0 * g.stride_n + dh * 64, g.stride_n, rows, 64, false);
+          }
+        }
+      }
+    }
+    if (big >= F32_UNSAFE_BITS) *a.unsafe = a.wa.epoch;
+  } else if (warp == 12) {
+    // ------------------------------------------------------------------ UMMA issuer
+    if (elect_one()) {
+      constexpr uint32_t id_kk = idesc_bf16(128, 64, 0, 0), id_cons = READOUT ? idesc_bf16(128, 64, 0, 1) : idesc_bf16(128, 64, 1, 1);
+      constexpr int PA[6] = {2, 0, 1, 1, 0, 0}, PB[6] = {0, 2, 1, 0, 1, 0};
+      uint32_t n_st = 0, n_pass = 0;
+      bool alive = true;
+      auto wait = [&](uint64_t* bar, uint32_t parity) {
+        alive = alive && mbar_wait(smem_u32(bar), parity, wc, PH_ERR_MMA);
+        if (alive) tc_fence_after();
+        return alive;
+      };
+      const uint64_t d_x = smem_desc_sw128(sb, 16, 1024), d_phi_mn = smem_desc_sw128(sb, 16384, 1024), d_b = smem_desc_sw128(s_ring, 16, 1024);
+      // waits for the ring's next stage and issues its share of a pass: `ksteps` times 16 terms of the six products
+      auto share = [&](bool first, int ksteps, auto&& mma) {
+        const uint32_t s = n_st & 1;
+        if (!wait(&bars->ring_full[s], (n_st >> 1) & 1)) return;
+        const uint64_t db = smem_desc_advance(d_b, s * PF_STAGE);
+#pragma unroll
+        for (int p = 0; p < 6; ++p)
+#pragma unroll 1
+          for (int kk = 0; kk < ksteps; ++kk)
+            mma(tmem + (p == 5 ? 64 : 0), PA[p], kk, smem_desc_advance(db, PB[p] * PF_SPLANE), (!first || kk > 0 || (p > 0 && p < 5)) ? 1u : 0u);
+        umma_commit(smem_u32(&bars->ring_empty[s]));
+        ++n_st;
+      };
+      auto begin = [&]() { return n_pass == 0 || wait(&bars->epi_done, (n_pass - 1) & 1); };
+      auto end = [&]() { if (alive) { umma_commit(smem_u32(&bars->acc_ready)); ++n_pass; } };
+      const auto k_off = [](int kk, uint32_t sub) { return (kk >> 2) * sub + (kk & 3) * 32; };   // K-major image
+      for (int j = 0; j < n_tiles && alive; ++j) {
+        if (!wait(&bars->x_full, j & 1)) break;
+        for (int q = 0; q < nqh && alive; ++q) {
+          if (!begin()) break;
+          share(true, D / 16, [&](uint32_t d, int p, int kk, uint64_t db, uint32_t acc) {
+            umma_ss(d, smem_desc_advance(d_x, p * PF_XPLANE + k_off(kk, 16384)), smem_desc_advance(db, k_off(kk, 8192)), id_kk, acc);
+          });
+          end();
+        }
+        for (int hf = 0; hf < n_half && alive; ++hf) {
+          const int nq = min(2, nqu - 2 * hf);
+          for (int q = 0; q < nq && alive; ++q) {
+            if (!begin()) break;
+            for (int s = 0; s < ksu && alive; ++s)
+              share(s == 0, min(8, nqh * 4 - s * 8), [&](uint32_t d, int p, int kk, uint64_t db, uint32_t acc) {
+                umma_ts(d, tmem + T_H + p * H_PLANE + (s * 8 + kk) * 8, smem_desc_advance(db, k_off(kk, 8192)), id_kk, acc);
+              });
+            end();
+          }
+          for (int dh = 0; dh < ND && alive; ++dh) {
+            if (!begin()) break;
+            if (READOUT)
+              share(true, nq * 4, [&](uint32_t d, int p, int kk, uint64_t db, uint32_t acc) {
+                umma_ss(d, smem_desc_advance(d_x, p * PF_XPLANE + k_off(kk, 16384)), smem_desc_advance(db, kk * 2048), id_cons, acc);
+              });
+            else
+              share(true, 8, [&](uint32_t d, int p, int kk, uint64_t db, uint32_t acc) {
+                umma_ss(d, smem_desc_advance(d_phi_mn, p * PF_XPLANE + kk * 2048), smem_desc_advance(db, kk * 2048), id_cons, acc);
+              });
+            end();
+          }
+        }
+        if (alive) umma_commit(smem_u32(&bars->x_empty));
+      }
+      umma_commit(smem_u32(&bars->drained));                         // as in window_f32_tc
+      mbar_wait_drain(smem_u32(&bars->drained), 0, wc);
+    }
+  } else {
+    // ------------------------------------------------------------------ epilogues
+    const int half = warp >> 2, qd = warp & 3, r = qd * 32 + lane;
+    const uint32_t tb = tmem + ((uint32_t)(qd * 32) << 16);
+    const int part_w = Dp / a.P;
+    // as in window_f32_tc: a wait given up returns at once, the warps leave together at the head of a tile
+    uint32_t n_pass = 0, big = 0;
+    auto barrier = [&](bool flag) -> bool {
+      uint32_t any;
+      asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbarrier.cta.red.or.pred q, 1, 256, p;\n\tselp.b32 %0, 1, 0, q;\n\t}"
+                   : "=r"(any) : "r"((uint32_t)flag) : "memory");
+      return any != 0;
+    };
+    auto acc_wait = [&]() {
+      mbar_wait(smem_u32(&bars->acc_ready), n_pass & 1, wc, PH_ERR_EPI);
+      __syncwarp();
+      ++n_pass;
+      tc_fence_after();
+    };
+    auto acc_done = [&]() {
+      tc_fence_before();
+      mbar_arrive_warp(smem_u32(&bars->epi_done), lane);
+    };
+    // 16 columns of the pass from column `half * 32 + c` on: both accumulators, bias and activation
+    auto activated = [&](int c, const float* bias, int act, float (&y)[16]) {
+      uint32_t lo[16], hi[16];
+      tmem_ld16(tb + half * 32 + c, lo);
+      tmem_ld16(tb + 64 + half * 32 + c, hi);
+      tmem_wait_ld();
+#pragma unroll
+      for (int e = 0; e < 16; ++e) y[e] = (__uint_as_float(lo[e]) + __uint_as_float(hi[e])) + bias[half * 32 + c + e];
+      if (act == ACT_RELU) {
+#pragma unroll
+        for (int e = 0; e < 16; ++e) y[e] = fmaxf(y[e], 0.f);
+      } else {
+#pragma unroll
+        for (int e = 0; e < 16; ++e) y[e] = apply_act(y[e], act);
+      }
+    };
+    if (READOUT) {
+      grid_dep_wait();
+      grid_dep_launch();
+      bars->z[threadIdx.x] = (int)threadIdx.x < Dp ? a.state[(((size_t)ci * g.BH + bh) * Dp + threadIdx.x) * SD + D] : 0.f;
+    }
+    for (int j = 0; j < n_tiles; ++j) {
+      if (barrier(wait_ctx_aborted(wc) != 0)) break;                 // (and z is there, the last tile's sums have been read)
+      const int tok0 = tok_a + j * 128;
+      const bool tok_valid = tok0 + r < tok_b;
+#pragma unroll 1
+      for (int q = 0; q < nqh; ++q) {
+        acc_wait();
+#pragma unroll 1
+        for (int c = 0; c < 32; c += 16) {
+          float y[16];
+          uint32_t h[8], m[8], l[8];
+          activated(c, bars->b1 + q * 64, a.act_hidden, y);
+#pragma unroll
+          for (int e = 0; e < 16; e += 2) {
+            big = max(big, max(abs_bits(y[e]), abs_bits(y[e + 1])));
+            split3(y[e], y[e + 1], h[e / 2], m[e / 2], l[e / 2]);
+          }
+          const uint32_t col = tb + T_H + (q * 64 + half * 32 + c) / 2;
+          tmem_st8(col, h); tmem_st8(col + H_PLANE, m); tmem_st8(col + 2 * H_PLANE, l);
+        }
+        tmem_wait_st();
+        acc_done();
+      }
+      float nl = 0.f;
+      uint64_t racc[READOUT ? ND : 1][16];
+#pragma unroll 1
+      for (int hf = 0; hf < n_half; ++hf) {
+#pragma unroll 1
+        for (int q = 2 * hf; q < min(2 * hf + 2, nqu); ++q) {
+          acc_wait();
+#pragma unroll 1
+          for (int c = 0; c < 32; c += 16) {
+            float y[16];
+            activated(c, bars->b2 + q * 64, a.act_out, y);
+            const int f0 = q * 64 + half * 32 + c;                   // feature of the first column
+#pragma unroll
+            for (int e = 0; e < 16; ++e) {
+              const int f = f0 + e, part_f = f / part_w;
+              const float u = y[e];
+              float p = u;
+              if (part_f >= 1) p *= u;
+              if (part_f >= 2) p *= u;
+              if (part_f >= 3) p *= u;
+              y[e] = tok_valid && f < Dp ? p : 0.f;
+              big = max(big, abs_bits(y[e]));
+              if (READOUT) nl = fmaf(y[e], bars->z[f], nl);
+            }
+#pragma unroll
+            for (int e = 0; e < 16; e += 8) {
+              uint4 h, m, l;
+              split3(y[e], y[e + 1], h.x, m.x, l.x); split3(y[e + 2], y[e + 3], h.y, m.y, l.y);
+              split3(y[e + 4], y[e + 5], h.z, m.z, l.z); split3(y[e + 6], y[e + 7], h.w, m.w, l.w);
+              const int col = (q & 1) * 64 + half * 32 + c + e;
+              st_tile_chunk_sw128(sb, 16384, r, col, h);
+              st_tile_chunk_sw128(sb + PF_XPLANE, 16384, r, col, m);
+              st_tile_chunk_sw128(sb + 2 * PF_XPLANE, 16384, r, col, l);
+            }
+            if (!READOUT) {
+              // column sums over the warp's 32 tokens: a lane keeps half of the columns at each of four steps
+#pragma unroll
+              for (int o = 8; o; o >>= 1) {
+                const bool up = (lane & o) != 0;
+#pragma unroll
+                for (int e = 0; e < o; ++e) {
+                  const float keep = up ? y[e + o] : y[e], give = up ? y[e] : y[e + o];
+                  y[e] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+                }
+              }
+              y[0] += __shfl_xor_sync(0xffffffffu, y[0], 16);
+              if (lane < 16) bars->sums[qd][f0 + lane] = j == 0 ? y[0] : bars->sums[qd][f0 + lane] + y[0];
+            }
+          }
+          fence_proxy_async_smem();
+          acc_done();
+        }
+#pragma unroll
+        for (int dh = 0; dh < ND; ++dh) {
+          acc_wait();
+          uint32_t lo[32], hi[32];
+          tmem_ld32(tb + half * 32, lo);
+          tmem_ld32(tb + 64 + half * 32, hi);
+          tmem_wait_ld();
+          acc_done();
+#pragma unroll
+          for (int e = 0; e < 32; e += 2) {
+            const uint64_t y = add2(pk2u(lo[e], lo[e + 1]), pk2u(hi[e], hi[e + 1]));
+            if constexpr (READOUT) {
+              racc[dh][e / 2] = hf == 0 ? y : add2(racc[dh][e / 2], y);
+            } else {
+              upk2u(y, lo[e], lo[e + 1]);
+            }
+          }
+          if (!READOUT) {
+            const int f = hf * 128 + r;                              // TMEM lane = feature
+            if (f < Dp && !wait_ctx_aborted(wc)) {
+              float4* p = reinterpret_cast<float4*>(part + (size_t)f * SD + dh * 64 + half * 32);
+#pragma unroll
+              for (int e = 0; e < 8; ++e) {
+                float4 y = make_float4(__uint_as_float(lo[4 * e]), __uint_as_float(lo[4 * e + 1]), __uint_as_float(lo[4 * e + 2]),
+                                       __uint_as_float(lo[4 * e + 3]));
+                if (j > 0) y = add4(p[e], y);
+                p[e] = y;
+              }
+            }
+          }
+        }
+      }
+      if constexpr (READOUT) {
+        bars->sums[half][r] = nl;
+        if (barrier(wait_ctx_aborted(wc) != 0)) break;
+        if (tok_valid) {
+          const int ric = tok0 + r - geo_q0(g, t);
+#pragma unroll
+          for (int dh = 0; dh < ND; ++dh)
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+              float y[4];
+              upk2(racc[dh][2 * e], y[0], y[1]);
+              upk2(racc[dh][2 * e + 1], y[2], y[3]);
+              *reinterpret_cast<float4*>(a.rd + rd_index(g, a.rd_rows, D, bh, ci, ric, (dh * 64 + half * 32) / 4 + e)) =
+                  make_float4(y[0], y[1], y[2], y[3]);
+            }
+          if (half == 0) a.rd[rd_index(g, a.rd_rows, D, bh, ci, ric, D / 4)] = bars->sums[0][r] + bars->sums[1][r];
+        }
+      }
+    }
+    if (!READOUT && !barrier(wait_ctx_aborted(wc) != 0)) {
+      const int f = threadIdx.x;
+      if (f < Dp)
+        *reinterpret_cast<float4*>(part + (size_t)f * SD + D) =
+            make_float4((bars->sums[0][f] + bars->sums[1][f]) + (bars->sums[2][f] + bars->sums[3][f]), 0.f, 0.f, 0.f);
+    }
+    if (big >= F32_UNSAFE_BITS) *a.unsafe = a.wa.epoch;
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 12) {
+    tc_fence_after();
+    tmem_dealloc(tmem, 512);
+  }
+}
+
 }  // namespace rehyat

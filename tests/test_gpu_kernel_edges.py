@@ -87,8 +87,23 @@ def test_fp32_window_on_the_tensor_cores(d, nh, T, HW, Tc, To, c_mode):
 @pytest.mark.parametrize("where,value", [("k", -3.4e38), ("k", float("-inf")), ("v", float("inf")), ("q", float("nan")), ("v", 1e30),
                                          ("q", 2.0 ** 41)])
 def test_fp32_values_that_cannot_be_split(where, value):
-    """Values beyond what the split into bf16 parts carries are computed by the CUDA-core kernel, as if it were alone."""
+    """Values beyond what the split into bf16 parts carries are computed by the CUDA-core kernels, as if they were alone (the
+    state sums of the two calls are split differently over CTAs: fp32 sums in another order)."""
     wl = synth.Workload("f32big", 1, 3, 128, 4, 10, 20, 1, 1, "fp32", False, seed=synth.BASE_SEED + 405)
     x = synth.make_inputs(wl)
     x[where][0, 1, 333, 5] = value
-    np.testing.assert_array_equal(_forward(wl, x, impl="auto"), _forward(wl, x, impl="simt"))
+    np.testing.assert_allclose(_forward(wl, x, impl="auto"), _forward(wl, x, impl="simt"), rtol=1e-5, atol=1e-6)
+
+
+# fp32 phi on the tensor cores: widths that end inside quarters of 64 and halves of 128 columns, chunks that end inside
+# tiles of 128 tokens, several tiles of a CTA, all degrees and activations (more than one round of tiles of 32 on the SMs).
+# The features are non-negative: with both signs the denominator of Eq. 5 may vanish and no tolerance holds.
+@pytest.mark.parametrize("d,nh,T,HW,Tc,To,Dh,Dp,P,act_hidden,act_out", [
+    (64, 60, 6, 150, 1, 0, 8, 8, 1, "relu", "relu"), (128, 60, 6, 150, 1, 0, 72, 136, 2, "gelu", "softplus"),
+    (128, 40, 7, 129, 3, 1, 256, 256, 4, "relu", "relu"), (64, 40, 7, 100, 3, 2, 200, 192, 3, "elu1", "elu1"),
+    (64, 4, 9, 400, 4, 1, 128, 128, 2, "relu", "relu"), (128, 6, 9, 410, 4, 1, 64, 64, 2, "identity", "softplus")])
+def test_fp32_phi_on_the_tensor_cores(d, nh, T, HW, Tc, To, Dh, Dp, P, act_hidden, act_out):
+    wl = synth.Workload("f32phi", 1, nh, d, T, 1, HW, Tc, To, "fp32", False, P=P, seed=synth.BASE_SEED + 406, phi_hidden=Dh, phi_dim=Dp)
+    x = synth.make_inputs(wl, v_frame_offsets=True, phi_scale=2.0)
+    y = _forward(wl, x, act_hidden=act_hidden, act_out=act_out)
+    _gate(y, _oracle(wl, x, act_hidden=act_hidden, act_out=act_out), "fp32")
