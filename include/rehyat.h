@@ -60,8 +60,9 @@ typedef enum { REHYAT_C_ROWMAX = 0, REHYAT_C_ZERO = 1 } rehyat_c_mode;
 /* Kernel family.  AUTO: tensor-core (tcgen05) kernels when dtype is bf16 (head_dim 64 or 128 for
  * the softmax window; for phi, state and read-out also D_h and D' multiples of 32 with
  * 64 <= D_h <= 256, 32 <= D' <= 256; other widths keep the window on the tensor cores and run
- * the linear branch on the fp32 kernels), SIMT fp32 kernels otherwise.  SIMT / TENSOR force one (TENSOR fails with REHYAT_ERR_UNSUPPORTED
- * where it does not apply).  TENSOR_WINDOW: tensor-core window, SIMT linear branch (a cross-check). */
+ * the linear branch on the fp32 kernels).  fp32: by size, tensor-core kernels that split every operand into three bf16
+ * parts (fp32 precision; values of 2^40 and more or not finite are left to the SIMT kernels) or SIMT fp32 kernels.
+ * SIMT / TENSOR force one (TENSOR fails with REHYAT_ERR_UNSUPPORTED where it does not apply, for fp32 always).  TENSOR_WINDOW: tensor-core window, SIMT linear branch (a cross-check). */
 typedef enum {
   REHYAT_IMPL_AUTO = 0, REHYAT_IMPL_SIMT = 1, REHYAT_IMPL_TENSOR = 2, REHYAT_IMPL_TENSOR_WINDOW = 3
 } rehyat_impl;
@@ -287,7 +288,8 @@ int rehyat_last_launches(const rehyat_ctx* ctx);
 
 /* Kernels of the last forward: 2 = every step on the tensor cores, 1 = the softmax window on the tensor cores
  * and phi, state and read-out on the fp32 SIMT kernels (phi widths the tensor-core kernels do not cover, or
- * REHYAT_IMPL_TENSOR_WINDOW), 0 = SIMT kernels throughout. */
+ * REHYAT_IMPL_TENSOR_WINDOW), 0 = the fp32 operator (each step on the tensor cores, with fp32 operands split into bf16
+ * parts, or on the SIMT kernels, by size) or SIMT kernels throughout (REHYAT_IMPL_SIMT). */
 int rehyat_last_impl(const rehyat_ctx* ctx);
 
 /* Query tiles per work item of the last tensor-core window launch: 2 (window_tc) or 1 (window_tc1);

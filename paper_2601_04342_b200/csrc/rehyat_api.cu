@@ -427,11 +427,8 @@ void launch_qk_prepare(rehyat_ctx* ctx, const void* q, const void* k, void* qo, 
   pa.wq = ctx->qk.q_norm_weight; pa.wk = ctx->qk.k_norm_weight;
   pa.cos = ctx->qk.rope_cos; pa.sin = ctx->qk.rope_sin;
   pa.eps = ctx->qk.norm_eps; pa.rms_norm = ctx->qk.rms_norm;
-  const int rows_per_block = 256 / (c.head_dim / 8);
-  // about thirty-two CTAs per SM over the whole grid, every thread walking several pairs of rows of its columns
-  const long long want = (32LL * ctx->tc.n_sm + 2 * BH - 1) / (2 * BH), need = (pa.rows + 2 * rows_per_block - 1) / (2 * rows_per_block);
-  const unsigned blocks = (unsigned)(need < want ? need : (want > 0 ? want : 1));
-  const dim3 grid(blocks, BH, 2);
+  const int rows_per_block = 256 / (c.head_dim / 8), groups = (pa.n_heads + QK_HEADS - 1) / QK_HEADS;
+  const dim3 grid((unsigned)((pa.rows + rows_per_block - 1) / rows_per_block), BH / pa.n_heads * groups);
   ctx->prof.begin(REHYAT_PROF_QKPREP, st);
   if (c.dtype == REHYAT_DTYPE_FP32) {
     if (c.head_dim == 64) launch_kernel(qk_prepare<float, 64>, grid, 256, 0, st, (const float*)q, (const float*)k, (float*)qo, (float*)ko, pa);

@@ -577,7 +577,11 @@ readout_simt(const T* q, PhiPtrs<T> wq, PhiDims pd, Geo g, const float* state, f
 // normalisation x / sqrt(mean(x^2) + eps) * weight, then the rotary embedding with caller-supplied tables (the
 // pair (x[2i], x[2i+1]) of token n turned by the angle of cos[n][i], sin[n][i]).  One pass over q and k, bound by
 // HBM: every element is read once and written once, in the layout it came in.
-// grid (row blocks, BH, 2: q / k), 256 threads; a row of d elements is shared by d/8 lanes, eight elements each.
+// grid (row blocks, batch * head groups), 256 threads; a row of d elements is shared by d/8 lanes, eight elements each.
+// A thread takes one token's rows of QK_HEADS heads, of q and of k: the rotation tables (twice the bytes of a bf16 row) are
+// loaded once for eight rows instead of once for each, and four rows are in flight.  12 heads x 32,760 tokens of 128
+// channels, bf16: 99 -> 87 us between two events (a copy of the same bytes: 60).
+constexpr int QK_HEADS = 4;
 struct QkPrepArgs {
   const void* wq; const void* wk;       // [n_heads][d] in the operator dtype, or null
   const float* cos; const float* sin;   // [positions][d/2], or null
@@ -595,74 +599,54 @@ qk_prepare(const T* q, const T* k, T* qo, T* ko, QkPrepArgs a) {
   ptx::grid_dep_wait();
   ptx::grid_dep_launch();
   constexpr int LPR = D / 8;                                        // lanes per row
-  const T* src = blockIdx.z ? k : q;
-  T* dst = blockIdx.z ? ko : qo;
-  const T* wgt = static_cast<const T*>(blockIdx.z ? a.wk : a.wq);
-  const int bh = blockIdx.y, head = bh % a.n_heads, bat = bh / a.n_heads;
-  const long long hoff = (long long)bat * a.sb + (long long)head * a.sh;
-  const long long doff = blockIdx.z ? (long long)bat * a.kb + (long long)head * a.kh : (long long)bat * a.qb + (long long)head * a.qh;
-  const long long dn = blockIdx.z ? a.kn : a.qn;
-  const int lane_in_row = threadIdx.x % LPR, col = lane_in_row * 8;
-  const int rows_per_block = 256 / LPR;
-  // a thread keeps its eight columns for all its rows: their norm weights are loaded once
-  float wv[8] = {1.f, 1.f, 1.f, 1.f, 1.f, 1.f, 1.f, 1.f};
-  if (a.rms_norm && wgt != nullptr) {
-    const float4 w0 = ld4(wgt + (size_t)head * D + col), w1 = ld4(wgt + (size_t)head * D + col + 4);
-    wv[0] = w0.x; wv[1] = w0.y; wv[2] = w0.z; wv[3] = w0.w; wv[4] = w1.x; wv[5] = w1.y; wv[6] = w1.z; wv[7] = w1.w;
+  const int groups = (a.n_heads + QK_HEADS - 1) / QK_HEADS;
+  const int bat = blockIdx.y / groups, h0 = blockIdx.y % groups * QK_HEADS, n_here = min(QK_HEADS, a.n_heads - h0);
+  const int col = threadIdx.x % LPR * 8, row = blockIdx.x * (256 / LPR) + threadIdx.x / LPR;
+  const bool ok = row < a.rows;                                     // rows beyond the end take part in the shuffles, nothing else
+  float cs[4] = {1.f, 1.f, 1.f, 1.f}, sn[4] = {0.f, 0.f, 0.f, 0.f};
+  if (a.cos != nullptr && ok) {
+    const size_t at = (size_t)(a.pos0 + row) * (D / 2) + col / 2;
+    const float4 c = *reinterpret_cast<const float4*>(a.cos + at), s = *reinterpret_cast<const float4*>(a.sin + at);
+    cs[0] = c.x; cs[1] = c.y; cs[2] = c.z; cs[3] = c.w;
+    sn[0] = s.x; sn[1] = s.y; sn[2] = s.z; sn[3] = s.w;
   }
-  // the lanes that share a row reduce among themselves: row groups of one warp may leave the loop at different times
-  const unsigned row_lanes = (LPR >= 32 ? 0xffffffffu : ((1u << LPR) - 1u) << ((threadIdx.x & 31) / LPR * LPR));
-  // two rows per step, both loaded before either is worked on: twice the bytes in flight per thread
-  const int stride = gridDim.x * rows_per_block;
-  const int first = blockIdx.x * rows_per_block + threadIdx.x / LPR;
-  // the addresses of a thread's rows advance by constants: pointers of the first of the two rows, stepped per turn
-  const T* sp = src + hoff + (long long)first * a.sn + col;
-  T* dp = dst + doff + (long long)first * dn + col;
-  const float* cp = a.cos != nullptr ? a.cos + (size_t)(a.pos0 + first) * (D / 2) + col / 2 : nullptr;
-  const float* np_ = a.cos != nullptr ? a.sin + (size_t)(a.pos0 + first) * (D / 2) + col / 2 : nullptr;
-  const long long s_row = (long long)stride * a.sn, d_row = (long long)stride * dn;       // one row group further
-  const size_t t_row = (size_t)stride * (D / 2);
-  for (int row0 = first; row0 < a.rows; row0 += 2 * stride, sp += 2 * s_row, dp += 2 * d_row, cp += 2 * t_row, np_ += 2 * t_row) {
-    float x[2][8];
+#pragma unroll 1
+  for (int z = 0; z < 2; ++z) {
+    const T* src = (z ? k : q) + (long long)bat * a.sb + (long long)h0 * a.sh + (long long)row * a.sn + col;
+    T* dst = z ? ko + (long long)bat * a.kb + (long long)h0 * a.kh + (long long)row * a.kn + col
+               : qo + (long long)bat * a.qb + (long long)h0 * a.qh + (long long)row * a.qn + col;
+    const long long dh = z ? a.kh : a.qh;
+    const T* wgt = static_cast<const T*>(z ? a.wk : a.wq);
+    float x[QK_HEADS][8];
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      const int row = row0 + u * stride;
-      if (row < a.rows) {
-        const T* p = sp + u * s_row;
-        const float4 x0 = ld4(p), x1 = ld4(p + 4);
-        x[u][0] = x0.x; x[u][1] = x0.y; x[u][2] = x0.z; x[u][3] = x0.w;
-        x[u][4] = x1.x; x[u][5] = x1.y; x[u][6] = x1.z; x[u][7] = x1.w;
-      } else {
+    for (int h = 0; h < QK_HEADS; ++h) {
 #pragma unroll
-        for (int e = 0; e < 8; ++e) x[u][e] = 0.f;
-      }
+      for (int e = 0; e < 8; ++e) x[h][e] = 0.f;
+      if (ok && h < n_here) ld8(src + h * a.sh, x[h]);
     }
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      const int row = row0 + u * stride;                 // rows beyond the end take part in the shuffles, nothing else
+    for (int h = 0; h < QK_HEADS; ++h) {
       if (a.rms_norm) {
         float ss = 0.f;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) ss = fmaf(x[u][e], x[u][e], ss);
+        for (int e = 0; e < 8; ++e) ss = fmaf(x[h][e], x[h][e], ss);
 #pragma unroll
-        for (int o = 1; o < LPR; o <<= 1) ss += __shfl_xor_sync(row_lanes, ss, o);
+        for (int o = 1; o < LPR; o <<= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
         const float inv = rsqrtf(ss * (1.f / D) + a.eps);
+        float w[8] = {1.f, 1.f, 1.f, 1.f, 1.f, 1.f, 1.f, 1.f};
+        if (wgt != nullptr && h < n_here) ld8(wgt + (size_t)(h0 + h) * D + col, w);
 #pragma unroll
-        for (int e = 0; e < 8; ++e) x[u][e] *= inv * wv[e];
+        for (int e = 0; e < 8; ++e) x[h][e] *= inv * w[e];
       }
-      if (row >= a.rows) continue;
       if (a.cos != nullptr) {
-        const float4 c = *reinterpret_cast<const float4*>(cp + u * t_row);
-        const float4 s = *reinterpret_cast<const float4*>(np_ + u * t_row);
-        const float cs[4] = {c.x, c.y, c.z, c.w}, sn[4] = {s.x, s.y, s.z, s.w};
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          const float p0 = x[u][2 * e], p1 = x[u][2 * e + 1];
-          x[u][2 * e] = p0 * cs[e] - p1 * sn[e];
-          x[u][2 * e + 1] = p0 * sn[e] + p1 * cs[e];
+          const float p0 = x[h][2 * e], p1 = x[h][2 * e + 1];
+          x[h][2 * e] = p0 * cs[e] - p1 * sn[e];
+          x[h][2 * e + 1] = p0 * sn[e] + p1 * cs[e];
         }
       }
-      st8(dp + u * d_row, x[u]);
+      if (ok && h < n_here) st8(dst + h * dh, x[h]);
     }
   }
 }
