@@ -7,6 +7,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "rehyat_ptx.cuh"
+
 namespace rehyat {
 
 // Activations of the phi MLP (same numbering as rehyat_act in the public header).
@@ -154,23 +156,44 @@ __device__ __forceinline__ float apply_act(float x, int act) {
 __device__ __forceinline__ float sfu_ex2(float x) { float y; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
 __device__ __forceinline__ float sfu_rcp(float x) { float y; asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
 
+// A polynomial with the coefficients c[0] (highest) ... c[N - 1] at two points, one packed multiply-add per step: the
+// epilogues of the phi kernels are bound by issue slots when the activation is not ReLU, and a packed multiply-add does
+// two at the cost of one (same rounding).
+template <int N>
+__device__ __forceinline__ uint64_t poly2(const float (&c)[N], uint64_t x) {
+  uint64_t p = ptx::pk2(c[0], c[0]);
+#pragma unroll
+  for (int i = 1; i < N; ++i) p = ptx::fma2(p, x, ptx::pk2(c[i], c[i]));
+  return p;
+}
 // log(1 + exp(x)) = max(x, 0) + log1p(e), e = exp(-|x|) in (0, 1]: log1p(e) / e as a polynomial fitted to the minimax
 // relative error on (0, 1] (2e-7), so that small results keep their relative accuracy.
-__device__ __forceinline__ float softplus_fast(float x) {
-  const float e = sfu_ex2(-1.4426950408889634f * fabsf(x));
-  float p = -0.0085390963f;
-  p = fmaf(p, e, 0.044089238f); p = fmaf(p, e, -0.10768117f); p = fmaf(p, e, 0.17745204f);
-  p = fmaf(p, e, -0.2449545f); p = fmaf(p, e, 0.33275478f); p = fmaf(p, e, -0.49997405f); p = fmaf(p, e, 0.9999998f);
-  return fmaf(p, e, fmaxf(x, 0.f));
+__device__ __forceinline__ void softplus_fast2(float& x0, float& x1) {
+  constexpr float c[8] = {-0.0085390963f, 0.044089238f, -0.10768117f, 0.17745204f, -0.2449545f, 0.33275478f, -0.49997405f, 0.9999998f};
+  const uint64_t e = ptx::pk2(sfu_ex2(-1.4426950408889634f * fabsf(x0)), sfu_ex2(-1.4426950408889634f * fabsf(x1)));
+  ptx::upk2(ptx::fma2(poly2(c, e), e, ptx::pk2(fmaxf(x0, 0.f), fmaxf(x1, 0.f))), x0, x1);
 }
 // x Phi(x) = max(x, 0) - |x| Q(|x|) with the normal tail Q(a) = exp(-a^2 / 2) g(t), t = 1 / (1 + a / 4); g as a
 // polynomial fitted to the minimax relative error for 0 <= a <= 9.5 (1.2e-7); beyond that exp(-a^2 / 2) < 3e-20.
-__device__ __forceinline__ float gelu_fast(float x) {
-  const float a = fabsf(x) > 64.f ? 64.f : fabsf(x), t = sfu_rcp(fmaf(0.25f, a, 1.f)), e = sfu_ex2(-0.72134752044448170f * a * a);
-  float p = -0.098380317f;
-  p = fmaf(p, t, 0.37461082f); p = fmaf(p, t, -0.33402116f); p = fmaf(p, t, 0.35451113f); p = fmaf(p, t, -0.02167429f);
-  p = fmaf(p, t, 0.12915299f); p = fmaf(p, t, 0.095545365f); p = fmaf(p, t, 0.00025551728f);
-  return fmaf(-a * e, p, fmaxf(x, 0.f));
+__device__ __forceinline__ void gelu_fast2(float& x0, float& x1) {
+  constexpr float c[8] = {-0.098380317f, 0.37461082f, -0.33402116f, 0.35451113f, -0.02167429f, 0.12915299f, 0.095545365f, 0.00025551728f};
+  const float a0 = fabsf(x0) > 64.f ? 64.f : fabsf(x0), a1 = fabsf(x1) > 64.f ? 64.f : fabsf(x1);
+  const uint64_t a = ptx::pk2(a0, a1);
+  float d0, d1, g0, g1;
+  ptx::upk2(ptx::fma2(a, ptx::pk2(0.25f, 0.25f), ptx::pk2(1.f, 1.f)), d0, d1);
+  ptx::upk2(ptx::mul2(ptx::mul2(a, ptx::pk2(-0.72134752044448170f, -0.72134752044448170f)), a), g0, g1);
+  const uint64_t t = ptx::pk2(sfu_rcp(d0), sfu_rcp(d1)), e = ptx::pk2(-sfu_ex2(g0), -sfu_ex2(g1));
+  ptx::upk2(ptx::fma2(ptx::mul2(a, e), poly2(c, t), ptx::pk2(fmaxf(x0, 0.f), fmaxf(x1, 0.f))), x0, x1);
+}
+// y = accumulators + bias (16-byte aligned), N columns
+template <int N>
+__device__ __forceinline__ void add_bias(const uint32_t (&x)[N], const float* bias, float (&y)[N]) {
+#pragma unroll
+  for (int e = 0; e < N; e += 4) {
+    const float4 b = *reinterpret_cast<const float4*>(bias + e);
+    ptx::upk2(ptx::add2(ptx::pk2u(x[e], x[e + 1]), ptx::pk2(b.x, b.y)), y[e], y[e + 1]);
+    ptx::upk2(ptx::add2(ptx::pk2u(x[e + 2], x[e + 3]), ptx::pk2(b.z, b.w)), y[e + 2], y[e + 3]);
+  }
 }
 // The activation of a block of values, for the kernels that round it to bf16 (2^-9): within 5e-7 of apply_act.
 // The selection is outside the loop over the block, and the library functions (log1pf, expf, erff: tens of
@@ -185,7 +208,7 @@ __device__ __forceinline__ void act_block(float (&y)[N], int act) {
     case ACT_IDENTITY: break;
     case ACT_SOFTPLUS:
 #pragma unroll
-      for (int e = 0; e < N; ++e) y[e] = softplus_fast(y[e]);
+      for (int e = 0; e < N; e += 2) softplus_fast2(y[e], y[e + 1]);
       break;
     case ACT_ELU1:
 #pragma unroll
@@ -193,7 +216,7 @@ __device__ __forceinline__ void act_block(float (&y)[N], int act) {
       break;
     default:
 #pragma unroll
-      for (int e = 0; e < N; ++e) y[e] = gelu_fast(y[e]);
+      for (int e = 0; e < N; e += 2) gelu_fast2(y[e], y[e + 1]);
       break;
   }
 }

@@ -399,7 +399,7 @@ phi_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtenso
           // Rolled over blocks of 16 columns with the selection of the activation outside the block.  Inlined per column
           // and unrolled (the library's erff, log1pf and expf, a loop and a division per power) this role was
           // thousands of instructions long: 12 heads x 13,440 tokens of a three-layer GELU / softplus map took 1,796 us
-          // here and 804 us in the read-out kernel, in this form 308 and 237 us.
+          // here and 804 us in the read-out kernel, in this form 308 and 237 us (285 and 219 with packed polynomials).
 #pragma unroll 1
           for (int cb = 0; cb < 4; ++cb) {
             const int col0 = half * 128 + ch * 64 + cb * 16;
@@ -407,8 +407,7 @@ phi_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtenso
             float y[16];
             tmem_ld16(tmem + lane_off + T_SCR + ch * 64 + cb * 16, x);
             tmem_wait_ld();
-#pragma unroll
-            for (int e = 0; e < 16; ++e) y[e] = __uint_as_float(x[e]) + bias[ch * 64 + cb * 16 + e];
+            add_bias(x, bias + ch * 64 + cb * 16, y);
             act_power_block(y, is_u ? a.act_out : a.act_hidden, is_u, col0, part_w, Dp);
             if (is_u && !tok_valid) {
 #pragma unroll
