@@ -21,19 +21,28 @@
 
 namespace rehyat {
 
-constexpr int RD_RING = 7;
+constexpr int RD_RING_MAX = 7;
 constexpr int RD_WT_BYTES = 128 * 64 * 2;                        // one weight / state tile: 16 KB
-constexpr int RD_OFF_X = 0;
-constexpr int RD_OFF_PHI0 = RD_OFF_X + PH_TILE_BYTES;
-constexpr int RD_OFF_PHI1 = RD_OFF_PHI0 + PH_TILE_BYTES;
-constexpr int RD_OFF_RING = RD_OFF_PHI1 + PH_TILE_BYTES;
-constexpr int RD_OFF_BIAS = RD_OFF_RING + RD_RING * RD_WT_BYTES;  // b1[256], b2[256], z[256], two partial phi.z sums per token (x2: by tile parity), bmid[2][256]
-constexpr int RD_OFF_BARS = RD_OFF_BIAS + (5 + PH_MAX_MID) * 256 * 4;
-constexpr int RD_SMEM = RD_OFF_BARS + 512 + 1024;
+// The two forms of the kernel.  NARROW serves heads of 64 with widths up to 128, where H, U and R are one half each and
+// nothing is left to overlap inside a tile: with three ring stages, no second phi half and 256 TMEM columns two CTAs fit an
+// SM, and one works on the tensor core while the other's epilogues run: 24 heads x 32,760 tokens, one-frame chunks,
+// 308 -> 169 us.
+template <bool NARROW>
+struct RdShape {
+  static constexpr int RING = NARROW ? 3 : RD_RING_MAX;
+  static constexpr int OFF_X = 0;
+  static constexpr int OFF_PHI0 = OFF_X + (NARROW ? PH_SUB : PH_TILE_BYTES);
+  static constexpr int OFF_PHI1 = OFF_PHI0 + PH_TILE_BYTES;      // not used if NARROW
+  static constexpr int OFF_RING = OFF_PHI1 + (NARROW ? 0 : PH_TILE_BYTES);
+  static constexpr int OFF_BIAS = OFF_RING + RING * RD_WT_BYTES;  // b1[256], b2[256], z[256], two partial phi.z sums per token (x2: by tile parity), bmid[2][256]
+  static constexpr int OFF_BARS = OFF_BIAS + (5 + PH_MAX_MID) * 256 * 4;
+  static constexpr int SMEM = OFF_BARS + 512 + 1024;
+  static constexpr uint32_t T_H = NARROW ? 128 : 256, T_R = NARROW ? 192 : 384, COLS = NARROW ? 256 : 512;
+};
 
 struct RdBars {
   uint64_t x_full, x_empty;
-  uint64_t ring_full[RD_RING], ring_empty[RD_RING];
+  uint64_t ring_full[RD_RING_MAX], ring_empty[RD_RING_MAX];
   uint64_t acc_ready[2], epi_done[2], out_ready, out_read;
   uint64_t nl_ready;           // both halves of a tile's phi.z sums are in shared memory
   uint64_t drained;            // every tcgen05.mma of the issuer has completed
@@ -46,17 +55,19 @@ struct RdBars {
 // PC: polynomial degree known at compile time (0: read it from the arguments; 2 needs D' = 256).
 // A hidden layer of a deeper map (GEN only) reads H from TMEM and writes it back there: both halves of its GEMM
 // have completed before the first column of H is overwritten.
-template <bool RELU, int PC, bool GEN>
-__global__ void __launch_bounds__(PH_THREADS, 1)
+template <bool RELU, int PC, bool GEN, bool NARROW>
+__global__ void __launch_bounds__(PH_THREADS, NARROW ? 2 : 1)
 readout_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w1,
            const __grid_constant__ CUtensorMap tm_w2, const __grid_constant__ CUtensorMap tm_wm,
            const __grid_constant__ CUtensorMap tm_s, Geo g, PhiTcArgs a) {
   using namespace ptx;
+  using SH = RdShape<NARROW>;
+  constexpr int RD_RING = SH::RING;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t sb = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* smem = smem_raw + (sb - smem_u32(smem_raw));
-  RdBars* bars = reinterpret_cast<RdBars*>(smem + RD_OFF_BARS);
-  float* s_b1 = reinterpret_cast<float*>(smem + RD_OFF_BIAS);
+  RdBars* bars = reinterpret_cast<RdBars*>(smem + SH::OFF_BARS);
+  float* s_b1 = reinterpret_cast<float*>(smem + SH::OFF_BIAS);
   float* s_b2 = s_b1 + 256;
   float* s_z = s_b2 + 256;
   float* s_nl = s_z + 256;
@@ -95,15 +106,15 @@ readout_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUt
       s_bm[m * 256 + i] = i < ex.Dh ? __bfloat162float(a.bm[((size_t)h_idx * n_mid + m) * ex.Dh + i]) : 0.f;
   }
   if (warp == 9) {
-    tmem_alloc(smem_u32(&bars->tmem_base), 512);
+    tmem_alloc(smem_u32(&bars->tmem_base), SH::COLS);
     tmem_relinquish();
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = bars->tmem_base;
-  constexpr uint32_t T_SCR = 0, T_H = 256, T_R = 384;
-  const uint32_t sX = sb + RD_OFF_X, sPhi0 = sb + RD_OFF_PHI0, sPhi1 = sb + RD_OFF_PHI1, sRing = sb + RD_OFF_RING;
+  constexpr uint32_t T_SCR = 0, T_H = SH::T_H, T_R = SH::T_R;
+  const uint32_t sX = sb + SH::OFF_X, sPhi0 = sb + SH::OFF_PHI0, sPhi1 = sb + SH::OFF_PHI1, sRing = sb + SH::OFF_RING;
 
   if (warp == 8) {
     // ------------------------------------------------------------------ TMA producer
@@ -454,7 +465,7 @@ readout_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUt
   __syncthreads();
   if (warp == 9) {
     tc_fence_after();
-    tmem_dealloc(tmem, 512);
+    tmem_dealloc(tmem, SH::COLS);
   }
 }
 

@@ -588,11 +588,13 @@ inline int tc_set_attributes() {
             cudaFuncSetAttribute(phi_tc<false, 0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PH_SMEM) == cudaSuccess &&
             cudaFuncSetAttribute(phi_tc<true, 0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, PH_SMEM) == cudaSuccess &&
             cudaFuncSetAttribute(phi_tc<false, 0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, PH_SMEM) == cudaSuccess &&
-            cudaFuncSetAttribute(readout_tc<true, 2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, RD_SMEM) == cudaSuccess &&
-            cudaFuncSetAttribute(readout_tc<true, 0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, RD_SMEM) == cudaSuccess &&
-            cudaFuncSetAttribute(readout_tc<false, 0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, RD_SMEM) == cudaSuccess &&
-            cudaFuncSetAttribute(readout_tc<true, 0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, RD_SMEM) == cudaSuccess &&
-            cudaFuncSetAttribute(readout_tc<false, 0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, RD_SMEM) == cudaSuccess;
+            cudaFuncSetAttribute(readout_tc<true, 2, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, RdShape<false>::SMEM) == cudaSuccess &&
+            cudaFuncSetAttribute(readout_tc<true, 0, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, RdShape<false>::SMEM) == cudaSuccess &&
+            cudaFuncSetAttribute(readout_tc<false, 0, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, RdShape<false>::SMEM) == cudaSuccess &&
+            cudaFuncSetAttribute(readout_tc<true, 0, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, RdShape<false>::SMEM) == cudaSuccess &&
+            cudaFuncSetAttribute(readout_tc<false, 0, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, RdShape<false>::SMEM) == cudaSuccess &&
+            cudaFuncSetAttribute(readout_tc<true, 0, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, RdShape<true>::SMEM) == cudaSuccess &&
+            cudaFuncSetAttribute(readout_tc<false, 0, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, RdShape<true>::SMEM) == cudaSuccess;
   return ok ? REHYAT_OK : REHYAT_ERR_CUDA;
 }
 
@@ -711,7 +713,10 @@ inline int tc_launch_readout(const TcWorkspace* w, const void* q, const rehyat_p
   a.P = P; a.act_hidden = act_hidden; a.act_out = act_out;
   a.d = d; a.Dh = Dh; a.Dp = Dp; a.n_mid = n_mid;
   a.state = state; a.rd = rd; a.rd_rows = rd_rows; a.wa = wa;
-  // One CTA per SM: split a chunk's query tiles over as many CTAs as costs the fewest tile-times over all waves.
+  const bool narrow = d == 64 && Dh <= 128 && Dp <= 128;
+  // One CTA per SM (two of the narrow form): split a chunk's query tiles over as many CTAs as costs the fewest tile-times
+  // over all waves.
+  const int slots = w->n_sm * (narrow ? 2 : 1);
   const int tiles = (g.Np + 127) / 128;
   int busy = 0;
   for (int t = g.t0; t < g.t0 + g.G; ++t) busy += geo_linear(g, t);
@@ -719,19 +724,22 @@ inline int tc_launch_readout(const TcWorkspace* w, const void* q, const rehyat_p
   long long best = -1;
   int best_s = 1;
   for (int s = 1; s <= 16; ++s) {
-    const long long cost = ((units * s + w->n_sm - 1) / w->n_sm) * ((tiles + s - 1) / s);
+    const long long cost = ((units * s + slots - 1) / slots) * ((tiles + s - 1) / s);
     if (best < 0 || cost < best) { best = cost; best_s = s; }
   }
   a.tiles_per_cta = (tiles + best_s - 1) / best_s;
   const int ctas = (tiles + a.tiles_per_cta - 1) / a.tiles_per_cta;
   const PhiKernelChoice ch = tc_phi_choice(d, Dh, Dp, P, n_mid, act_hidden, act_out);
   const dim3 grid(ctas, g.G, g.BH);
-#define REHYAT_LAUNCH_RD(R, PC, GEN) launch_kernel(readout_tc<R, PC, GEN>, grid, PH_THREADS, RD_SMEM, st, tq, tw1, tw2, twm, ts, g, a)
-  if (ch.gen) { if (ch.relu) REHYAT_LAUNCH_RD(true, 0, true); else REHYAT_LAUNCH_RD(false, 0, true); }
+#define REHYAT_LAUNCH_RD_N(R, PC, GEN, N) launch_kernel(readout_tc<R, PC, GEN, N>, grid, PH_THREADS, RdShape<N>::SMEM, st, tq, tw1, tw2, twm, ts, g, a)
+#define REHYAT_LAUNCH_RD(R, PC, GEN) REHYAT_LAUNCH_RD_N(R, PC, GEN, false)
+  if (narrow) { if (ch.relu) REHYAT_LAUNCH_RD_N(true, 0, true, true); else REHYAT_LAUNCH_RD_N(false, 0, true, true); }
+  else if (ch.gen) { if (ch.relu) REHYAT_LAUNCH_RD(true, 0, true); else REHYAT_LAUNCH_RD(false, 0, true); }
   else if (ch.pc == 2) REHYAT_LAUNCH_RD(true, 2, false);
   else if (ch.relu) REHYAT_LAUNCH_RD(true, 0, false);
   else REHYAT_LAUNCH_RD(false, 0, false);
 #undef REHYAT_LAUNCH_RD
+#undef REHYAT_LAUNCH_RD_N
   return cudaGetLastError() == cudaSuccess ? REHYAT_OK : REHYAT_ERR_CUDA;
 }
 
