@@ -208,7 +208,11 @@ struct PhiPlan { int parts; bool f32_tc; };
 // needs fewer rounds: 24 heads of 64, chunks of 192 tokens 93 -> 66 us a call; one chunk of 64 tokens stays (54 us, not 65).
 PhiPlan plan_phi(const rehyat_ctx* ctx, long long tokens, long long units, int most) {
   const int n_sm = ctx->tc.n_sm;
-  if (ctx->tensor_ok && ctx->tc.phi_ok) return {pick_parts((tokens + 127) / 128, units, most, n_sm), false};
+  if (ctx->tensor_ok && ctx->tc.phi_ok) {
+    const rehyat_config& c = ctx->cfg;
+    const int per_sm = tc_state_narrow(c.head_dim, c.phi_hidden, c.phi_dim, c.phi_layers > 2 ? c.phi_layers - 2 : 0) ? 2 : 1;
+    return {pick_parts((tokens + 127) / 128, units, most, per_sm * n_sm), false};
+  }
   long long simt = 0, tc = 0;
   const int simt_parts = pick_parts((tokens + SIMT_TM - 1) / SIMT_TM, units, most, n_sm, &simt);
   if (ctx->status_dev == nullptr || ctx->cfg.impl == REHYAT_IMPL_SIMT || ctx->cfg.dtype != REHYAT_DTYPE_FP32 || ctx->cfg.phi_layers > 2)

@@ -33,27 +33,36 @@ namespace rehyat {
 
 constexpr int PH_D = 128, PH_DH = 256, PH_DP = 256, PH_SD = PH_D + 4;
 constexpr int PH_THREADS = 320;            // 8 epilogue warps, TMA producer, UMMA issuer
-constexpr int PH_RING = 3;                // weight tiles in flight
+constexpr int PH_RING_MAX = 3;             // weight tiles in flight
 constexpr int PH_WT_BYTES = 128 * 64 * 2;          // one weight / state tile: 16 KB
 constexpr int PH_TILE_BYTES = 128 * 128 * 2;       // X, V, phi half: 32 KB (two swizzled sub-tiles)
 constexpr int PH_SUB = PH_TILE_BYTES / 2;
-// shared memory map (bytes from the 1024-aligned base)
-constexpr int PH_OFF_X = 0;
-constexpr int PH_OFF_V = PH_OFF_X + PH_TILE_BYTES;
-constexpr int PH_OFF_HB = PH_OFF_V + PH_TILE_BYTES;            // 64 KB; one of its halves doubles as phi half 1
-constexpr int PH_OFF_PHI0 = PH_OFF_HB + 2 * PH_TILE_BYTES;
-constexpr int PH_OFF_RING = PH_OFF_PHI0 + PH_TILE_BYTES;
-constexpr int PH_OFF_ONES = PH_OFF_RING + PH_RING * PH_WT_BYTES; // [16 x 128] K-major, row 0 = 1
-constexpr int PH_OFF_BIAS = PH_OFF_ONES + 4096;                 // b1[256], b2[256], bmid[2][256] fp32
-constexpr int PH_MAX_MID = 2;                                   // hidden layers between the first and the last
-constexpr int PH_OFF_BARS = PH_OFF_BIAS + (2 + PH_MAX_MID) * 256 * 4;
-constexpr int PH_SMEM = PH_OFF_BARS + 512 + 1024;
+constexpr int PH_MAX_MID = 2;                      // hidden layers between the first and the last
+// Shared memory map (bytes from the 1024-aligned base).  NARROW serves two-layer maps of heads of 64 with widths up to 128:
+// one half of H and U each, phi written over H (which its GEMM has read), two ring stages and 256 TMEM columns, so that
+// two CTAs fit an SM and one works on the tensor core while the other's epilogues run: 24 heads x 32,760 tokens, one-frame
+// chunks, 217 -> 187 us.
+template <bool NARROW>
+struct PhShape {
+  static constexpr int RING = NARROW ? 2 : PH_RING_MAX;
+  static constexpr int XV_BYTES = NARROW ? PH_SUB : PH_TILE_BYTES;
+  static constexpr int OFF_X = 0;
+  static constexpr int OFF_V = OFF_X + XV_BYTES;
+  static constexpr int OFF_HB = OFF_V + XV_BYTES;                  // 64 KB; one of its halves doubles as phi half 1
+  static constexpr int OFF_PHI0 = NARROW ? OFF_HB : OFF_HB + 2 * PH_TILE_BYTES;
+  static constexpr int OFF_RING = OFF_PHI0 + PH_TILE_BYTES;
+  static constexpr int OFF_ONES = OFF_RING + RING * PH_WT_BYTES;   // [16 x 128] K-major, row 0 = 1
+  static constexpr int OFF_BIAS = OFF_ONES + 4096;                 // b1[256], b2[256], bmid[2][256] fp32
+  static constexpr int OFF_BARS = OFF_BIAS + (2 + PH_MAX_MID) * 256 * 4;
+  static constexpr int SMEM = OFF_BARS + 512 + 1024;
+  static constexpr uint32_t T_Z = NARROW ? 192 : 384, COLS = NARROW ? 256 : 512;
+};
 
 enum PhErr : int { PH_ERR_LOAD = 16, PH_ERR_MMA = 32, PH_ERR_EPI = 64 };
 
 struct PhBars {
   uint64_t x_full, x_empty, v_full, v_empty;
-  uint64_t ring_full[PH_RING], ring_empty[PH_RING];
+  uint64_t ring_full[PH_RING_MAX], ring_empty[PH_RING_MAX];
   uint64_t acc_ready, epi_done, out_ready;
   uint64_t drained;            // every tcgen05.mma of the issuer has completed
   uint32_t tmem_base;
@@ -92,17 +101,19 @@ struct PhiExtents {
 // tm_x: K, tm_v: V, 4-D like the window kernel's maps.  tm_w1: (d, D_h, heads), tm_w2: (D_h, D', heads),
 // tm_wm: (D_h, D_h, heads * n_mid) (any valid map when n_mid = 0), boxes [64 x 128].  PC: polynomial degree known
 // at compile time (0: read it from the arguments; 2 needs D' = 256).
-template <bool RELU, int PC, bool GEN>
-__global__ void __launch_bounds__(PH_THREADS, 1)
+template <bool RELU, int PC, bool GEN, bool NARROW>
+__global__ void __launch_bounds__(PH_THREADS, NARROW ? 2 : 1)
 phi_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_v,
        const __grid_constant__ CUtensorMap tm_w1, const __grid_constant__ CUtensorMap tm_w2,
        const __grid_constant__ CUtensorMap tm_wm, Geo g, PhiTcArgs a) {
   using namespace ptx;
+  using SH = PhShape<NARROW>;
+  constexpr int PH_RING = SH::RING;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t sb = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* smem = smem_raw + (sb - smem_u32(smem_raw));
-  PhBars* bars = reinterpret_cast<PhBars*>(smem + PH_OFF_BARS);
-  float* s_b1 = reinterpret_cast<float*>(smem + PH_OFF_BIAS);
+  PhBars* bars = reinterpret_cast<PhBars*>(smem + SH::OFF_BARS);
+  float* s_b1 = reinterpret_cast<float*>(smem + SH::OFF_BIAS);
   float* s_b2 = s_b1 + 256;
   const uint32_t wc = smem_u32(&bars->wctx);
 
@@ -142,7 +153,7 @@ phi_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtenso
     fence_mbar_init();
   }
   if (warp == 9) {
-    tmem_alloc(smem_u32(&bars->tmem_base), 512);
+    tmem_alloc(smem_u32(&bars->tmem_base), SH::COLS);
     tmem_relinquish();
   }
   grid_dep_wait();
@@ -155,7 +166,7 @@ phi_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtenso
       s_b2[(1 + m) * 256 + i] = i < ex.Dh ? __bfloat162float(a.bm[((size_t)h_idx * n_mid + m) * ex.Dh + i]) : 0.f;
   }
   {
-    uint32_t* ones = reinterpret_cast<uint32_t*>(smem + PH_OFF_ONES);
+    uint32_t* ones = reinterpret_cast<uint32_t*>(smem + SH::OFF_ONES);
     for (int i = threadIdx.x; i < 1024; i += PH_THREADS) {
       const int byte = i * 4, sub = byte / 2048, within = byte % 2048;
       ones[i] = (within < 128 && sub < 2) ? 0x3F803F80u : 0u;       // two bf16 ones
@@ -167,11 +178,11 @@ phi_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtenso
   tc_fence_after();
   const uint32_t tmem = bars->tmem_base;
   // TMEM columns: scratch [0,128), S half 0 [128,256), S half 1 [256,384), z half 0 [384,400), z half 1 [400,416)
-  constexpr uint32_t T_SCR = 0, T_ACC = 128, T_Z = 384;
+  constexpr uint32_t T_SCR = 0, T_ACC = 128, T_Z = SH::T_Z;
   constexpr int RING = PH_RING;
 
-  const uint32_t sX = sb + PH_OFF_X, sV = sb + PH_OFF_V, sHb = sb + PH_OFF_HB, sPhi0 = sb + PH_OFF_PHI0,
-                 sRing = sb + PH_OFF_RING, sOnes = sb + PH_OFF_ONES;
+  const uint32_t sX = sb + SH::OFF_X, sV = sb + SH::OFF_V, sHb = sb + SH::OFF_HB, sPhi0 = sb + SH::OFF_PHI0,
+                 sRing = sb + SH::OFF_RING, sOnes = sb + SH::OFF_ONES;
   auto ring_addr = [&](int s) -> uint32_t { return sRing + s * PH_WT_BYTES; };
   // The two buffers of hidden activations, each four [128 x 64] sub-tiles: 0 = the H buffer, 1 = the X tile
   // followed by the phi half 0 tile.  The first layer writes buffer 0, hidden layer m reads m % 2 and writes the other.
@@ -357,7 +368,7 @@ phi_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtenso
         wait(&bars->acc_ready, n_acc & 1);
         ++n_acc;
         tc_fence_after();
-        if constexpr (RELU) {
+        if constexpr (RELU && !NARROW) {
           uint32_t x[2][32];
           tmem_ld32(tmem + lane_off + T_SCR + ch * 64, x[0]);
           tmem_ld32(tmem + lane_off + T_SCR + ch * 64 + 32, x[1]);
@@ -408,7 +419,7 @@ phi_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtenso
             tmem_ld16(tmem + lane_off + T_SCR + ch * 64 + cb * 16, x);
             tmem_wait_ld();
             add_bias(x, bias + ch * 64 + cb * 16, y);
-            act_power_block(y, is_u ? a.act_out : a.act_hidden, is_u, col0, part_w, Dp);
+            act_power_block(y, RELU ? (int)ACT_RELU : is_u ? a.act_out : a.act_hidden, is_u, col0, part_w, Dp);
             if (is_u && !tok_valid) {
 #pragma unroll
               for (int e = 0; e < 16; ++e) y[e] = 0.f;
@@ -478,7 +489,7 @@ phi_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtenso
   __syncthreads();
   if (warp == 9) {
     tc_fence_after();
-    tmem_dealloc(tmem, 512);
+    tmem_dealloc(tmem, SH::COLS);
   }
 }
 

@@ -519,6 +519,8 @@ inline bool tc_phi_supported(int d, int Dh, int Dp, int P, int n_mid) {
   return (d == 64 || d == 128) && Dh >= 64 && Dh <= PH_DH && Dh % 32 == 0 && Dp >= 32 && Dp <= PH_DP && Dp % 32 == 0 &&
          P >= 1 && Dp % P == 0 && n_mid >= 0 && n_mid <= PH_MAX_MID;
 }
+// Does the narrow form of phi_tc (two CTAs per SM) serve a map?
+inline bool tc_state_narrow(int d, int Dh, int Dp, int n_mid) { return d == 64 && Dh <= 128 && Dp <= 128 && n_mid == 0; }
 // Which instantiation serves a map: the fixed-shape kernels for the two-layer map of 128 / 256 / 256, the ones
 // that read their extents otherwise; the ReLU fast path needs polynomial parts that end on 32-column blocks.
 struct PhiKernelChoice { bool gen, relu; int pc; };
@@ -583,11 +585,13 @@ inline int tc_set_attributes() {
             cudaFuncSetAttribute(window_tc<1, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, WinShape<64>::SMEM) == cudaSuccess &&
             cudaFuncSetAttribute(window_tc<2, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, WinShape<64>::SMEM) == cudaSuccess &&
             cudaFuncSetAttribute(window_tc<3, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, WinShape<64>::SMEM) == cudaSuccess &&
-            cudaFuncSetAttribute(phi_tc<true, 2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PH_SMEM) == cudaSuccess &&
-            cudaFuncSetAttribute(phi_tc<true, 0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PH_SMEM) == cudaSuccess &&
-            cudaFuncSetAttribute(phi_tc<false, 0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PH_SMEM) == cudaSuccess &&
-            cudaFuncSetAttribute(phi_tc<true, 0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, PH_SMEM) == cudaSuccess &&
-            cudaFuncSetAttribute(phi_tc<false, 0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, PH_SMEM) == cudaSuccess &&
+            cudaFuncSetAttribute(phi_tc<true, 2, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PhShape<false>::SMEM) == cudaSuccess &&
+            cudaFuncSetAttribute(phi_tc<true, 0, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PhShape<false>::SMEM) == cudaSuccess &&
+            cudaFuncSetAttribute(phi_tc<false, 0, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PhShape<false>::SMEM) == cudaSuccess &&
+            cudaFuncSetAttribute(phi_tc<true, 0, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PhShape<false>::SMEM) == cudaSuccess &&
+            cudaFuncSetAttribute(phi_tc<false, 0, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PhShape<false>::SMEM) == cudaSuccess &&
+            cudaFuncSetAttribute(phi_tc<true, 0, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, PhShape<true>::SMEM) == cudaSuccess &&
+            cudaFuncSetAttribute(phi_tc<false, 0, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, PhShape<true>::SMEM) == cudaSuccess &&
             cudaFuncSetAttribute(readout_tc<true, 2, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, RdShape<false>::SMEM) == cudaSuccess &&
             cudaFuncSetAttribute(readout_tc<true, 0, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, RdShape<false>::SMEM) == cudaSuccess &&
             cudaFuncSetAttribute(readout_tc<false, 0, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, RdShape<false>::SMEM) == cudaSuccess &&
@@ -687,12 +691,15 @@ inline int tc_launch_state(const TcWorkspace* w, const void* k, const void* v, c
   a.n_split = n_split; a.partial = partial; a.wa = wa;
   const PhiKernelChoice ch = tc_phi_choice(d, Dh, Dp, P, n_mid, act_hidden, act_out);
   const dim3 grid(n_split, g.G, g.BH);
-#define REHYAT_LAUNCH_PHI(R, PC, GEN) launch_kernel(phi_tc<R, PC, GEN>, grid, PH_THREADS, PH_SMEM, st, tk, tv, tw1, tw2, twm, g, a)
-  if (ch.gen) { if (ch.relu) REHYAT_LAUNCH_PHI(true, 0, true); else REHYAT_LAUNCH_PHI(false, 0, true); }
+#define REHYAT_LAUNCH_PHI_N(R, PC, GEN, N) launch_kernel(phi_tc<R, PC, GEN, N>, grid, PH_THREADS, PhShape<N>::SMEM, st, tk, tv, tw1, tw2, twm, g, a)
+#define REHYAT_LAUNCH_PHI(R, PC, GEN) REHYAT_LAUNCH_PHI_N(R, PC, GEN, false)
+  if (tc_state_narrow(d, Dh, Dp, n_mid)) { if (ch.relu) REHYAT_LAUNCH_PHI_N(true, 0, true, true); else REHYAT_LAUNCH_PHI_N(false, 0, true, true); }
+  else if (ch.gen) { if (ch.relu) REHYAT_LAUNCH_PHI(true, 0, true); else REHYAT_LAUNCH_PHI(false, 0, true); }
   else if (ch.pc == 2) REHYAT_LAUNCH_PHI(true, 2, false);
   else if (ch.relu) REHYAT_LAUNCH_PHI(true, 0, false);
   else REHYAT_LAUNCH_PHI(false, 0, false);
 #undef REHYAT_LAUNCH_PHI
+#undef REHYAT_LAUNCH_PHI_N
   return cudaGetLastError() == cudaSuccess ? REHYAT_OK : REHYAT_ERR_CUDA;
 }
 
