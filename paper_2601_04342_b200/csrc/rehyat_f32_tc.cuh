@@ -19,6 +19,7 @@
 //
 // Values beyond 2^40 (or not finite) cannot be split safely: whoever sees one leaves the launch's epoch in *unsafe, and
 // window_simt, launched behind this kernel, computes the call again; otherwise it ends at once.
+// At the other end the third part of a value below 2^-110 is a bf16 subnormal: such values keep fewer than 24 bits.
 #pragma once
 
 #include "rehyat_simt.cuh"
