@@ -7,6 +7,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "rehyat_ptx.cuh"
 
 namespace rehyat {
@@ -152,39 +154,6 @@ __device__ __forceinline__ float apply_act(float x, int act) {
   }
 }
 
-// 2^x and 1/x by the special-function unit.
-__device__ __forceinline__ float sfu_ex2(float x) { float y; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
-__device__ __forceinline__ float sfu_rcp(float x) { float y; asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
-
-// A polynomial with the coefficients c[0] (highest) ... c[N - 1] at two points, one packed multiply-add per step: the
-// epilogues of the phi kernels are bound by issue slots when the activation is not ReLU, and a packed multiply-add does
-// two at the cost of one (same rounding).
-template <int N>
-__device__ __forceinline__ uint64_t poly2(const float (&c)[N], uint64_t x) {
-  uint64_t p = ptx::pk2(c[0], c[0]);
-#pragma unroll
-  for (int i = 1; i < N; ++i) p = ptx::fma2(p, x, ptx::pk2(c[i], c[i]));
-  return p;
-}
-// log(1 + exp(x)) = max(x, 0) + log1p(e), e = exp(-|x|) in (0, 1]: log1p(e) / e as a polynomial fitted to the minimax
-// relative error on (0, 1] (2e-7), so that small results keep their relative accuracy.
-__device__ __forceinline__ void softplus_fast2(float& x0, float& x1) {
-  constexpr float c[8] = {-0.0085390963f, 0.044089238f, -0.10768117f, 0.17745204f, -0.2449545f, 0.33275478f, -0.49997405f, 0.9999998f};
-  const uint64_t e = ptx::pk2(sfu_ex2(-1.4426950408889634f * fabsf(x0)), sfu_ex2(-1.4426950408889634f * fabsf(x1)));
-  ptx::upk2(ptx::fma2(poly2(c, e), e, ptx::pk2(fmaxf(x0, 0.f), fmaxf(x1, 0.f))), x0, x1);
-}
-// x Phi(x) = max(x, 0) - |x| Q(|x|) with the normal tail Q(a) = exp(-a^2 / 2) g(t), t = 1 / (1 + a / 4); g as a
-// polynomial fitted to the minimax relative error for 0 <= a <= 9.5 (1.2e-7); beyond that exp(-a^2 / 2) < 3e-20.
-__device__ __forceinline__ void gelu_fast2(float& x0, float& x1) {
-  constexpr float c[8] = {-0.098380317f, 0.37461082f, -0.33402116f, 0.35451113f, -0.02167429f, 0.12915299f, 0.095545365f, 0.00025551728f};
-  const float a0 = fabsf(x0) > 64.f ? 64.f : fabsf(x0), a1 = fabsf(x1) > 64.f ? 64.f : fabsf(x1);
-  const uint64_t a = ptx::pk2(a0, a1);
-  float d0, d1, g0, g1;
-  ptx::upk2(ptx::fma2(a, ptx::pk2(0.25f, 0.25f), ptx::pk2(1.f, 1.f)), d0, d1);
-  ptx::upk2(ptx::mul2(ptx::mul2(a, ptx::pk2(-0.72134752044448170f, -0.72134752044448170f)), a), g0, g1);
-  const uint64_t t = ptx::pk2(sfu_rcp(d0), sfu_rcp(d1)), e = ptx::pk2(-sfu_ex2(g0), -sfu_ex2(g1));
-  ptx::upk2(ptx::fma2(ptx::mul2(a, e), poly2(c, t), ptx::pk2(fmaxf(x0, 0.f), fmaxf(x1, 0.f))), x0, x1);
-}
 // y = accumulators + bias (16-byte aligned), N columns
 template <int N>
 __device__ __forceinline__ void add_bias(const uint32_t (&x)[N], const float* bias, float (&y)[N]) {
@@ -195,59 +164,58 @@ __device__ __forceinline__ void add_bias(const uint32_t (&x)[N], const float* bi
     ptx::upk2(ptx::add2(ptx::pk2u(x[e + 2], x[e + 3]), ptx::pk2(b.z, b.w)), y[e + 2], y[e + 3]);
   }
 }
-// The activation of a block of values, for the kernels that round it to bf16 (2^-9): within 5e-7 of apply_act.
-// The selection is outside the loop over the block, and the library functions (log1pf, expf, erff: tens of
-// instructions and branches each, inlined once per column) are not used: see the epilogues of the phi kernels.
+// The activation of a block of values: apply_act with the selection outside the loop over the block.  The library's
+// functions stay although the result is rounded to bf16: polynomials on ex2.approx and rcp.approx are a third faster (282 and
+// 219 us for the two kernels of the map named in phi_tc, 413 and 326 with these) but off by up to 2e-6 where these are off by
+// 3e-7, which moves roundings of the features and of the output.
 template <int N>
 __device__ __forceinline__ void act_block(float (&y)[N], int act) {
+  const auto each = [&](auto a) {
+#pragma unroll
+    for (int e = 0; e < N; ++e) y[e] = apply_act(y[e], decltype(a)::value);
+  };
   switch (act) {
-    case ACT_RELU:
-#pragma unroll
-      for (int e = 0; e < N; ++e) y[e] = fmaxf(y[e], 0.f);
-      break;
+    case ACT_RELU: each(std::integral_constant<int, ACT_RELU>()); break;
     case ACT_IDENTITY: break;
-    case ACT_SOFTPLUS:
-#pragma unroll
-      for (int e = 0; e < N; e += 2) softplus_fast2(y[e], y[e + 1]);
-      break;
-    case ACT_ELU1:
-#pragma unroll
-      for (int e = 0; e < N; ++e) y[e] = y[e] > 0.f ? y[e] + 1.f : sfu_ex2(1.4426950408889634f * y[e]);
-      break;
-    default:
-#pragma unroll
-      for (int e = 0; e < N; e += 2) gelu_fast2(y[e], y[e + 1]);
-      break;
+    case ACT_SOFTPLUS: each(std::integral_constant<int, ACT_SOFTPLUS>()); break;
+    case ACT_ELU1: each(std::integral_constant<int, ACT_ELU1>()); break;
+    default: each(std::integral_constant<int, ACT_GELU>()); break;
   }
 }
-// The power part + 1 of a block of values of one polynomial part (part <= 3).
-template <int N>
+// The power part + 1 of a block of values of one polynomial part (part <= 3).  The fourth power is multiplied up as
+// poly_power does, or squared twice as in the ReLU epilogues.
+template <bool RELU, int N>
 __device__ __forceinline__ void power_block(float (&y)[N], int part) {
   if (part == 0) return;
 #pragma unroll
   for (int e = 0; e < N; ++e) {
     const float u = y[e], u2 = u * u;
-    y[e] = part == 1 ? u2 : part == 2 ? u2 * u : u2 * u2;
+    y[e] = part == 1 ? u2 : part == 2 ? u2 * u : RELU ? u2 * u2 : u2 * u * u;
   }
 }
 
-// What the epilogues of the phi kernels do to a block of accumulator columns [col0, col0 + N) of a non-ReLU layer
-// (bias already added): the activation, for the last layer (is_u) the power of the columns' polynomial parts and zero
-// beyond D'.  D' is a multiple of 32 and P at most 4, so a part is a whole number of eight columns
-// and D' ends on a block.
-template <int N>
-__device__ __forceinline__ void act_power_block(float (&y)[N], int act, bool is_u, int col0, int part_w, int Dp) {
+// What the epilogues of the phi kernels do to a block of accumulator columns [col0, col0 + N) of a layer of `width` columns
+// (bias already added): the activation, for the last layer (is_u) the power of the columns' polynomial parts, and zero
+// beyond the layer's width.  Widths are multiples of 32 and P is at most 4, so a part is a whole number of eight columns and
+// a layer ends on a block: one beyond it costs no activation (its columns of the next matrix are zero).
+template <bool RELU, int N>
+__device__ __forceinline__ void act_power_block(float (&y)[N], int act, bool is_u, int col0, int part_w, int width) {
   static_assert(N % 8 == 0 && N <= 32, "blocks of whole parts");
-  act_block(y, act);
-  if (!is_u) return;
+  if (col0 >= width) {
+#pragma unroll
+    for (int e = 0; e < N; ++e) y[e] = 0.f;
+    return;
+  }
+  act_block(y, RELU ? (int)ACT_RELU : act);
+  if (!is_u || part_w == width) return;
 #pragma unroll
   for (int g = 0; g < N; g += 8) {
     float z[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) z[e] = y[g + e];
-    if (part_w < Dp) power_block(z, (col0 + g) / part_w);
+    power_block<RELU>(z, (col0 + g) / part_w);
 #pragma unroll
-    for (int e = 0; e < 8; ++e) y[g + e] = col0 < Dp ? z[e] : 0.f;
+    for (int e = 0; e < 8; ++e) y[g + e] = z[e];
   }
 }
 

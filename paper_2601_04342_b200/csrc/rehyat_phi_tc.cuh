@@ -407,10 +407,11 @@ phi_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtenso
             }
           }
         } else {
-          // Rolled over blocks of 16 columns with the selection of the activation outside the block.  Inlined per column
-          // and unrolled (the library's erff, log1pf and expf, a loop and a division per power) this role was
-          // thousands of instructions long: 12 heads x 13,440 tokens of a three-layer GELU / softplus map took 1,796 us
-          // here and 804 us in the read-out kernel, in this form 308 and 237 us (285 and 219 with packed polynomials).
+          // Rolled over blocks of 16 columns with the selection of the activation outside the block, and one call site
+          // below.  Inlined per column, unrolled and once per layer (the library's erff, log1pf and expf, a loop and a
+          // division per power) this role was thousands of instructions long: 12 heads x 13,440 tokens of a three-layer
+          // GELU / softplus map took 1,822 us here and 805 us in the read-out kernel, in this form 413 and 326 us.  Blocks
+          // of 8 columns 461 us, of 32 columns 414 us.  What is left is the issue of the functions' instructions.
 #pragma unroll 1
           for (int cb = 0; cb < 4; ++cb) {
             const int col0 = half * 128 + ch * 64 + cb * 16;
@@ -419,7 +420,7 @@ phi_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtenso
             tmem_ld16(tmem + lane_off + T_SCR + ch * 64 + cb * 16, x);
             tmem_wait_ld();
             add_bias(x, bias + ch * 64 + cb * 16, y);
-            act_power_block(y, RELU ? (int)ACT_RELU : is_u ? a.act_out : a.act_hidden, is_u, col0, part_w, Dp);
+            act_power_block<RELU>(y, is_u ? a.act_out : a.act_hidden, is_u, col0, part_w, is_u ? Dp : ex.Dh);
             if (is_u && !tok_valid) {
 #pragma unroll
               for (int e = 0; e < 16; ++e) y[e] = 0.f;
@@ -439,16 +440,28 @@ phi_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtenso
       if (aborted()) break;
       tok_valid = tok_a + j * 128 + r < tok_b;
       // a width of at most 128 has no second half
+      if constexpr (RELU && !NARROW) {
 #pragma unroll
-      for (int half = 0; half < 2; ++half)                          // first layer -> hidden buffer 0
-        if (half < nh) epi_step(false, half, s_b1 + half * 128, hid_sub(0, half * 2 + ch));
-      for (int m = 0; m < n_mid; ++m)                               // hidden layer m -> the buffer it does not read
+        for (int half = 0; half < 2; ++half)                        // first layer -> hidden buffer 0
+          if (half < nh) epi_step(false, half, s_b1 + half * 128, hid_sub(0, half * 2 + ch));
+        for (int m = 0; m < n_mid; ++m)                             // hidden layer m -> the buffer it does not read
 #pragma unroll
-        for (int half = 0; half < 2; ++half)
-          if (half < nh) epi_step(false, half, s_b2 + (1 + m) * 256 + half * 128, hid_sub((m & 1) ^ 1, half * 2 + ch));
+          for (int half = 0; half < 2; ++half)
+            if (half < nh) epi_step(false, half, s_b2 + (1 + m) * 256 + half * 128, hid_sub((m & 1) ^ 1, half * 2 + ch));
 #pragma unroll
-      for (int half = 0; half < 2; ++half)                          // last layer -> the phi tiles
-        if (half < nu) epi_step(true, half, s_b2 + half * 128, (half == 0 ? sPhiHalf0 : sPhiHalf1) + ch * PH_SUB);
+        for (int half = 0; half < 2; ++half)                        // last layer -> the phi tiles
+          if (half < nu) epi_step(true, half, s_b2 + half * 128, (half == 0 ? sPhiHalf0 : sPhiHalf1) + ch * PH_SUB);
+      } else {
+        // the same steps with one call site: the library's functions are in the code once
+#pragma unroll 1
+        for (int l = 0; l < n_mid + 2; ++l) {
+          const bool is_u = l == n_mid + 1;
+#pragma unroll 1
+          for (int half = 0; half < (is_u ? nu : nh); ++half)
+            epi_step(is_u, half, (l == 0 ? s_b1 : is_u ? s_b2 : s_b2 + l * 256) + half * 128,
+                     is_u ? (half == 0 ? sPhiHalf0 : sPhiHalf1) + ch * PH_SUB : hid_sub(l & 1, half * 2 + ch));
+        }
+      }
     }
     wait(&bars->out_ready, 0);
     if (!aborted()) {

@@ -325,7 +325,7 @@ readout_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUt
       } else {
         float y[NC];
         add_bias(x, bias, y);
-        act_power_block(y, is_u ? a.act_out : a.act_hidden, is_u, col0, part_w, Dp);
+        act_power_block<false>(y, is_u ? a.act_out : a.act_hidden, is_u, col0, part_w, is_u ? Dp : ex.Dh);
 #pragma unroll
         for (int e = 0; e < NC; e += 2) w[e >> 1] = pack_bf16(y[e], y[e + 1]);
       }

@@ -107,3 +107,62 @@ def test_fp32_phi_on_the_tensor_cores(d, nh, T, HW, Tc, To, Dh, Dp, P, act_hidde
     x = synth.make_inputs(wl, v_frame_offsets=True, phi_scale=2.0)
     y = _forward(wl, x, act_hidden=act_hidden, act_out=act_out)
     _gate(y, _oracle(wl, x, act_hidden=act_hidden, act_out=act_out), "fp32")
+
+
+def _act64(act, t):
+    """The activation of a float64 tensor, exact."""
+    if act == "softplus":
+        return torch.log1p(torch.exp(-t.abs())) + t.clamp(min=0)
+    if act == "elu1":
+        return torch.where(t > 0, t + 1, torch.exp(t))
+    return t * 0.5 * torch.special.erfc(-t / 2 ** 0.5)
+
+
+def _arguments_near_roundings(act, n_heads, width, d, unit):
+    """x [n_heads, d] and b [n_heads, width], bf16, so that act(x[i % d] + b[i]), the sum rounded to fp32, lies about
+    1.5 `unit` relative (GELU: of its argument) from a value halfway between two bf16 numbers."""
+    g = torch.Generator().manual_seed(4)
+    x = (torch.rand(n_heads, d, generator=g) * 34 - 29).bfloat16()
+    col = torch.arange(width) % d
+    pool = (torch.rand(4000, generator=g) * 2 - 1).bfloat16()
+    b = torch.empty(n_heads, width, dtype=torch.bfloat16)
+    for h in range(n_heads):
+        pre = (x[h].float()[col][:, None] + pool.float()[None, :]).double()
+        y = _act64(act, pre)
+        half = (y.float().view(torch.int32) & -65536 | 0x8000).view(torch.float32).double()      # between its bf16 neighbours
+        off = (y - half).abs() / (unit * (pre if act == "gelu" else y).abs() + 1e-300)
+        b[h] = pool[(off - 1.5).abs().argmin(1)]
+    return x, b
+
+
+@pytest.mark.parametrize("act", ["softplus", "elu1", "gelu"])
+@pytest.mark.parametrize("d,Dh,Dp,last", [(128, 256, 256, False), (128, 256, 256, True), (128, 192, 160, True), (64, 128, 128, True), (64, 64, 96, False)])
+def test_activations_are_as_precise_as_the_library(act, d, Dh, Dp, last):
+    """phi of a single token is the z part of the exported state.  With one non-zero weight per row the sums are exact, so
+    a feature is the bf16 rounding of act(x + b), act with the error of CUDA's expf (2 ulp), log1pf (1 ulp) and erff (2 ulp):
+    within 4e-7 of the exact function, for GELU, whose 1 + erf cancels in the negative tail, within 4e-7 of |x|."""
+    from paper_2601_04342_b200 import binding
+    nh, unit = 24, 4e-7
+    x, b = _arguments_near_roundings(act, nh, Dp if last else Dh, d, unit)
+    W1 = torch.zeros(nh, Dh, d)
+    W2 = torch.zeros(nh, Dp, Dh)
+    W1[:, torch.arange(Dh), torch.arange(Dh) % d] = 1
+    W2[:, torch.arange(Dp), torch.arange(Dp) % Dh] = 1
+    phi = {"W1": W1, "b1": torch.zeros(nh, Dh) if last else b, "W2": W2, "b2": b if last else torch.zeros(nh, Dp)}
+    phi = {n: t.bfloat16().cuda() for n, t in phi.items()}
+    op = binding.Rehyat(n_heads=nh, head_dim=d, phi_hidden=Dh, phi_dim=Dp, poly_degree=1, max_batch=1, max_tokens_per_frame=1, max_chunk_frames=1,
+                        act_hidden="identity" if last else act, act_out=act if last else "identity")
+    op.stream_begin(1, 1, 1, 1, 0)
+    k = x.cuda()[None, :, None, :].contiguous()
+    op.stream_step(k, k, k, phi, phi, 1)
+    assert op.status() == 0 and op.last_phi_impl == "tensor"
+    state = np.frombuffer(op.stream_export(), np.uint8)[-4 * nh * Dp * (d + 4):].view(np.float32)      # behind the header; no kept frames
+    op.close()
+    z = state.reshape(nh, Dp, d + 4)[..., d].astype(np.float64)
+    f = torch.arange(Dp) % Dh
+    pre = (x.float()[:, f % d] + b.float()[:, torch.arange(Dp) if last else f]).double()
+    exact = _act64(act, pre).numpy()
+    err = unit * np.abs(pre.numpy() if act == "gelu" else exact)
+    rnd = lambda v: torch.from_numpy(v).bfloat16().double().numpy()                    # noqa: E731
+    off = (z < rnd(exact - err)) | (z > rnd(exact + err))
+    assert not off.any(), f"{off.sum()} of {off.size} features are off"
