@@ -180,7 +180,7 @@ int rehyat_forward_host(rehyat_ctx* ctx, const void* q_host, const void* k_host,
  * rehyat_stream_begin starts a sequence (s_0 = 0, z_0 = 0, Eq. 14-15) for chunks of at most `chunk` frames
  * with `overlap` frames of overlap, and sizes two buffers (k and v) of (overlap + 4*chunk)*H*W tokens per
  * (batch, head) - more chunks where overlap > 3*chunk: the only allocation of this API, repeated only when a
- * later sequence needs more.  The softmax window slides through these buffers: a step appends its chunk's k and
+ * later sequence needs more (the sequence before it is over then, also where the allocation fails).  The softmax window slides through these buffers: a step appends its chunk's k and
  * v behind the kept overlap frames, the frames that stay are addressed rather than moved, and only at the end
  * of the buffers (every few steps) are they copied back to the front.  q and out are read and written in place.
  * rehyat_stream_step takes the next chunk,

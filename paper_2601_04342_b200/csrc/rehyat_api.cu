@@ -93,7 +93,7 @@ struct rehyat_ctx {
     void* vbuf = nullptr;
     void* qbuf = nullptr;         // the chunk's q after the q/k transform (contexts made with qk_transform only)
     int chunk_cap = 0;            // tokens per (batch, head) qbuf holds
-    size_t bytes = 0;
+    size_t kv_bytes = 0, q_bytes = 0;   // what kbuf and vbuf hold each, and qbuf
   } stream;
 };
 
@@ -892,14 +892,25 @@ int rehyat_stream_begin(rehyat_ctx* ctx, int32_t batch, int32_t H, int32_t W, in
   rehyat_ctx::Stream& s = ctx->stream;
   const size_t one = (size_t)batch * c.n_heads * cap * c.head_dim * elem_size(c.dtype);
   const size_t qone = c.qk_transform ? (size_t)batch * c.n_heads * chunk * HW * c.head_dim * elem_size(c.dtype) : 0;
-  if (one * 2 + qone > s.bytes) {                   // grow the buffers (the only allocation of this API)
+  // Grown when any of the buffers is too small, whatever the others hold (the only allocation of this API); a sequence in
+  // progress ends with its buffers.
+  if (one > s.kv_bytes || qone > s.q_bytes) {
     if (cudaStreamSynchronize(st) != cudaSuccess) return REHYAT_ERR_CUDA;
-    void** all[3] = {&s.kbuf, &s.vbuf, &s.qbuf};
-    for (void** p : all) { cudaFree(*p); *p = nullptr; }
-    s.bytes = 0;
-    if (cudaMalloc(&s.kbuf, one) != cudaSuccess || cudaMalloc(&s.vbuf, one) != cudaSuccess ||
-        (qone && cudaMalloc(&s.qbuf, qone) != cudaSuccess)) { cudaGetLastError(); return REHYAT_ERR_ALLOC; }
-    s.bytes = one * 2 + qone;
+    s.active = false;
+    // neither size shrinks, so that alternating sequences settle; short of memory, no more than this one needs
+    const size_t kv_max = one > s.kv_bytes ? one : s.kv_bytes, q_max = qone > s.q_bytes ? qone : s.q_bytes;
+    bool ok = false;
+    for (int least = 0; least < 2 && !ok; ++least) {
+      const size_t kv = least ? one : kv_max, qb = least ? qone : q_max;
+      void** all[3] = {&s.kbuf, &s.vbuf, &s.qbuf};
+      for (void** p : all) { cudaFree(*p); *p = nullptr; }
+      ok = cudaMalloc(&s.kbuf, kv) == cudaSuccess && cudaMalloc(&s.vbuf, kv) == cudaSuccess &&
+           (qb == 0 || cudaMalloc(&s.qbuf, qb) == cudaSuccess);
+      if (!ok) cudaGetLastError();
+      s.kv_bytes = ok ? kv : 0;
+      s.q_bytes = ok ? qb : 0;
+    }
+    if (!ok) return REHYAT_ERR_ALLOC;
   }
   s.chunk_cap = (int)(chunk * HW);
   s.active = true;

@@ -165,3 +165,61 @@ def test_chunks_as_views_of_the_whole_sequence(layout):
         assert op.status() == 0
     op.close()
     gate(out.double().cpu().numpy(), ref, "bf16")
+
+
+def _steps(op, wl, d, chunk, overlap, n_steps):
+    """The outputs of the first `n_steps` steps of a sequence on a context that may have served others before."""
+    op.stream_begin(wl.B, wl.H, wl.W, chunk, overlap)
+    out = []
+    for t in range(n_steps):
+        sl = slice(t * chunk * wl.HW, (t + 1) * chunk * wl.HW)
+        q, k, v = (d[n][:, :, sl].contiguous() for n in ("q", "k", "v"))
+        out.append(op.stream_step(q, k, v, d["phi_q"], d["phi_k"], chunk))
+    assert op.status() == 0
+    return torch.cat(out, 2)
+
+
+@pytest.mark.parametrize("qk", [False, True])
+def test_sequences_of_other_sizes_on_one_context(qk):
+    """k and v want overlap + rounds * chunk frames, the transformed q one chunk: a sequence of short chunks and a long
+    overlap has larger buffers in all but smaller ones for q than one of long chunks.  Each is sized by itself; every
+    sequence gives the bits of a fresh context."""
+    from paper_2601_04342_b200 import binding
+    wl = synth.Workload("sizes", 1, 2, 128, 12, 9, 17, 3, 1, "bf16", True, seed=synth.BASE_SEED + 98)
+    d = _dev(synth.make_inputs(wl, phi_scale=1.5, v_frame_offsets=True))
+    ang = torch.arange(wl.N, dtype=torch.float64)[:, None] * 10000.0 ** (-torch.arange(64, dtype=torch.float64) / 64)[None, :]
+    cos, sin = ang.cos().float().cuda(), ang.sin().float().cuda()
+
+    def make():
+        op = binding.for_workload(wl, qk_transform=qk)
+        if qk:
+            op.set_qk_transform(cos=cos, sin=sin)
+        return op
+
+    sizes = [(1, 10, 6), (3, 1, 4), (2, 0, 6), (1, 10, 12), (3, 3, 4)]          # chunk, overlap, steps
+    op = make()
+    for chunk, overlap, steps in sizes:
+        fresh = make()
+        want = _steps(fresh, wl, d, chunk, overlap, steps)
+        fresh.close()
+        assert torch.equal(_steps(op, wl, d, chunk, overlap, steps), want), (chunk, overlap)
+    op.close()
+
+
+def test_a_sequence_that_does_not_fit_ends_the_one_before():
+    """268 GB of window buffers cannot be had: the call says so, the sequence whose buffers it gave up is over, and the
+    context serves the next one."""
+    from paper_2601_04342_b200 import binding
+    wl = synth.Workload("nofit", 1, 64, 128, 6, 10, 10, 2, 1, "bf16", True, seed=synth.BASE_SEED + 99)
+    d = _dev(synth.make_inputs(wl, phi_scale=1.5))
+    op = binding.for_workload(wl)
+    want = _steps(op, wl, d, 2, 1, 3)
+    with pytest.raises(binding.RehyatError) as e:
+        op.stream_begin(1, wl.H, wl.W, 1, 80000)
+    assert e.value.code == binding.ERR_ALLOC
+    q = d["q"][:, :, :2 * wl.HW].contiguous()
+    with pytest.raises(binding.RehyatError) as e:
+        op.stream_step(q, q, q, d["phi_q"], d["phi_k"], 2)
+    assert e.value.code == binding.ERR_INVALID_ARG
+    assert torch.equal(_steps(op, wl, d, 2, 1, 3), want)
+    op.close()
