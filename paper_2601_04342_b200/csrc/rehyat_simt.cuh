@@ -469,11 +469,16 @@ readout_simt(const T* q, PhiPtrs<T> wq, PhiDims pd, Geo g, const float* state, f
   const int rg = lane >> 3, cg = lane & 7, cb = warp % NCB, row0 = warp / NCB * (4 * RR);
   uint8_t* const slab_ptr = slabs + warp * SIMT_STAGES * SIMT_SLAB;
   const uint32_t slab = ptx::smem_u32(slab_ptr);
-  auto issue_state = [&](int s) {                      // features [16 s, 16 s + 16) x 32 columns, rows of 128 bytes
+  // Features [16 s, 16 s + 16) x 32 columns, rows of 128 bytes; one commit group per call, also when there is nothing to copy.
+  // Nothing is copied beyond the last slab: no wait covers such a copy, and the next tile's weights go into the same slots.
+  const int n_slab = (pd.Dp + 15) / 16;
+  auto issue_state = [&](int s) {
+    if (s < n_slab) {
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int c = lane + 32 * u, f = s * 16 + (c >> 3);
-      cp_async16(slab + (s % SIMT_STAGES) * SIMT_SLAB + c * 16, S + (size_t)(f < pd.Dp ? f : 0) * SD + cb * 32 + (c & 7) * 4, f < pd.Dp);
+      for (int u = 0; u < 4; ++u) {
+        const int c = lane + 32 * u, f = s * 16 + (c >> 3);
+        cp_async16(slab + (s % SIMT_STAGES) * SIMT_SLAB + c * 16, S + (size_t)(f < pd.Dp ? f : 0) * SD + cb * 32 + (c & 7) * 4, f < pd.Dp);
+      }
     }
     cp_async_commit();
   };
@@ -520,7 +525,6 @@ readout_simt(const T* q, PhiPtrs<T> wq, PhiDims pd, Geo g, const float* state, f
 #pragma unroll
     for (int i = 0; i < RR; ++i) acc[i][0] = acc[i][1] = 0ull;
     const float* fr = F + (row0 + rg) * ldh;
-    const int n_slab = (pd.Dp + 15) / 16;
 #pragma unroll 1
     for (int s = 0; s < n_slab; ++s) {
       cp_async_wait<SIMT_STAGES - 2>();

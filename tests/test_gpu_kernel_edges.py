@@ -166,3 +166,15 @@ def test_activations_are_as_precise_as_the_library(act, d, Dh, Dp, last):
     rnd = lambda v: torch.from_numpy(v).bfloat16().double().numpy()                    # noqa: E731
     off = (z < rnd(exact - err)) | (z > rnd(exact + err))
     assert not off.any(), f"{off.sum()} of {off.size} features are off"
+
+
+# The read-out on the CUDA cores with five tiles per CTA (148 units of a chunk and a head take one CTA each): the slabs of
+# the state, then of the next tile's weights, go through the same slots.  One, seven, thirteen and sixteen slabs of a state.
+@pytest.mark.parametrize("dtype,d,Dh,Dp", [("fp32", 128, 256, 256), ("fp32", 64, 64, 8), ("bf16", 64, 136, 104), ("bf16", 128, 256, 200)])
+def test_several_tiles_per_cta_of_the_cuda_core_readout(dtype, d, Dh, Dp):
+    wl = synth.Workload("rdtiles", 1, 37, d, 5, 10, 15, 1, 0, dtype, dtype == "bf16", seed=synth.BASE_SEED + 407, phi_hidden=Dh, phi_dim=Dp)
+    x = synth.make_inputs(wl, v_frame_offsets=True)
+    y = _forward(wl, x, impl="simt")
+    _gate(y, _oracle(wl, x), dtype)
+    for _ in range(5):
+        np.testing.assert_array_equal(_forward(wl, x, impl="simt"), y)
