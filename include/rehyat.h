@@ -61,7 +61,7 @@ typedef enum { REHYAT_C_ROWMAX = 0, REHYAT_C_ZERO = 1 } rehyat_c_mode;
  * the softmax window; for phi, state and read-out also D_h and D' multiples of 32 with
  * 64 <= D_h <= 256, 32 <= D' <= 256; other widths keep the window on the tensor cores and run
  * the linear branch on the fp32 kernels).  fp32: by size, tensor-core kernels that split every operand into three bf16
- * parts (fp32 precision; values of 2^40 and more or not finite are left to the SIMT kernels) or SIMT fp32 kernels.
+ * parts (fp32 precision at all magnitudes; values of 2^39 and more or not finite are left to the SIMT kernels) or SIMT fp32 kernels.
  * SIMT / TENSOR force one (TENSOR fails with REHYAT_ERR_UNSUPPORTED where it does not apply, for fp32 always).  TENSOR_WINDOW: tensor-core window, SIMT linear branch (a cross-check). */
 typedef enum {
   REHYAT_IMPL_AUTO = 0, REHYAT_IMPL_SIMT = 1, REHYAT_IMPL_TENSOR = 2, REHYAT_IMPL_TENSOR_WINDOW = 3

@@ -17,9 +17,11 @@
 //   Q K^T of tile j + 1 is in the queue before P V of tile j, so that softmax j + 1 and the sum of O run beside MMAs.
 // Bound by the MMAs: 3,072 cycles per key tile of 128 x 64 at D = 128.  The same layer: 4,783 -> 1,051 us (0.56 ms of MMAs).
 //
-// Values beyond 2^40 (or not finite) cannot be split safely: whoever sees one leaves the launch's epoch in *unsafe, and
-// window_simt, launched behind this kernel, computes the call again; otherwise it ends at once.
-// At the other end the third part of a value below 2^-110 is a bf16 subnormal: such values keep fewer than 24 bits.
+// Every operand is multiplied by 2^20 as it is split, so that the parts of the smallest fp32 numbers are bf16 numbers too
+// (without it values below 2^-110 keep fewer than 24 bits), and what leaves an accumulator by 2^-40: both are exact.
+// Values from 2^39 on (or not finite) cannot be split safely, as 256 products of them would no longer fit an accumulator:
+// whoever sees one leaves the launch's epoch in *unsafe, and window_simt, launched behind this kernel, computes the call
+// again; otherwise it ends at once.
 #pragma once
 
 #include "rehyat_simt.cuh"
@@ -29,7 +31,8 @@ namespace rehyat {
 
 constexpr int F32_BN = 64, F32_STAGES = 2, F32_SOFTMAX_WARPS = 8, F32_LOAD_WARPS = 4;
 constexpr int F32_THREADS = (F32_SOFTMAX_WARPS + F32_LOAD_WARPS + 1) * 32;
-constexpr uint32_t F32_UNSAFE_BITS = 0x53800000u;     // 2^40
+constexpr uint32_t F32_UNSAFE_BITS = 0x53000000u;     // 2^39
+constexpr float F32_UP = 0x1p20f, F32_DOWN = 0x1p-40f;  // scale of the split operands, and what takes it out of a product
 
 struct F32Bars {
   uint64_t q_ready, k_full[F32_STAGES], k_empty[F32_STAGES], v_full[F32_STAGES], v_empty[F32_STAGES];
@@ -46,8 +49,9 @@ struct F32Shape {
   static constexpr uint32_t T_S = 3 * D / 2, T_O = T_S + 2 * 96;
 };
 
-// Two floats into the bf16 pairs of their three parts.
+// Two floats, scaled, into the bf16 pairs of their three parts.
 __device__ __forceinline__ void split3(float x0, float x1, uint32_t& h, uint32_t& m, uint32_t& l) {
+  ptx::upk2(ptx::mul2(ptx::pk2(x0, x1), ptx::pk2(F32_UP, F32_UP)), x0, x1);
   h = ptx::pack_bf16(x0, x1);
   x0 -= __uint_as_float(h << 16); x1 -= __uint_as_float(h & 0xffff0000u);
   m = ptx::pack_bf16(x0, x1);
@@ -270,7 +274,7 @@ window_f32_tc(const float* q, const float* k, const float* v, float* out, Geo g,
         const int n_here = w.hi - (w.lo + j * F32_BN + half * 32);   // keys of the window among this thread's
         float s[32], tmax = -INFINITY;
 #pragma unroll
-        for (int e = 0; e < 32; ++e) s[e] = __uint_as_float(x[e]) * scale;
+        for (int e = 0; e < 32; ++e) s[e] = __uint_as_float(x[e]) * (scale * F32_DOWN);
         if (n_here < 32) {
 #pragma unroll
           for (int e = 0; e < 32; ++e)
@@ -331,8 +335,8 @@ window_f32_tc(const float* q, const float* k, const float* v, float* out, Geo g,
           float4 aL = make_float4(0.f, 0.f, 0.f, 0.f);
           if (w.linear) aL = *reinterpret_cast<const float4*>(rd + rd_index(g, rd_rows, D, w.bh, w.ci, row - w.q0, (half * (D / 2) + c) >> 2));
           float y[4];
-          upk2(o[c / 2], y[0], y[1]);
-          upk2(o[c / 2 + 1], y[2], y[3]);
+          upk2(mul2(o[c / 2], pk2(F32_DOWN, F32_DOWN)), y[0], y[1]);
+          upk2(mul2(o[c / 2 + 1], pk2(F32_DOWN, F32_DOWN)), y[2], y[3]);
           st4(orow + c, (y[0] * ws + lam * aL.x) * inv, (y[1] * ws + lam * aL.y) * inv, (y[2] * ws + lam * aL.z) * inv,
               (y[3] * ws + lam * aL.w) * inv);
         }
@@ -628,7 +632,7 @@ phi_f32_tc(Geo g, PhiF32Args a) {
       tmem_ld16(tb + 64 + half * 32 + c, hi);
       tmem_wait_ld();
 #pragma unroll
-      for (int e = 0; e < 16; ++e) y[e] = (__uint_as_float(lo[e]) + __uint_as_float(hi[e])) + bias[half * 32 + c + e];
+      for (int e = 0; e < 16; ++e) y[e] = fmaf(__uint_as_float(lo[e]) + __uint_as_float(hi[e]), F32_DOWN, bias[half * 32 + c + e]);
       if (act == ACT_RELU) {
 #pragma unroll
         for (int e = 0; e < 16; ++e) y[e] = fmaxf(y[e], 0.f);
@@ -731,7 +735,7 @@ phi_f32_tc(Geo g, PhiF32Args a) {
             if constexpr (READOUT) {
               racc[dh][e / 2] = hf == 0 ? y : add2(racc[dh][e / 2], y);
             } else {
-              upk2u(y, lo[e], lo[e + 1]);
+              upk2u(mul2(y, pk2(F32_DOWN, F32_DOWN)), lo[e], lo[e + 1]);
             }
           }
           if (!READOUT) {
@@ -762,7 +766,7 @@ phi_f32_tc(Geo g, PhiF32Args a) {
               upk2(racc[dh][2 * e], y[0], y[1]);
               upk2(racc[dh][2 * e + 1], y[2], y[3]);
               *reinterpret_cast<float4*>(a.rd + rd_index(g, a.rd_rows, D, bh, ci, ric, (dh * 64 + half * 32) / 4 + e)) =
-                  make_float4(y[0], y[1], y[2], y[3]);
+                  make_float4(y[0] * F32_DOWN, y[1] * F32_DOWN, y[2] * F32_DOWN, y[3] * F32_DOWN);
             }
           if (half == 0) a.rd[rd_index(g, a.rd_rows, D, bh, ci, ric, D / 4)] = bars->sums[0][r] + bars->sums[1][r];
         }

@@ -178,3 +178,21 @@ def test_several_tiles_per_cta_of_the_cuda_core_readout(dtype, d, Dh, Dp):
     _gate(y, _oracle(wl, x), dtype)
     for _ in range(5):
         np.testing.assert_array_equal(_forward(wl, x, impl="simt"), y)
+
+
+@pytest.mark.parametrize("small", ["k", "v"])
+def test_fp32_keeps_its_precision_at_the_smallest_magnitudes(small):
+    """v, or k, near the smallest normal numbers (elements below it among them), with k the weights of phi_k and phi_q
+    scaled by powers of two so that half of the output stays linear: window, state and read-out on the tensor cores
+    have to carry 24 bits there too.  1e-6: three times the error at magnitude one."""
+    wl = synth.Workload("f32small", 1, 60, 128, 6, 10, 15, 1, 0, "fp32", False, P=1, seed=synth.BASE_SEED + 408)
+    x = synth.make_inputs(wl, v_frame_offsets=True, phi_scale=2.0)
+    x[small] = x[small] * 2.0 ** -122
+    for m, w, h in (("phi_k", 41, -81), ("phi_q", 19, 19)) if small == "k" else ():   # exponents of the weights, of the hidden units:
+        p = x[m]                                                  # phi_k(k) times 2^-40, phi_q(q) times 2^38
+        p["W1"], p["W2"] = p["W1"] * 2.0 ** w, p["W2"] * 2.0 ** w
+        p["b1"], p["b2"] = p["b1"] * 2.0 ** h, p["b2"] * 2.0 ** (h + w)
+    y, ref = _forward(wl, x), _oracle(wl, x)
+    back = 2.0 ** (122 if small == "v" else 0)
+    rel = np.linalg.norm(y * back - ref * back) / np.linalg.norm(ref * back)
+    assert rel <= 1e-6, f"relative error {rel:.2e}"
