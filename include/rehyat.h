@@ -23,6 +23,10 @@
  *     allocation, in the causal and in the bidirectional form.  A context serves one stream at a
  *     time (it owns the workspace).  The library keeps no process-wide state and reads no
  *     environment variable.
+ *   - rehyat_forward, rehyat_forward_static and the steps of a sequence (with the rehyat_stream_begin in front of
+ *     them, where its buffers are large enough already) can be captured into a CUDA graph after a first call outside.
+ *     A replay carries the settings and pointers of the capture; after one whose device-side wait ran out,
+ *     rehyat_status has to be read before the next.
  *   - There is no CPU fallback: on a machine without an sm_100 device rehyat_create fails.
  */
 #ifndef REHYAT_H

@@ -52,7 +52,8 @@ struct rehyat_ctx {
   float* state = nullptr;      // [Gmax][BHmax][Dp][d+4]
   float* partial = nullptr;    // [partial_units][BHmax][Dp][d+4]
   float* readout = nullptr;    // linear read-out of one chunk group, rd_cap rows per (batch, head), laid out by rd_index
-  int* status_dev = nullptr;
+  int* status_dev = nullptr;   // [0] sticky error bits, [1] epoch of a launch that gave up (ptx::WaitCtx); [2], [3] epochs of an fp32 window
+                               // and a phi launch with values that cannot be split, [4], [5] counters (simt_takes_over)
   float* cum = nullptr;        // bidirectional mode: [frames + 1][BHmax][Dp][d+4] states summed over whole frames
   int cum_frames = 0;
   TcWorkspace tc;              // extra buffers of the tensor-core path
@@ -244,7 +245,7 @@ int launch_group_simt(rehyat_ctx* ctx, const T* q, const T* k, const T* v, T* ou
     PhiPtrs<T> wk = {(const T*)phi->k_W1, (const T*)phi->k_b1, (const T*)phi->k_W2, (const T*)phi->k_b2,
                      (const T*)phi->k_Wmid, (const T*)phi->k_bmid};
     ctx->prof.begin(REHYAT_PROF_STATE, st);
-    const int* unsafe = nullptr;
+    int* unsafe = nullptr;
     int epoch = 0;
     if constexpr (sizeof(T) == 4) {
       if (split.f32_tc) {
@@ -272,7 +273,7 @@ int launch_group_simt(rehyat_ctx* ctx, const T* q, const T* k, const T* v, T* ou
     const PhiPlan plan = plan_phi(ctx, g.Np, (long long)busy_readout(g) * g.BH, 64);
     const int per_cta = (tiles + plan.parts - 1) / plan.parts;
     ctx->prof.begin(REHYAT_PROF_READOUT, st);
-    const int* unsafe = nullptr;
+    int* unsafe = nullptr;
     int epoch = 0;
     if constexpr (sizeof(T) == 4) {
       if (plan.f32_tc) {

@@ -57,6 +57,20 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
+// Of the kernels launched behind a tensor-core kernel of the fp32 operator: does this one have to compute the step, because
+// a value could not be split and *unsafe holds the launch's epoch?  The last CTA to have looked takes the mark away
+// (unsafe[2] counts them): a replay of a captured launch carries the same epoch, and would otherwise compute every step
+// twice ever after.  For all threads of a CTA.
+__device__ __forceinline__ bool simt_takes_over(int* unsafe, int epoch) {
+  if (*reinterpret_cast<volatile int*>(unsafe) != epoch) return false;
+  __syncthreads();
+  if (threadIdx.x == 0 && atomicAdd(unsafe + 2, 1) == (int)(gridDim.x * gridDim.y * gridDim.z) - 1) {
+    unsafe[2] = 0;
+    *unsafe = 0;
+  }
+  return true;
+}
+
 // Four consecutive elements in shared memory as two pairs of floats.
 __device__ __forceinline__ void ld_pairs(const float* p, uint64_t& a, uint64_t& b) {
   const ulonglong2 u = *reinterpret_cast<const ulonglong2*>(p);
@@ -250,12 +264,12 @@ __device__ __forceinline__ void load_rows_simt(float* dst, int ld, const __nv_bf
 // column d holding the z part.
 template <typename T, int D>
 __global__ void __launch_bounds__(SIMT_THREADS)
-state_partial_simt(const T* k, const T* v, PhiPtrs<T> wk, PhiDims pd, Geo g, int n_split, float* partial, const int* unsafe,
+state_partial_simt(const T* k, const T* v, PhiPtrs<T> wk, PhiDims pd, Geo g, int n_split, float* partial, int* unsafe,
                    int epoch) {
   extern __shared__ __align__(16) float smem[];
   ptx::grid_dep_wait();
   ptx::grid_dep_launch();
-  if (unsafe != nullptr && *unsafe != epoch) return;   // behind phi_f32_tc, which could do all of it
+  if (unsafe != nullptr && !simt_takes_over(unsafe, epoch)) return;   // behind phi_f32_tc, which could do all of it
   constexpr int SD = D + 4;
   const int ldh = simt_act_ld(pd.Dh, pd.Dp);
   float* Xs = smem;
@@ -436,12 +450,12 @@ combine_bidirectional(const float* cum, float* state, size_t per_slot, Geo g, in
 template <typename T, int D>
 __global__ void __launch_bounds__(SIMT_THREADS)
 readout_simt(const T* q, PhiPtrs<T> wq, PhiDims pd, Geo g, const float* state, float* rd, int rd_rows, int rd_half,
-             int tiles_per_cta, const int* unsafe, int epoch) {
+             int tiles_per_cta, int* unsafe, int epoch) {
   extern __shared__ __align__(16) float smem[];
   if (unsafe != nullptr) {                             // behind phi_f32_tc, which could do all of it
     ptx::grid_dep_wait();
     ptx::grid_dep_launch();
-    if (*unsafe != epoch) return;
+    if (!simt_takes_over(unsafe, epoch)) return;
   }
   constexpr int SD = D + 4;
   const int ldh = simt_act_ld(pd.Dh, pd.Dp);
@@ -676,9 +690,9 @@ struct WinSimt {
 template <typename T, int D, int WK>
 __global__ void __launch_bounds__(SIMT_THREADS)
 window_simt(const T* q, const T* k, const T* v, T* out, Geo g, const float* rd, int rd_rows, float scale, int c_mode,
-            float* share, int wait_first, const int* unsafe, int epoch) {
+            float* share, int wait_first, int* unsafe, int epoch) {
   if (wait_first) ptx::grid_dep_wait();                        // q, k, v may come from the direct predecessor
-  if (unsafe != nullptr && *unsafe != epoch) return;           // behind window_f32_tc, which could do all of it
+  if (unsafe != nullptr && !simt_takes_over(unsafe, epoch)) return;   // behind window_f32_tc, which could do all of it
   using S = WinSimt<T, D, WK>;
   extern __shared__ __align__(16) float smem[];
   constexpr int KJ = S::KJ, NQ = D / 32, RGS = 8 / WK;          // RGS: row groups of 16 per CTA
