@@ -275,7 +275,8 @@ size_t rehyat_workspace_bytes(const rehyat_ctx* ctx);
 /* Synchronises `cuda_stream`, reads the device status word and clears it.  Returns REHYAT_OK,
  * REHYAT_ERR_DEVICE_TIMEOUT or REHYAT_ERR_CUDA.
  * Every wait inside the tensor-core kernels (on an mbarrier: for a TMA load, a tcgen05.mma, another
- * role of the CTA) is bounded in wall time.  A wait that runs out makes its CTA stop issuing work,
+ * role of the CTA) is bounded in wall time; what a CTA waits for the kernel before it on the stream (a kernel may start
+ * early) is not counted.  A wait that runs out makes its CTA stop issuing work,
  * wait for what it has already put in flight, free its TMEM and return; the other CTAs of the same
  * launch follow at their next wait.  The output of that launch is then undefined, the status word
  * records the time-out until it is read here, and later launches are not affected. */

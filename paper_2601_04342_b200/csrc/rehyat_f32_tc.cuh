@@ -203,6 +203,7 @@ window_f32_tc(const float* q, const float* k, const float* v, float* out, Geo g,
       // TMEM is not freed, nor does the CTA exit, with an MMA still running: this wait is not cut short by the abort flag
       umma_commit(smem_u32(&bars->drained));
       mbar_wait_drain(smem_u32(&bars->drained), 0, wc);
+      grid_dep_wait();                                               // nor before the predecessor, where the epilogues were given up
     }
   } else {
     // ------------------------------------------------------------------ softmax, sum of O, epilogue
@@ -311,7 +312,7 @@ window_f32_tc(const float* q, const float* k, const float* v, float* out, Geo g,
       }
       add_o(n - 1, a_prev);
       bars->ls[half][r] = l;
-      grid_dep_wait();                                               // the read-out is the predecessor's result
+      grid_dep_wait_role(wc);                                        // the read-out is the predecessor's result
       grid_dep_launch();
       if (barrier(wait_ctx_aborted(wc) != 0)) break;
       l += bars->ls[half ^ 1][r];
@@ -527,7 +528,7 @@ phi_f32_tc(Geo g, PhiF32Args a) {
 #pragma unroll 1
         for (int dh = 0; dh < ND; ++dh) {
           if (READOUT) {
-            grid_dep_wait();                                         // the states are the predecessor's results
+            grid_dep_wait_role(wc);                                  // the states are the predecessor's results
             stage(S + (size_t)hf * 128 * SD + dh * 64, SD, Dp - hf * 128, 64, false);
           } else {
             stage(V + (long long)tok0 * g.stride_n + dh * 64, g.stride_n, rows, 64, false);
@@ -642,7 +643,7 @@ phi_f32_tc(Geo g, PhiF32Args a) {
       }
     };
     if (READOUT) {
-      grid_dep_wait();
+      grid_dep_wait_role(wc);
       grid_dep_launch();
       bars->z[threadIdx.x] = (int)threadIdx.x < Dp ? a.state[(((size_t)ci * g.BH + bh) * Dp + threadIdx.x) * SD + D] : 0.f;
     }

@@ -4,6 +4,7 @@
 
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
+#include <stddef.h>
 #include <stdint.h>
 
 namespace rehyat {
@@ -22,6 +23,16 @@ __device__ __forceinline__ bool elect_one() {
       : "=r"(pred));
   return pred != 0;
 }
+
+// ----------------------------------------------------------------------------- dependent launch
+// Programmatic dependent launch.  Every kernel of the library is launched as one that may start before its predecessor
+// on the stream has ended (launch_kernel in rehyat_tc.cuh).  grid_dep_wait returns when that predecessor is complete and
+// its writes are visible; grid_dep_launch lets the next kernel start once all CTAs of this grid have called it or ended.
+// The rule that makes early work safe: a CTA calls grid_dep_launch only after its grid_dep_wait, so that a kernel that
+// has started may use everything but the results of its direct predecessor, and no kernel ends before its predecessor.
+// (Loads of a predecessor's results must not go through pointers the compiler may take for read-only.)
+__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // ----------------------------------------------------------------------------- mbarrier
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
@@ -76,13 +87,16 @@ __device__ __forceinline__ bool mbar_try_wait_hint(uint32_t bar, uint32_t parity
 // must not issue anything further (no TMA load, no tcgen05.mma, no barrier arrival it owes): it leaves its loops
 // and goes to the common exit of the kernel.  A later launch carries another epoch, so one timeout does not
 // poison the launches that follow; the sticky bits stay until the host reads them.
+// What a CTA waits for its grid's predecessor does not count: see grid_dep_wait_role.
 // The context lives in the CTA's shared memory (set up by one thread before the first __syncthreads) and the
 // waits take its shared-memory address, so that it costs the hot loops no registers.
 struct WaitCtx {
   int abort_flag;                  // set by whichever thread of the CTA first gives up
   int epoch;                       // of this launch (never 0)
-  unsigned long long limit_ns;     // wall-time limit of one wait
+  unsigned long long limit_ns;     // wall-time limit of one wait, as it stands
   int* status;                     // global: [0] sticky error bits, [1] epoch of a launch in which a CTA gave up
+  unsigned long long own_limit_ns; // what the host asked for
+  unsigned long long start_ns;     // time of wait_ctx_init; 0 once the predecessor is known to have ended
 };
 // What a kernel receives from the host about waiting (and, for the one test that makes a wait run out, the
 // switch that makes the TMA producer withhold every load so that nothing is ever in flight).
@@ -92,16 +106,32 @@ struct WaitArgs {
   unsigned int limit_us;
   int withhold_loads;
 };
-__device__ __forceinline__ void wait_ctx_init(WaitCtx* w, const WaitArgs& a) {
-  w->abort_flag = 0;
-  w->epoch = a.epoch;
-  w->limit_ns = (unsigned long long)a.limit_us * 1000ull;
-  w->status = a.status;
-}
 __device__ __forceinline__ unsigned long long global_timer_ns() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
+}
+__device__ __forceinline__ void wait_ctx_init(WaitCtx* w, const WaitArgs& a) {
+  w->abort_flag = 0;
+  w->epoch = a.epoch;
+  w->limit_ns = w->own_limit_ns = (unsigned long long)a.limit_us * 1000ull;
+  w->start_ns = global_timer_ns();
+  w->status = a.status;
+}
+// grid_dep_wait of a role whose fellows may be waiting on barriers behind it.  How long the predecessor takes says nothing
+// about this grid, so the limit of their waits is lifted meanwhile, and is longer afterwards by what the CTA has been
+// running: every wait that has begun has the whole of its limit left.  Warps that come together write about the same;
+// whoever comes later finds the predecessor ended.
+__device__ __forceinline__ void grid_dep_wait_role(uint32_t wctx) {
+  constexpr uint32_t o_start = offsetof(WaitCtx, start_ns), o_limit = offsetof(WaitCtx, limit_ns), o_own = offsetof(WaitCtx, own_limit_ns);
+  unsigned long long start, own;
+  asm volatile("ld.volatile.shared.u64 %0, [%1];" : "=l"(start) : "r"(wctx + o_start));
+  if (start != 0ull) asm volatile("st.volatile.shared.u64 [%0], %1;" ::"r"(wctx + o_limit), "l"(~0ull) : "memory");
+  grid_dep_wait();
+  if (start == 0ull) return;
+  asm volatile("ld.volatile.shared.u64 %0, [%1];" : "=l"(own) : "r"(wctx + o_own));
+  asm volatile("st.volatile.shared.u64 [%0], %1;" ::"r"(wctx + o_limit), "l"(own + (global_timer_ns() - start)) : "memory");
+  asm volatile("st.volatile.shared.u64 [%0], %1;" ::"r"(wctx + o_start), "l"(0ull) : "memory");
 }
 __device__ __forceinline__ int wait_ctx_aborted(uint32_t wctx) {     // abort_flag is the first word of the context
   int f;
@@ -138,7 +168,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_
 // Wait of a role for what it has itself put in flight (its TMA loads, its tcgen05.mma through a commit) before
 // the CTA may free TMEM and exit.  The abort flag does not cut it short; only the time limit does.
 __device__ __forceinline__ bool mbar_wait_drain(uint32_t bar, uint32_t parity, uint32_t wctx) {
-  const unsigned long long limit_ns = reinterpret_cast<volatile WaitCtx*>(__cvta_shared_to_generic(wctx))->limit_ns;
+  const unsigned long long limit_ns = reinterpret_cast<volatile WaitCtx*>(__cvta_shared_to_generic(wctx))->own_limit_ns;
   const unsigned long long t0 = global_timer_ns();
   for (uint32_t i = 0;; ++i) {
     if (mbar_try_wait(bar, parity)) return true;
@@ -150,14 +180,6 @@ __device__ __forceinline__ bool mbar_wait_drain(uint32_t bar, uint32_t parity, u
 }
 
 // ----------------------------------------------------------------------------- TMA
-// Programmatic dependent launch.  Every kernel of the library is launched as one that may start before its predecessor
-// on the stream has ended (launch_kernel in rehyat_api.cu).  grid_dep_wait returns when that predecessor is complete and
-// its writes are visible; grid_dep_launch lets the next kernel start once all CTAs of this grid have called it or ended.
-// The rule that makes early work safe: a CTA calls grid_dep_launch only after its grid_dep_wait, so that a kernel that
-// has started may use everything but the results of its direct predecessor, and no kernel ends before its predecessor.
-// (Loads of a predecessor's results must not go through pointers the compiler may take for read-only.)
-__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ uint4 ld_global_v4(const void* p) {
   uint4 v;
   asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");

@@ -144,7 +144,7 @@ readout_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUt
           for (int ks = 0; ks < ks1; ++ks) tma_load_3d(dst + ks * 8192, &tm_s, full, ks * 64, f * 64, ci * g.BH + bh);
       };
       auto state_half = [&](int c) {                                // the blocks of features [128 c, 128 c + 128)
-        grid_dep_wait();                                            // the states are the predecessor's results
+        grid_dep_wait_role(wc);                                     // the states are the predecessor's results
         for (int f = 2 * c; f < 2 * c + 2 && f < nf; ++f) state_load(f);
       };
       for (int j = 0; j < n_tiles && alive; ++j) {
@@ -295,7 +295,7 @@ readout_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUt
     auto aborted = [&]() -> bool { return __any_sync(0xffffffffu, wait_ctx_aborted(wc) != 0); };
     auto wait = [&](uint64_t* bar, uint32_t parity) { mbar_wait(smem_u32(bar), parity, wc, PH_ERR_EPI); };
     // z_t: the first result of the predecessor that is needed; the loads and GEMMs of the first tile's H run meanwhile
-    grid_dep_wait();
+    grid_dep_wait_role(wc);
     grid_dep_launch();
     s_z[threadIdx.x] = (int)threadIdx.x < Dp ? a.state[(((size_t)ci * g.BH + bh) * Dp + threadIdx.x) * SD + d] : 0.f;
     asm volatile("bar.sync 1, 256;" ::: "memory");                  // the eight epilogue warps

@@ -383,6 +383,7 @@ window_tc(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
       // abort flag: TMEM must not be freed, nor the CTA exit, with a tcgen05.mma still running.
       umma_commit(smem_u32(&bars->drained));
       mbar_wait_drain(smem_u32(&bars->drained), 0, wc);
+      grid_dep_wait();                                               // nor before the predecessor, where the epilogues were given up
     }
   } else if (warp >= 4) {
     // ------------------------------------------------------------------ softmax + epilogue
@@ -424,7 +425,7 @@ window_tc(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
       uint4 rdv[D / 8];                                              // fp16 pairs of aL / nL
       float nL = 0.f;
       if (w.linear) {
-        grid_dep_wait();                                             // the read-out is the predecessor's result
+        grid_dep_wait_role(wc);                                      // the read-out is the predecessor's result
         grid_dep_launch();
         const int ric = (valid ? row : w.q0) - w.q0, ci = w.ci;      // row inside the chunk: consecutive threads, consecutive pieces
         const uint4* rdh = reinterpret_cast<const uint4*>(rd);

@@ -67,6 +67,60 @@ def test_a_wait_that_runs_out_is_reported_and_the_context_stays_usable(both_wind
     op.close()
 
 
+# 148 units would take an SM each; with 140 the window kernel starts on the SMs that are left and gets to its epilogue
+# while every other SM has milliseconds of read-out to do.
+@pytest.mark.parametrize("dtype,d,H,W,limit_us", [("bf16", 128, 64, 128, 500), ("fp32", 64, 32, 32, 1000)])
+def test_a_long_predecessor_does_not_run_out_the_limit(dtype, d, H, W, limit_us):
+    """Waits that last because the read-out kernel is still running are not counted against the wait limit."""
+    from paper_2601_04342_b200 import binding
+    wl = synth.Workload("longrd", 1, 35, d, 5, H, W, 1, 0, dtype, dtype == "bf16", seed=synth.BASE_SEED + 73, phi_hidden=256, phi_dim=256, phi_layers=4)
+    g = torch.Generator(device="cuda").manual_seed(7)
+    t = torch.bfloat16 if dtype == "bf16" else torch.float32
+    q, k, v = (torch.randn((1, 35, wl.N, d), generator=g, device="cuda").to(t) for _ in range(3))
+    sizes = {"W1": (35, 256, d), "b1": (35, 256), "Wmid": (35, 2, 256, 256), "bmid": (35, 2, 256), "W2": (35, 256, 256), "b2": (35, 256)}
+    phi = [{n: (0.05 * torch.randn(s, generator=g, device="cuda")).to(t) for n, s in sizes.items()} for _ in range(2)]
+    op = binding.for_workload(wl, group_tokens=wl.N, act_hidden="gelu", act_out="softplus")
+    args = (q, k, v, *phi, wl.T, wl.H, wl.W, wl.Tc, wl.To)
+    want = op.forward(*args)
+    op.profile_enable(True)
+    op.forward(*args)
+    assert op.profile_read()["readout"][0] > 2e-3 * limit_us   # the read-out alone takes more than twice the limit
+    op.profile_enable(False)
+    op.set_wait_limit(limit_us)
+    for _ in range(3):
+        y = op.forward(*args)
+        assert op.status() == binding.OK
+        assert torch.equal(y, want)
+    op.close()
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_a_wait_that_runs_out_in_the_fp32_kernels(d):
+    """The same for the fp32 operator on the tensor cores: state, read-out and window give up, the CUDA-core kernels behind
+    them have nothing to do, and the next call gives the bits of the one before."""
+    from paper_2601_04342_b200 import binding
+    wl = synth.Workload("timeout32", 1, 60, d, 6, 10, 15, 1, 0, "fp32", False, seed=synth.BASE_SEED + 74)
+    x = synth.make_inputs(wl, phi_scale=1.5, v_frame_offsets=True)
+    dev = _dev(x)
+    op = binding.for_workload(wl)
+    args = (dev["q"], dev["k"], dev["v"], dev["phi_q"], dev["phi_k"], wl.T, wl.H, wl.W, wl.Tc, wl.To)
+    before = op.forward(*args).clone()
+    assert op.status() == binding.OK and op.last_launches == 7   # scan, and three steps on the tensor cores with their stand-ins
+    assert np.abs(before.double().cpu().numpy() - _oracle(wl, x)).max() <= 1e-4
+    op.set_wait_limit(2000, withhold_loads=True)
+    t0 = torch.cuda.Event(enable_timing=True); t1 = torch.cuda.Event(enable_timing=True)
+    t0.record()
+    op.forward(*args)
+    t1.record()
+    assert op.status() == binding.ERR_DEVICE_TIMEOUT
+    assert t0.elapsed_time(t1) < 500.0
+    assert op.status() == binding.OK
+    op.set_wait_limit(0, withhold_loads=False)
+    assert torch.equal(op.forward(*args), before)
+    assert op.status() == binding.OK
+    op.close()
+
+
 def test_contexts_with_different_phi_widths_live_side_by_side():
     """The shared-memory limit of a kernel belongs to the function, not to a context: a context with narrow phi
     widths created (or a static call made) while a wider one is alive must not break the wider one."""
