@@ -16,7 +16,8 @@ def _built():
     build.build()
 
 
-def _forward(wl, x, layout="bhnd", **kw):
+def _forward(wl, x, layout="bhnd", launches=None, **kw):
+    """The operator's output; `launches`: how many kernels the call has to take (see F32_LAUNCHES)."""
     from paper_2601_04342_b200 import binding
     op = binding.for_workload(wl, **kw)
     q, k, v = (x[n].cuda() for n in ("q", "k", "v"))
@@ -25,6 +26,7 @@ def _forward(wl, x, layout="bhnd", **kw):
     pq, pk = ({n: t.cuda() for n, t in x[m].items()} for m in ("phi_q", "phi_k"))
     y = op.forward(q, k, v, pq, pk, wl.T, wl.H, wl.W, wl.Tc, wl.To, layout=layout)
     assert op.status() == 0
+    assert launches is None or op.last_launches == launches, f"{op.last_launches} kernels"
     op.close()
     return (y.transpose(1, 2) if layout == "bnhd" else y).double().cpu().numpy()
 
@@ -73,40 +75,152 @@ def test_cuda_core_kernels(dtype, d, nh, T, H, W, Tc, To, Dh, Dp, P, layers):
     _gate(_forward(wl, x, impl="simt"), _oracle(wl, x), dtype)
 
 
-# fp32 windows on the tensor cores: one to seven key tiles of 64 with remainders, several items of a CTA one after the
-# other with odd and even numbers of tiles, moving row maxima, both conventions for c.
-@pytest.mark.parametrize("d,nh,T,HW,Tc,To,c_mode", [(64, 3, 4, 129, 1, 0, "rowmax"), (128, 2, 5, 65, 1, 1, "zero"), (64, 160, 3, 65, 1, 1, "rowmax"),
-                                                    (128, 100, 6, 100, 3, 1, "rowmax"), (64, 61, 9, 43, 3, 2, "zero"), (64, 2, 3, 43, 1, 1, "rowmax"), (128, 7, 3, 150, 1, 2, "rowmax")])
-def test_fp32_window_on_the_tensor_cores(d, nh, T, HW, Tc, To, c_mode):
+# Kernels of an fp32 call of one group of chunks with a linear set: state, scan, read-out and window on the CUDA cores are 4;
+# a step on the tensor cores is one more, as the CUDA-core kernel stands behind it.
+F32_LAUNCHES = {"cuda cores": 4, "window": 5, "phi": 6, "phi and window": 7}
+
+
+def _rel(y, ref):
+    return np.linalg.norm(y - ref) / np.linalg.norm(ref)
+
+
+# fp32 windows on the tensor cores (and one that is too small for them): one to seven key tiles of 64 with remainders, several items of a CTA one after the
+# other with odd and even numbers of tiles, moving row maxima, both conventions for c.  Operands of two bf16 parts instead of
+# three (the inputs rounded to 16 bits in the oracle) are 2.6e-6 to 3.3e-6 off, with logits of half the size and c = 0
+# 5.6e-7 to 7.3e-7; the kernel is 1.5e-7 to 3.3e-7 and 1.0e-7 off.
+@pytest.mark.parametrize("d,nh,T,HW,Tc,To,c_mode,launches", [
+    (64, 3, 4, 129, 1, 0, "rowmax", 5), (128, 2, 5, 65, 1, 1, "zero", 5), (64, 160, 3, 65, 1, 1, "rowmax", 7), (128, 100, 6, 100, 3, 1, "rowmax", 7),
+    (64, 61, 9, 43, 3, 2, "zero", 7), (64, 2, 3, 43, 1, 1, "rowmax", 4), (64, 40, 6, 43, 1, 3, "rowmax", 7), (128, 3, 6, 64, 1, 5, "zero", 2), (128, 7, 3, 150, 1, 2, "rowmax", 2)])
+def test_fp32_window_on_the_tensor_cores(d, nh, T, HW, Tc, To, c_mode, launches):
     wl = synth.Workload("f32tc", 1, nh, d, T, 1, HW, Tc, To, "fp32", False, seed=synth.BASE_SEED + 404)
     x = synth.make_inputs(wl, v_frame_offsets=True)
     x["q"] = x["q"] * (2 if c_mode == "rowmax" else 0.5)
-    _gate(_forward(wl, x, impl="auto", c_mode=c_mode), _oracle(wl, x, c_mode=c_mode), "fp32")
+    y, ref = _forward(wl, x, impl="auto", c_mode=c_mode, launches=launches), _oracle(wl, x, c_mode=c_mode)
+    _gate(y, ref, "fp32")
+    rel = _rel(y, ref)
+    assert rel <= (1e-6 if c_mode == "rowmax" else 3e-7), f"relative error {rel:.2e}"
 
 
+# A value that cannot be split, in each place where one may come up: an input, a weight of either map, the power of a feature,
+# a state.  3 heads: only the window runs on the tensor cores; 60 heads: phi, state and read-out too.
+@pytest.mark.parametrize("nh,T,HW,To,token,launches", [(3, 4, 200, 1, 333, 5), (60, 6, 150, 0, 183, 7)])
 @pytest.mark.parametrize("where,value", [("k", -3.4e38), ("k", float("-inf")), ("v", float("inf")), ("q", float("nan")), ("v", 1e30),
-                                         ("q", 2.0 ** 41)])
-def test_fp32_values_that_cannot_be_split(where, value):
+                                         ("q", 2.0 ** 41), ("k", 2.0 ** 39), ("phi_k.W1", 2.0 ** 40), ("phi_k.W2", -2.0 ** 40), ("phi_q.W1", 2.0 ** 40),
+                                         ("phi_q.W2", 2.0 ** 40), ("power", 2.0 ** 11), ("state", 2.0 ** 38)])
+def test_fp32_values_that_cannot_be_split(nh, T, HW, To, token, launches, where, value):
     """Values beyond what the split into bf16 parts carries are computed by the CUDA-core kernels, as if they were alone (the
-    state sums of the two calls are split differently over CTAs: fp32 sums in another order)."""
-    wl = synth.Workload("f32big", 1, 3, 128, 4, 10, 20, 1, 1, "fp32", False, seed=synth.BASE_SEED + 405)
+    state sums of the two calls are split differently over CTAs: fp32 sums in another order, compared by the row where
+    large terms cancel)."""
+    P = 4 if where == "power" else 1 if where == "state" else 2
+    wl = synth.Workload("f32big", 1, nh, 128, T, 1, HW, 1, To, "fp32", False, P=P, seed=synth.BASE_SEED + 405)
     x = synth.make_inputs(wl)
-    x[where][0, 1, 333, 5] = value
-    np.testing.assert_allclose(_forward(wl, x, impl="auto"), _forward(wl, x, impl="simt"), rtol=1e-5, atol=1e-6)
+    if where == "power":                                       # u^4 of 2^44
+        x["phi_k"]["b2"][1] = value
+    elif where == "state":                                     # features of 16 and a v of 2^38: each fits, their product does not
+        x["phi_k"]["b2"][1] = 16.0
+        x["v"][0, 1, token, 5] = value
+    elif "." in where:
+        m, n = where.split(".")
+        x[m][n][1, 7, 5] = value
+    else:
+        x[where][0, 1, token, 5] = value
+    y, alone = _forward(wl, x, impl="auto", launches=launches), _forward(wl, x, impl="simt", launches=4)
+    if where in ("q", "k", "v"):
+        np.testing.assert_allclose(y, alone, rtol=1e-5, atol=1e-6)
+        return
+    assert np.isfinite(alone).all()
+    np.testing.assert_array_less(np.abs(y - alone), np.broadcast_to(1e-5 * np.abs(alone).max(-1, keepdims=True) + 1e-6, y.shape))
 
 
 # fp32 phi on the tensor cores: widths that end inside quarters of 64 and halves of 128 columns, chunks that end inside
 # tiles of 128 tokens, several tiles of a CTA, all degrees and activations (more than one round of tiles of 32 on the SMs).
 # The features are non-negative: with both signs the denominator of Eq. 5 may vanish and no tolerance holds.
-@pytest.mark.parametrize("d,nh,T,HW,Tc,To,Dh,Dp,P,act_hidden,act_out", [
-    (64, 60, 6, 150, 1, 0, 8, 8, 1, "relu", "relu"), (128, 60, 6, 150, 1, 0, 72, 136, 2, "gelu", "softplus"),
-    (128, 40, 7, 129, 3, 1, 256, 256, 4, "relu", "relu"), (64, 40, 7, 100, 3, 2, 200, 192, 3, "elu1", "elu1"),
-    (64, 4, 9, 400, 4, 1, 128, 128, 2, "relu", "relu"), (128, 6, 9, 410, 4, 1, 64, 64, 2, "identity", "softplus")])
-def test_fp32_phi_on_the_tensor_cores(d, nh, T, HW, Tc, To, Dh, Dp, P, act_hidden, act_out):
+F32_PHI = [(64, 60, 6, 150, 1, 0, 8, 8, 1, "relu", "relu", 7), (128, 60, 6, 150, 1, 0, 72, 136, 2, "gelu", "softplus", 7),
+           (128, 40, 7, 129, 3, 1, 256, 256, 4, "relu", "relu", 7), (64, 40, 7, 100, 3, 2, 200, 192, 3, "elu1", "elu1", 7),
+           (64, 4, 9, 400, 4, 1, 128, 128, 2, "relu", "relu", 7), (128, 6, 9, 410, 4, 1, 64, 64, 2, "identity", "softplus", 7)]
+
+
+@pytest.mark.parametrize("d,nh,T,HW,Tc,To,Dh,Dp,P,act_hidden,act_out,launches", F32_PHI)
+def test_fp32_phi_on_the_tensor_cores(d, nh, T, HW, Tc, To, Dh, Dp, P, act_hidden, act_out, launches):
     wl = synth.Workload("f32phi", 1, nh, d, T, 1, HW, Tc, To, "fp32", False, P=P, seed=synth.BASE_SEED + 406, phi_hidden=Dh, phi_dim=Dp)
     x = synth.make_inputs(wl, v_frame_offsets=True, phi_scale=2.0)
-    y = _forward(wl, x, act_hidden=act_hidden, act_out=act_out)
-    _gate(y, _oracle(wl, x, act_hidden=act_hidden, act_out=act_out), "fp32")
+    y, ref = _forward(wl, x, act_hidden=act_hidden, act_out=act_out, launches=launches), _oracle(wl, x, act_hidden=act_hidden, act_out=act_out)
+    _gate(y, ref, "fp32")
+    rel = _rel(y, ref)
+    assert rel <= 1e-6, f"relative error {rel:.2e}"
+
+
+@pytest.mark.parametrize("d,Dh,Dp", [(128, 64, 8), (64, 64, 8), (128, 256, 8), (128, 256, 256)])
+def test_fp32_phi_carries_24_bits(d, Dh, Dp):
+    """In the operator's output the errors of many features and tokens average out.  Here they do not: the state of a
+    sequence whose tokens are all the same (operands of two parts: 3.9e-6 to 5.7e-6 off), and the linear share of the
+    normaliser with a few features (two-part weights of phi_q alone: 1.2e-6 to 1.8e-6)."""
+    from paper_2601_04342_b200 import binding
+    wl = synth.Workload("f32bits", 1, 400, d, 1, 1, 33, 1, 0, "fp32", False, P=1, seed=synth.BASE_SEED + 411, phi_hidden=Dh, phi_dim=Dp)
+    x = synth.make_inputs(wl, phi_scale=4.0)
+    k, v = (x[n][:, :, :1] for n in ("k", "v"))
+    dev = [t.expand(-1, -1, 33, -1).contiguous().cuda() for t in (x["q"][:, :, :1], k, v)]
+    pk = {n: t.cuda() for n, t in x["phi_k"].items()}
+    op = binding.for_workload(wl)
+    op.stream_begin(1, 1, 33, 1, 0)
+    op.stream_step(*dev, pk, pk, 1)
+    assert op.last_launches == 4 and op.status() == 0          # window, scan, and the state on the tensor cores with its stand-in
+    state = np.frombuffer(op.stream_export(), np.uint8)[-4 * 400 * Dp * (d + 4):].view(np.float32).reshape(400, Dp, d + 4).astype(np.float64)
+    op.close()
+    f = synth.to_f64(x)["phi_k"]
+    h = np.maximum(np.einsum("hd,hed->he", k[0, :, 0].double().numpy(), f["W1"]) + f["b1"], 0)
+    z = 33 * np.maximum(np.einsum("he,hfe->hf", h, f["W2"]) + f["b2"], 0)
+    assert _rel(state[..., d], z) <= 1e-6 and _rel(state[..., :d], z[..., None] * v[0, :, 0].double().numpy()[:, None]) <= 1e-6
+    if Dp > 8:
+        return
+    wl = wl.with_(n_heads=60, T=2, W=150)
+    x = synth.make_inputs(wl, phi_scale=4.0)
+    op = binding.for_workload(wl)
+    share = torch.zeros(1, 60, wl.N, device="cuda")
+    op.set_linear_share_output(share)
+    op.forward(*(x[n].cuda() for n in ("q", "k", "v")), *({n: t.cuda() for n, t in x[m].items()} for m in ("phi_q", "phi_k")), 2, 1, 150, 1, 0)
+    assert op.last_launches == F32_LAUNCHES["phi and window"] and op.status() == 0
+    op.close()
+    _, ref = _oracle(wl, x, return_parts=True)
+    got = share.double().cpu().numpy()
+    assert np.abs(got[..., :150]).max() == 0 and 0.3 < ref[..., 150:].mean() < 0.9
+    assert _rel(got[..., 150:], ref[..., 150:]) <= 6e-7
+
+
+@pytest.mark.parametrize("d,Tc,To", [(128, 2, 1), (64, 3, 0), (128, 1, 3)])
+def test_fp32_stream_on_the_tensor_cores(d, Tc, To):
+    """Steps of a sequence: increments of "chunk 1" into the running state, read-outs of a state alone."""
+    from paper_2601_04342_b200 import binding
+    wl = synth.Workload("f32stream", 1, 60, d, 7, 10, 15, Tc, To, "fp32", False, seed=synth.BASE_SEED + 409)
+    x = synth.make_inputs(wl, v_frame_offsets=True, phi_scale=2.0)
+    q, k, v = (x[n].cuda() for n in ("q", "k", "v"))
+    pq, pk = ({n: t.cuda() for n, t in x[m].items()} for m in ("phi_q", "phi_k"))
+    out = torch.empty_like(q)
+    op = binding.for_workload(wl)
+    op.stream_begin(1, wl.H, wl.W, Tc, To)
+    took = []
+    for f0 in range(0, wl.T, Tc):
+        f1 = min(f0 + Tc, wl.T)
+        sl = slice(f0 * wl.HW, f1 * wl.HW)
+        op.stream_step(q[:, :, sl], k[:, :, sl], v[:, :, sl], pq, pk, f1 - f0, out=out[:, :, sl])
+        took.append(op.last_launches)
+    assert op.status() == 0
+    op.close()
+    assert max(took) == F32_LAUNCHES["phi and window"], took
+    y, ref = out.double().cpu().numpy(), _oracle(wl, x)
+    _gate(y, ref, "fp32")
+    assert _rel(y, ref) <= 1e-6, f"relative error {_rel(y, ref):.2e}"
+
+
+def test_fp32_bidirectional_on_the_tensor_cores():
+    """States summed frame by frame in two groups, one combination of them per chunk, read-outs with every prefix."""
+    wl = synth.Workload("f32bidir", 1, 24, 128, 18, 10, 15, 2, 1, "fp32", False, seed=synth.BASE_SEED + 410)
+    x = synth.make_inputs(wl, v_frame_offsets=True, phi_scale=2.0)
+    f = synth.to_f64(x)
+    y = _forward(wl, x, bidirectional=True, launches=3 + 3 + 1 + 4)
+    ref = orc.hybrid_direct(f["q"], f["k"], f["v"], f["phi_q"], f["phi_k"], wl.T, wl.HW, wl.Tc, wl.To, P=wl.P, causal=False)
+    _gate(y, ref, "fp32")
+    assert _rel(y, ref) <= 1e-6, f"relative error {_rel(y, ref):.2e}"
 
 
 def _act64(act, t):
