@@ -15,7 +15,8 @@
 //     warp 12     UMMA issuer: S = Q K^T (48 MMAs of N = 64), O = P V (24 of N = D), Q and P read from TMEM
 //   TMEM: Q planes [0, 3D/2), two S slots of 96 columns (64 of S; the three planes of P overwrite them), O [3D/2 + 192, + D).
 //   Q K^T of tile j + 1 is in the queue before P V of tile j, so that softmax j + 1 and the sum of O run beside MMAs.
-// Bound by the MMAs: 3,072 cycles per key tile of 128 x 64 at D = 128.  The same layer: 4,783 -> 1,051 us (0.56 ms of MMAs).
+// Bound by the MMAs: 3,072 cycles per key tile of 128 x 64 at D = 128.  The same layer: 4,783 -> 1,106 us (0.56 ms of MMAs;
+// 1,053 without the multiplication by 2^20 below).
 //
 // Every operand is multiplied by 2^20 as it is split, so that the parts of the smallest fp32 numbers are bf16 numbers too
 // (without it values below 2^-110 keep fewer than 24 bits), and what leaves an accumulator by 2^-40: both are exact.
@@ -371,7 +372,7 @@ window_f32_tc(const float* q, const float* k, const float* v, float* out, Geo g,
 //   TMEM: accumulators [0, 128), H planes [128, 512).
 // A pass waits for the epilogue of the one before: the chain is what bounds a tile (37,000 cycles of MMAs at the default
 // widths, about as long again in hand-overs and epilogues).  12 heads x 12,600 tokens of 128 channels against the
-// CUDA-core kernels: state 1,319 -> 445 us, read-out 1,284 -> 402 us.
+// CUDA-core kernels: state 1,319 -> 458 us, read-out 1,284 -> 406 us.
 // ---------------------------------------------------------------------------------------------
 struct PhiF32Args {
   const float *x, *v, *W1, *b1, *W2, *b2, *state;

@@ -673,7 +673,7 @@ qk_prepare(const T* q, const T* k, T* qo, T* ko, QkPrepArgs a) {
 // read-out `rd`.  grid (tiles per chunk of BM rows, G, BH), SIMT_THREADS threads.
 // A warp has 16 query rows and 1/WK of the keys of every key tile (BM = 128 / WK rows per CTA); the WK warps of the same
 // rows keep maxima and sums of their own and are merged at the end.  WK = 1 needs the fewest loads per multiply-add,
-// WK = 4 gives a short sequence four times as many CTAs (window_simt_split chooses).  Per key tile two barriers: V is
+// WK = 4 gives a short sequence four times as many CTAs (launch_group_simt chooses).  Per key tile two barriers: V is
 // copied in while Q K^T runs, the next K while P V runs.
 template <typename T, int D, int WK>
 struct WinSimt {
