@@ -164,10 +164,52 @@ __device__ __forceinline__ void add_bias(const uint32_t (&x)[N], const float* bi
     ptx::upk2(ptx::add2(ptx::pk2u(x[e + 2], x[e + 3]), ptx::pk2(b.z, b.w)), y[e + 2], y[e + 3]);
   }
 }
-// The activation of a block of values: apply_act with the selection outside the loop over the block.  The library's
-// functions stay although the result is rounded to bf16: polynomials on ex2.approx and rcp.approx are a third faster (282 and
-// 219 us for the two kernels of the map named in phi_tc, 413 and 326 with these) but off by up to 2e-6 where these are off by
-// 3e-7, which moves roundings of the features and of the output.
+// GELU and softplus of a pair of values of bounded magnitude on packed multiply-adds; both polynomials are least-maximum
+// fits whose own error (2e-9, 2e-10) is far below what the fp32 roundings leave.
+//   GELU, |x| <= 2:      x Phi(x),  Phi(x) = 1/2 + x Q(x^2)
+//   softplus, |x| <= 1:  ln 2 + x/2 + x^2 R(x^2)             (the even part is ln(2 cosh(x/2)))
+// Largest error over 2^24 arguments of the range, relative to the exact value (GELU: to x), theirs and that of the library's
+// functions in apply_act: GELU 1.05e-7 and 1.08e-7, softplus 1.20e-7 and 1.74e-7; root mean square 2.2e-8 and 2.3e-8,
+// 3.7e-8 and 4.0e-8.  Wider ranges would need terms that cancel (softplus at -2: 7e-7).
+constexpr float GELU_RANGE = 2.f, SOFTPLUS_RANGE = 1.f;
+__device__ __forceinline__ void gelu2_near(float& y0, float& y1) {
+  using namespace ptx;
+  const auto both = [](float c) { return pk2(c, c); };
+  const uint64_t x = pk2(y0, y1), s = mul2(x, x);
+  uint64_t p = fma2(both(-1.6666440671997407e-08f), s, both(5.219349645813054e-07f));
+  p = fma2(p, s, both(-8.957101272244472e-06f));
+  p = fma2(p, s, both(1.1446127609815449e-04f));
+  p = fma2(p, s, both(-1.1862065875902772e-03f));
+  p = fma2(p, s, both(9.97286569327116e-03f));
+  p = fma2(p, s, both(-6.649018824100494e-02f));
+  p = fma2(p, s, both(3.989422619342804e-01f));
+  upk2(mul2(x, fma2(p, x, both(0.5f))), y0, y1);
+}
+__device__ __forceinline__ void softplus2_near(float& y0, float& y1) {
+  using namespace ptx;
+  const auto both = [](float c) { return pk2(c, c); };
+  const uint64_t x = pk2(y0, y1), s = mul2(x, x);
+  uint64_t p = fma2(both(1.6702316543160123e-06f), s, both(-2.585325637483038e-05f));
+  p = fma2(p, s, both(3.469709772616625e-04f));
+  p = fma2(p, s, both(-5.208276677876711e-03f));
+  p = fma2(p, s, both(1.249999925494194e-01f));
+  upk2(fma2(p, s, fma2(x, both(0.5f), both(0.69314718055994531f))), y0, y1);
+}
+// Largest magnitude of a block of values (one that is not a number does not count).
+template <int N>
+__device__ __forceinline__ float max_abs(const float (&y)[N]) {
+  static_assert(N % 2 == 0, "");
+  float m = fabsf(y[0]);
+#pragma unroll
+  for (int e = 1; e + 1 < N; e += 2) m = ptx::fmax3(m, fabsf(y[e]), fabsf(y[e + 1]));
+  return fmaxf(m, fabsf(y[N - 1]));
+}
+// The activation of a block of values: apply_act with the selection outside the loop over the block.  GELU and softplus take
+// the polynomials above where the whole warp's block lies in their range, which the pre-activations of these maps mostly do
+// (weights of 0.02 and inputs of magnitude one: standard deviation 0.2), and the library's functions otherwise; the vote
+// costs half an instruction per value.  The issue of the library's instructions was what bounded the kernels of such maps: 12
+// heads x 13,440 tokens of a three-layer GELU / softplus map, state 414 -> 252 us, read-out 328 -> 194 us.  (Functions good to
+// 2e-6 would do no better, 282 and 219 us, and move the roundings to bf16 that follow.)  All 32 lanes call it.
 template <int N>
 __device__ __forceinline__ void act_block(float (&y)[N], int act) {
   const auto each = [&](auto a) {
@@ -177,9 +219,23 @@ __device__ __forceinline__ void act_block(float (&y)[N], int act) {
   switch (act) {
     case ACT_RELU: each(std::integral_constant<int, ACT_RELU>()); break;
     case ACT_IDENTITY: break;
-    case ACT_SOFTPLUS: each(std::integral_constant<int, ACT_SOFTPLUS>()); break;
+    case ACT_SOFTPLUS:
+      if (__all_sync(0xffffffffu, max_abs(y) <= SOFTPLUS_RANGE)) {
+#pragma unroll
+        for (int e = 0; e < N; e += 2) softplus2_near(y[e], y[e + 1]);
+      } else {
+        each(std::integral_constant<int, ACT_SOFTPLUS>());
+      }
+      break;
     case ACT_ELU1: each(std::integral_constant<int, ACT_ELU1>()); break;
-    default: each(std::integral_constant<int, ACT_GELU>()); break;
+    default:
+      if (__all_sync(0xffffffffu, max_abs(y) <= GELU_RANGE)) {
+#pragma unroll
+        for (int e = 0; e < N; e += 2) gelu2_near(y[e], y[e + 1]);
+      } else {
+        each(std::integral_constant<int, ACT_GELU>());
+      }
+      break;
   }
 }
 // The power part + 1 of a block of values of one polynomial part (part <= 3).  The fourth power is multiplied up as

@@ -411,7 +411,8 @@ phi_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtenso
           // below.  Inlined per column, unrolled and once per layer (the library's erff, log1pf and expf, a loop and a
           // division per power) this role was thousands of instructions long: 12 heads x 13,440 tokens of a three-layer
           // GELU / softplus map took 1,822 us here and 805 us in the read-out kernel, in this form 413 and 326 us.  Blocks
-          // of 8 columns 461 us, of 32 columns 414 us.  What is left is the issue of the functions' instructions.
+          // of 8 columns 461 us, of 32 columns 414 us.  What was left was the issue of the functions' instructions: 252 and
+          // 194 us with the polynomials of act_block.
 #pragma unroll 1
           for (int cb = 0; cb < 4; ++cb) {
             const int col0 = half * 128 + ch * 64 + cb * 16;

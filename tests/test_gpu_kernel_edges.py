@@ -232,13 +232,13 @@ def _act64(act, t):
     return t * 0.5 * torch.special.erfc(-t / 2 ** 0.5)
 
 
-def _arguments_near_roundings(act, n_heads, width, d, unit):
+def _arguments_near_roundings(act, n_heads, width, d, unit, lo=-29, hi=5, spread=1):
     """x [n_heads, d] and b [n_heads, width], bf16, so that act(x[i % d] + b[i]), the sum rounded to fp32, lies about
     1.5 `unit` relative (GELU: of its argument) from a value halfway between two bf16 numbers."""
     g = torch.Generator().manual_seed(4)
-    x = (torch.rand(n_heads, d, generator=g) * 34 - 29).bfloat16()
+    x = (torch.rand(n_heads, d, generator=g) * (hi - lo) + lo).bfloat16()
     col = torch.arange(width) % d
-    pool = (torch.rand(4000, generator=g) * 2 - 1).bfloat16()
+    pool = ((torch.rand(4000, generator=g) * 2 - 1) * spread).bfloat16()
     b = torch.empty(n_heads, width, dtype=torch.bfloat16)
     for h in range(n_heads):
         pre = (x[h].float()[col][:, None] + pool.float()[None, :]).double()
@@ -255,9 +255,27 @@ def test_activations_are_as_precise_as_the_library(act, d, Dh, Dp, last):
     """phi of a single token is the z part of the exported state.  With one non-zero weight per row the sums are exact, so
     a feature is the bf16 rounding of act(x + b), act with the error of CUDA's expf (2 ulp), log1pf (1 ulp) and erff (2 ulp):
     within 4e-7 of the exact function, for GELU, whose 1 + erf cancels in the negative tail, within 4e-7 of |x|."""
-    from paper_2601_04342_b200 import binding
     nh, unit = 24, 4e-7
     x, b = _arguments_near_roundings(act, nh, Dp if last else Dh, d, unit)
+    _check_features(act, nh, d, Dh, Dp, last, x, b, unit)
+
+
+@pytest.mark.parametrize("act,reach", [("softplus", 1.0), ("gelu", 2.0)])
+@pytest.mark.parametrize("d,Dh,Dp,last", [(128, 256, 256, True), (128, 192, 160, False), (64, 128, 96, True)])
+def test_activations_of_small_arguments(act, reach, d, Dh, Dp, last):
+    """Blocks of arguments of at most `reach` take polynomials: largest error 1.2e-7 (softplus, relative) and 1.05e-7 (GELU, of
+    the argument) over 2^24 arguments, within 2e-7.  Heads 0 and 1: arguments of exactly +-reach; head 2: the next bf16
+    numbers beyond, whose blocks take the library's functions (1.7e-7 there)."""
+    nh, unit = 24, 2e-7
+    x, b = _arguments_near_roundings(act, nh, Dp if last else Dh, d, unit, -reach / 2, reach / 2, reach / 2)
+    assert (x.float().abs().max() + b.float().abs().max()) <= reach
+    x[0], x[1], b[:3] = reach, -reach, 0
+    x[2, ::17] = reach * (1 + 2 ** -7)
+    _check_features(act, nh, d, Dh, Dp, last, x, b, unit)
+
+
+def _check_features(act, nh, d, Dh, Dp, last, x, b, unit):
+    from paper_2601_04342_b200 import binding
     W1 = torch.zeros(nh, Dh, d)
     W2 = torch.zeros(nh, Dp, Dh)
     W1[:, torch.arange(Dh), torch.arange(Dh) % d] = 1
