@@ -11,12 +11,13 @@
 //   Persistent: CTAs walk items (batch*head, chunk, tile of 128 queries), key tiles of 64.
 //     warps 0-7   two threads per row (TMEM lane), each with 32 of a tile's keys and half of the output columns: Q into
 //                 TMEM, softmax, split of P, sum of O, epilogue
-//     warps 8-11  loaders: K and V rows from global memory, split, into swizzled shared-memory tiles (two stages)
-//     warp 12     UMMA issuer: S = Q K^T (48 MMAs of N = 64), O = P V (24 of N = D), Q and P read from TMEM
+//     warps 8-15  loaders: K and V rows from global memory, split, into swizzled shared-memory tiles (two stages)
+//     warp 16     UMMA issuer: S = Q K^T (48 MMAs of N = 64), O = P V (24 of N = D), Q and P read from TMEM
 //   TMEM: Q planes [0, 3D/2), two S slots of 96 columns (64 of S; the three planes of P overwrite them), O [3D/2 + 192, + D).
 //   Q K^T of tile j + 1 is in the queue before P V of tile j, so that softmax j + 1 and the sum of O run beside MMAs.
-// Bound by the MMAs: 3,072 cycles per key tile of 128 x 64 at D = 128.  The same layer: 4,783 -> 1,106 us (0.56 ms of MMAs;
-// 1,053 without the multiplication by 2^20 below).
+// The MMAs take 3,072 cycles per key tile of 128 x 64 at D = 128, the kernel 4,900 (issue slots 64 % busy, tensor pipe 63 %).
+// The same layer: 4,783 us on the CUDA cores, 1,090 with four loader warps (one per scheduler: the split of a tile then took
+// longer than its MMAs), 990 with eight; two more threads per row instead: 1,164.
 //
 // Every operand is multiplied by 2^20 as it is split, so that the parts of the smallest fp32 numbers are bf16 numbers too
 // (without it values below 2^-110 keep fewer than 24 bits), and what leaves an accumulator by 2^-40: both are exact.
@@ -30,8 +31,11 @@
 
 namespace rehyat {
 
-constexpr int F32_BN = 64, F32_STAGES = 2, F32_SOFTMAX_WARPS = 8, F32_LOAD_WARPS = 4;
-constexpr int F32_THREADS = (F32_SOFTMAX_WARPS + F32_LOAD_WARPS + 1) * 32;
+constexpr int F32_BN = 64, F32_STAGES = 2, F32_SOFTMAX_WARPS = 8, F32_LOAD_WARPS = 8;
+constexpr int F32_W_LOAD = F32_SOFTMAX_WARPS, F32_W_MMA = F32_W_LOAD + F32_LOAD_WARPS;   // first loader warp, issuer warp
+constexpr int F32_THREADS = (F32_W_MMA + 4) * 32, F32_LOADERS = F32_LOAD_WARPS * 32;     // whole warpgroups
+constexpr int F32_REGS = 96, F32_REGS_SOFTMAX = 136, F32_REGS_LOAD = 80, F32_REGS_MMA = 48;   // at launch, then by role (setmaxnreg)
+static_assert(F32_SOFTMAX_WARPS * F32_REGS_SOFTMAX + F32_LOAD_WARPS * F32_REGS_LOAD + 4 * F32_REGS_MMA <= F32_THREADS / 32 * F32_REGS, "");
 constexpr uint32_t F32_UNSAFE_BITS = 0x53000000u;     // 2^39
 constexpr float F32_UP = 0x1p20f, F32_DOWN = 0x1p-40f;  // scale of the split operands, and what takes it out of a product
 
@@ -89,7 +93,7 @@ window_f32_tc(const float* q, const float* k, const float* v, float* out, Geo g,
     wait_ctx_init(&bars->wctx, wa);
     fence_mbar_init();
   }
-  if (warp == 12) {
+  if (warp == F32_W_MMA) {
     tmem_alloc(smem_u32(&bars->tmem_base), 512);
     tmem_relinquish();
   }
@@ -103,10 +107,11 @@ window_f32_tc(const float* q, const float* k, const float* v, float* out, Geo g,
   }
   const auto n_tiles_of = [](const WinItem& w) { return (w.hi - w.lo + F32_BN - 1) / F32_BN; };
 
-  if (warp >= 8 && warp < 12) {
+  if (warp >= F32_W_LOAD && warp < F32_W_MMA) {
     // ------------------------------------------------------------------ loaders
-    constexpr int CH = D / 8, U = F32_BN * CH / 128;                 // 8-column chunks of a row; chunks per thread and tile
-    const int t = threadIdx.x - 256;
+    setmaxnreg_dec<F32_REGS_LOAD>();
+    constexpr int CH = D / 8, U = F32_BN * CH / F32_LOADERS;                 // 8-column chunks of a row; chunks per thread and tile
+    const int t = threadIdx.x - F32_W_LOAD * 32;
     uint32_t n = 0, big = 0;                                         // key tiles so far; largest magnitude seen
     bool alive = !wa.withhold_loads;
     for (int item = blockIdx.x; item < n_items && alive; item += gridDim.x) {
@@ -122,7 +127,7 @@ window_f32_tc(const float* q, const float* k, const float* v, float* out, Geo g,
           float4 x[U][2];
 #pragma unroll
           for (int u = 0; u < U; ++u) {
-            const int c = t + 128 * u, key = w.lo + j * F32_BN + c / CH;
+            const int c = t + F32_LOADERS * u, key = w.lo + j * F32_BN + c / CH;
             const float* p = src + (long long)key * g.stride_n + (c % CH) * 8;
             x[u][0] = x[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (key < w.hi) { x[u][0] = ld4(p); x[u][1] = ld4(p + 4); }
@@ -132,7 +137,7 @@ window_f32_tc(const float* q, const float* k, const float* v, float* out, Geo g,
           const uint32_t dst = sb + st * SH::STAGE + kv * 3 * SH::PLANE;
 #pragma unroll
           for (int u = 0; u < U; ++u) {
-            const int c = t + 128 * u;
+            const int c = t + F32_LOADERS * u;
             big = max_bits(max_bits(big, x[u][0]), x[u][1]);
             uint4 h, m, l;
             split3(x[u][0].x, x[u][0].y, h.x, m.x, l.x); split3(x[u][0].z, x[u][0].w, h.y, m.y, l.y);
@@ -147,9 +152,10 @@ window_f32_tc(const float* q, const float* k, const float* v, float* out, Geo g,
       }
     }
     if (big >= F32_UNSAFE_BITS) *unsafe = wa.epoch;
-  } else if (warp == 12) {
+  } else if (warp >= F32_W_MMA) {
     // ------------------------------------------------------------------ UMMA issuer
-    if (elect_one()) {
+    setmaxnreg_dec<F32_REGS_MMA>();
+    if (warp == F32_W_MMA && elect_one()) {
       constexpr uint32_t id_qk = idesc_bf16(TC_BM, F32_BN, 0, 0), id_pv = idesc_bf16(TC_BM, D, 0, 1);
       constexpr int PA[6] = {2, 0, 1, 1, 0, 0}, PB[6] = {0, 2, 1, 0, 1, 0};   // planes of A and B, small terms first
       const uint64_t d_k = smem_desc_sw128(sb, 16, 1024), d_v = smem_desc_sw128(sb + 3 * SH::PLANE, SH::SUB, 1024);
@@ -208,6 +214,7 @@ window_f32_tc(const float* q, const float* k, const float* v, float* out, Geo g,
     }
   } else {
     // ------------------------------------------------------------------ softmax, sum of O, epilogue
+    setmaxnreg_inc<F32_REGS_SOFTMAX>();
     const int half = warp >> 2, r = (warp & 3) * 32 + lane;
     const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16, tb = tmem + lane_off;
     // Waits that were given up return at once; these warps then run through the rest of their item (the barrier below
@@ -349,7 +356,7 @@ window_f32_tc(const float* q, const float* k, const float* v, float* out, Geo g,
 
   tc_fence_before();
   __syncthreads();
-  if (warp == 12) {
+  if (warp == F32_W_MMA) {
     tc_fence_after();
     tmem_dealloc(tmem, 512);
   }
@@ -367,12 +374,12 @@ window_f32_tc(const float* q, const float* k, const float* v, float* out, Geo g,
 //     consumer     phi s_t         -> added to the read-out in registers            (READOUT)
 //                  phi^T V         -> added to the CTA's partial state in global memory (L2), fp32
 //   warps 0-7   epilogues, two threads per token (TMEM lane) with 32 columns each
-//   warps 8-11  loaders: X, and weights, states or V through a ring of two stages of three planes, split on the way
-//   warp 12     UMMA issuer
+//   warps 8-15  loaders: X, and weights, states or V through a ring of two stages of three planes, split on the way
+//   warp 16     UMMA issuer
 //   TMEM: accumulators [0, 128), H planes [128, 512).
 // A pass waits for the epilogue of the one before: the chain is what bounds a tile (37,000 cycles of MMAs at the default
 // widths, about as long again in hand-overs and epilogues).  12 heads x 12,600 tokens of 128 channels against the
-// CUDA-core kernels: state 1,319 -> 458 us, read-out 1,284 -> 406 us.
+// CUDA-core kernels: state 1,319 -> 430 us, read-out 1,284 -> 399 us (458 and 406 with four loader warps).
 // ---------------------------------------------------------------------------------------------
 struct PhiF32Args {
   const float *x, *v, *W1, *b1, *W2, *b2, *state;
@@ -438,7 +445,7 @@ phi_f32_tc(Geo g, PhiF32Args a) {
     wait_ctx_init(&bars->wctx, a.wa);
     fence_mbar_init();
   }
-  if (warp == 12) {
+  if (warp == F32_W_MMA) {
     tmem_alloc(smem_u32(&bars->tmem_base), 512);
     tmem_relinquish();
   }
@@ -456,17 +463,19 @@ phi_f32_tc(Geo g, PhiF32Args a) {
   const uint32_t tmem = bars->tmem_base;
   constexpr uint32_t T_H = 128, H_PLANE = 128;
 
-  if (warp >= 8 && warp < 12) {
+  if (warp >= F32_W_LOAD && warp < F32_W_MMA) {
     // ------------------------------------------------------------------ loaders
-    const int tl = threadIdx.x - 256;
+    setmaxnreg_dec<F32_REGS_LOAD>();
+    const int tl = threadIdx.x - F32_W_LOAD * 32;
     uint32_t big = 0, n_st = 0;
     bool alive = !a.wa.withhold_loads;
-    float4 x[8][2];
+    constexpr int U = 1024 / F32_LOADERS;
+    float4 x[U][2];
     // 1,024 chunks of eight columns, of 64 rows x 128 columns (wide) or 128 rows x 64; zeros beyond rows and cols
     auto fetch = [&](const float* src, long long stride, int rows, int cols, bool wide) {
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int c = tl + 128 * u, r = wide ? c >> 4 : c >> 3, col = (wide ? c & 15 : c & 7) * 8;
+      for (int u = 0; u < U; ++u) {
+        const int c = tl + F32_LOADERS * u, r = wide ? c >> 4 : c >> 3, col = (wide ? c & 15 : c & 7) * 8;
         x[u][0] = x[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (r < rows && col < cols) {
           const float* p = src + (long long)r * stride + col;
@@ -476,8 +485,8 @@ phi_f32_tc(Geo g, PhiF32Args a) {
     };
     auto put = [&](uint32_t dst, uint32_t plane, uint32_t sub, int row0, bool wide) {
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int c = tl + 128 * u, r = row0 + (wide ? c >> 4 : c >> 3), col = (wide ? c & 15 : c & 7) * 8;
+      for (int u = 0; u < U; ++u) {
+        const int c = tl + F32_LOADERS * u, r = row0 + (wide ? c >> 4 : c >> 3), col = (wide ? c & 15 : c & 7) * 8;
         big = max_bits(max_bits(big, x[u][0]), x[u][1]);
         uint4 h, m, l;
         split3(x[u][0].x, x[u][0].y, h.x, m.x, l.x); split3(x[u][0].z, x[u][0].w, h.y, m.y, l.y);
@@ -538,9 +547,10 @@ phi_f32_tc(Geo g, PhiF32Args a) {
       }
     }
     if (big >= F32_UNSAFE_BITS) *a.unsafe = a.wa.epoch;
-  } else if (warp == 12) {
+  } else if (warp >= F32_W_MMA) {
     // ------------------------------------------------------------------ UMMA issuer
-    if (elect_one()) {
+    setmaxnreg_dec<F32_REGS_MMA>();
+    if (warp == F32_W_MMA && elect_one()) {
       constexpr uint32_t id_kk = idesc_bf16(128, 64, 0, 0), id_cons = READOUT ? idesc_bf16(128, 64, 0, 1) : idesc_bf16(128, 64, 1, 1);
       constexpr int PA[6] = {2, 0, 1, 1, 0, 0}, PB[6] = {0, 2, 1, 0, 1, 0};
       uint32_t n_st = 0, n_pass = 0;
@@ -606,6 +616,7 @@ phi_f32_tc(Geo g, PhiF32Args a) {
     }
   } else {
     // ------------------------------------------------------------------ epilogues
+    setmaxnreg_inc<F32_REGS_SOFTMAX>();
     const int half = warp >> 2, qd = warp & 3, r = qd * 32 + lane;
     const uint32_t tb = tmem + ((uint32_t)(qd * 32) << 16);
     const int part_w = Dp / a.P;
@@ -785,7 +796,7 @@ phi_f32_tc(Geo g, PhiF32Args a) {
 
   tc_fence_before();
   __syncthreads();
-  if (warp == 12) {
+  if (warp == F32_W_MMA) {
     tc_fence_after();
     tmem_dealloc(tmem, 512);
   }
