@@ -251,7 +251,7 @@ int launch_group_simt(rehyat_ctx* ctx, const T* q, const T* k, const T* v, T* ou
       if (split.f32_tc) {
         PhiF32Args a = f32_args(ctx, wk, pd, k);
         a.v = v; a.partial = ctx->partial; a.n_split = n_split;
-        launch_kernel(phi_f32_tc<D, false>, dim3(n_split, g.G, g.BH), F32_THREADS, PF_SMEM, st, g, a);
+        launch_kernel(phi_f32_tc<D, false>, dim3(n_split, g.G, g.BH), PF_THREADS, PF_SMEM, st, g, a);
         ctx->last_launches += 1;
         unsafe = a.unsafe;
         epoch = a.wa.epoch;
@@ -280,7 +280,7 @@ int launch_group_simt(rehyat_ctx* ctx, const T* q, const T* k, const T* v, T* ou
         PhiF32Args a = f32_args(ctx, wq, pd, q);
         a.state = ctx->state; a.rd = ctx->readout; a.rd_rows = ctx->rd_cap;
         a.tiles_per_cta = (tc_tiles + plan.parts - 1) / plan.parts;
-        launch_kernel(phi_f32_tc<D, true>, dim3((tc_tiles + a.tiles_per_cta - 1) / a.tiles_per_cta, g.G, g.BH), F32_THREADS, PF_SMEM, st, g, a);
+        launch_kernel(phi_f32_tc<D, true>, dim3((tc_tiles + a.tiles_per_cta - 1) / a.tiles_per_cta, g.G, g.BH), PF_THREADS, PF_SMEM, st, g, a);
         ctx->last_launches += 1;
         unsafe = a.unsafe;
         epoch = a.wa.epoch;

@@ -373,13 +373,15 @@ window_f32_tc(const float* q, const float* k, const float* v, float* out, Geo g,
 //     U quarters   H W2^T          -> bias, activation, power, split -> phi planes in the space of X, 128 features at a time
 //     consumer     phi s_t         -> added to the read-out in registers            (READOUT)
 //                  phi^T V         -> added to the CTA's partial state in global memory (L2), fp32
-//   warps 0-7   epilogues, two threads per token (TMEM lane) with 32 columns each
-//   warps 8-15  loaders: X, and weights, states or V through a ring of two stages of three planes, split on the way
-//   warp 16     UMMA issuer
+//   warps 0-15   epilogues, four threads per token (TMEM lane) with 16 columns each
+//   warps 16-23  loaders: X, and weights, states or V through a ring of two stages of three planes, split on the way
+//   warp 24      UMMA issuer
 //   TMEM: accumulators [0, 128), H planes [128, 512).
-// A pass waits for the epilogue of the one before: the chain is what bounds a tile (37,000 cycles of MMAs at the default
-// widths, about as long again in hand-overs and epilogues).  12 heads x 12,600 tokens of 128 channels against the
-// CUDA-core kernels: state 1,319 -> 430 us, read-out 1,284 -> 399 us (458 and 406 with four loader warps).
+// A pass that needs no results of the epilogue before (the next quarter of a layer, the next columns of the consumer) starts
+// as soon as that has the accumulators in registers; H, phi and the next X have to be waited for.  31,000 cycles of a tile are
+// MMAs at the default widths, as many again those waits.  12 heads x 12,600 tokens of 128 channels, against two threads per
+// token and every pass behind the whole epilogue of the one before:
+// state 430 -> 404 us, read-out 399 -> 366 us (on the CUDA cores 1,319 and 1,284).
 // ---------------------------------------------------------------------------------------------
 struct PhiF32Args {
   const float *x, *v, *W1, *b1, *W2, *b2, *state;
@@ -389,17 +391,21 @@ struct PhiF32Args {
   int* unsafe;
 };
 struct PhiF32Bars {
-  uint64_t x_full, x_empty, ring_full[2], ring_empty[2], acc_ready, epi_done, drained;
+  uint64_t x_full, x_empty, ring_full[2], ring_empty[2], acc_ready, acc_free, epi_done[2], drained;   // see the issuer
   uint32_t tmem_base;
   ptx::WaitCtx wctx;
   float b1[256], b2[256], z[256];
-  float sums[4][256];          // READOUT: [half][token] shares of phi z_t; else [TMEM quadrant][feature] sums of phi
+  float sums[4][256];          // READOUT: [quarter][token] shares of phi z_t; else [TMEM quadrant][feature] sums of phi
 };
+constexpr int PF_EPI_WARPS = 16, PF_LOAD_WARPS = 8, PF_W_LOAD = PF_EPI_WARPS, PF_W_MMA = PF_W_LOAD + PF_LOAD_WARPS;
+constexpr int PF_THREADS = (PF_W_MMA + 4) * 32, PF_LOADERS = PF_LOAD_WARPS * 32;          // whole warpgroups
+constexpr int PF_REGS = 72, PF_REGS_EPI = 80, PF_REGS_LOAD = 64, PF_REGS_MMA = 48;       // at launch, then by role (setmaxnreg)
+static_assert(PF_EPI_WARPS * PF_REGS_EPI + PF_LOAD_WARPS * PF_REGS_LOAD + 4 * PF_REGS_MMA <= PF_THREADS / 32 * PF_REGS, "");
 constexpr int PF_XPLANE = 128 * 128 * 2, PF_SPLANE = 16384, PF_STAGE = 3 * PF_SPLANE;
 constexpr int PF_SMEM = 3 * PF_XPLANE + 2 * PF_STAGE + (int)sizeof(PhiF32Bars) + 16 + 1024;
 
 template <int D, bool READOUT>
-__global__ void __launch_bounds__(F32_THREADS, 1)
+__global__ void __launch_bounds__(PF_THREADS, 1)
 phi_f32_tc(Geo g, PhiF32Args a) {
   using namespace ptx;
   constexpr int SD = D + 4, ND = D / 64;
@@ -431,21 +437,22 @@ phi_f32_tc(Geo g, PhiF32Args a) {
     if (tok_a >= tok_b) {                                            // nothing admitted: the partial is zero
       grid_dep_wait();
       grid_dep_launch();
-      for (int i = threadIdx.x; i < Dp * SD / 4; i += F32_THREADS) reinterpret_cast<float4*>(part)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int i = threadIdx.x; i < Dp * SD / 4; i += PF_THREADS) reinterpret_cast<float4*>(part)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
       return;
     }
   }
   const int n_tiles = (tok_b - tok_a + 127) / 128;
 
   if (threadIdx.x == 0) {
-    mbar_init(smem_u32(&bars->x_full), F32_LOAD_WARPS); mbar_init(smem_u32(&bars->x_empty), 1);
-    for (int s = 0; s < 2; ++s) { mbar_init(smem_u32(&bars->ring_full[s]), F32_LOAD_WARPS); mbar_init(smem_u32(&bars->ring_empty[s]), 1); }
-    mbar_init(smem_u32(&bars->acc_ready), 1); mbar_init(smem_u32(&bars->epi_done), F32_SOFTMAX_WARPS);
+    mbar_init(smem_u32(&bars->x_full), PF_LOAD_WARPS); mbar_init(smem_u32(&bars->x_empty), 1);
+    for (int s = 0; s < 2; ++s) { mbar_init(smem_u32(&bars->ring_full[s]), PF_LOAD_WARPS); mbar_init(smem_u32(&bars->ring_empty[s]), 1); }
+    mbar_init(smem_u32(&bars->acc_ready), 1); mbar_init(smem_u32(&bars->acc_free), PF_EPI_WARPS);
+    mbar_init(smem_u32(&bars->epi_done[0]), PF_EPI_WARPS); mbar_init(smem_u32(&bars->epi_done[1]), PF_EPI_WARPS);
     mbar_init(smem_u32(&bars->drained), 1);
     wait_ctx_init(&bars->wctx, a.wa);
     fence_mbar_init();
   }
-  if (warp == F32_W_MMA) {
+  if (warp == PF_W_MMA) {
     tmem_alloc(smem_u32(&bars->tmem_base), 512);
     tmem_relinquish();
   }
@@ -453,7 +460,7 @@ phi_f32_tc(Geo g, PhiF32Args a) {
     grid_dep_wait();
     grid_dep_launch();
   }
-  for (int i = threadIdx.x; i < 256; i += F32_THREADS) {             // zero beyond the widths
+  for (int i = threadIdx.x; i < 256; i += PF_THREADS) {             // zero beyond the widths
     bars->b1[i] = i < Dh ? a.b1[(size_t)head * Dh + i] : 0.f;
     bars->b2[i] = i < Dp ? a.b2[(size_t)head * Dp + i] : 0.f;
   }
@@ -463,19 +470,19 @@ phi_f32_tc(Geo g, PhiF32Args a) {
   const uint32_t tmem = bars->tmem_base;
   constexpr uint32_t T_H = 128, H_PLANE = 128;
 
-  if (warp >= F32_W_LOAD && warp < F32_W_MMA) {
+  if (warp >= PF_W_LOAD && warp < PF_W_MMA) {
     // ------------------------------------------------------------------ loaders
-    setmaxnreg_dec<F32_REGS_LOAD>();
-    const int tl = threadIdx.x - F32_W_LOAD * 32;
+    setmaxnreg_dec<PF_REGS_LOAD>();
+    const int tl = threadIdx.x - PF_W_LOAD * 32;
     uint32_t big = 0, n_st = 0;
     bool alive = !a.wa.withhold_loads;
-    constexpr int U = 1024 / F32_LOADERS;
+    constexpr int U = 1024 / PF_LOADERS;
     float4 x[U][2];
     // 1,024 chunks of eight columns, of 64 rows x 128 columns (wide) or 128 rows x 64; zeros beyond rows and cols
     auto fetch = [&](const float* src, long long stride, int rows, int cols, bool wide) {
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const int c = tl + F32_LOADERS * u, r = wide ? c >> 4 : c >> 3, col = (wide ? c & 15 : c & 7) * 8;
+        const int c = tl + PF_LOADERS * u, r = wide ? c >> 4 : c >> 3, col = (wide ? c & 15 : c & 7) * 8;
         x[u][0] = x[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (r < rows && col < cols) {
           const float* p = src + (long long)r * stride + col;
@@ -486,7 +493,7 @@ phi_f32_tc(Geo g, PhiF32Args a) {
     auto put = [&](uint32_t dst, uint32_t plane, uint32_t sub, int row0, bool wide) {
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const int c = tl + F32_LOADERS * u, r = row0 + (wide ? c >> 4 : c >> 3), col = (wide ? c & 15 : c & 7) * 8;
+        const int c = tl + PF_LOADERS * u, r = row0 + (wide ? c >> 4 : c >> 3), col = (wide ? c & 15 : c & 7) * 8;
         big = max_bits(max_bits(big, x[u][0]), x[u][1]);
         uint4 h, m, l;
         split3(x[u][0].x, x[u][0].y, h.x, m.x, l.x); split3(x[u][0].z, x[u][0].w, h.y, m.y, l.y);
@@ -519,12 +526,13 @@ phi_f32_tc(Geo g, PhiF32Args a) {
     for (int j = 0; j < n_tiles && alive; ++j) {
       const int tok0 = tok_a + j * 128, rows = min(128, tok_b - tok0);
       constexpr int PIECES = D / 64;                                 // of 64 rows x 128 columns, or one of 128 x 64
-      if (!wait(&bars->x_empty, (j & 1) ^ 1)) break;
 #pragma unroll 1
       for (int p = 0; p < PIECES; ++p) {
         fetch(xh + (long long)(tok0 + p * 64) * xs, xs, rows - p * 64, D, D == 128);
+        if (p == 0 && !wait(&bars->x_empty, (j & 1) ^ 1)) break;     // (the first piece is on its way meanwhile)
         put(sb, PF_XPLANE, 16384, p * 64, D == 128);
       }
+      if (!alive) break;
       fence_proxy_async_smem();
       mbar_arrive_warp(smem_u32(&bars->x_full), lane);
 #pragma unroll 1
@@ -547,13 +555,17 @@ phi_f32_tc(Geo g, PhiF32Args a) {
       }
     }
     if (big >= F32_UNSAFE_BITS) *a.unsafe = a.wa.epoch;
-  } else if (warp >= F32_W_MMA) {
+  } else if (warp >= PF_W_MMA) {
     // ------------------------------------------------------------------ UMMA issuer
-    setmaxnreg_dec<F32_REGS_MMA>();
-    if (warp == F32_W_MMA && elect_one()) {
+    setmaxnreg_dec<PF_REGS_MMA>();
+    if (warp == PF_W_MMA && elect_one()) {
       constexpr uint32_t id_kk = idesc_bf16(128, 64, 0, 0), id_cons = READOUT ? idesc_bf16(128, 64, 0, 1) : idesc_bf16(128, 64, 1, 1);
       constexpr int PA[6] = {2, 0, 1, 1, 0, 0}, PB[6] = {0, 2, 1, 0, 1, 0};
-      uint32_t n_st = 0, n_pass = 0;
+      // acc_free: the epilogue of a pass has its accumulators in registers, the next pass may write them; epi_done: the
+      // planes an epilogue of an H or U pass (numbered n_data) writes are complete.  A pass that does not read those runs
+      // beside the arithmetic of the epilogue.  epi_done of pass n is waited for before pass n + 2 is issued, so neither of
+      // its two barriers is ever more than one phase ahead of this thread.
+      uint32_t n_st = 0, n_pass = 0, n_data = 0, n_epi = 0;
       bool alive = true;
       auto wait = [&](uint64_t* bar, uint32_t parity) {
         alive = alive && mbar_wait(smem_u32(bar), parity, wc, PH_ERR_MMA);
@@ -574,28 +586,39 @@ phi_f32_tc(Geo g, PhiF32Args a) {
         umma_commit(smem_u32(&bars->ring_empty[s]));
         ++n_st;
       };
-      auto begin = [&]() { return n_pass == 0 || wait(&bars->epi_done, (n_pass - 1) & 1); };
+      auto planes = [&](uint32_t n) {                                // the first n H and U passes' planes are complete
+        for (; n_epi < n && alive; ++n_epi) wait(&bars->epi_done[n_epi & 1], (n_epi >> 1) & 1);
+        return alive;
+      };
+      auto begin = [&]() { return n_pass == 0 || wait(&bars->acc_free, (n_pass - 1) & 1); };
+      auto begin_data = [&]() {
+        if ((n_data >= 2 && !planes(n_data - 1)) || !begin()) return false;
+        ++n_data;
+        return true;
+      };
       auto end = [&]() { if (alive) { umma_commit(smem_u32(&bars->acc_ready)); ++n_pass; } };
       const auto k_off = [](int kk, uint32_t sub) { return (kk >> 2) * sub + (kk & 3) * 32; };   // K-major image
       for (int j = 0; j < n_tiles && alive; ++j) {
         if (!wait(&bars->x_full, j & 1)) break;
         for (int q = 0; q < nqh && alive; ++q) {
-          if (!begin()) break;
+          if (!begin_data()) break;
           share(true, D / 16, [&](uint32_t d, int p, int kk, uint64_t db, uint32_t acc) {
             umma_ss(d, smem_desc_advance(d_x, p * PF_XPLANE + k_off(kk, 16384)), smem_desc_advance(db, k_off(kk, 8192)), id_kk, acc);
           });
           end();
         }
+        if (!planes(n_data)) break;                                  // H
         for (int hf = 0; hf < n_half && alive; ++hf) {
           const int nq = min(2, nqu - 2 * hf);
           for (int q = 0; q < nq && alive; ++q) {
-            if (!begin()) break;
+            if (!begin_data()) break;
             for (int s = 0; s < ksu && alive; ++s)
               share(s == 0, min(8, nqh * 4 - s * 8), [&](uint32_t d, int p, int kk, uint64_t db, uint32_t acc) {
                 umma_ts(d, tmem + T_H + p * H_PLANE + (s * 8 + kk) * 8, smem_desc_advance(db, k_off(kk, 8192)), id_kk, acc);
               });
             end();
           }
+          if (!planes(n_data)) break;                                // phi
           for (int dh = 0; dh < ND && alive; ++dh) {
             if (!begin()) break;
             if (READOUT)
@@ -616,15 +639,15 @@ phi_f32_tc(Geo g, PhiF32Args a) {
     }
   } else {
     // ------------------------------------------------------------------ epilogues
-    setmaxnreg_inc<F32_REGS_SOFTMAX>();
-    const int half = warp >> 2, qd = warp & 3, r = qd * 32 + lane;
+    setmaxnreg_inc<PF_REGS_EPI>();
+    const int qr = warp >> 2, qd = warp & 3, r = qd * 32 + lane;        // quarter of a pass's columns, TMEM quadrant, lane
     const uint32_t tb = tmem + ((uint32_t)(qd * 32) << 16);
     const int part_w = Dp / a.P;
-    // as in window_f32_tc: a wait given up returns at once, the warps leave together at the head of a tile
-    uint32_t n_pass = 0, big = 0;
+    // a wait given up returns at once; the sixteen warps leave together at the head of a tile
+    uint32_t n_pass = 0, n_data = 0, big = 0;
     auto barrier = [&](bool flag) -> bool {
       uint32_t any;
-      asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbarrier.cta.red.or.pred q, 1, 256, p;\n\tselp.b32 %0, 1, 0, q;\n\t}"
+      asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbarrier.cta.red.or.pred q, 1, 512, p;\n\tselp.b32 %0, 1, 0, q;\n\t}"
                    : "=r"(any) : "r"((uint32_t)flag) : "memory");
       return any != 0;
     };
@@ -634,18 +657,24 @@ phi_f32_tc(Geo g, PhiF32Args a) {
       ++n_pass;
       tc_fence_after();
     };
-    auto acc_done = [&]() {
+    auto acc_read = [&]() {
       tc_fence_before();
-      mbar_arrive_warp(smem_u32(&bars->epi_done), lane);
+      mbar_arrive_warp(smem_u32(&bars->acc_free), lane);
     };
-    // 16 columns of the pass from column `half * 32 + c` on: both accumulators, bias and activation
-    auto activated = [&](int c, const float* bias, int act, float (&y)[16]) {
+    auto planes_done = [&]() {
+      tc_fence_before();
+      mbar_arrive_warp(smem_u32(&bars->epi_done[n_data & 1]), lane);
+      ++n_data;
+    };
+    // this thread's 16 columns of the pass: both accumulators, bias and activation
+    auto activated = [&](const float* bias, int act, float (&y)[16]) {
       uint32_t lo[16], hi[16];
-      tmem_ld16(tb + half * 32 + c, lo);
-      tmem_ld16(tb + 64 + half * 32 + c, hi);
+      tmem_ld16(tb + qr * 16, lo);
+      tmem_ld16(tb + 64 + qr * 16, hi);
       tmem_wait_ld();
+      acc_read();
 #pragma unroll
-      for (int e = 0; e < 16; ++e) y[e] = fmaf(__uint_as_float(lo[e]) + __uint_as_float(hi[e]), F32_DOWN, bias[half * 32 + c + e]);
+      for (int e = 0; e < 16; ++e) y[e] = fmaf(__uint_as_float(lo[e]) + __uint_as_float(hi[e]), F32_DOWN, bias[qr * 16 + e]);
       if (act == ACT_RELU) {
 #pragma unroll
         for (int e = 0; e < 16; ++e) y[e] = fmaxf(y[e], 0.f);
@@ -657,7 +686,7 @@ phi_f32_tc(Geo g, PhiF32Args a) {
     if (READOUT) {
       grid_dep_wait_role(wc);
       grid_dep_launch();
-      bars->z[threadIdx.x] = (int)threadIdx.x < Dp ? a.state[(((size_t)ci * g.BH + bh) * Dp + threadIdx.x) * SD + D] : 0.f;
+      if (threadIdx.x < 256) bars->z[threadIdx.x] = (int)threadIdx.x < Dp ? a.state[(((size_t)ci * g.BH + bh) * Dp + threadIdx.x) * SD + D] : 0.f;
     }
     for (int j = 0; j < n_tiles; ++j) {
       if (barrier(wait_ctx_aborted(wc) != 0)) break;                 // (and z is there, the last tile's sums have been read)
@@ -666,84 +695,78 @@ phi_f32_tc(Geo g, PhiF32Args a) {
 #pragma unroll 1
       for (int q = 0; q < nqh; ++q) {
         acc_wait();
-#pragma unroll 1
-        for (int c = 0; c < 32; c += 16) {
-          float y[16];
-          uint32_t h[8], m[8], l[8];
-          activated(c, bars->b1 + q * 64, a.act_hidden, y);
+        float y[16];
+        uint32_t h[8], m[8], l[8];
+        activated(bars->b1 + q * 64, a.act_hidden, y);
 #pragma unroll
-          for (int e = 0; e < 16; e += 2) {
-            big = max(big, max(abs_bits(y[e]), abs_bits(y[e + 1])));
-            split3(y[e], y[e + 1], h[e / 2], m[e / 2], l[e / 2]);
-          }
-          const uint32_t col = tb + T_H + (q * 64 + half * 32 + c) / 2;
-          tmem_st8(col, h); tmem_st8(col + H_PLANE, m); tmem_st8(col + 2 * H_PLANE, l);
+        for (int e = 0; e < 16; e += 2) {
+          big = max(big, max(abs_bits(y[e]), abs_bits(y[e + 1])));
+          split3(y[e], y[e + 1], h[e / 2], m[e / 2], l[e / 2]);
         }
+        const uint32_t col = tb + T_H + (q * 64 + qr * 16) / 2;
+        tmem_st8(col, h); tmem_st8(col + H_PLANE, m); tmem_st8(col + 2 * H_PLANE, l);
         tmem_wait_st();
-        acc_done();
+        planes_done();
       }
       float nl = 0.f;
-      uint64_t racc[READOUT ? ND : 1][16];
+      uint64_t racc[READOUT ? ND : 1][8];
 #pragma unroll 1
       for (int hf = 0; hf < n_half; ++hf) {
 #pragma unroll 1
         for (int q = 2 * hf; q < min(2 * hf + 2, nqu); ++q) {
           acc_wait();
-#pragma unroll 1
-          for (int c = 0; c < 32; c += 16) {
-            float y[16];
-            activated(c, bars->b2 + q * 64, a.act_out, y);
-            const int f0 = q * 64 + half * 32 + c;                   // feature of the first column
+          float y[16];
+          activated(bars->b2 + q * 64, a.act_out, y);
+          const int f0 = q * 64 + qr * 16;                   // feature of the first column
 #pragma unroll
-            for (int e = 0; e < 16; ++e) {
-              const int f = f0 + e, part_f = f / part_w;
-              const float u = y[e];
-              float p = u;
-              if (part_f >= 1) p *= u;
-              if (part_f >= 2) p *= u;
-              if (part_f >= 3) p *= u;
-              y[e] = tok_valid && f < Dp ? p : 0.f;
-              big = max(big, abs_bits(y[e]));
-              if (READOUT) nl = fmaf(y[e], bars->z[f], nl);
-            }
+          for (int e = 0; e < 16; ++e) {
+            const int f = f0 + e, part_f = f / part_w;
+            const float u = y[e];
+            float p = u;
+            if (part_f >= 1) p *= u;
+            if (part_f >= 2) p *= u;
+            if (part_f >= 3) p *= u;
+            y[e] = tok_valid && f < Dp ? p : 0.f;
+            big = max(big, abs_bits(y[e]));
+            if (READOUT) nl = fmaf(y[e], bars->z[f], nl);
+          }
 #pragma unroll
-            for (int e = 0; e < 16; e += 8) {
-              uint4 h, m, l;
-              split3(y[e], y[e + 1], h.x, m.x, l.x); split3(y[e + 2], y[e + 3], h.y, m.y, l.y);
-              split3(y[e + 4], y[e + 5], h.z, m.z, l.z); split3(y[e + 6], y[e + 7], h.w, m.w, l.w);
-              const int col = (q & 1) * 64 + half * 32 + c + e;
-              st_tile_chunk_sw128(sb, 16384, r, col, h);
-              st_tile_chunk_sw128(sb + PF_XPLANE, 16384, r, col, m);
-              st_tile_chunk_sw128(sb + 2 * PF_XPLANE, 16384, r, col, l);
-            }
-            if (!READOUT) {
-              // column sums over the warp's 32 tokens: a lane keeps half of the columns at each of four steps
+          for (int e = 0; e < 16; e += 8) {
+            uint4 h, m, l;
+            split3(y[e], y[e + 1], h.x, m.x, l.x); split3(y[e + 2], y[e + 3], h.y, m.y, l.y);
+            split3(y[e + 4], y[e + 5], h.z, m.z, l.z); split3(y[e + 6], y[e + 7], h.w, m.w, l.w);
+            const int col = (q & 1) * 64 + qr * 16 + e;
+            st_tile_chunk_sw128(sb, 16384, r, col, h);
+            st_tile_chunk_sw128(sb + PF_XPLANE, 16384, r, col, m);
+            st_tile_chunk_sw128(sb + 2 * PF_XPLANE, 16384, r, col, l);
+          }
+          if (!READOUT) {
+            // column sums over the warp's 32 tokens: a lane keeps half of the columns at each of four steps
 #pragma unroll
-              for (int o = 8; o; o >>= 1) {
-                const bool up = (lane & o) != 0;
+            for (int o = 8; o; o >>= 1) {
+              const bool up = (lane & o) != 0;
 #pragma unroll
-                for (int e = 0; e < o; ++e) {
-                  const float keep = up ? y[e + o] : y[e], give = up ? y[e] : y[e + o];
-                  y[e] = keep + __shfl_xor_sync(0xffffffffu, give, o);
-                }
+              for (int e = 0; e < o; ++e) {
+                const float keep = up ? y[e + o] : y[e], give = up ? y[e] : y[e + o];
+                y[e] = keep + __shfl_xor_sync(0xffffffffu, give, o);
               }
-              y[0] += __shfl_xor_sync(0xffffffffu, y[0], 16);
-              if (lane < 16) bars->sums[qd][f0 + lane] = j == 0 ? y[0] : bars->sums[qd][f0 + lane] + y[0];
             }
+            y[0] += __shfl_xor_sync(0xffffffffu, y[0], 16);
+            if (lane < 16) bars->sums[qd][f0 + lane] = j == 0 ? y[0] : bars->sums[qd][f0 + lane] + y[0];
           }
           fence_proxy_async_smem();
-          acc_done();
+          planes_done();
         }
 #pragma unroll
         for (int dh = 0; dh < ND; ++dh) {
           acc_wait();
-          uint32_t lo[32], hi[32];
-          tmem_ld32(tb + half * 32, lo);
-          tmem_ld32(tb + 64 + half * 32, hi);
+          uint32_t lo[16], hi[16];
+          tmem_ld16(tb + qr * 16, lo);
+          tmem_ld16(tb + 64 + qr * 16, hi);
           tmem_wait_ld();
-          acc_done();
+          acc_read();
 #pragma unroll
-          for (int e = 0; e < 32; e += 2) {
+          for (int e = 0; e < 16; e += 2) {
             const uint64_t y = add2(pk2u(lo[e], lo[e + 1]), pk2u(hi[e], hi[e + 1]));
             if constexpr (READOUT) {
               racc[dh][e / 2] = hf == 0 ? y : add2(racc[dh][e / 2], y);
@@ -754,9 +777,9 @@ phi_f32_tc(Geo g, PhiF32Args a) {
           if (!READOUT) {
             const int f = hf * 128 + r;                              // TMEM lane = feature
             if (f < Dp && !wait_ctx_aborted(wc)) {
-              float4* p = reinterpret_cast<float4*>(part + (size_t)f * SD + dh * 64 + half * 32);
+              float4* p = reinterpret_cast<float4*>(part + (size_t)f * SD + dh * 64 + qr * 16);
 #pragma unroll
-              for (int e = 0; e < 8; ++e) {
+              for (int e = 0; e < 4; ++e) {
                 float4 y = make_float4(__uint_as_float(lo[4 * e]), __uint_as_float(lo[4 * e + 1]), __uint_as_float(lo[4 * e + 2]),
                                        __uint_as_float(lo[4 * e + 3]));
                 if (j > 0) y = add4(p[e], y);
@@ -767,21 +790,21 @@ phi_f32_tc(Geo g, PhiF32Args a) {
         }
       }
       if constexpr (READOUT) {
-        bars->sums[half][r] = nl;
+        bars->sums[qr][r] = nl;
         if (barrier(wait_ctx_aborted(wc) != 0)) break;
         if (tok_valid) {
           const int ric = tok0 + r - geo_q0(g, t);
 #pragma unroll
           for (int dh = 0; dh < ND; ++dh)
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
+            for (int e = 0; e < 4; ++e) {
               float y[4];
               upk2(racc[dh][2 * e], y[0], y[1]);
               upk2(racc[dh][2 * e + 1], y[2], y[3]);
-              *reinterpret_cast<float4*>(a.rd + rd_index(g, a.rd_rows, D, bh, ci, ric, (dh * 64 + half * 32) / 4 + e)) =
+              *reinterpret_cast<float4*>(a.rd + rd_index(g, a.rd_rows, D, bh, ci, ric, (dh * 64 + qr * 16) / 4 + e)) =
                   make_float4(y[0] * F32_DOWN, y[1] * F32_DOWN, y[2] * F32_DOWN, y[3] * F32_DOWN);
             }
-          if (half == 0) a.rd[rd_index(g, a.rd_rows, D, bh, ci, ric, D / 4)] = bars->sums[0][r] + bars->sums[1][r];
+          if (qr == 0) a.rd[rd_index(g, a.rd_rows, D, bh, ci, ric, D / 4)] = (bars->sums[0][r] + bars->sums[1][r]) + (bars->sums[2][r] + bars->sums[3][r]);
         }
       }
     }
@@ -796,7 +819,7 @@ phi_f32_tc(Geo g, PhiF32Args a) {
 
   tc_fence_before();
   __syncthreads();
-  if (warp == F32_W_MMA) {
+  if (warp == PF_W_MMA) {
     tc_fence_after();
     tmem_dealloc(tmem, 512);
   }
