@@ -381,7 +381,8 @@ window_f32_tc(const float* q, const float* k, const float* v, float* out, Geo g,
 // as soon as that has the accumulators in registers; H, phi and the next X have to be waited for.  31,000 cycles of a tile are
 // MMAs at the default widths, as many again those waits.  12 heads x 12,600 tokens of 128 channels, against two threads per
 // token and every pass behind the whole epilogue of the one before:
-// state 430 -> 404 us, read-out 399 -> 366 us (on the CUDA cores 1,319 and 1,284).
+// state 404 -> 373 us, read-out 366 -> 329 us with the straight-line issue
+// of the MMAs (on the CUDA cores 1,319 and 1,284).
 // ---------------------------------------------------------------------------------------------
 struct PhiF32Args {
   const float *x, *v, *W1, *b1, *W2, *b2, *state;
@@ -399,10 +400,13 @@ struct PhiF32Bars {
 };
 constexpr int PF_EPI_WARPS = 16, PF_LOAD_WARPS = 8, PF_W_LOAD = PF_EPI_WARPS, PF_W_MMA = PF_W_LOAD + PF_LOAD_WARPS;
 constexpr int PF_THREADS = (PF_W_MMA + 4) * 32, PF_LOADERS = PF_LOAD_WARPS * 32;          // whole warpgroups
-constexpr int PF_REGS = 72, PF_REGS_EPI = 80, PF_REGS_LOAD = 64, PF_REGS_MMA = 48;       // at launch, then by role (setmaxnreg)
+constexpr int PF_REGS = 72, PF_REGS_EPI = 80, PF_REGS_LOAD = 64, PF_REGS_MMA = 56;       // at launch, then by role (setmaxnreg)
 static_assert(PF_EPI_WARPS * PF_REGS_EPI + PF_LOAD_WARPS * PF_REGS_LOAD + 4 * PF_REGS_MMA <= PF_THREADS / 32 * PF_REGS, "");
 constexpr int PF_XPLANE = 128 * 128 * 2, PF_SPLANE = 16384, PF_STAGE = 3 * PF_SPLANE;
 constexpr int PF_SMEM = 3 * PF_XPLANE + 2 * PF_STAGE + (int)sizeof(PhiF32Bars) + 16 + 1024;
+
+// The products of phi_f32_tc: X W1^T, H W2^T, phi s and phi^T V.
+enum PhiPass : int { PASS_H, PASS_U, PASS_PHI_S, PASS_PHI_V };
 
 template <int D, bool READOUT>
 __global__ void __launch_bounds__(PF_THREADS, 1)
@@ -572,17 +576,38 @@ phi_f32_tc(Geo g, PhiF32Args a) {
         if (alive) tc_fence_after();
         return alive;
       };
-      const uint64_t d_x = smem_desc_sw128(sb, 16, 1024), d_phi_mn = smem_desc_sw128(sb, 16384, 1024), d_b = smem_desc_sw128(s_ring, 16, 1024);
-      // waits for the ring's next stage and issues its share of a pass: `ksteps` times 16 terms of the six products
-      auto share = [&](bool first, int ksteps, auto&& mma) {
+      // Descriptors differ in the start address only (low word, units of 16 bytes): built once, constants added per MMA.
+      uint32_t k_lo, k_hi, mn_lo, mn_hi, b_lo, b_hi;
+      upk2u(smem_desc_sw128(sb, 16, 1024), k_lo, k_hi);               // X, or phi with features as the reduction index
+      upk2u(smem_desc_sw128(sb, 16384, 1024), mn_lo, mn_hi);          // phi with tokens as the reduction index
+      upk2u(smem_desc_sw128(s_ring, 16, 1024), b_lo, b_hi);           // the ring, either way
+      // Waits for the ring's next stage and issues its share of a pass: 4 * `blocks` (at most 8) times 16 terms of the six
+      // products.  Straight-line code: rolled over the steps, with descriptors built for each, the issue took 99 cycles an
+      // MMA of which the tensor pipe was busy 27, and bounded the kernel.
+      auto share = [&](auto kind, bool first, int blocks, uint32_t a_col) {
+        constexpr int K = decltype(kind)::value;                      // PASS_H, PASS_U, PASS_PHI_S or PASS_PHI_V
+        constexpr uint32_t A_BLK = (K == PASS_PHI_V ? 8192 : 16384) >> 4, A_STEP = (K == PASS_PHI_V ? 2048 : 32) >> 4;
+        constexpr bool B_MN = K == PASS_PHI_S || K == PASS_PHI_V;
+        constexpr uint32_t B_BLK = 8192 >> 4, B_STEP = (B_MN ? 2048 : 32) >> 4;
         const uint32_t s = n_st & 1;
         if (!wait(&bars->ring_full[s], (n_st >> 1) & 1)) return;
-        const uint64_t db = smem_desc_advance(d_b, s * PF_STAGE);
+        const uint32_t b0 = b_lo + s * (PF_STAGE >> 4);
 #pragma unroll
         for (int p = 0; p < 6; ++p)
-#pragma unroll 1
-          for (int kk = 0; kk < ksteps; ++kk)
-            mma(tmem + (p == 5 ? 64 : 0), PA[p], kk, smem_desc_advance(db, PB[p] * PF_SPLANE), (!first || kk > 0 || (p > 0 && p < 5)) ? 1u : 0u);
+#pragma unroll
+          for (int blk = 0; blk < 2; ++blk) {
+            if (blk >= blocks) continue;
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) {
+              const uint32_t d = tmem + (p == 5 ? 64 : 0), acc = (p > 0 && p < 5) || (blk | kk) != 0 ? 1u : (first ? 0u : 1u);
+              const uint64_t db = pk2u(b0 + PB[p] * (PF_SPLANE >> 4) + blk * B_BLK + kk * B_STEP, b_hi);
+              if constexpr (K == PASS_U)
+                umma_ts(d, a_col + PA[p] * H_PLANE + (blk * 4 + kk) * 8, db, id_kk, acc);
+              else
+                umma_ss(d, pk2u((K == PASS_PHI_V ? mn_lo : k_lo) + PA[p] * (PF_XPLANE >> 4) + blk * A_BLK + kk * A_STEP, K == PASS_PHI_V ? mn_hi : k_hi),
+                        db, K == PASS_H ? id_kk : id_cons, acc);
+            }
+          }
         umma_commit(smem_u32(&bars->ring_empty[s]));
         ++n_st;
       };
@@ -597,14 +622,11 @@ phi_f32_tc(Geo g, PhiF32Args a) {
         return true;
       };
       auto end = [&]() { if (alive) { umma_commit(smem_u32(&bars->acc_ready)); ++n_pass; } };
-      const auto k_off = [](int kk, uint32_t sub) { return (kk >> 2) * sub + (kk & 3) * 32; };   // K-major image
       for (int j = 0; j < n_tiles && alive; ++j) {
         if (!wait(&bars->x_full, j & 1)) break;
         for (int q = 0; q < nqh && alive; ++q) {
           if (!begin_data()) break;
-          share(true, D / 16, [&](uint32_t d, int p, int kk, uint64_t db, uint32_t acc) {
-            umma_ss(d, smem_desc_advance(d_x, p * PF_XPLANE + k_off(kk, 16384)), smem_desc_advance(db, k_off(kk, 8192)), id_kk, acc);
-          });
+          share(std::integral_constant<int, PASS_H>(), true, D / 64, 0);
           end();
         }
         if (!planes(n_data)) break;                                  // H
@@ -613,22 +635,13 @@ phi_f32_tc(Geo g, PhiF32Args a) {
           for (int q = 0; q < nq && alive; ++q) {
             if (!begin_data()) break;
             for (int s = 0; s < ksu && alive; ++s)
-              share(s == 0, min(8, nqh * 4 - s * 8), [&](uint32_t d, int p, int kk, uint64_t db, uint32_t acc) {
-                umma_ts(d, tmem + T_H + p * H_PLANE + (s * 8 + kk) * 8, smem_desc_advance(db, k_off(kk, 8192)), id_kk, acc);
-              });
+              share(std::integral_constant<int, PASS_U>(), s == 0, min(2, nqh - s * 2), tmem + T_H + s * 64);
             end();
           }
           if (!planes(n_data)) break;                                // phi
           for (int dh = 0; dh < ND && alive; ++dh) {
             if (!begin()) break;
-            if (READOUT)
-              share(true, nq * 4, [&](uint32_t d, int p, int kk, uint64_t db, uint32_t acc) {
-                umma_ss(d, smem_desc_advance(d_x, p * PF_XPLANE + k_off(kk, 16384)), smem_desc_advance(db, kk * 2048), id_cons, acc);
-              });
-            else
-              share(true, 8, [&](uint32_t d, int p, int kk, uint64_t db, uint32_t acc) {
-                umma_ss(d, smem_desc_advance(d_phi_mn, p * PF_XPLANE + kk * 2048), smem_desc_advance(db, kk * 2048), id_cons, acc);
-              });
+            share(std::integral_constant<int, READOUT ? PASS_PHI_S : PASS_PHI_V>(), true, READOUT ? nq : 2, 0);
             end();
           }
         }
