@@ -17,7 +17,7 @@
 //   Q K^T of tile j + 1 is in the queue before P V of tile j, so that softmax j + 1 and the sum of O run beside MMAs.
 // The MMAs take 3,072 cycles per key tile of 128 x 64 at D = 128, the kernel 4,900 (issue slots 64 % busy, tensor pipe 63 %).
 // The same layer: 4,783 us on the CUDA cores, 1,090 with four loader warps (one per scheduler: the split of a tile then took
-// longer than its MMAs), 990 with eight; two more threads per row instead: 1,164.
+// longer than its MMAs), 1,000 with eight, 980 with the whole warp issuing (ptx::Umma); two more threads per row instead: 1,164.
 //
 // Every operand is multiplied by 2^20 as it is split, so that the parts of the smallest fp32 numbers are bf16 numbers too
 // (without it values below 2^-110 keep fewer than 24 bits), and what leaves an accumulator by 2^-40: both are exact.
@@ -155,14 +155,15 @@ window_f32_tc(const float* q, const float* k, const float* v, float* out, Geo g,
   } else if (warp >= F32_W_MMA) {
     // ------------------------------------------------------------------ UMMA issuer
     setmaxnreg_dec<F32_REGS_MMA>();
-    if (warp == F32_W_MMA && elect_one()) {
+    if (warp == F32_W_MMA) {
+      const Umma umma;
       constexpr uint32_t id_qk = idesc_bf16(TC_BM, F32_BN, 0, 0), id_pv = idesc_bf16(TC_BM, D, 0, 1);
       constexpr int PA[6] = {2, 0, 1, 1, 0, 0}, PB[6] = {0, 2, 1, 0, 1, 0};   // planes of A and B, small terms first
       const uint64_t d_k = smem_desc_sw128(sb, 16, 1024), d_v = smem_desc_sw128(sb + 3 * SH::PLANE, SH::SUB, 1024);
       uint32_t n0 = 0, n_q = 0;                                      // key tiles of finished items, items
       bool alive = true;
       auto wait = [&](uint64_t* bar, uint32_t parity) {
-        alive = alive && mbar_wait(smem_u32(bar), parity, wc, TC_ERR_MMA, TC_HINT_I);
+        alive = alive && __all_sync(0xffffffffu, mbar_wait(smem_u32(bar), parity, wc, TC_ERR_MMA, TC_HINT_I));
         return alive;
       };
       for (int item = blockIdx.x; item < n_items && alive; item += gridDim.x) {
@@ -181,10 +182,10 @@ window_f32_tc(const float* q, const float* k, const float* v, float* out, Geo g,
           for (int t = 0; t < 6; ++t)
 #pragma unroll
             for (int kk = 0; kk < D / 16; ++kk)
-              umma_ts(acc, tmem + PA[t] * (D / 2) + kk * 8, smem_desc_advance(db, PB[t] * SH::PLANE + (kk >> 2) * SH::SUB + (kk & 3) * 32),
+              umma.ts(acc, tmem + PA[t] * (D / 2) + kk * 8, smem_desc_advance(db, PB[t] * SH::PLANE + (kk >> 2) * SH::SUB + (kk & 3) * 32),
                       id_qk, (t | kk) != 0);
-          umma_commit(smem_u32(&bars->s_ready[st]));
-          umma_commit(smem_u32(&bars->k_empty[st]));
+          umma.commit(smem_u32(&bars->s_ready[st]));
+          umma.commit(smem_u32(&bars->k_empty[st]));
         };
         qk(n0);
         if (n_kv > 1 && alive) qk(n0 + 1);
@@ -199,16 +200,16 @@ window_f32_tc(const float* q, const float* k, const float* v, float* out, Geo g,
           for (int t = 0; t < 6; ++t)
 #pragma unroll
             for (int kk = 0; kk < F32_BN / 16; ++kk)
-              umma_ts(tmem + SH::T_O, pa + PA[t] * (F32_BN / 2) + kk * 8, smem_desc_advance(db, PB[t] * SH::PLANE + kk * 2048), id_pv,
+              umma.ts(tmem + SH::T_O, pa + PA[t] * (F32_BN / 2) + kk * 8, smem_desc_advance(db, PB[t] * SH::PLANE + kk * 2048), id_pv,
                       (t | kk) != 0);
-          umma_commit(smem_u32(&bars->pv_done));
-          umma_commit(smem_u32(&bars->v_empty[st]));
+          umma.commit(smem_u32(&bars->pv_done));
+          umma.commit(smem_u32(&bars->v_empty[st]));
           if (j + 2 < n_kv) qk(n + 2);                               // into the slot this P V reads
         }
         n0 += n_kv;
       }
       // TMEM is not freed, nor does the CTA exit, with an MMA still running: this wait is not cut short by the abort flag
-      umma_commit(smem_u32(&bars->drained));
+      umma.commit(smem_u32(&bars->drained));
       mbar_wait_drain(smem_u32(&bars->drained), 0, wc);
       grid_dep_wait();                                               // nor before the predecessor, where the epilogues were given up
     }
@@ -381,8 +382,7 @@ window_f32_tc(const float* q, const float* k, const float* v, float* out, Geo g,
 // as soon as that has the accumulators in registers; H, phi and the next X have to be waited for.  31,000 cycles of a tile are
 // MMAs at the default widths, as many again those waits.  12 heads x 12,600 tokens of 128 channels, against two threads per
 // token and every pass behind the whole epilogue of the one before:
-// state 404 -> 373 us, read-out 366 -> 329 us with the straight-line issue
-// of the MMAs (on the CUDA cores 1,319 and 1,284).
+// state 364 us, read-out 318 us (on the CUDA cores 1,319 and 1,284).
 // ---------------------------------------------------------------------------------------------
 struct PhiF32Args {
   const float *x, *v, *W1, *b1, *W2, *b2, *state;
@@ -562,7 +562,8 @@ phi_f32_tc(Geo g, PhiF32Args a) {
   } else if (warp >= PF_W_MMA) {
     // ------------------------------------------------------------------ UMMA issuer
     setmaxnreg_dec<PF_REGS_MMA>();
-    if (warp == PF_W_MMA && elect_one()) {
+    if (warp == PF_W_MMA) {
+      const Umma umma;
       constexpr uint32_t id_kk = idesc_bf16(128, 64, 0, 0), id_cons = READOUT ? idesc_bf16(128, 64, 0, 1) : idesc_bf16(128, 64, 1, 1);
       constexpr int PA[6] = {2, 0, 1, 1, 0, 0}, PB[6] = {0, 2, 1, 0, 1, 0};
       // acc_free: the epilogue of a pass has its accumulators in registers, the next pass may write them; epi_done: the
@@ -572,7 +573,7 @@ phi_f32_tc(Geo g, PhiF32Args a) {
       uint32_t n_st = 0, n_pass = 0, n_data = 0, n_epi = 0;
       bool alive = true;
       auto wait = [&](uint64_t* bar, uint32_t parity) {
-        alive = alive && mbar_wait(smem_u32(bar), parity, wc, PH_ERR_MMA);
+        alive = alive && __all_sync(0xffffffffu, mbar_wait(smem_u32(bar), parity, wc, PH_ERR_MMA));
         if (alive) tc_fence_after();
         return alive;
       };
@@ -602,13 +603,13 @@ phi_f32_tc(Geo g, PhiF32Args a) {
               const uint32_t d = tmem + (p == 5 ? 64 : 0), acc = (p > 0 && p < 5) || (blk | kk) != 0 ? 1u : (first ? 0u : 1u);
               const uint64_t db = pk2u(b0 + PB[p] * (PF_SPLANE >> 4) + blk * B_BLK + kk * B_STEP, b_hi);
               if constexpr (K == PASS_U)
-                umma_ts(d, a_col + PA[p] * H_PLANE + (blk * 4 + kk) * 8, db, id_kk, acc);
+                umma.ts(d, a_col + PA[p] * H_PLANE + (blk * 4 + kk) * 8, db, id_kk, acc);
               else
-                umma_ss(d, pk2u((K == PASS_PHI_V ? mn_lo : k_lo) + PA[p] * (PF_XPLANE >> 4) + blk * A_BLK + kk * A_STEP, K == PASS_PHI_V ? mn_hi : k_hi),
+                umma.ss(d, pk2u((K == PASS_PHI_V ? mn_lo : k_lo) + PA[p] * (PF_XPLANE >> 4) + blk * A_BLK + kk * A_STEP, K == PASS_PHI_V ? mn_hi : k_hi),
                         db, K == PASS_H ? id_kk : id_cons, acc);
             }
           }
-        umma_commit(smem_u32(&bars->ring_empty[s]));
+        umma.commit(smem_u32(&bars->ring_empty[s]));
         ++n_st;
       };
       auto planes = [&](uint32_t n) {                                // the first n H and U passes' planes are complete
@@ -621,7 +622,7 @@ phi_f32_tc(Geo g, PhiF32Args a) {
         ++n_data;
         return true;
       };
-      auto end = [&]() { if (alive) { umma_commit(smem_u32(&bars->acc_ready)); ++n_pass; } };
+      auto end = [&]() { if (alive) { umma.commit(smem_u32(&bars->acc_ready)); ++n_pass; } };
       for (int j = 0; j < n_tiles && alive; ++j) {
         if (!wait(&bars->x_full, j & 1)) break;
         for (int q = 0; q < nqh && alive; ++q) {
@@ -645,9 +646,9 @@ phi_f32_tc(Geo g, PhiF32Args a) {
             end();
           }
         }
-        if (alive) umma_commit(smem_u32(&bars->x_empty));
+        if (alive) umma.commit(smem_u32(&bars->x_empty));
       }
-      umma_commit(smem_u32(&bars->drained));                         // as in window_f32_tc
+      umma.commit(smem_u32(&bars->drained));                         // as in window_f32_tc
       mbar_wait_drain(smem_u32(&bars->drained), 0, wc);
     }
   } else {

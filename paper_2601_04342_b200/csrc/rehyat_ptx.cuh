@@ -249,6 +249,42 @@ __device__ __forceinline__ void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64
       : "memory");
 }
 
+// The same for a role that a whole warp runs: all 32 lanes go through it (every decision a vote), the instructions execute in
+// the one lane with `leader` set.  Addresses and descriptors then are values of the warp, which is how tcgen05.mma takes
+// them: issued by a single thread an MMA costs 45 cycles whatever its size, this way 128 x 64 x 16 takes 32 and 128 x 32 x 16
+// takes 16 (A in TMEM, 256 of them back to back).  For MMAs of N = 128, which take 64 either way, the single thread is the
+// better form: its waits are shorter (24 heads of 64: window kernel 977 us, in this form 1,018; 320 x 480 layer 312 and 327).
+struct Umma {
+  uint32_t leader;
+  __device__ __forceinline__ Umma() : leader(elect_one()) {}
+  // arrives on `bar` once every tcgen05.mma issued so far has completed
+  __device__ __forceinline__ void commit(uint32_t bar) const {
+    asm volatile(
+        "{\n\t.reg .pred q;\n\t"
+        "setp.ne.b32 q, %1, 0;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
+        ::"r"(bar), "r"(leader) : "memory");
+  }
+  // D[tmem] (+)= A[smem] * B[smem]
+  __device__ __forceinline__ void ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) const {
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "setp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(leader) : "memory");
+  }
+  // D[tmem] (+)= A[tmem] * B[smem]
+  __device__ __forceinline__ void ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) const {
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "setp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(leader) : "memory");
+  }
+};
+
 // 32 lanes x 32 consecutive 32-bit columns: thread i of the warp gets lane (base lane + i).
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
   asm volatile(
