@@ -36,7 +36,7 @@ constexpr int F32_W_LOAD = F32_SOFTMAX_WARPS, F32_W_MMA = F32_W_LOAD + F32_LOAD_
 constexpr int F32_THREADS = (F32_W_MMA + 4) * 32, F32_LOADERS = F32_LOAD_WARPS * 32;     // whole warpgroups
 constexpr int F32_REGS = 96, F32_REGS_SOFTMAX = 136, F32_REGS_LOAD = 80, F32_REGS_MMA = 48;   // at launch, then by role (setmaxnreg)
 static_assert(F32_SOFTMAX_WARPS * F32_REGS_SOFTMAX + F32_LOAD_WARPS * F32_REGS_LOAD + 4 * F32_REGS_MMA <= F32_THREADS / 32 * F32_REGS, "");
-constexpr uint32_t F32_UNSAFE_BITS = 0x53000000u;     // 2^39
+constexpr uint32_t F32_UNSAFE_BF16 = 0x5d00u;         // 2^39, scaled, as bf16
 constexpr float F32_UP = 0x1p20f, F32_DOWN = 0x1p-40f;  // scale of the split operands, and what takes it out of a product
 
 struct F32Bars {
@@ -56,17 +56,22 @@ struct F32Shape {
 
 // Two floats, scaled, into the bf16 pairs of their three parts.
 __device__ __forceinline__ void split3(float x0, float x1, uint32_t& h, uint32_t& m, uint32_t& l) {
-  ptx::upk2(ptx::mul2(ptx::pk2(x0, x1), ptx::pk2(F32_UP, F32_UP)), x0, x1);
+  uint64_t x = ptx::mul2(ptx::pk2(x0, x1), ptx::pk2(F32_UP, F32_UP));
+  ptx::upk2(x, x0, x1);
   h = ptx::pack_bf16(x0, x1);
-  x0 -= __uint_as_float(h << 16); x1 -= __uint_as_float(h & 0xffff0000u);
+  x = ptx::sub2(x, ptx::pk2u(h << 16, h & 0xffff0000u));
+  ptx::upk2(x, x0, x1);
   m = ptx::pack_bf16(x0, x1);
-  x0 -= __uint_as_float(m << 16); x1 -= __uint_as_float(m & 0xffff0000u);
+  ptx::upk2(ptx::sub2(x, ptx::pk2u(m << 16, m & 0xffff0000u)), x0, x1);
   l = ptx::pack_bf16(x0, x1);
 }
-__device__ __forceinline__ uint32_t abs_bits(float x) { return __float_as_uint(x) & 0x7fffffffu; }
-__device__ __forceinline__ uint32_t max_bits(uint32_t m, float4 x) {
-  return max(max(m, max(abs_bits(x.x), abs_bits(x.y))), max(abs_bits(x.z), abs_bits(x.w)));
+// Largest magnitude seen among the first parts of split values, in two halves; what is not a number stays.
+__device__ __forceinline__ uint32_t max_part(uint32_t big, uint32_t h) {
+  uint32_t r;
+  asm("{\n\t.reg .b32 t;\n\tabs.bf16x2 t, %2;\n\tmax.NaN.bf16x2 %0, %1, t;\n\t}" : "=r"(r) : "r"(big), "r"(h));
+  return r;
 }
+__device__ __forceinline__ bool unsafe_parts(uint32_t big) { return (big & 0xffffu) >= F32_UNSAFE_BF16 || (big >> 16) >= F32_UNSAFE_BF16; }
 
 template <int D>
 __global__ void __launch_bounds__(F32_THREADS, 1)
@@ -138,10 +143,10 @@ window_f32_tc(const float* q, const float* k, const float* v, float* out, Geo g,
 #pragma unroll
           for (int u = 0; u < U; ++u) {
             const int c = t + F32_LOADERS * u;
-            big = max_bits(max_bits(big, x[u][0]), x[u][1]);
             uint4 h, m, l;
             split3(x[u][0].x, x[u][0].y, h.x, m.x, l.x); split3(x[u][0].z, x[u][0].w, h.y, m.y, l.y);
             split3(x[u][1].x, x[u][1].y, h.z, m.z, l.z); split3(x[u][1].z, x[u][1].w, h.w, m.w, l.w);
+            big = max_part(max_part(max_part(max_part(big, h.x), h.y), h.z), h.w);
             st_tile_chunk_sw128(dst, SH::SUB, c / CH, (c % CH) * 8, h);
             st_tile_chunk_sw128(dst + SH::PLANE, SH::SUB, c / CH, (c % CH) * 8, m);
             st_tile_chunk_sw128(dst + 2 * SH::PLANE, SH::SUB, c / CH, (c % CH) * 8, l);
@@ -151,7 +156,7 @@ window_f32_tc(const float* q, const float* k, const float* v, float* out, Geo g,
         }
       }
     }
-    if (big >= F32_UNSAFE_BITS) *unsafe = wa.epoch;
+    if (unsafe_parts(big)) *unsafe = wa.epoch;
   } else if (warp >= F32_W_MMA) {
     // ------------------------------------------------------------------ UMMA issuer
     setmaxnreg_dec<F32_REGS_MMA>();
@@ -243,9 +248,9 @@ window_f32_tc(const float* q, const float* k, const float* v, float* out, Geo g,
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
             const float4 x = valid ? ld4(qp + c + u * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
-            big = max_bits(big, x);
             split3(x.x, x.y, h[2 * u], m[2 * u], l[2 * u]);
             split3(x.z, x.w, h[2 * u + 1], m[2 * u + 1], l[2 * u + 1]);
+            big = max_part(max_part(big, h[2 * u]), h[2 * u + 1]);
           }
           const uint32_t col = (half * (D / 2) + c) / 2;
           tmem_st8(tb + col, h); tmem_st8(tb + D / 2 + col, m); tmem_st8(tb + D + col, l);
@@ -352,7 +357,7 @@ window_f32_tc(const float* q, const float* k, const float* v, float* out, Geo g,
         }
       }
     }
-    if (big >= F32_UNSAFE_BITS) *unsafe = wa.epoch;
+    if (unsafe_parts(big)) *unsafe = wa.epoch;
   }
 
   tc_fence_before();
@@ -382,7 +387,7 @@ window_f32_tc(const float* q, const float* k, const float* v, float* out, Geo g,
 // as soon as that has the accumulators in registers; H, phi and the next X have to be waited for.  31,000 cycles of a tile are
 // MMAs at the default widths, as many again those waits.  12 heads x 12,600 tokens of 128 channels, against two threads per
 // token and every pass behind the whole epilogue of the one before:
-// state 364 us, read-out 318 us (on the CUDA cores 1,319 and 1,284).
+// state 362 us, read-out 303 us (on the CUDA cores 1,319 and 1,284).
 // ---------------------------------------------------------------------------------------------
 struct PhiF32Args {
   const float *x, *v, *W1, *b1, *W2, *b2, *state;
@@ -498,10 +503,10 @@ phi_f32_tc(Geo g, PhiF32Args a) {
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int c = tl + PF_LOADERS * u, r = row0 + (wide ? c >> 4 : c >> 3), col = (wide ? c & 15 : c & 7) * 8;
-        big = max_bits(max_bits(big, x[u][0]), x[u][1]);
         uint4 h, m, l;
         split3(x[u][0].x, x[u][0].y, h.x, m.x, l.x); split3(x[u][0].z, x[u][0].w, h.y, m.y, l.y);
         split3(x[u][1].x, x[u][1].y, h.z, m.z, l.z); split3(x[u][1].z, x[u][1].w, h.w, m.w, l.w);
+        big = max_part(max_part(max_part(max_part(big, h.x), h.y), h.z), h.w);
         st_tile_chunk_sw128(dst, sub, r, col, h);
         st_tile_chunk_sw128(dst + plane, sub, r, col, m);
         st_tile_chunk_sw128(dst + 2 * plane, sub, r, col, l);
@@ -530,6 +535,8 @@ phi_f32_tc(Geo g, PhiF32Args a) {
     for (int j = 0; j < n_tiles && alive; ++j) {
       const int tok0 = tok_a + j * 128, rows = min(128, tok_b - tok0);
       constexpr int PIECES = D / 64;                                 // of 64 rows x 128 columns, or one of 128 x 64
+      stage(W1, D, Dh, D, true);                                     // its slot is free before the space of X is
+      if (!alive) break;
 #pragma unroll 1
       for (int p = 0; p < PIECES; ++p) {
         fetch(xh + (long long)(tok0 + p * 64) * xs, xs, rows - p * 64, D, D == 128);
@@ -540,7 +547,7 @@ phi_f32_tc(Geo g, PhiF32Args a) {
       fence_proxy_async_smem();
       mbar_arrive_warp(smem_u32(&bars->x_full), lane);
 #pragma unroll 1
-      for (int q = 0; q < nqh; ++q) stage(W1 + (size_t)q * 64 * D, D, Dh - q * 64, D, true);
+      for (int q = 1; q < nqh; ++q) stage(W1 + (size_t)q * 64 * D, D, Dh - q * 64, D, true);
 #pragma unroll 1
       for (int hf = 0; hf < n_half; ++hf) {
 #pragma unroll 1
@@ -558,7 +565,7 @@ phi_f32_tc(Geo g, PhiF32Args a) {
         }
       }
     }
-    if (big >= F32_UNSAFE_BITS) *a.unsafe = a.wa.epoch;
+    if (unsafe_parts(big)) *a.unsafe = a.wa.epoch;
   } else if (warp >= PF_W_MMA) {
     // ------------------------------------------------------------------ UMMA issuer
     setmaxnreg_dec<PF_REGS_MMA>();
@@ -714,8 +721,8 @@ phi_f32_tc(Geo g, PhiF32Args a) {
         activated(bars->b1 + q * 64, a.act_hidden, y);
 #pragma unroll
         for (int e = 0; e < 16; e += 2) {
-          big = max(big, max(abs_bits(y[e]), abs_bits(y[e + 1])));
           split3(y[e], y[e + 1], h[e / 2], m[e / 2], l[e / 2]);
+          big = max_part(big, h[e / 2]);
         }
         const uint32_t col = tb + T_H + (q * 64 + qr * 16) / 2;
         tmem_st8(col, h); tmem_st8(col + H_PLANE, m); tmem_st8(col + 2 * H_PLANE, l);
@@ -734,14 +741,13 @@ phi_f32_tc(Geo g, PhiF32Args a) {
           const int f0 = q * 64 + qr * 16;                   // feature of the first column
 #pragma unroll
           for (int e = 0; e < 16; ++e) {
-            const int f = f0 + e, part_f = f / part_w;
+            const int f = f0 + e;
             const float u = y[e];
             float p = u;
-            if (part_f >= 1) p *= u;
-            if (part_f >= 2) p *= u;
-            if (part_f >= 3) p *= u;
+            if (f >= part_w) p *= u;                                 // part f / part_w has the power of its number plus one
+            if (f >= 2 * part_w) p *= u;
+            if (f >= 3 * part_w) p *= u;
             y[e] = tok_valid && f < Dp ? p : 0.f;
-            big = max(big, abs_bits(y[e]));
             if (READOUT) nl = fmaf(y[e], bars->z[f], nl);
           }
 #pragma unroll
@@ -749,6 +755,7 @@ phi_f32_tc(Geo g, PhiF32Args a) {
             uint4 h, m, l;
             split3(y[e], y[e + 1], h.x, m.x, l.x); split3(y[e + 2], y[e + 3], h.y, m.y, l.y);
             split3(y[e + 4], y[e + 5], h.z, m.z, l.z); split3(y[e + 6], y[e + 7], h.w, m.w, l.w);
+            big = max_part(max_part(max_part(max_part(big, h.x), h.y), h.z), h.w);
             const int col = (q & 1) * 64 + qr * 16 + e;
             st_tile_chunk_sw128(sb, 16384, r, col, h);
             st_tile_chunk_sw128(sb + PF_XPLANE, 16384, r, col, m);
@@ -828,7 +835,7 @@ phi_f32_tc(Geo g, PhiF32Args a) {
         *reinterpret_cast<float4*>(part + (size_t)f * SD + D) =
             make_float4((bars->sums[0][f] + bars->sums[1][f]) + (bars->sums[2][f] + bars->sums[3][f]), 0.f, 0.f, 0.f);
     }
-    if (big >= F32_UNSAFE_BITS) *a.unsafe = a.wa.epoch;
+    if (unsafe_parts(big)) *a.unsafe = a.wa.epoch;
   }
 
   tc_fence_before();
