@@ -143,8 +143,12 @@ int check_config(const rehyat_config* c) {
 template <typename T, int D>
 int set_simt_attributes() {
   const auto smem = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  if (cudaFuncSetAttribute(state_partial_simt<T, D>, smem, simt_phi_smem(D, 256, 256, true)) != cudaSuccess ||
-      cudaFuncSetAttribute(readout_simt<T, D>, smem, simt_phi_smem(D, 256, 256, false)) != cudaSuccess ||
+  const auto set = [&](auto tile) {
+    constexpr int TM = decltype(tile)::value;
+    return cudaFuncSetAttribute(state_partial_simt<T, D, TM>, smem, simt_phi_smem(TM, D, 256, 256, true)) == cudaSuccess &&
+           cudaFuncSetAttribute(readout_simt<T, D, TM>, smem, simt_phi_smem(TM, D, 256, 256, false)) == cudaSuccess;
+  };
+  if (!set(std::integral_constant<int, 32>()) || !set(std::integral_constant<int, 16>()) || !set(std::integral_constant<int, 8>()) ||
       cudaFuncSetAttribute(window_simt<T, D, 1>, smem, WinSimt<T, D, 1>::SMEM) != cudaSuccess ||
       cudaFuncSetAttribute(window_simt<T, D, 4>, smem, WinSimt<T, D, 4>::SMEM) != cudaSuccess)
     return REHYAT_ERR_CUDA;
@@ -202,25 +206,74 @@ bool use_f32_tc(const rehyat_ctx* ctx, const Geo& g) {
 }
 
 // How phi and what follows it are cut into CTAs: `parts` per (chunk, batch*head) unit, for fp32 on the tensor cores
-// (phi_f32_tc, tiles of 128 tokens) or not (tiles of 32).
-struct PhiPlan { int parts; bool f32_tc; };
-// A tile of phi_f32_tc takes about 1.2 times as long as a tile of the CUDA-core kernels (12 heads x 12,600 tokens of 128
-// channels, state: 55 us for each of 8 rounds of tiles on the SMs against 47 us for each of 28), so it is taken where it
-// needs fewer rounds: 24 heads of 64, chunks of 192 tokens 93 -> 66 us a call; one chunk of 64 tokens stays (54 us, not 65).
-PhiPlan plan_phi(const rehyat_ctx* ctx, long long tokens, long long units, int most) {
+// (phi_f32_tc, tiles of 128 tokens) or not (tiles of `tm` tokens: 32, 16 or 8).  `cost` and `ctas` of the fp32 forms: rounds of
+// tiles on the SMs times the time of a tile, in sixteenths of that of a tile of 32; CTAs that have work.
+struct PhiPlan { int parts; bool f32_tc; int tm; long long cost, ctas; };
+
+// The smaller tiles of the CUDA-core kernels give short sequences more CTAs.  Time of a tile of 32 / 16 / 8 tokens, two-layer
+// maps of default widths in fp32: heads of 64 15 / 10.5 / 9 us, of 128 48 / 26 / 18.
+struct PhiTile { int tm, cost64, cost128; };
+constexpr PhiTile SIMT_TILES[] = {{SIMT_TM, 16, 16}, {16, 11, 9}, {8, 9, 6}};
+PhiPlan simt_plan(const rehyat_ctx* ctx, const PhiTile& t, long long tokens, long long units, int most) {
+  PhiPlan p = {1, false, t.tm, 0, 0};
+  p.parts = pick_parts((tokens + t.tm - 1) / t.tm, units, most, ctx->tc.n_sm, &p.cost);
+  p.cost *= ctx->cfg.head_dim == 64 ? t.cost64 : t.cost128;
+  p.ctas = p.parts * units;
+  return p;
+}
+// The read-out's phi starts beside the state kernel if its CTAs find room, and behind it if not.
+long long cost_behind(const rehyat_ctx* ctx, const PhiPlan& state, const PhiPlan& readout) {
+  return state.ctas + readout.ctas <= ctx->tc.n_sm ? (state.cost > readout.cost ? state.cost : readout.cost) : state.cost + readout.cost;
+}
+// `state`: the plan of the state kernel ahead of a read-out (null: none).
+// A tile of phi_f32_tc takes about as long as one of the CUDA-core kernels (a round of 128-token tiles of the default map 45 us),
+// but two more launches, and is taken where it needs fewer rounds: 24 heads of 64, chunks of 192 tokens 93 -> 66 us a call; one
+// chunk of 64 tokens stays (54 us, not 65).
+PhiPlan plan_phi(const rehyat_ctx* ctx, long long tokens, long long units, int most, const PhiPlan* state = nullptr) {
   const int n_sm = ctx->tc.n_sm;
   if (ctx->tensor_ok && ctx->tc.phi_ok) {
     const rehyat_config& c = ctx->cfg;
     const int per_sm = tc_state_narrow(c.head_dim, c.phi_hidden, c.phi_dim, c.phi_layers > 2 ? c.phi_layers - 2 : 0) ? 2 : 1;
-    return {pick_parts((tokens + 127) / 128, units, most, per_sm * n_sm), false};
+    return {pick_parts((tokens + 127) / 128, units, most, per_sm * n_sm), false, SIMT_TM, 0, 0};
   }
-  long long simt = 0, tc = 0;
-  const int simt_parts = pick_parts((tokens + SIMT_TM - 1) / SIMT_TM, units, most, n_sm, &simt);
-  if (ctx->status_dev == nullptr || ctx->cfg.impl == REHYAT_IMPL_SIMT || ctx->cfg.dtype != REHYAT_DTYPE_FP32 || ctx->cfg.phi_layers > 2)
-    return {simt_parts, false};
-  const int tc_parts = pick_parts((tokens + 127) / 128, units, most, n_sm, &tc);
-  if (6 * tc < 5 * simt) return {tc_parts, true};
-  return {simt_parts, false};
+  PhiPlan best = simt_plan(ctx, SIMT_TILES[0], tokens, units, most);
+  if (ctx->status_dev != nullptr && ctx->cfg.impl != REHYAT_IMPL_SIMT && ctx->cfg.dtype == REHYAT_DTYPE_FP32 && ctx->cfg.phi_layers <= 2) {
+    long long tc = 0;
+    const int tc_parts = pick_parts((tokens + 127) / 128, units, most, n_sm, &tc);
+    if (6 * 16 * tc < 5 * best.cost) return {tc_parts, true, SIMT_TM, 15 * tc, tc_parts * units};
+  }
+  const PhiPlan none = {0, false, 0, 0, 0};
+  const PhiPlan& before = state ? *state : none;
+  for (const PhiTile& t : SIMT_TILES) {
+    const PhiPlan p = simt_plan(ctx, t, tokens, units, most);
+    if (cost_behind(ctx, before, p) < cost_behind(ctx, before, best)) best = p;
+  }
+  return best;
+}
+// The state kernel's plan.  rd_tokens: tokens a unit of the read-out that follows (0: none); small tiles of the one may leave the
+// other no room.  Tiles of 16 and 8 are for chunks whose tiles need no more than a quarter of the SMs: how the sums over the
+// tokens are cut then does not depend on the number of chunks in the call, and a sequence taken chunk by chunk adds up in the
+// same order.  2 heads of 64 in frames of 8 x 8: 45.1 -> 35.3 us a call, 1 head of 128 104 -> 59; two chunks of 459 tokens for 2
+// heads of 64 (bf16) stay at 60 + 60 CTAs and 64 us, with tiles of 16 in the read-out it would take 77.
+PhiPlan plan_state(const rehyat_ctx* ctx, long long tokens, long long units, int most, long long chunk_tokens, int BH, long long rd_tokens) {
+  PhiPlan best = plan_phi(ctx, tokens, units, most);
+  if (best.f32_tc || best.ctas == 0) return best;                     // the tensor cores
+  const PhiPlan none = {0, false, 0, 0, 0};
+  long long best_cost = -1;
+  for (const PhiTile& t : SIMT_TILES) {
+    if (t.tm < SIMT_TM && 4 * BH * ((chunk_tokens + t.tm - 1) / t.tm) > ctx->tc.n_sm) continue;
+    const PhiPlan p = simt_plan(ctx, t, tokens, units, most);
+    const long long cost = cost_behind(ctx, p, rd_tokens > 0 ? plan_phi(ctx, rd_tokens, units, 64, &p) : none);
+    if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = p; }
+  }
+  return best;
+}
+// The tile sizes of the CUDA-core phi kernels: calls f with the chosen one as a constant.
+template <typename F>
+void with_tile(int tm, F&& f) {
+  if (tm == 32) f(std::integral_constant<int, 32>());
+  else if (tm == 16) f(std::integral_constant<int, 16>());
+  else f(std::integral_constant<int, 8>());
 }
 PhiF32Args f32_args(rehyat_ctx* ctx, const PhiPtrs<float>& w, const PhiDims& pd, const float* x) {
   PhiF32Args a = {};
@@ -257,8 +310,11 @@ int launch_group_simt(rehyat_ctx* ctx, const T* q, const T* k, const T* v, T* ou
         epoch = a.wa.epoch;
       }
     }
-    launch_kernel(state_partial_simt<T, D>, dim3(n_split, g.G, g.BH), SIMT_THREADS, simt_phi_smem(D, pd.Dh, pd.Dp, true), st,
-                  k, v, wk, pd, g, n_split, ctx->partial, unsafe, epoch);
+    with_tile(split.tm, [&](auto tile) {
+      constexpr int TM = decltype(tile)::value;
+      launch_kernel(state_partial_simt<T, D, TM>, dim3(n_split, g.G, g.BH), SIMT_THREADS, simt_phi_smem(TM, D, pd.Dh, pd.Dp, true), st,
+                    k, v, wk, pd, g, n_split, ctx->partial, unsafe, epoch);
+    });
     ctx->prof.end(REHYAT_PROF_STATE, st);
     const size_t per_slot = (size_t)g.BH * pd.Dp * SD;
     ctx->prof.begin(REHYAT_PROF_SCAN, st);
@@ -269,8 +325,8 @@ int launch_group_simt(rehyat_ctx* ctx, const T* q, const T* k, const T* v, T* ou
   if (parts & PART_READOUT) {
     PhiPtrs<T> wq = {(const T*)phi->q_W1, (const T*)phi->q_b1, (const T*)phi->q_W2, (const T*)phi->q_b2,
                      (const T*)phi->q_Wmid, (const T*)phi->q_bmid};
-    const int tiles = (g.Np + SIMT_TM - 1) / SIMT_TM, tc_tiles = (g.Np + 127) / 128;
-    const PhiPlan plan = plan_phi(ctx, g.Np, (long long)busy_readout(g) * g.BH, 64);
+    const PhiPlan plan = plan_phi(ctx, g.Np, (long long)busy_readout(g) * g.BH, 64, parts & PART_STATE ? &split : nullptr);
+    const int tiles = (g.Np + plan.tm - 1) / plan.tm, tc_tiles = (g.Np + 127) / 128;
     const int per_cta = (tiles + plan.parts - 1) / plan.parts;
     ctx->prof.begin(REHYAT_PROF_READOUT, st);
     int* unsafe = nullptr;
@@ -286,8 +342,12 @@ int launch_group_simt(rehyat_ctx* ctx, const T* q, const T* k, const T* v, T* ou
         epoch = a.wa.epoch;
       }
     }
-    launch_kernel(readout_simt<T, D>, dim3((tiles + per_cta - 1) / per_cta, g.G, g.BH), SIMT_THREADS, simt_phi_smem(D, pd.Dh, pd.Dp, false), st,
-                  q, wq, pd, g, ctx->state, ctx->readout, ctx->rd_cap, rd_half, per_cta, unsafe, epoch);
+    with_tile(plan.tm, [&](auto tile) {
+      constexpr int TM = decltype(tile)::value;
+      launch_kernel(readout_simt<T, D, TM>, dim3((tiles + per_cta - 1) / per_cta, g.G, g.BH), SIMT_THREADS,
+                    simt_phi_smem(TM, D, pd.Dh, pd.Dp, false), st, q, wq, pd, g, ctx->state, ctx->readout, ctx->rd_cap, rd_half, per_cta,
+                    unsafe, epoch);
+    });
     ctx->prof.end(REHYAT_PROF_READOUT, st);
     ctx->last_launches += 1;
   }
@@ -326,8 +386,9 @@ int launch_group_simt(rehyat_ctx* ctx, const T* q, const T* k, const T* v, T* ou
   return cudaGetLastError() == cudaSuccess ? REHYAT_OK : REHYAT_ERR_CUDA;
 }
 
-// Split of a chunk's state increment over CTAs: one CTA per (split, chunk, head) and one CTA per SM.
-PhiPlan pick_state_split(const rehyat_ctx* ctx, const Geo& g, int n_chunks_in_group, int tokens_per_increment) {
+// Split of a chunk's state increment over CTAs: one CTA per (split, chunk, head) and one CTA per SM.  chunk_tokens: of a
+// full chunk; rd_tokens: queries per chunk of the read-out that follows (0: none).
+PhiPlan pick_state_split(const rehyat_ctx* ctx, const Geo& g, int n_chunks_in_group, int tokens_per_increment, int chunk_tokens, int rd_tokens) {
   // the buffer holds partial_units increments of bh_max problems; a call with fewer of them (one head of
   // rehyat_forward_host) has room for more splits
   const long long units = (long long)ctx->partial_units * ctx->bh_max / g.BH;
@@ -336,7 +397,7 @@ PhiPlan pick_state_split(const rehyat_ctx* ctx, const Geo& g, int n_chunks_in_gr
   if (most < 1) most = 1;
   int busy = 0;                                     // chunks of the group that admit keys into the state
   for (int t = g.t0 > 1 ? g.t0 : 1; t < g.t0 + n_chunks_in_group; ++t) busy += geo_lo(g, t) > geo_lo(g, t - 1);
-  return plan_phi(ctx, tokens_per_increment, (long long)(busy > 0 ? busy : 1) * g.BH, most);
+  return plan_state(ctx, tokens_per_increment, (long long)(busy > 0 ? busy : 1) * g.BH, most, chunk_tokens, g.BH, rd_tokens);
 }
 
 // Enqueues the requested steps for the chunks [g.t0, g.t0 + g.G) with whichever kernel family the context uses.
@@ -698,7 +759,7 @@ int rehyat_forward(rehyat_ctx* ctx, const void* q, const void* k, const void* v,
   if (G < 1) return REHYAT_ERR_INVALID_ARG;   // cannot happen: rd_rows >= max chunk size
   if (G > ctx->Gmax) G = ctx->Gmax;
   g.t0 = 0;
-  const PhiPlan split = pick_state_split(ctx, g, G < n_chunks ? G : n_chunks, g.Np);
+  const PhiPlan split = pick_state_split(ctx, g, G < n_chunks ? G : n_chunks, g.Np, g.Np, g.Np);
 
   ctx->last_launches = 0;
   ctx->last_impl = ctx->tensor_ok ? (ctx->tc.phi_ok ? 2 : 1) : 0;
@@ -724,7 +785,7 @@ int rehyat_forward(rehyat_ctx* ctx, const void* q, const void* k, const void* v,
     for (int f0 = 1; f0 <= frames; f0 += ctx->Gmax) {
       gs.t0 = f0;                                // "chunk" f admits frame f-1: [lo_{f-1}, lo_f) = [(f-1) HW, f HW)
       gs.G = frames + 1 - f0 < ctx->Gmax ? frames + 1 - f0 : ctx->Gmax;
-      const PhiPlan ns = pick_state_split(ctx, gs, gs.G, (int)HW);
+      const PhiPlan ns = pick_state_split(ctx, gs, gs.G, (int)HW, (int)HW, 0);
       float* cum = ctx->cum + (size_t)f0 * per_slot;
       const int rc = run_parts(ctx, nullptr, k, v, nullptr, phi, gs, batch, ns, cum, f0 > 1 ? cum - per_slot : nullptr, PART_STATE, st);
       if (rc != REHYAT_OK) return rc;
@@ -737,7 +798,7 @@ int rehyat_forward(rehyat_ctx* ctx, const void* q, const void* k, const void* v,
           ctx->cum, ctx->state, per_slot, g, (int)HW, frames,
           (ctx->tensor_ok && ctx->tc.phi_ok) ? ctx->tc.state_bf16 : nullptr, c.head_dim);
       ctx->last_launches += 1;
-      const int rc = run_parts(ctx, q, k, v, out, phi, g, batch, {1, false}, nullptr, nullptr, PART_READOUT | PART_WINDOW, st);
+      const int rc = run_parts(ctx, q, k, v, out, phi, g, batch, {1, false, SIMT_TM, 0, 0}, nullptr, nullptr, PART_READOUT | PART_WINDOW, st);
       if (rc != REHYAT_OK) return rc;
     }
     return REHYAT_OK;
@@ -990,7 +1051,7 @@ int rehyat_stream_step(rehyat_ctx* ctx, const void* q_chunk, const void* k_chunk
   g.q_off = h; g.Nq = Np;
   ctx->share_now = nullptr;
   ctx->last_impl = ctx->tensor_ok ? (ctx->tc.phi_ok ? 2 : 1) : 0;
-  int rc = run_parts(ctx, q_used, kwin, vwin, out_chunk, phi, g, s.batch, {1, false}, nullptr, nullptr, (s.has_state ? PART_READOUT : 0) | PART_WINDOW, st);
+  int rc = run_parts(ctx, q_used, kwin, vwin, out_chunk, phi, g, s.batch, {1, false, SIMT_TM, 0, 0}, nullptr, nullptr, (s.has_state ? PART_READOUT : 0) | PART_WINDOW, st);
   if (rc != REHYAT_OK) return rc;
   // 3. Eq. 17-18: the tokens that leave the window before the next chunk enter the running state
   const int keep = (long long)s.overlap * HW < (long long)h + Np ? s.overlap * HW : h + Np;
@@ -998,7 +1059,7 @@ int rehyat_stream_step(rehyat_ctx* ctx, const void* q_chunk, const void* k_chunk
   if (leave > 0) {
     Geo gs = g;
     gs.Np = leave; gs.ToHW = 0; gs.q_shift = 0; gs.prefix = 0; gs.t0 = 1; gs.G = 1;   // increment of "chunk 1" = [0, leave)
-    const PhiPlan split = pick_state_split(ctx, gs, 1, leave);
+    const PhiPlan split = pick_state_split(ctx, gs, 1, leave, s.chunk * HW, 0);
     rc = run_parts(ctx, nullptr, kwin, vwin, nullptr, phi, gs, s.batch, split, ctx->state, s.has_state ? ctx->state : nullptr,
                    PART_STATE, st);
     if (rc != REHYAT_OK) return rc;

@@ -22,7 +22,9 @@
 
 namespace rehyat {
 
-constexpr int SIMT_TM = 32;         // tokens per phi tile
+// Tokens per phi tile: 32 need the fewest loads per multiply-add, 16 and 8 give a short sequence two and four times as many
+// CTAs (plan_phi chooses).
+constexpr int SIMT_TM = 32;
 constexpr int SIMT_THREADS = 256;
 // Weights of the phi layers and the state reach the FMA pipe through slabs of 32 rows x 64 bytes, private to a warp
 // (a warp owns 32 output columns): no barrier but the warp's own between a slab's copy and its use.
@@ -45,8 +47,8 @@ struct PhiPtrs {
 // Row stride (floats) of the two buffers of activations, and the bytes of shared memory of the phi kernels:
 // X [TM][d + 4], two activation buffers, optionally V [TM][d], the slabs, TM floats.
 __host__ __device__ inline int simt_act_ld(int Dh, int Dp) { return (Dh > Dp ? Dh : Dp) + 4; }
-__host__ __device__ inline int simt_phi_smem(int d, int Dh, int Dp, bool with_v) {
-  return 4 * (SIMT_TM * (d + 4) + 2 * SIMT_TM * simt_act_ld(Dh, Dp) + (with_v ? SIMT_TM * d : 0) + SIMT_TM) + SIMT_SLAB_BYTES;
+__host__ __device__ inline int simt_phi_smem(int tm, int d, int Dh, int Dp, bool with_v) {
+  return 4 * (tm * (d + 4) + 2 * tm * simt_act_ld(Dh, Dp) + (with_v ? tm * d : 0) + tm) + SIMT_SLAB_BYTES;
 }
 
 // 16 bytes global -> shared, zeros if !valid (the address must be readable memory or is not touched then).
@@ -155,7 +157,7 @@ __device__ __forceinline__ void simt_unit_gemm(const SimtUnit<T>& un, const floa
 }
 
 // Bias, activation and, for the last layer, power and the mask of valid rows; into out [TM][ldo].
-template <typename T, int RT>
+template <typename T, int RT, int TM>
 __device__ __forceinline__ void simt_unit_finish(const SimtUnit<T>& un, const T* bias, int act, bool last, int part_w, int row0,
                                                  int valid, float* out, int ldo, int lane, const uint64_t (&acc)[RT][4]) {
   const int rg = lane >> 3, cg = lane & 7;
@@ -170,7 +172,7 @@ __device__ __forceinline__ void simt_unit_finish(const SimtUnit<T>& un, const T*
       out[(row0 + rg + 4 * i) * ldo + j] = act == ACT_RELU ? fmaxf(y, 0.f) : y;
     }
   }
-  if (act == ACT_RELU && !(last && (part_w < un.N || valid < SIMT_TM))) return;
+  if (act == ACT_RELU && !(last && (part_w < un.N || valid < TM))) return;
   // rolled: the library's log1pf, expf and erff inlined once, not once per accumulator.  A lane reads back its own values.
 #pragma unroll 1
   for (int e = 0; e < RT * 4; ++e) {
@@ -184,10 +186,10 @@ __device__ __forceinline__ void simt_unit_finish(const SimtUnit<T>& un, const T*
   }
 }
 
-// phi of SIMT_TM tokens held in Xs [TM][d + 4]; h0, h1 are the two activation buffers [TM][ldh].  Returns the one that
+// phi of TM tokens held in Xs [TM][d + 4]; h0, h1 are the two activation buffers [TM][ldh].  Returns the one that
 // holds the features [TM][D'], rows from `valid` on forced to zero.  `x_free` runs once Xs has been read by all warps
 // (after a barrier).  Ends without a barrier.
-template <typename T, typename XFree>
+template <typename T, int TM, typename XFree>
 __device__ __forceinline__ float* phi_tile_simt(const float* Xs, float* h0, float* h1, int ldh, uint8_t* slabs,
                                                 const PhiPtrs<T>& w, const PhiDims& pd, int valid, XFree&& x_free) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, rg = lane >> 3;
@@ -206,7 +208,7 @@ __device__ __forceinline__ float* phi_tile_simt(const float* Xs, float* h0, floa
     un.K = first ? pd.d : pd.Dh;
     const T* bias = first ? w.b1 : last ? w.b2 : w.bm + (size_t)(l - 1) * pd.Dh;
     const int act = last ? pd.act_out : pd.act_hidden;
-    // a warp per 32 columns and all 32 rows; widths up to 128 give it 16 rows, so that up to eight warps have work
+    // a warp per 32 columns and all rows; widths up to 128 give it half of them, so that up to eight warps have work
     const int n_cb = (un.N + 31) >> 5, row_units = n_cb > 4 ? 1 : 2;
     un.cb = warp % n_cb;
     un.active = warp / n_cb < row_units;
@@ -218,14 +220,14 @@ __device__ __forceinline__ float* phi_tile_simt(const float* Xs, float* h0, floa
     if (l == 1) x_free();
     if (un.active) {
       if (row_units == 1) {
-        uint64_t acc[8][4];
-        simt_unit_gemm<T, 8>(un, in + rg * ldi, ldi, lane, acc);
-        simt_unit_finish<T, 8>(un, bias, act, last, part_w, 0, valid, out, ldh, lane, acc);
+        uint64_t acc[TM / 4][4];
+        simt_unit_gemm<T, TM / 4>(un, in + rg * ldi, ldi, lane, acc);
+        simt_unit_finish<T, TM / 4, TM>(un, bias, act, last, part_w, 0, valid, out, ldh, lane, acc);
       } else {
-        const int row0 = warp / n_cb * 16;
-        uint64_t acc[4][4];
-        simt_unit_gemm<T, 4>(un, in + (row0 + rg) * ldi, ldi, lane, acc);
-        simt_unit_finish<T, 4>(un, bias, act, last, part_w, row0, valid, out, ldh, lane, acc);
+        const int row0 = warp / n_cb * (TM / 2);
+        uint64_t acc[TM / 8][4];
+        simt_unit_gemm<T, TM / 8>(un, in + (row0 + rg) * ldi, ldi, lane, acc);
+        simt_unit_finish<T, TM / 8, TM>(un, bias, act, last, part_w, row0, valid, out, ldh, lane, acc);
       }
     }
     in = out;
@@ -237,19 +239,19 @@ __device__ __forceinline__ float* phi_tile_simt(const float* Xs, float* h0, floa
 
 // Loads rows [tok0, tok0+TM) x [0, D) of one head into shared memory as floats (row stride ld), zero beyond tok_end:
 // fp32 by cp.async (complete after the caller's next wait), bf16 converted on the way.
-template <int D>
+template <int D, int TM>
 __device__ __forceinline__ void load_rows_simt(float* dst, int ld, const float* base, long long stride_n, int tok0, int tok_end) {
 #pragma unroll
-  for (int idx = threadIdx.x; idx < SIMT_TM * (D / 4); idx += SIMT_THREADS) {
+  for (int idx = threadIdx.x; idx < TM * (D / 4); idx += SIMT_THREADS) {
     const int r = idx / (D / 4), c = (idx % (D / 4)) * 4;
     const bool ok = tok0 + r < tok_end;
     cp_async16(ptx::smem_u32(dst + r * ld + c), base + (ok ? (long long)(tok0 + r) * stride_n + c : 0), ok);
   }
 }
-template <int D>
+template <int D, int TM>
 __device__ __forceinline__ void load_rows_simt(float* dst, int ld, const __nv_bfloat16* base, long long stride_n, int tok0, int tok_end) {
 #pragma unroll
-  for (int idx = threadIdx.x; idx < SIMT_TM * (D / 4); idx += SIMT_THREADS) {
+  for (int idx = threadIdx.x; idx < TM * (D / 4); idx += SIMT_THREADS) {
     const int r = idx / (D / 4), c = (idx % (D / 4)) * 4;
     float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
     if (tok0 + r < tok_end) x = ld4(base + (long long)(tok0 + r) * stride_n + c);
@@ -262,7 +264,7 @@ __device__ __forceinline__ void load_rows_simt(float* dst, int ld, const __nv_bf
 // newly admitted tokens).  Split s takes a contiguous share of them and writes
 // partial[blockIdx.y][s][bh] = sum_j phi_k(k_j) [v_j | 1]  as [Dp][SD] floats, SD = d + 4,
 // column d holding the z part.
-template <typename T, int D>
+template <typename T, int D, int TM>
 __global__ void __launch_bounds__(SIMT_THREADS)
 state_partial_simt(const T* k, const T* v, PhiPtrs<T> wk, PhiDims pd, Geo g, int n_split, float* partial, int* unsafe,
                    int epoch) {
@@ -273,17 +275,17 @@ state_partial_simt(const T* k, const T* v, PhiPtrs<T> wk, PhiDims pd, Geo g, int
   constexpr int SD = D + 4;
   const int ldh = simt_act_ld(pd.Dh, pd.Dp);
   float* Xs = smem;
-  float* Vs = Xs + SIMT_TM * (D + 4);
-  float* h0 = Vs + SIMT_TM * D;
-  float* h1 = h0 + SIMT_TM * ldh;
-  uint8_t* slabs = reinterpret_cast<uint8_t*>(h1 + SIMT_TM * ldh);
+  float* Vs = Xs + TM * (D + 4);
+  float* h0 = Vs + TM * D;
+  float* h1 = h0 + TM * ldh;
+  uint8_t* slabs = reinterpret_cast<uint8_t*>(h1 + TM * ldh);
 
   const int s = blockIdx.x, ci = blockIdx.y, bh = blockIdx.z, t = g.t0 + ci;
   const int head = bh % g.n_heads, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int lo_prev = t > 0 ? geo_lo(g, t - 1) : 0, lo = geo_lo(g, t);
   const int len = lo - lo_prev;
   int per = (len + n_split - 1) / n_split;
-  per = (per + SIMT_TM - 1) / SIMT_TM * SIMT_TM;
+  per = (per + TM - 1) / TM * TM;
   const int a = min(lo_prev + s * per, lo), b = min(a + per, lo);
 
   PhiPtrs<T> w = {wk.W1 + (size_t)head * pd.Dh * D, wk.b1 + (size_t)head * pd.Dh,
@@ -306,26 +308,26 @@ state_partial_simt(const T* k, const T* v, PhiPtrs<T> wk, PhiDims pd, Geo g, int
       for (int q = 0; q < NQ * 2; ++q) acc[n][u][q] = 0ull;
 
   if (a < b) {
-    load_rows_simt<D>(Xs, D + 4, k + hoff, g.stride_n, a, b);
-    load_rows_simt<D>(Vs, D, v + hoff, g.stride_n, a, b);
+    load_rows_simt<D, TM>(Xs, D + 4, k + hoff, g.stride_n, a, b);
+    load_rows_simt<D, TM>(Vs, D, v + hoff, g.stride_n, a, b);
     cp_async_commit();
   }
 #pragma unroll 1
-  for (int tok0 = a; tok0 < b; tok0 += SIMT_TM) {
-    const float* F = phi_tile_simt<T>(Xs, h0, h1, ldh, slabs, w, pd, b - tok0, [&]() {
-      if (tok0 + SIMT_TM < b) load_rows_simt<D>(Xs, D + 4, k + hoff, g.stride_n, tok0 + SIMT_TM, b);
+  for (int tok0 = a; tok0 < b; tok0 += TM) {
+    const float* F = phi_tile_simt<T, TM>(Xs, h0, h1, ldh, slabs, w, pd, b - tok0, [&]() {
+      if (tok0 + TM < b) load_rows_simt<D, TM>(Xs, D + 4, k + hoff, g.stride_n, tok0 + TM, b);
     });
     __syncthreads();
     if (threadIdx.x < pd.Dp)
 #pragma unroll 8
-      for (int r = 0; r < SIMT_TM; ++r) zacc += F[r * ldh + threadIdx.x];
+      for (int r = 0; r < TM; ++r) zacc += F[r * ldh + threadIdx.x];
 #pragma unroll
     for (int n = 0; n < NB; ++n) {
       const int f0 = (warp + 8 * n) * (FT * 4);
       if (f0 >= pd.Dp) continue;                       // the same for the whole warp
       const float* fp = F + f0 + fg * FT;
 #pragma unroll 2
-      for (int r = 0; r < SIMT_TM; ++r) {
+      for (int r = 0; r < TM; ++r) {
         uint64_t vv[NQ * 2], ff[FT];
 #pragma unroll
         for (int q = 0; q < NQ; ++q) ld_pairs(Vs + r * D + cg * 4 + 32 * q, vv[2 * q], vv[2 * q + 1]);
@@ -342,7 +344,7 @@ state_partial_simt(const T* k, const T* v, PhiPtrs<T> wk, PhiDims pd, Geo g, int
       }
     }
     __syncthreads();
-    if (tok0 + SIMT_TM < b) load_rows_simt<D>(Vs, D, v + hoff, g.stride_n, tok0 + SIMT_TM, b);
+    if (tok0 + TM < b) load_rows_simt<D, TM>(Vs, D, v + hoff, g.stride_n, tok0 + TM, b);
     cp_async_commit();
   }
   float* dst = partial + (((size_t)ci * n_split + s) * g.BH + bh) * pd.Dp * SD;
@@ -444,10 +446,10 @@ combine_bidirectional(const float* cum, float* state, size_t per_slot, Geo g, in
 }
 
 // grid (CTAs per chunk, G, BH), SIMT_THREADS threads, dynamic smem simt_phi_smem(.., false).  Linear read-out of
-// `tiles_per_cta` tiles of SIMT_TM queries of chunk t: rd[bh][row in group][0..d) = phi_q(q_i) s_t,
+// `tiles_per_cta` tiles of TM queries of chunk t: rd[bh][row in group][0..d) = phi_q(q_i) s_t,
 // [d] = phi_q(q_i) z_t, in the fp32 layout of rd_index or (rd_half, for the tensor-core window kernels) as fp16 ratios
 // in the layout of rdh_index.
-template <typename T, int D>
+template <typename T, int D, int TM>
 __global__ void __launch_bounds__(SIMT_THREADS)
 readout_simt(const T* q, PhiPtrs<T> wq, PhiDims pd, Geo g, const float* state, float* rd, int rd_rows, int rd_half,
              int tiles_per_cta, int* unsafe, int epoch) {
@@ -460,15 +462,15 @@ readout_simt(const T* q, PhiPtrs<T> wq, PhiDims pd, Geo g, const float* state, f
   constexpr int SD = D + 4;
   const int ldh = simt_act_ld(pd.Dh, pd.Dp);
   float* Xs = smem;
-  float* h0 = Xs + SIMT_TM * (D + 4);
-  float* h1 = h0 + SIMT_TM * ldh;
-  float* nl_s = h1 + SIMT_TM * ldh;                    // phi_q(q_i) z_t of the tile's rows
-  uint8_t* slabs = reinterpret_cast<uint8_t*>(nl_s + SIMT_TM);
+  float* h0 = Xs + TM * (D + 4);
+  float* h1 = h0 + TM * ldh;
+  float* nl_s = h1 + TM * ldh;                    // phi_q(q_i) z_t of the tile's rows
+  uint8_t* slabs = reinterpret_cast<uint8_t*>(nl_s + TM);
 
   const int ci = blockIdx.y, bh = blockIdx.z, t = g.t0 + ci, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (!geo_linear(g, t)) return;                       // empty linear set: nothing to read out
   const int q0 = geo_q0(g, t), q1 = geo_q1(g, t);
-  const int a = q0 + (int)blockIdx.x * tiles_per_cta * SIMT_TM, b = min(a + tiles_per_cta * SIMT_TM, q1);
+  const int a = q0 + (int)blockIdx.x * tiles_per_cta * TM, b = min(a + tiles_per_cta * TM, q1);
   if (a >= b) return;
   const int head = bh % g.n_heads;
   PhiPtrs<T> w = {wq.W1 + (size_t)head * pd.Dh * D, wq.b1 + (size_t)head * pd.Dh,
@@ -478,14 +480,15 @@ readout_simt(const T* q, PhiPtrs<T> wq, PhiDims pd, Geo g, const float* state, f
   const T* qh = q + q_row_offset(g, bh, 0);
   const float* S = state + ((size_t)ci * g.BH + bh) * pd.Dp * SD;
 
-  // phi s_t: a warp has 32 columns and TM * (D/32) / 8 rows, a lane four consecutive columns of RR rows
-  constexpr int NCB = D / 32, RR = D / 32;
+  // phi s_t: a warp has 32 columns and 4 RR rows, a lane four consecutive columns of RR rows (8 tokens of 64 channels are
+  // work for four warps only)
+  constexpr int NCB = D / 32, RR = TM * D >= 1024 ? TM * D / 1024 : 1;
   const int rg = lane >> 3, cg = lane & 7, cb = warp % NCB, row0 = warp / NCB * (4 * RR);
   uint8_t* const slab_ptr = slabs + warp * SIMT_STAGES * SIMT_SLAB;
   const uint32_t slab = ptx::smem_u32(slab_ptr);
   // Features [16 s, 16 s + 16) x 32 columns, rows of 128 bytes; one commit group per call, also when there is nothing to copy.
   // Nothing is copied beyond the last slab: no wait covers such a copy, and the next tile's weights go into the same slots.
-  const int n_slab = (pd.Dp + 15) / 16;
+  const int n_slab = row0 < TM ? (pd.Dp + 15) / 16 : 0;
   auto issue_state = [&](int s) {
     if (s < n_slab) {
 #pragma unroll
@@ -497,12 +500,12 @@ readout_simt(const T* q, PhiPtrs<T> wq, PhiDims pd, Geo g, const float* state, f
     cp_async_commit();
   };
 
-  load_rows_simt<D>(Xs, D + 4, qh, g.qstride_n, a, b);
+  load_rows_simt<D, TM>(Xs, D + 4, qh, g.qstride_n, a, b);
   cp_async_commit();
 #pragma unroll 1
-  for (int tok0 = a; tok0 < b; tok0 += SIMT_TM) {
-    const float* F = phi_tile_simt<T>(Xs, h0, h1, ldh, slabs, w, pd, b - tok0, [&]() {
-      if (tok0 + SIMT_TM < b) load_rows_simt<D>(Xs, D + 4, qh, g.qstride_n, tok0 + SIMT_TM, b);
+  for (int tok0 = a; tok0 < b; tok0 += TM) {
+    const float* F = phi_tile_simt<T, TM>(Xs, h0, h1, ldh, slabs, w, pd, b - tok0, [&]() {
+      if (tok0 + TM < b) load_rows_simt<D, TM>(Xs, D + 4, qh, g.qstride_n, tok0 + TM, b);
     });
     __syncwarp();                                      // the warp's slabs are free
     if (tok0 == a) {                                   // phi of the first tile runs while the states are still being summed
@@ -514,7 +517,7 @@ readout_simt(const T* q, PhiPtrs<T> wq, PhiDims pd, Geo g, const float* state, f
     __syncthreads();
     // nL of the warp's four rows, the lanes sharing the features
     {
-      constexpr int RW = SIMT_TM / (SIMT_THREADS / 32);
+      constexpr int RW = TM / (SIMT_THREADS / 32);
       float nl[RW] = {};
       for (int f = lane; f < pd.Dp; f += 32) {
         const float z = S[(size_t)f * SD + D];
@@ -571,7 +574,7 @@ readout_simt(const T* q, PhiPtrs<T> wq, PhiDims pd, Geo g, const float* state, f
 #pragma unroll
     for (int i = 0; i < RR; ++i) {
       const int r = row0 + rg + 4 * i, tok = tok0 + r;
-      if (tok >= b) continue;
+      if (r >= TM || tok >= b) continue;
       float y[4];
       ptx::upk2(acc[i][0], y[0], y[1]);
       ptx::upk2(acc[i][1], y[2], y[3]);

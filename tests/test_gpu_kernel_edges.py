@@ -328,3 +328,16 @@ def test_fp32_keeps_its_precision_at_the_smallest_magnitudes(small):
     back = 2.0 ** (122 if small == "v" else 0)
     rel = np.linalg.norm(y * back - ref * back) / np.linalg.norm(ref * back)
     assert rel <= 1e-6, f"relative error {rel:.2e}"
+
+# Tiles of 8, 16 and 32 tokens of the CUDA-core phi kernels (a quarter of the SMs bounds the state's, the rounds of tiles decide
+# on the read-out's): chunks that end inside a tile, two tiles of 8 a CTA, widths of one column block to eight.
+@pytest.mark.parametrize("dtype,d,nh,T,H,W,Tc,To,Dh,Dp,P", [
+    ("fp32", 64, 1, 5, 3, 5, 1, 1, 128, 128, 2), ("fp32", 128, 2, 4, 8, 16, 1, 1, 256, 256, 2), ("fp32", 64, 2, 6, 7, 11, 2, 1, 8, 40, 1),
+    ("fp32", 128, 3, 5, 9, 17, 1, 0, 256, 192, 3), ("bf16", 64, 2, 5, 7, 9, 1, 1, 136, 200, 2), ("bf16", 128, 1, 4, 5, 7, 2, 1, 72, 24, 4),
+    ("bf16", 64, 4, 7, 16, 17, 1, 1, 24, 104, 1)])
+def test_tiles_of_the_cuda_core_phi_kernels(dtype, d, nh, T, H, W, Tc, To, Dh, Dp, P):
+    wl = synth.Workload("phitiles", 1, nh, d, T, H, W, Tc, To, dtype, dtype == "bf16", P=P, seed=synth.BASE_SEED + 409, phi_hidden=Dh, phi_dim=Dp)
+    x = synth.make_inputs(wl, phi_scale=2.0, v_frame_offsets=True)
+    y = _forward(wl, x, impl="simt")
+    _gate(y, _oracle(wl, x), dtype)
+    np.testing.assert_array_equal(_forward(wl, x, impl="simt"), y)
