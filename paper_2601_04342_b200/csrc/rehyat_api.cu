@@ -441,10 +441,10 @@ int run_parts(rehyat_ctx* ctx, const void* q, const void* k, const void* v, void
     }
     if (rc == REHYAT_OK && (parts & PART_WINDOW)) {
       ctx->prof.begin(REHYAT_PROF_WINDOW, st);
-      rc = tc_launch_window(&ctx->tc, q, k, v, out, g, batch, ctx->readout, ctx->rd_cap, c.c_mode, next_wait(ctx), ctx->share_now,
-                            !(parts & PART_READOUT), st);
+      const ptx::WaitArgs wa = next_wait(ctx);
+      rc = tc_launch_window(&ctx->tc, q, k, v, out, g, batch, ctx->readout, ctx->rd_cap, c.c_mode, wa, next_wait(ctx), ctx->share_now,
+                            !(parts & PART_READOUT), &ctx->last_launches, st);
       ctx->prof.end(REHYAT_PROF_WINDOW, st);
-      ctx->last_launches += 1;
     }
   } else if (c.dtype == REHYAT_DTYPE_FP32) {
     rc = c.head_dim == 64

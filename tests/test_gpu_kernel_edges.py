@@ -341,3 +341,20 @@ def test_tiles_of_the_cuda_core_phi_kernels(dtype, d, nh, T, H, W, Tc, To, Dh, D
     y = _forward(wl, x, impl="simt")
     _gate(y, _oracle(wl, x), dtype)
     np.testing.assert_array_equal(_forward(wl, x, impl="simt"), y)
+
+# Windows in two launches: full waves of pairs of tiles, then the rest tile by tile.  Nine tiles a chunk, all 864 pairs first and
+# the ninth tiles left; eleven tiles a chunk, 888 of 900 pairs first; short last chunks of an odd and of an even number of tiles.
+@pytest.mark.parametrize("d,nh,T,H,W,Tc,To", [(128, 72, 5, 20, 26, 2, 0), (64, 60, 5, 1, 641, 2, 0)])
+def test_window_in_two_launches(d, nh, T, H, W, Tc, To):
+    wl = synth.Workload("rest", 1, nh, d, T, H, W, Tc, To, "bf16", True, seed=synth.BASE_SEED + 410, phi_hidden=64, phi_dim=64)
+    x = synth.make_inputs(wl, phi_scale=2.0, v_frame_offsets=True)
+    y, pairs = _forward(wl, x, launches=5), _forward(wl, x, window_tiles=2, launches=4)
+    some = [0, 7, nh // 2, nh - 1]                              # heads
+    xs = {n: x[n][:, some] for n in ("q", "k", "v")} | {m: {n: p[some] for n, p in x[m].items()} for m in ("phi_q", "phi_k")}
+    ref, size = _oracle(wl, xs), _oracle(wl, {**xs, "v": xs["v"].abs()})
+    # The roundings to bf16 (weights, features, states) change the weights of Eq. 5 by a few 2^-9 of themselves, so they move y
+    # by that part of the mean of |v| under the same weights, which is more than |y| where the v of the offset frames cancel.
+    for z in (y[:, some], pairs[:, some]):
+        assert (np.abs(z - ref) <= 3e-3 + 2.0 ** -7 * size).all() and np.sqrt(((z - ref) ** 2).mean() / (ref ** 2).mean()) <= 1e-2
+    assert np.abs(y - pairs).max() <= 2.0 ** -6 * np.abs(pairs).max()      # every row: two roundings of the weights and of the output
+    np.testing.assert_array_equal(_forward(wl, x), y)
