@@ -231,11 +231,7 @@ long long cost_behind(const rehyat_ctx* ctx, const PhiPlan& state, const PhiPlan
 // chunk of 64 tokens stays (54 us, not 65).
 PhiPlan plan_phi(const rehyat_ctx* ctx, long long tokens, long long units, int most, const PhiPlan* state = nullptr) {
   const int n_sm = ctx->tc.n_sm;
-  if (ctx->tensor_ok && ctx->tc.phi_ok) {
-    const rehyat_config& c = ctx->cfg;
-    const int per_sm = tc_state_narrow(c.head_dim, c.phi_hidden, c.phi_dim, c.phi_layers > 2 ? c.phi_layers - 2 : 0) ? 2 : 1;
-    return {pick_parts((tokens + 127) / 128, units, most, per_sm * n_sm), false, SIMT_TM, 0, 0};
-  }
+  if (ctx->tensor_ok && ctx->tc.phi_ok) return {1, false, SIMT_TM, 0, 0};   // phi_tc and readout_tc share out their tiles themselves
   PhiPlan best = simt_plan(ctx, SIMT_TILES[0], tokens, units, most);
   if (ctx->status_dev != nullptr && ctx->cfg.impl != REHYAT_IMPL_SIMT && ctx->cfg.dtype == REHYAT_DTYPE_FP32 && ctx->cfg.phi_layers <= 2) {
     long long tc = 0;
@@ -318,7 +314,7 @@ int launch_group_simt(rehyat_ctx* ctx, const T* q, const T* k, const T* v, T* ou
     ctx->prof.end(REHYAT_PROF_STATE, st);
     const size_t per_slot = (size_t)g.BH * pd.Dp * SD;
     ctx->prof.begin(REHYAT_PROF_SCAN, st);
-    launch_kernel(scan_states, dim3(scan_blocks(per_slot)), SCAN_THREADS, 0, st, ctx->partial, state_out, per_slot, g.G, n_split, carry, nullptr, D);
+    launch_kernel(scan_states<false>, dim3(scan_blocks(per_slot)), SCAN_THREADS, 0, st, ctx->partial, state_out, per_slot, g.G, n_split, carry, nullptr, D, g, StateWalk());
     ctx->prof.end(REHYAT_PROF_SCAN, st);
     ctx->last_launches += 2;
   }
@@ -406,7 +402,6 @@ PhiPlan pick_state_split(const rehyat_ctx* ctx, const Geo& g, int n_chunks_in_gr
 int run_parts(rehyat_ctx* ctx, const void* q, const void* k, const void* v, void* out, const rehyat_phi_params* phi,
               const Geo& g, int batch, PhiPlan split, float* state_out, const float* carry, int parts, cudaStream_t st) {
   const rehyat_config& c = ctx->cfg;
-  const int n_split = split.parts;
   int rc = REHYAT_OK;
   if (ctx->tensor_ok) {
     using B = __nv_bfloat16;
@@ -418,15 +413,18 @@ int run_parts(rehyat_ctx* ctx, const void* q, const void* k, const void* v, void
                                            parts & (PART_STATE | PART_READOUT), st);
     } else {
       if (parts & PART_STATE) {
+        // as many partial states per chunk as there is room for, up to 16
+        const int n_mid = c.phi_layers > 2 ? c.phi_layers - 2 : 0;
+        const long long room = (long long)ctx->partial_units * ctx->bh_max / g.BH / g.G;
+        const StateWalk walk = state_walk(g, ctx->tc.n_sm * (tc_state_narrow(c.head_dim, c.phi_hidden, c.phi_dim, n_mid) ? 2 : 1), room < 16 ? (int)room : 16);
         ctx->prof.begin(REHYAT_PROF_STATE, st);
         rc = tc_launch_state(&ctx->tc, k, v, phi, g, batch, c.phi_hidden, c.phi_dim, c.poly_degree,
-                             c.phi_layers > 2 ? c.phi_layers - 2 : 0, c.act_hidden, c.act_out, n_split,
-                             ctx->partial, next_wait(ctx), st);
+                             n_mid, c.act_hidden, c.act_out, walk, ctx->partial, next_wait(ctx), st);
         ctx->prof.end(REHYAT_PROF_STATE, st);
         const size_t per_slot = (size_t)g.BH * c.phi_dim * (c.head_dim + 4);
         ctx->prof.begin(REHYAT_PROF_SCAN, st);
-        launch_kernel(scan_states, dim3(scan_blocks(per_slot)), SCAN_THREADS, 0, st, ctx->partial, state_out, per_slot, g.G, n_split, carry,
-                                                                    state_out == ctx->state ? ctx->tc.state_bf16 : nullptr, c.head_dim);
+        launch_kernel(walk.even ? scan_states<false> : scan_states<true>, dim3(scan_blocks(per_slot)), SCAN_THREADS, 0, st, ctx->partial,
+                      state_out, per_slot, g.G, walk.slots, carry, state_out == ctx->state ? ctx->tc.state_bf16 : nullptr, c.head_dim, g, walk);
         ctx->prof.end(REHYAT_PROF_SCAN, st);
         ctx->last_launches += 2;
       }
@@ -577,7 +575,7 @@ int rehyat_create(rehyat_ctx** out, const rehyat_config* cfg) {
   const int np_max = c.max_tokens_per_frame * c.max_chunk_frames;
   const int want = c.group_tokens > 0 ? c.group_tokens : 32768;
   ctx->rd_rows = ((want > np_max ? want : np_max) + 127) / 128 * 128 + 128;
-  ctx->Gmax = 16;
+  ctx->Gmax = STATE_CHUNKS;
   ctx->rd_cap = ctx->rd_rows + ctx->Gmax * 128;          // every chunk's last 128-row tile may be partly empty
   ctx->partial_units = 32;
   ctx->bh_max = c.max_batch * c.n_heads;
@@ -1135,8 +1133,8 @@ int rehyat_stream_import(rehyat_ctx* ctx, const void* host_buf, size_t bytes, vo
   if (s.has_state && ctx->tensor_ok && ctx->tc.phi_ok) {
     // the bf16 copy of the state that the tensor-core read-out multiplies with: a scan over zero increments
     const size_t per_slot = stream_state_floats(ctx);
-    launch_kernel(scan_states, dim3(scan_blocks(per_slot)), SCAN_THREADS, 0, st, ctx->partial, ctx->state, per_slot, 1, 0, ctx->state,
-                                                                ctx->tc.state_bf16, c.head_dim);
+    launch_kernel(scan_states<false>, dim3(scan_blocks(per_slot)), SCAN_THREADS, 0, st, ctx->partial, ctx->state, per_slot, 1, 0, ctx->state,
+                  ctx->tc.state_bf16, c.head_dim, Geo(), StateWalk());
   }
   const size_t es = elem_size(c.dtype), width = (size_t)s.halo * c.head_dim * es, pitch = (size_t)s.cap_tokens * c.head_dim * es;
   const int BH = s.batch * c.n_heads;

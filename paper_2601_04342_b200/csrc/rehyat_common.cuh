@@ -52,6 +52,99 @@ __host__ __device__ inline int geo_lo(const Geo& g, int t) {
 // Does chunk t have a non-empty linear set TL_t?
 __host__ __device__ inline bool geo_linear(const Geo& g, int t) { return geo_lo(g, t) > 0 || g.prefix != 0; }
 
+// The key tiles of a state launch, numbered over (batch*head, chunk, tile); CTA c takes the numbers [c per, (c + 1) per).
+// Every chunk it meets gets a partial state of its own, numbered from the first CTA that has tiles of it; `slots` is the largest
+// number of them.  state_walk numbers the tiles either without gaps, so that all CTAs have the same share across chunks and
+// heads, or gives every chunk slots * per numbers (`even`), so that no CTA has to end one chunk and begin another, every chunk
+// has `slots` partial states and those of CTAs without tiles are zero.
+constexpr int STATE_CHUNKS = 16;       // most chunks of a group
+struct StateWalk {
+  int per = 0, slots = 0, even = 1;
+  int off[STATE_CHUNKS + 1] = {};      // number of a chunk's first tile within its (batch*head); last: of all
+};
+// keys chunk t0 + ci newly admits
+__host__ __device__ inline void state_range(const Geo& g, int ci, int& lo_prev, int& lo) {
+  const int t = g.t0 + ci;
+  lo_prev = t > 0 ? geo_lo(g, t - 1) : 0;
+  lo = geo_lo(g, t);
+}
+__host__ __device__ inline int state_tiles(const Geo& g, int ci) {
+  int a, b;
+  state_range(g, ci, a, b);
+  return (b - a + 127) / 128;
+}
+// `ctas` at a time, at most `most` (at least 2) partial states per chunk.  Costs in times of a tile, of which a CTA loses about one
+// in every chunk it works on (pipeline fill, the sums' way out).  Heads of 128, state kernel, numbered by chunk and without
+// gaps: 24 heads x 7 chunks of 37 tiles (twice) 692 and 546 us, 12 heads x 16 frames of 5 tiles 242 and 227; one chunk of 37 tiles for
+// 12 heads (4 + 1 against 3 + 2 tiles) 36 and 42, 12 heads x 7 chunks of 15 tiles (8 + 1, 7 + 2) 64 and 67.
+inline StateWalk state_walk(const Geo& g, int ctas, int most) {
+  StateWalk w;
+  long long total = 0, units = 0;
+  int longest = 0;
+  for (int ci = 0; ci < g.G; ++ci) {
+    const int n = state_tiles(g, ci);
+    total += n;
+    units += n > 0;
+    longest = n > longest ? n : longest;
+  }
+  if (longest == 0) return w;
+  total *= g.BH;
+  units *= g.BH;
+  const int share = (int)((total + ctas - 1) / ctas), least = (longest - 1 + most - 2) / (most - 1);
+  w.per = share > least ? share : least;
+  w.slots = (longest - 1 + w.per - 1) / w.per + 1;
+  w.even = 0;
+  long long best = w.per + 1 + (w.per + longest - 1) / longest;
+  for (int s = 1; s <= most; ++s) {
+    const int per = (longest + s - 1) / s;
+    const long long cost = (units * s + ctas - 1) / ctas * (per + 1);
+    if (cost < best || (cost == best && !w.even)) { best = cost; w.even = 1; w.per = per; w.slots = (longest + per - 1) / per; }
+  }
+  for (int ci = 0; ci < g.G; ++ci) {
+    w.off[ci + 1] = w.off[ci] + (w.even ? w.slots * w.per : state_tiles(g, ci));
+  }
+  for (int ci = g.G; ci < STATE_CHUNKS; ++ci) w.off[ci + 1] = w.off[ci];
+  return w;
+}
+inline int state_ctas(const Geo& g, const StateWalk& w) { return w.per == 0 ? 0 : (w.off[STATE_CHUNKS] * g.BH + w.per - 1) / w.per; }
+// Partial states of chunk ci of bh (not `even`).
+__device__ __forceinline__ int state_slots(const Geo& g, const StateWalk& w, int bh, int ci) {
+  const int n = state_tiles(g, ci), first = bh * w.off[STATE_CHUNKS] + w.off[ci];
+  return n == 0 ? 0 : (first + n - 1) / w.per - first / w.per + 1;
+}
+
+// The query tiles of a launch, numbered over (batch*head, chunk with a linear set, tile); CTA c takes the numbers
+// [c per, (c + 1) per).  `stride` numbers per chunk: its tiles, so that all CTAs have the same share across chunks and heads (only
+// the last chunk may have fewer tiles than the others), or (`even`) a multiple of `per`, so that no CTA changes chunks.
+struct RdTile {
+  int bh, ci, tok, tok_end;    // first token of the tile, end of its chunk
+};
+struct RdWalk {
+  int first = 0, per = 0, stride = 0, per_bh = 0, even = 0;   // first: chunk of the group with a linear set
+};
+// `ctas` at a time.  Costs in tenths of the time of a tile: about one tile to fill the pipeline, 0.3 to change chunks (biases and
+// z_t), 0.05 per tile for keeping track of them.  Read-out kernel, chunks cut evenly and tiles numbered through: 24 heads of 64, 21
+// chunks of 13 tiles 169 and 125 us, 12 heads of 128, 11 chunks of 10 tiles (GELU) 193 and 158, 24 heads x 14 chunks of 37 tiles 554
+// and 529, one chunk of 37 tiles for 12 heads (4 tiles, 3) 28 and 27; 12 heads x 7 chunks of 37 tiles (19, 18) 127 and 138, of 15
+// tiles (8 either way) 59 and 62.
+inline RdWalk rd_walk(const Geo& g, int ctas) {
+  RdWalk w;
+  const int full = (g.Np + 127) / 128, last = g.t0 + g.G - 1, short_one = (geo_q1(g, last) - geo_q0(g, last) + 127) / 128;
+  while (w.first < g.G && !geo_linear(g, g.t0 + w.first)) ++w.first;
+  const int chunks = g.G - w.first;
+  if (chunks == 0) return w;
+  w.stride = full;
+  w.per_bh = (chunks - 1) * full + short_one;
+  w.per = (int)(((long long)w.per_bh * g.BH + ctas - 1) / ctas);
+  long long best = 10LL * (w.per + 1) + w.per / 2 + 3 * ((w.per + full - 1) / full);
+  for (int s = 1; s <= 16; ++s) {
+    const int per = (full + s - 1) / s;
+    const long long cost = ((long long)chunks * g.BH * s + ctas - 1) / ctas * 10 * (per + 1);
+    if (cost < best || (cost == best && !w.even)) { best = cost; w.even = 1; w.per = per; }
+  }
+  if (w.even) { w.stride = (full + w.per - 1) / w.per * w.per; w.per_bh = chunks * w.stride; }
+  return w;
+}
 // Linear read-out workspace (phi_q(q_i) s_t in columns [0, d), phi_q(q_i) z_t in column d).  Per (batch*head)
 // it is cut into tiles of 128 query rows - tile k of chunk ci of the group has index ci*ceil(Np/128) + k - and a
 // tile into d/4 + 1 pieces of four columns, each piece holding the tile's 128 rows contiguously (16 bytes per row).

@@ -2,8 +2,8 @@
 //
 // phi_tc evaluates the feature map phi_k of Section 3.2 ("Characterization of phi") on tiles of 128 keys with
 // tcgen05.mma and feeds it straight into the contraction that consumes it: phi_k(K tile)^T [V | 1] accumulated
-// in TMEM over the CTA's share of the keys a chunk newly admits (Eq. 17-18), flushed once as an fp32 partial
-// state.  (The read-out kernel, readout_tc, has a file of its own; it shares the constants and PhiTcArgs.)
+// in TMEM over the CTA's share of the keys a chunk newly admits (Eq. 17-18), flushed once per chunk as an fp32
+// partial state.  (The read-out kernel, readout_tc, has a file of its own; it shares the constants and PhiTcArgs.)
 //
 // Per tile the chain is  H = act(X W1^T + b1) -> U = act(H W2^T + b2) -> phi = U^(1..P)  with the
 // two GEMMs done as 128x128 halves through one 128-column TMEM scratch accumulator (the state accumulators
@@ -68,6 +68,7 @@ struct PhBars {
   uint64_t x_full, x_empty, v_full, v_empty;
   uint64_t ring_full[PH_RING_MAX], ring_empty[PH_RING_MAX];
   uint64_t acc_ready, acc_free, epi_done[2], out_ready;   // see the issuer
+  uint64_t out_free;           // a chunk's sums have left TMEM
   uint64_t drained;            // every tcgen05.mma of the issuer has completed
   uint32_t tmem_base;
   ptx::WaitCtx wctx;
@@ -80,14 +81,34 @@ struct PhiTcArgs {
   int d, Dh, Dp;               // head_dim (64 or 128), phi widths (read by the GEN = true kernels)
   int n_mid;                   // hidden layers between the first and the last (GEN = true kernels), at most PH_MAX_MID
   const __nv_bfloat16* bm;     // [heads][n_mid][D_h]
-  int n_split;                 // state kernel: splits of a chunk's increment
-  float* partial;              // state kernel: [G][n_split][BH][D'][d + 4]
+  StateWalk walk;              // state kernel: who has which tiles
+  float* partial;              // state kernel: [G][walk.slots][BH][D'][d + 4]
   const float* state;          // read-out kernel: fp32 states (z column is read)
   float* rd;                   // read-out kernel: the read-out workspace (see rdh_index)
   int rd_rows;
-  int tiles_per_cta;           // read-out kernel
+  RdWalk rd_walk;              // read-out kernel: who has which tiles
   ptx::WaitArgs wa;            // status word, launch epoch, wait limit
 };
+
+// What a CTA has of one chunk, from tile number n on, and the number behind it (past the gap, if there is one).
+struct StateSeg {
+  int bh, ci, tok, tok_end, n_tiles, slot, next;
+};
+__device__ __forceinline__ StateSeg state_seg(const Geo& g, const StateWalk& w, int n, int n_end) {
+  StateSeg s;
+  const int all = w.off[STATE_CHUNKS];
+  s.bh = n / all;
+  const int rest = n % all;
+  for (s.ci = 0; rest >= w.off[s.ci + 1]; ++s.ci) {}
+  int lo_prev;
+  state_range(g, s.ci, lo_prev, s.tok_end);
+  const int tile = rest - w.off[s.ci];
+  s.tok = lo_prev + tile * 128;
+  s.next = min(n_end, n - rest + w.off[s.ci + 1]);
+  s.n_tiles = min(s.next - n, (s.tok_end - s.tok + 127) / 128);
+  s.slot = n / w.per - (n - tile) / w.per;
+  return s;
+}
 
 // Extents of one launch: constants for the default shape, read from the arguments otherwise.
 template <bool GEN>
@@ -105,7 +126,7 @@ struct PhiExtents {
 // tm_x: K, tm_v: V, 4-D like the window kernel's maps.  tm_w1: (d, D_h, heads), tm_w2: (D_h, D', heads),
 // tm_wm: (D_h, D_h, heads * n_mid) (any valid map when n_mid = 0), boxes [64 x 128].  PC: polynomial degree known
 // at compile time (0: read it from the arguments; 2 needs D' = 256).
-template <bool RELU, int PC, bool GEN, bool NARROW>
+template <bool RELU, int PC, bool GEN, bool NARROW, bool EVEN>
 __global__ void __launch_bounds__(PH_THREADS, NARROW ? 2 : 1)
 phi_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_v,
        const __grid_constant__ CUtensorMap tm_w1, const __grid_constant__ CUtensorMap tm_w2,
@@ -122,28 +143,22 @@ phi_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtenso
   const uint32_t wc = smem_u32(&bars->wctx);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int ci = blockIdx.y, bh = blockIdx.z, t = g.t0 + ci;
-  const int b_idx = bh / g.n_heads, h_idx = bh % g.n_heads;
   const PhiExtents<GEN> ex(a);
   const int Dp = ex.Dp, SD = ex.sd(), ks1 = ex.ks1(), ks2 = ex.ks2(), nh = ex.nh(), nu = ex.nu(), n_mid = ex.n_mid;
 
-  // token range [tok_a, tok_b) of this CTA
-  const int lo_prev = t > 0 ? geo_lo(g, t - 1) : 0, lo = geo_lo(g, t);
-  int per = (lo - lo_prev + a.n_split - 1) / a.n_split;
-  per = (per + 127) / 128 * 128;
-  const int tok_a = min(lo_prev + (int)blockIdx.x * per, lo);
-  const int tok_b = min(tok_a + per, lo);
-  const int n_tiles = (tok_b - tok_a + 127) / 128;
+  const int n_begin = (int)blockIdx.x * a.walk.per, n_end = min(n_begin + a.walk.per, a.walk.off[STATE_CHUNKS] * g.BH);
 
-  if (n_tiles == 0) {                          // nothing admitted: the partial is zero
-    grid_dep_wait();
-    grid_dep_launch();
-    float* dst = a.partial + (((size_t)ci * a.n_split + blockIdx.x) * g.BH + bh) * Dp * SD;
-    for (int i = threadIdx.x; i < Dp * SD / 4; i += PH_THREADS)
-      reinterpret_cast<float4*>(dst)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    return;
+  const StateSeg sg0 = state_seg(g, a.walk, n_begin, n_end);
+  if constexpr (EVEN) {
+    if (sg0.n_tiles <= 0) {                     // nothing admitted: the partial is zero
+      grid_dep_wait();
+      grid_dep_launch();
+      float* dst = a.partial + (((size_t)sg0.ci * a.walk.slots + sg0.slot) * g.BH + sg0.bh) * Dp * SD;
+      for (int i = threadIdx.x; i < Dp * SD / 4; i += PH_THREADS)
+        reinterpret_cast<float4*>(dst)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      return;
+    }
   }
-
   if (threadIdx.x == 0) {
     mbar_init(smem_u32(&bars->x_full), 1); mbar_init(smem_u32(&bars->x_empty), 1);
     mbar_init(smem_u32(&bars->v_full), 1); mbar_init(smem_u32(&bars->v_empty), 1);
@@ -152,7 +167,7 @@ phi_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtenso
     }
     mbar_init(smem_u32(&bars->acc_ready), 1); mbar_init(smem_u32(&bars->acc_free), 8);
     mbar_init(smem_u32(&bars->epi_done[0]), 8); mbar_init(smem_u32(&bars->epi_done[1]), 8);
-    mbar_init(smem_u32(&bars->out_ready), 1);
+    mbar_init(smem_u32(&bars->out_ready), 1); mbar_init(smem_u32(&bars->out_free), 8);
     mbar_init(smem_u32(&bars->drained), 1);
     wait_ctx_init(&bars->wctx, a.wa);
     fence_mbar_init();
@@ -163,13 +178,17 @@ phi_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtenso
   }
   grid_dep_wait();
   grid_dep_launch();
-  // biases as fp32; the ones tile: row 0 of both 64-column sub-tiles is 1, the rest 0
-  for (int i = threadIdx.x; i < 256; i += PH_THREADS) {          // zero beyond the widths
-    s_b1[i] = i < ex.Dh ? __bfloat162float(a.b1[(size_t)h_idx * ex.Dh + i]) : 0.f;
-    s_b2[i] = i < Dp ? __bfloat162float(a.b2[(size_t)h_idx * Dp + i]) : 0.f;
-    for (int m = 0; m < n_mid; ++m)
-      s_b2[(1 + m) * 256 + i] = i < ex.Dh ? __bfloat162float(a.bm[((size_t)h_idx * n_mid + m) * ex.Dh + i]) : 0.f;
-  }
+  auto load_biases = [&](const StateSeg& sg, int threads) {         // as fp32, zero beyond the widths
+    const int h_idx = sg.bh % g.n_heads;
+    for (int i = threadIdx.x; i < 256; i += threads) {
+      s_b1[i] = i < ex.Dh ? __bfloat162float(a.b1[(size_t)h_idx * ex.Dh + i]) : 0.f;
+      s_b2[i] = i < Dp ? __bfloat162float(a.b2[(size_t)h_idx * Dp + i]) : 0.f;
+      for (int m = 0; m < n_mid; ++m)
+        s_b2[(1 + m) * 256 + i] = i < ex.Dh ? __bfloat162float(a.bm[((size_t)h_idx * n_mid + m) * ex.Dh + i]) : 0.f;
+    }
+  };
+  load_biases(sg0, PH_THREADS);
+  // the ones tile: row 0 of both 64-column sub-tiles is 1, the rest 0
   {
     uint32_t* ones = reinterpret_cast<uint32_t*>(smem + SH::OFF_ONES);
     for (int i = threadIdx.x; i < 1024; i += PH_THREADS) {
@@ -218,8 +237,14 @@ phi_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtenso
         tma_load_3d(ring_addr(s), tm, full, x, y, z);
         ++ring_i;
       };
-      for (int j = 0; j < n_tiles && alive; ++j) {
-        const int tok0 = tok_a + j * 128;
+      StateSeg sg = sg0;
+      for (int j = 0, k = 0; alive; ++j, ++k) {                     // tile of the CTA, of the segment
+        if (k == sg.n_tiles) {
+          if (EVEN || sg.next == n_end) break;
+          sg = state_seg(g, a.walk, sg.next, n_end);
+          k = 0;
+        }
+        const int tok0 = sg.tok + k * 128, h_idx = sg.bh % g.n_heads, b_idx = sg.bh / g.n_heads;
         alive = mbar_wait(smem_u32(&bars->x_empty), (j & 1) ^ 1, wc, PH_ERR_LOAD);
         if (!alive) break;
         const uint32_t xf = smem_u32(&bars->x_full);
@@ -314,42 +339,50 @@ phi_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtenso
         }
       };
       auto run = [&]() {
-        for (int j = 0; j < n_tiles; ++j) {
-          if (!wait(&bars->x_full, j & 1)) return;
-          const bool owe_half1 = j > 0 && nu == 2;                    // phi half 1 of tile j-1 is not yet in the state
-          if (owe_half1 && last_hid == 1) {                           // before the half-GEMM whose epilogue writes over it
-            if (!wait_epi() || !wait(&bars->v_full, (j - 1) & 1)) return;
-            consume_half(1, sPhiHalf1, j == 1);
-            umma_commit(smem_u32(&bars->v_empty));
-          }
-          if (!mlp_half(-1, ks1)) return;                             // H[:, 0:128]
-          if (owe_half1 && last_hid == 0) {                           // behind the half-GEMM: it runs during that half's epilogue
-            if (!wait_epi_but_last() || !wait(&bars->v_full, (j - 1) & 1)) return;
-            consume_half(1, sPhiHalf1, j == 1);
-            umma_commit(smem_u32(&bars->v_empty));
-          }
-          if (nh == 2 && !mlp_half(-1, ks1)) return;                  // H[:, 128:256]
-          // The X tile is free after its last reader: the first layer, or the last GEMMs that read hidden buffer 1.
-          if (n_mid == 0) umma_commit(smem_u32(&bars->x_empty));
-          for (int m = 0; m < n_mid; ++m) {                           // hidden layer m: buffer m % 2 -> the other
+        int j = 0;                                                    // tile of the CTA
+        for (int n = n_begin, seg = 0; n < n_end && (!EVEN || seg == 0); ++seg) {
+          const StateSeg sg = EVEN ? sg0 : state_seg(g, a.walk, n, n_end);
+          const int n_tiles = sg.n_tiles;
+          n = sg.next;
+          for (int k = 0; k < n_tiles; ++k, ++j) {                     // tile of the segment
+            if (!wait(&bars->x_full, j & 1)) return;
+            const bool owe_half1 = k > 0 && nu == 2;                    // phi half 1 of tile j-1 is not yet in the state
+            if (owe_half1 && last_hid == 1) {                           // before the half-GEMM whose epilogue writes over it
+              if (!wait_epi() || !wait(&bars->v_full, (j - 1) & 1)) return;
+              consume_half(1, sPhiHalf1, k == 1);
+              umma_commit(smem_u32(&bars->v_empty));
+            }
+            if (!mlp_half(-1, ks1)) return;                             // H[:, 0:128]
+            if (owe_half1 && last_hid == 0) {                           // behind the half-GEMM: it runs during that half's epilogue
+              if (!wait_epi_but_last() || !wait(&bars->v_full, (j - 1) & 1)) return;
+              consume_half(1, sPhiHalf1, k == 1);
+              umma_commit(smem_u32(&bars->v_empty));
+            }
+            if (nh == 2 && !mlp_half(-1, ks1)) return;                  // H[:, 128:256]
+            // The X tile is free after its last reader: the first layer, or the last GEMMs that read hidden buffer 1.
+            if (n_mid == 0) umma_commit(smem_u32(&bars->x_empty));
+            for (int m = 0; m < n_mid; ++m) {                           // hidden layer m: buffer m % 2 -> the other
+              if (!wait_epi()) return;
+              if (!mlp_half(m & 1, ks2)) return;
+              if (nh == 2 && !mlp_half(m & 1, ks2)) return;
+              if (m == n_mid - 1 && last_hid == 0) umma_commit(smem_u32(&bars->x_empty));
+            }
             if (!wait_epi()) return;
-            if (!mlp_half(m & 1, ks2)) return;
-            if (nh == 2 && !mlp_half(m & 1, ks2)) return;
-            if (m == n_mid - 1 && last_hid == 0) umma_commit(smem_u32(&bars->x_empty));
+            if (!mlp_half(last_hid, ks2)) return;                       // U[:, 0:128]
+            if (nu == 2 && !mlp_half(last_hid, ks2)) return;            // U[:, 128:256]
+            if (last_hid == 1) umma_commit(smem_u32(&bars->x_empty));
+            if (!(nu == 2 ? wait_epi_but_last() : wait_epi()) || !wait(&bars->v_full, j & 1)) return;
+            if (k == 0 && seg > 0 && !wait(&bars->out_free, (seg - 1) & 1)) return;   // the sums of the chunk before have left
+            consume_half(0, sPhiHalf0, k == 0);
+            if (nu == 1) umma_commit(smem_u32(&bars->v_empty));         // no second half: V is free once these have run
           }
-          if (!wait_epi()) return;
-          if (!mlp_half(last_hid, ks2)) return;                       // U[:, 0:128]
-          if (nu == 2 && !mlp_half(last_hid, ks2)) return;            // U[:, 128:256]
-          if (last_hid == 1) umma_commit(smem_u32(&bars->x_empty));
-          if (!(nu == 2 ? wait_epi_but_last() : wait_epi()) || !wait(&bars->v_full, j & 1)) return;
-          consume_half(0, sPhiHalf0, j == 0);
-          if (nu == 1) umma_commit(smem_u32(&bars->v_empty));         // no second half: V is free once these have run
+          if (nu == 2) {
+            if (!wait_epi()) return;
+            consume_half(1, sPhiHalf1, n_tiles == 1);
+            umma_commit(smem_u32(&bars->v_empty));
+          }
+          umma_commit(smem_u32(&bars->out_ready));
         }
-        if (nu == 2) {
-          if (!wait_epi()) return;
-          consume_half(1, sPhiHalf1, n_tiles == 1);
-        }
-        umma_commit(smem_u32(&bars->out_ready));
       };
       run();
       // Everything this thread has issued is complete once `drained` flips; the abort flag does not cut this
@@ -455,65 +488,83 @@ phi_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtenso
         mbar_arrive_warp(smem_u32(&bars->epi_done[n_acc & 1]), lane);
         ++n_acc;
     };
-    for (int j = 0; j < n_tiles; ++j) {
-      if (aborted()) break;
-      tok_valid = tok_a + j * 128 + r < tok_b;
-      // a width of at most 128 has no second half
-      if constexpr (RELU && !NARROW) {
-#pragma unroll
-        for (int half = 0; half < 2; ++half)                        // first layer -> hidden buffer 0
-          if (half < nh) epi_step(false, half, s_b1 + half * 128, hid_sub(0, half * 2 + ch));
-        for (int m = 0; m < n_mid; ++m)                             // hidden layer m -> the buffer it does not read
-#pragma unroll
-          for (int half = 0; half < 2; ++half)
-            if (half < nh) epi_step(false, half, s_b2 + (1 + m) * 256 + half * 128, hid_sub((m & 1) ^ 1, half * 2 + ch));
-#pragma unroll
-        for (int half = 0; half < 2; ++half)                        // last layer -> the phi tiles
-          if (half < nu) epi_step(true, half, s_b2 + half * 128, (half == 0 ? sPhiHalf0 : sPhiHalf1) + ch * PH_SUB);
-      } else {
-        // the same steps with one call site: the library's functions are in the code once
-#pragma unroll 1
-        for (int l = 0; l < n_mid + 2; ++l) {
-          const bool is_u = l == n_mid + 1;
-#pragma unroll 1
-          for (int half = 0; half < (is_u ? nu : nh); ++half)
-            epi_step(is_u, half, (l == 0 ? s_b1 : is_u ? s_b2 : s_b2 + l * 256) + half * 128,
-                     is_u ? (half == 0 ? sPhiHalf0 : sPhiHalf1) + ch * PH_SUB : hid_sub(l & 1, half * 2 + ch));
-        }
+    // Of the eight warps; true if any thread's flag is.  No warp leaves but behind one of these, so none waits in vain.
+    auto barrier = [&](bool flag) -> bool {
+      uint32_t any;
+      asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbarrier.cta.red.or.pred q, 1, 256, p;\n\tselp.b32 %0, 1, 0, q;\n\t}"
+                   : "=r"(any) : "r"((uint32_t)flag) : "memory");
+      return any != 0;
+    };
+    for (int n = n_begin, seg = 0; n < n_end && (!EVEN || seg == 0); ++seg) {
+      const StateSeg sg = EVEN ? sg0 : state_seg(g, a.walk, n, n_end);
+      n = sg.next;
+      if (seg > 0) {
+        if (barrier(wait_ctx_aborted(wc) != 0)) break;              // (all warps are done with the biases of the segment before)
+        load_biases(sg, 256);
+        barrier(false);
       }
-    }
-    wait(&bars->out_ready, 0);
-    if (!aborted()) {
-      // flush: lane r holds feature c*128 + r of half c; this thread writes its share of the d columns
-      tc_fence_after();
-      float* base = a.partial + (((size_t)ci * a.n_split + blockIdx.x) * g.BH + bh) * Dp * SD;
+      for (int j = 0; j < sg.n_tiles; ++j) {
+        if (aborted()) break;
+        tok_valid = sg.tok + j * 128 + r < sg.tok_end;
+        // a width of at most 128 has no second half
+        if constexpr (RELU && !NARROW) {
 #pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        if (c >= nu) continue;
-        const bool feat_valid = c * 128 + r < Dp;
-        float* dst = base + (size_t)(c * 128 + r) * SD;
+          for (int half = 0; half < 2; ++half)                        // first layer -> hidden buffer 0
+            if (half < nh) epi_step(false, half, s_b1 + half * 128, hid_sub(0, half * 2 + ch));
+          for (int m = 0; m < n_mid; ++m)                             // hidden layer m -> the buffer it does not read
 #pragma unroll
-        for (int cb = 0; cb < 2; ++cb) {
-          const int col = ch * 64 + cb * 32;
-          if (col >= ex.d) continue;                                // the same for the whole warp
-          uint32_t x[32];
-          tmem_ld32(tmem + lane_off + T_ACC + c * 128 + col, x);
-          tmem_wait_ld();
-          if (feat_valid) {
+            for (int half = 0; half < 2; ++half)
+              if (half < nh) epi_step(false, half, s_b2 + (1 + m) * 256 + half * 128, hid_sub((m & 1) ^ 1, half * 2 + ch));
 #pragma unroll
-            for (int e = 0; e < 32; e += 4)
-              *reinterpret_cast<float4*>(dst + col + e) =
-                  make_float4(__uint_as_float(x[e]), __uint_as_float(x[e + 1]), __uint_as_float(x[e + 2]),
-                              __uint_as_float(x[e + 3]));
+          for (int half = 0; half < 2; ++half)                        // last layer -> the phi tiles
+            if (half < nu) epi_step(true, half, s_b2 + half * 128, (half == 0 ? sPhiHalf0 : sPhiHalf1) + ch * PH_SUB);
+        } else {
+          // the same steps with one call site: the library's functions are in the code once
+#pragma unroll 1
+          for (int l = 0; l < n_mid + 2; ++l) {
+            const bool is_u = l == n_mid + 1;
+#pragma unroll 1
+            for (int half = 0; half < (is_u ? nu : nh); ++half)
+              epi_step(is_u, half, (l == 0 ? s_b1 : is_u ? s_b2 : s_b2 + l * 256) + half * 128,
+                       is_u ? (half == 0 ? sPhiHalf0 : sPhiHalf1) + ch * PH_SUB : hid_sub(l & 1, half * 2 + ch));
           }
         }
-        if (ch == 1) {
-          uint32_t zc[16];
-          tmem_ld16(tmem + lane_off + T_Z + c * 16, zc);
-          tmem_wait_ld();
-          if (feat_valid) *reinterpret_cast<float4*>(dst + ex.d) = make_float4(__uint_as_float(zc[0]), 0.f, 0.f, 0.f);
+      }
+      wait(&bars->out_ready, seg & 1);
+      if (!aborted()) {
+        // flush: lane r holds feature c*128 + r of half c; this thread writes its share of the d columns
+        tc_fence_after();
+        float* base = a.partial + (((size_t)sg.ci * a.walk.slots + sg.slot) * g.BH + sg.bh) * Dp * SD;
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          if (c >= nu) continue;
+          const bool feat_valid = c * 128 + r < Dp;
+          float* dst = base + (size_t)(c * 128 + r) * SD;
+#pragma unroll
+          for (int cb = 0; cb < 2; ++cb) {
+            const int col = ch * 64 + cb * 32;
+            if (col >= ex.d) continue;                                // the same for the whole warp
+            uint32_t x[32];
+            tmem_ld32(tmem + lane_off + T_ACC + c * 128 + col, x);
+            tmem_wait_ld();
+            if (feat_valid) {
+#pragma unroll
+              for (int e = 0; e < 32; e += 4)
+                *reinterpret_cast<float4*>(dst + col + e) =
+                    make_float4(__uint_as_float(x[e]), __uint_as_float(x[e + 1]), __uint_as_float(x[e + 2]),
+                                __uint_as_float(x[e + 3]));
+            }
+          }
+          if (ch == 1) {
+            uint32_t zc[16];
+            tmem_ld16(tmem + lane_off + T_Z + c * 16, zc);
+            tmem_wait_ld();
+            if (feat_valid) *reinterpret_cast<float4*>(dst + ex.d) = make_float4(__uint_as_float(zc[0]), 0.f, 0.f, 0.f);
+          }
         }
       }
+      tc_fence_before();
+      mbar_arrive_warp(smem_u32(&bars->out_free), lane);
     }
   }
 

@@ -50,12 +50,26 @@ struct RdBars {
   ptx::WaitCtx wctx;
 };
 
-// tm_x: Q, 4-D like the window kernel's maps.  tm_w1: (d, D_h, heads), tm_w2: (D_h, D', heads), tm_wm: (D_h, D_h,
-// heads * n_mid) (any valid map when n_mid = 0), boxes [64 x 128].  tm_s: bf16 states (d, D', G*BH), box [64 x 64].
+__device__ __forceinline__ RdTile rd_tile(const Geo& g, const RdWalk& w, int n) {
+  const int rest = n % w.per_bh;
+  RdTile t;
+  t.bh = n / w.per_bh;
+  t.ci = w.first + rest / w.stride;
+  t.tok = geo_q0(g, g.t0 + t.ci) + rest % w.stride * 128;
+  t.tok_end = geo_q1(g, g.t0 + t.ci);
+  return t;
+}
+// ... of tile n, given that of n - 1 (the divisions above take as long as a twentieth of a tile).
+template <bool EVEN>
+__device__ __forceinline__ void rd_next(const Geo& g, const RdWalk& w, int n, RdTile& t) {
+  t.tok += 128;
+  if (!EVEN && t.tok >= t.tok_end) t = rd_tile(g, w, n);
+}
+
 // PC: polynomial degree known at compile time (0: read it from the arguments; 2 needs D' = 256).
 // A hidden layer of a deeper map (GEN only) reads H from TMEM and writes it back there: both halves of its GEMM
 // have completed before the first column of H is overwritten.
-template <bool RELU, int PC, bool GEN, bool NARROW>
+template <bool RELU, int PC, bool GEN, bool NARROW, bool EVEN>
 __global__ void __launch_bounds__(PH_THREADS, NARROW ? 2 : 1)
 readout_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w1,
            const __grid_constant__ CUtensorMap tm_w2, const __grid_constant__ CUtensorMap tm_wm,
@@ -75,18 +89,17 @@ readout_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUt
   const uint32_t wc = smem_u32(&bars->wctx);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int ci = blockIdx.y, bh = blockIdx.z, t = g.t0 + ci;
-  const int b_idx = bh / g.n_heads, h_idx = bh % g.n_heads;
-  if (!geo_linear(g, t)) return;                                    // empty linear set
   const PhiExtents<GEN> ex(a);
   const int d = ex.d, Dp = ex.Dp, SD = ex.sd(), ks1 = ex.ks1(), ks2 = ex.ks2(), nh = ex.nh(), nu = ex.nu();
   const int nf = (Dp + 63) / 64;                                    // 64-feature blocks of the state
   const int n_mid = ex.n_mid;
-  const int q0 = geo_q0(g, t), q1 = geo_q1(g, t);
-  const int tok_a = min(q0 + (int)blockIdx.x * a.tiles_per_cta * 128, q1);
-  const int tok_b = min(tok_a + a.tiles_per_cta * 128, q1);
-  if (tok_a >= tok_b) return;
-  const int n_tiles = (tok_b - tok_a + 127) / 128;
+  const int n0 = (int)blockIdx.x * a.rd_walk.per;
+  int n_tiles = min(a.rd_walk.per, a.rd_walk.per_bh * g.BH - n0);
+  const RdTile t0 = rd_tile(g, a.rd_walk, n0);
+  if constexpr (EVEN) {
+    n_tiles = min(n_tiles, (t0.tok_end - t0.tok + 127) / 128);
+    if (n_tiles <= 0) return;                                        // a short last chunk
+  }
 
   if (threadIdx.x == 0) {
     mbar_init(smem_u32(&bars->x_full), 1); mbar_init(smem_u32(&bars->x_empty), 1);
@@ -99,12 +112,16 @@ readout_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUt
     wait_ctx_init(&bars->wctx, a.wa);
     fence_mbar_init();
   }
-  for (int i = threadIdx.x; i < 256; i += PH_THREADS) {             // biases as fp32, zero beyond the widths
-    s_b1[i] = i < ex.Dh ? __bfloat162float(a.b1[(size_t)h_idx * ex.Dh + i]) : 0.f;
-    s_b2[i] = i < Dp ? __bfloat162float(a.b2[(size_t)h_idx * Dp + i]) : 0.f;
-    for (int m = 0; m < n_mid; ++m)
-      s_bm[m * 256 + i] = i < ex.Dh ? __bfloat162float(a.bm[((size_t)h_idx * n_mid + m) * ex.Dh + i]) : 0.f;
-  }
+  auto load_biases = [&](const RdTile& tl, int threads) {             // as fp32, zero beyond the widths
+    const int h_idx = tl.bh % g.n_heads;
+    for (int i = threadIdx.x; i < 256; i += threads) {
+      s_b1[i] = i < ex.Dh ? __bfloat162float(a.b1[(size_t)h_idx * ex.Dh + i]) : 0.f;
+      s_b2[i] = i < Dp ? __bfloat162float(a.b2[(size_t)h_idx * Dp + i]) : 0.f;
+      for (int m = 0; m < n_mid; ++m)
+        s_bm[m * 256 + i] = i < ex.Dh ? __bfloat162float(a.bm[((size_t)h_idx * n_mid + m) * ex.Dh + i]) : 0.f;
+    }
+  };
+  load_biases(t0, PH_THREADS);
   if (warp == 9) {
     tmem_alloc(smem_u32(&bars->tmem_base), SH::COLS);
     tmem_relinquish();
@@ -137,23 +154,27 @@ readout_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUt
         const uint32_t dst = ring_slot(full, RD_WT_BYTES);
         if (dst) tma_load_3d(dst, tm, full, x, y, plane);
       };
+      int plane = 0;                                                // of the state the tile before is read out with
       auto state_load = [&](int f) {                                // [64 features x d] as 64-column boxes
         uint32_t full = 0;
         const uint32_t dst = ring_slot(full, 8192u * ks1);
         if (dst)
-          for (int ks = 0; ks < ks1; ++ks) tma_load_3d(dst + ks * 8192, &tm_s, full, ks * 64, f * 64, ci * g.BH + bh);
+          for (int ks = 0; ks < ks1; ++ks) tma_load_3d(dst + ks * 8192, &tm_s, full, ks * 64, f * 64, plane);
       };
       auto state_half = [&](int c) {                                // the blocks of features [128 c, 128 c + 128)
         grid_dep_wait_role(wc);                                     // the states are the predecessor's results
         for (int f = 2 * c; f < 2 * c + 2 && f < nf; ++f) state_load(f);
       };
+      RdTile tl = t0;
       for (int j = 0; j < n_tiles && alive; ++j) {
+        if (j > 0) rd_next<EVEN>(g, a.rd_walk, n0 + j, tl);
+        const int h_idx = tl.bh % g.n_heads, b_idx = tl.bh / g.n_heads;
         alive = mbar_wait(smem_u32(&bars->x_empty), (j & 1) ^ 1, wc, PH_ERR_LOAD);
         if (!alive) break;
         const uint32_t xf = smem_u32(&bars->x_full);
         mbar_expect_tx(xf, PH_SUB * ks1);
         for (int ks = 0; ks < ks1; ++ks)
-          tma_load_4d(sX + ks * PH_SUB, &tm_x, xf, ks * 64, tok_a - g.q_off + j * 128, h_idx, b_idx);
+          tma_load_4d(sX + ks * PH_SUB, &tm_x, xf, ks * 64, tl.tok - g.q_off, h_idx, b_idx);
         ++n_x;
         // the ring follows the issue order of the MMAs: read-out of the previous tile between this tile's H halves
         for (int ks = 0; ks < ks1; ++ks) weight_load(&tm_w1, ks * 64, 0, h_idx);
@@ -166,6 +187,7 @@ readout_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUt
             for (int ks = 0; ks < ks2; ++ks) weight_load(&tm_wm, ks * 64, half * 128, h_idx * n_mid + m);
         for (int half = 0; half < nu; ++half)
           for (int ks = 0; ks < ks2; ++ks) weight_load(&tm_w2, ks * 64, half * 128, h_idx);
+        plane = tl.ci * g.BH + tl.bh;
       }
       for (int c = 0; c < nu && alive; ++c) state_half(c);
       if (!alive) {
@@ -295,10 +317,15 @@ readout_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUt
     auto aborted = [&]() -> bool { return __any_sync(0xffffffffu, wait_ctx_aborted(wc) != 0); };
     auto wait = [&](uint64_t* bar, uint32_t parity) { mbar_wait(smem_u32(bar), parity, wc, PH_ERR_EPI); };
     // z_t: the first result of the predecessor that is needed; the loads and GEMMs of the first tile's H run meanwhile
+    const auto all_warps = []() { asm volatile("bar.sync 1, 256;" ::: "memory"); };   // the eight epilogue warps
+    auto load_z = [&](const RdTile& tl) {
+      s_z[threadIdx.x] = (int)threadIdx.x < Dp ? a.state[(((size_t)tl.ci * g.BH + tl.bh) * Dp + threadIdx.x) * SD + d] : 0.f;
+      all_warps();
+    };
+    RdTile cur = t0, prev = t0;
     grid_dep_wait_role(wc);
     grid_dep_launch();
-    s_z[threadIdx.x] = (int)threadIdx.x < Dp ? a.state[(((size_t)ci * g.BH + bh) * Dp + threadIdx.x) * SD + d] : 0.f;
-    asm volatile("bar.sync 1, 256;" ::: "memory");                  // the eight epilogue warps
+    load_z(cur);
     // bias + activation (+ power) of 32 accumulator columns -> 16 bf16 pairs
     auto activate = [&](const auto& x, const float* bias, bool is_u, int col0, auto& w) {
       constexpr int NC = sizeof(x) / sizeof(x[0]);                 // columns of this block
@@ -330,14 +357,14 @@ readout_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUt
         for (int e = 0; e < NC; e += 2) w[e >> 1] = pack_bf16(y[e], y[e + 1]);
       }
     };
-    auto readout_store = [&](int jt) {                              // fp32 read-out of tile jt leaves TMEM
+    auto readout_store = [&](int jt) {                              // fp32 read-out of tile jt (`prev`) leaves TMEM
       wait(&bars->out_ready, jt & 1);
       tc_fence_after();
       wait(&bars->nl_ready, jt & 1);                                 // both halves of the tile's phi.z sums are written
       if (aborted()) return;                                         // nothing of an abandoned launch is stored
       const float* nlp = s_nl + (jt & 1) * 256;
-      const bool tok_valid = tok_a + jt * 128 + r < tok_b;
-      const int ric = tok_a + jt * 128 + r - q0;                    // row inside the chunk; its tile is 128-aligned
+      const bool tok_valid = prev.tok + r < prev.tok_end;
+      const int bh = prev.bh, ci = prev.ci, ric = prev.tok + r - geo_q0(g, g.t0 + ci);   // row inside the chunk; its tile is 128-aligned
       uint4* rdh = reinterpret_cast<uint4*>(a.rd);
       const float nl_row = nlp[r] + nlp[128 + r];
       const float inv_nl = nl_row != 0.f ? 1.f / nl_row : 0.f;       // the read-out is stored as the ratio aL / nL
@@ -373,8 +400,23 @@ readout_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUt
       tc_fence_after();
     };
     for (int j = 0; j <= n_tiles; ++j) {
+      if (j > 0) prev = cur;
       if (j < n_tiles) {
-        if (aborted()) break;
+        if (j > 0) rd_next<EVEN>(g, a.rd_walk, n0 + j, cur);
+        const bool change = !EVEN && (cur.bh != prev.bh || cur.ci != prev.ci);
+        if (aborted()) {                                             // the other warps may still pass the barriers of the changes
+          for (; !EVEN && j < n_tiles; ++j) {
+            cur = rd_tile(g, a.rd_walk, n0 + j);                     // (again, for this one)
+            if (cur.bh != prev.bh || cur.ci != prev.ci) { all_warps(); all_warps(); }
+            prev = cur;
+          }
+          break;
+        }
+        if (change) {                                                // another (chunk, batch*head): all warps are done with the last
+          all_warps();
+          load_biases(cur, 256);
+          load_z(cur);
+        }
         // H halves: bias, activation, bf16, back to TMEM as the A operand of the second GEMM
 #pragma unroll 1
         for (int half = 0; half < nh; ++half) {                     // a width of at most 128 has no second half
@@ -416,7 +458,7 @@ readout_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUt
         }
       }
       // U halves: bias, activation, power, bf16, to the swizzled phi tiles; phi . z_t on the way
-      const bool tok_valid = tok_a + j * 128 + r < tok_b;
+      const bool tok_valid = cur.tok + r < cur.tok_end;
       float nl4[4] = {0.f, 0.f, 0.f, 0.f};                          // four chains: the sum is not one dependent sequence
 #pragma unroll 1
       for (int half = 0; half < nu; ++half) {

@@ -576,6 +576,14 @@ inline int tc_launch_window1(int head_dim, int exp_poly, int n_sm, const CUtenso
                              const ptx::WaitArgs& wa, float* share, int wait_first, int n_items, int pairs, int n_done, cudaStream_t st);
 inline bool tc_set_attributes1();
 
+template <bool RELU, int PC, bool GEN, bool N>
+inline bool tc_set_phi_attributes() {
+  const auto smem = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  return cudaFuncSetAttribute(phi_tc<RELU, PC, GEN, N, true>, smem, PhShape<N>::SMEM) == cudaSuccess &&
+         cudaFuncSetAttribute(phi_tc<RELU, PC, GEN, N, false>, smem, PhShape<N>::SMEM) == cudaSuccess &&
+         cudaFuncSetAttribute(readout_tc<RELU, PC, GEN, N, true>, smem, RdShape<N>::SMEM) == cudaSuccess &&
+         cudaFuncSetAttribute(readout_tc<RELU, PC, GEN, N, false>, smem, RdShape<N>::SMEM) == cudaSuccess;
+}
 inline int tc_set_attributes() {
   bool ok = tc_set_attributes1() &&
             cudaFuncSetAttribute(window_tc<0, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, WinShape<128>::SMEM) == cudaSuccess &&
@@ -586,20 +594,10 @@ inline int tc_set_attributes() {
             cudaFuncSetAttribute(window_tc<1, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, WinShape<64>::SMEM) == cudaSuccess &&
             cudaFuncSetAttribute(window_tc<2, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, WinShape<64>::SMEM) == cudaSuccess &&
             cudaFuncSetAttribute(window_tc<3, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, WinShape<64>::SMEM) == cudaSuccess &&
-            cudaFuncSetAttribute(phi_tc<true, 2, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PhShape<false>::SMEM) == cudaSuccess &&
-            cudaFuncSetAttribute(phi_tc<true, 0, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PhShape<false>::SMEM) == cudaSuccess &&
-            cudaFuncSetAttribute(phi_tc<false, 0, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PhShape<false>::SMEM) == cudaSuccess &&
-            cudaFuncSetAttribute(phi_tc<true, 0, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PhShape<false>::SMEM) == cudaSuccess &&
-            cudaFuncSetAttribute(phi_tc<false, 0, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PhShape<false>::SMEM) == cudaSuccess &&
-            cudaFuncSetAttribute(phi_tc<true, 0, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, PhShape<true>::SMEM) == cudaSuccess &&
-            cudaFuncSetAttribute(phi_tc<false, 0, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, PhShape<true>::SMEM) == cudaSuccess &&
-            cudaFuncSetAttribute(readout_tc<true, 2, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, RdShape<false>::SMEM) == cudaSuccess &&
-            cudaFuncSetAttribute(readout_tc<true, 0, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, RdShape<false>::SMEM) == cudaSuccess &&
-            cudaFuncSetAttribute(readout_tc<false, 0, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, RdShape<false>::SMEM) == cudaSuccess &&
-            cudaFuncSetAttribute(readout_tc<true, 0, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, RdShape<false>::SMEM) == cudaSuccess &&
-            cudaFuncSetAttribute(readout_tc<false, 0, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, RdShape<false>::SMEM) == cudaSuccess &&
-            cudaFuncSetAttribute(readout_tc<true, 0, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, RdShape<true>::SMEM) == cudaSuccess &&
-            cudaFuncSetAttribute(readout_tc<false, 0, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, RdShape<true>::SMEM) == cudaSuccess;
+            tc_set_phi_attributes<true, 2, false, false>() && tc_set_phi_attributes<true, 0, false, false>() &&
+            tc_set_phi_attributes<false, 0, false, false>() && tc_set_phi_attributes<true, 0, true, false>() &&
+            tc_set_phi_attributes<false, 0, true, false>() && tc_set_phi_attributes<true, 0, true, true>() &&
+            tc_set_phi_attributes<false, 0, true, true>();
   return ok ? REHYAT_OK : REHYAT_ERR_CUDA;
 }
 
@@ -698,7 +696,7 @@ inline int tc_launch_window(TcWorkspace* w, const void* q, const void* k, const 
 // phi_k + chunk-state partial sums of one group (Eq. 17-18).
 inline int tc_launch_state(const TcWorkspace* w, const void* k, const void* v, const rehyat_phi_params* phi,
                            const Geo& g, int batch, int Dh, int Dp, int P, int n_mid, int act_hidden, int act_out,
-                           int n_split, float* partial, const ptx::WaitArgs& wa, cudaStream_t st) {
+                           const StateWalk& walk, float* partial, const ptx::WaitArgs& wa, cudaStream_t st) {
   const int d = w->head_dim;
   CUtensorMap tk, tv, tw1, tw2, twm;
   if (!tc_make_tmap(w, &tk, k, g, batch) || !tc_make_tmap(w, &tv, v, g, batch) ||
@@ -711,10 +709,12 @@ inline int tc_launch_state(const TcWorkspace* w, const void* k, const void* v, c
   a.b1 = (const __nv_bfloat16*)phi->k_b1; a.b2 = (const __nv_bfloat16*)phi->k_b2; a.bm = (const __nv_bfloat16*)phi->k_bmid;
   a.P = P; a.act_hidden = act_hidden; a.act_out = act_out;
   a.d = d; a.Dh = Dh; a.Dp = Dp; a.n_mid = n_mid;
-  a.n_split = n_split; a.partial = partial; a.wa = wa;
+  a.walk = walk; a.partial = partial; a.wa = wa;
   const PhiKernelChoice ch = tc_phi_choice(d, Dh, Dp, P, n_mid, act_hidden, act_out);
-  const dim3 grid(n_split, g.G, g.BH);
-#define REHYAT_LAUNCH_PHI_N(R, PC, GEN, N) launch_kernel(phi_tc<R, PC, GEN, N>, grid, PH_THREADS, PhShape<N>::SMEM, st, tk, tv, tw1, tw2, twm, g, a)
+  if (walk.per == 0) return REHYAT_OK;                               // no chunk of the group admits a key
+  const dim3 grid(state_ctas(g, walk));
+#define REHYAT_LAUNCH_PHI_N(R, PC, GEN, N) \
+  launch_kernel(walk.even ? phi_tc<R, PC, GEN, N, true> : phi_tc<R, PC, GEN, N, false>, grid, PH_THREADS, PhShape<N>::SMEM, st, tk, tv, tw1, tw2, twm, g, a)
 #define REHYAT_LAUNCH_PHI(R, PC, GEN) REHYAT_LAUNCH_PHI_N(R, PC, GEN, false)
   if (tc_state_narrow(d, Dh, Dp, n_mid)) { if (ch.relu) REHYAT_LAUNCH_PHI_N(true, 0, true, true); else REHYAT_LAUNCH_PHI_N(false, 0, true, true); }
   else if (ch.gen) { if (ch.relu) REHYAT_LAUNCH_PHI(true, 0, true); else REHYAT_LAUNCH_PHI(false, 0, true); }
@@ -744,24 +744,13 @@ inline int tc_launch_readout(const TcWorkspace* w, const void* q, const rehyat_p
   a.d = d; a.Dh = Dh; a.Dp = Dp; a.n_mid = n_mid;
   a.state = state; a.rd = rd; a.rd_rows = rd_rows; a.wa = wa;
   const bool narrow = d == 64 && Dh <= 128 && Dp <= 128;
-  // One CTA per SM (two of the narrow form): split a chunk's query tiles over as many CTAs as costs the fewest tile-times
-  // over all waves.
-  const int slots = w->n_sm * (narrow ? 2 : 1);
-  const int tiles = (g.Np + 127) / 128;
-  int busy = 0;
-  for (int t = g.t0; t < g.t0 + g.G; ++t) busy += geo_linear(g, t);
-  const long long units = (long long)(busy > 0 ? busy : 1) * g.BH;
-  long long best = -1;
-  int best_s = 1;
-  for (int s = 1; s <= 16; ++s) {
-    const long long cost = ((units * s + slots - 1) / slots) * ((tiles + s - 1) / s);
-    if (best < 0 || cost < best) { best = cost; best_s = s; }
-  }
-  a.tiles_per_cta = (tiles + best_s - 1) / best_s;
-  const int ctas = (tiles + a.tiles_per_cta - 1) / a.tiles_per_cta;
+  a.rd_walk = rd_walk(g, w->n_sm * (narrow ? 2 : 1));               // one CTA per SM, two of the narrow form
+  if (a.rd_walk.per == 0) return REHYAT_OK;
+  const int ctas = (a.rd_walk.per_bh * g.BH + a.rd_walk.per - 1) / a.rd_walk.per;
   const PhiKernelChoice ch = tc_phi_choice(d, Dh, Dp, P, n_mid, act_hidden, act_out);
-  const dim3 grid(ctas, g.G, g.BH);
-#define REHYAT_LAUNCH_RD_N(R, PC, GEN, N) launch_kernel(readout_tc<R, PC, GEN, N>, grid, PH_THREADS, RdShape<N>::SMEM, st, tq, tw1, tw2, twm, ts, g, a)
+  const dim3 grid(ctas);
+#define REHYAT_LAUNCH_RD_N(R, PC, GEN, N) \
+  launch_kernel(a.rd_walk.even ? readout_tc<R, PC, GEN, N, true> : readout_tc<R, PC, GEN, N, false>, grid, PH_THREADS, RdShape<N>::SMEM, st, tq, tw1, tw2, twm, ts, g, a)
 #define REHYAT_LAUNCH_RD(R, PC, GEN) REHYAT_LAUNCH_RD_N(R, PC, GEN, false)
   if (narrow) { if (ch.relu) REHYAT_LAUNCH_RD_N(true, 0, true, true); else REHYAT_LAUNCH_RD_N(false, 0, true, true); }
   else if (ch.gen) { if (ch.relu) REHYAT_LAUNCH_RD(true, 0, true); else REHYAT_LAUNCH_RD(false, 0, true); }

@@ -358,3 +358,28 @@ def test_window_in_two_launches(d, nh, T, H, W, Tc, To):
         assert (np.abs(z - ref) <= 3e-3 + 2.0 ** -7 * size).all() and np.sqrt(((z - ref) ** 2).mean() / (ref ** 2).mean()) <= 1e-2
     assert np.abs(y - pairs).max() <= 2.0 ** -6 * np.abs(pairs).max()      # every row: two roundings of the weights and of the output
     np.testing.assert_array_equal(_forward(wl, x), y)
+
+# phi_tc and readout_tc with tiles numbered through all chunks and heads (40 heads x 4 chunks of 5 tiles are two waves of whole
+# chunks, 6 tiles for each of 134 CTAs): short last chunks, chunks without keys for the state (overlap beyond the chunk), a
+# first chunk with fewer tiles, two batch items, one-half and three-layer maps, the narrow form (3 CTAs' worth of chunks each).
+@pytest.mark.parametrize("B,d,nh,T,H,W,Tc,To,Dh,Dp,layers", [
+    (1, 128, 40, 9, 16, 20, 2, 1, 256, 256, 2), (2, 128, 20, 10, 16, 20, 2, 3, 256, 256, 2), (1, 128, 40, 9, 16, 19, 2, 0, 192, 96, 3),
+    (1, 64, 80, 10, 16, 20, 2, 1, 128, 128, 2), (1, 64, 40, 9, 13, 25, 2, 1, 256, 192, 4)])
+def test_phi_tiles_numbered_through(B, d, nh, T, H, W, Tc, To, Dh, Dp, layers):
+    wl = synth.Workload("through", B, nh, d, T, H, W, Tc, To, "bf16", True, seed=synth.BASE_SEED + 411, phi_hidden=Dh, phi_dim=Dp,
+                        phi_layers=layers)
+    x = synth.make_inputs(wl, phi_scale=2.0)
+    y = _forward(wl, x)
+    some = [0, 3, 4, nh // 2, nh - 1]                           # heads
+    xs = {n: x[n][:, some] for n in ("q", "k", "v")} | {m: {n: p[some] for n, p in x[m].items()} for m in ("phi_q", "phi_k")}
+    _gate(y[:, some], _oracle(wl, xs), "bf16")
+    np.testing.assert_array_equal(_forward(wl, x), y)
+    # bidirectional: 16 frames' increments of 3 tiles a launch
+    wl = synth.Workload("throughb", 1, 24, d, 18, 16, 20, 3, 1, "bf16", True, seed=synth.BASE_SEED + 412, phi_hidden=Dh, phi_dim=Dp,
+                        phi_layers=layers)
+    x = synth.make_inputs(wl, phi_scale=2.0)
+    y = _forward(wl, x, bidirectional=True)
+    some = [0, 11, 23]
+    f = synth.to_f64({n: x[n][:, some] for n in ("q", "k", "v")} | {m: {n: p[some] for n, p in x[m].items()} for m in ("phi_q", "phi_k")})
+    _gate(y[:, some], orc.hybrid_direct(f["q"], f["k"], f["v"], f["phi_q"], f["phi_k"], wl.T, wl.HW, wl.Tc, wl.To, P=wl.P,
+                                        causal=False), "bf16")
