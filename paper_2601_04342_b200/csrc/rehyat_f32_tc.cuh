@@ -21,7 +21,8 @@
 //
 // Every operand is multiplied by 2^20 as it is split, so that the parts of the smallest fp32 numbers are bf16 numbers too
 // (without it values below 2^-110 keep fewer than 24 bits), and what leaves an accumulator by 2^-40: both are exact.
-// Values from 2^39 on (or not finite) cannot be split safely, as 256 products of them would no longer fit an accumulator:
+// Values whose first part is 2^39 or more (or not finite) cannot be split safely, as 256 products of them would no longer fit an
+// accumulator:
 // whoever sees one leaves the launch's epoch in *unsafe, and window_simt, launched behind this kernel, computes the call
 // again; otherwise it ends at once.
 #pragma once
