@@ -613,8 +613,9 @@ int rehyat_create(rehyat_ctx** out, const rehyat_config* cfg) {
   if (!ok) { cudaGetLastError(); rehyat_destroy(ctx); return REHYAT_ERR_ALLOC; }
   if (cudaMemset(ctx->status_dev, 0, 256) != cudaSuccess) { rehyat_destroy(ctx); return REHYAT_ERR_CUDA; }
 
-  rc = set_simt_attributes_for(c.dtype, c.head_dim);
-  if (rc == REHYAT_OK && ctx->tensor_ok) rc = tc_set_attributes();
+  if (!(ctx->tensor_ok && ctx->tc.phi_ok)) rc = set_simt_attributes_for(c.dtype, c.head_dim);   // the others launch none of those
+  if (rc == REHYAT_OK && ctx->tensor_ok)
+    rc = tc_set_attributes(&ctx->tc, c.phi_hidden, c.phi_dim, c.poly_degree, c.phi_layers > 2 ? c.phi_layers - 2 : 0, c.act_hidden, c.act_out);
   if (rc != REHYAT_OK) { rehyat_destroy(ctx); return rc; }
   *out = ctx;
   return REHYAT_OK;

@@ -522,6 +522,8 @@ inline bool tc_phi_supported(int d, int Dh, int Dp, int P, int n_mid) {
 }
 // Does the narrow form of phi_tc (two CTAs per SM) serve a map?
 inline bool tc_state_narrow(int d, int Dh, int Dp, int n_mid) { return d == 64 && Dh <= 128 && Dp <= 128 && n_mid == 0; }
+// And that of readout_tc?
+inline bool tc_readout_narrow(int d, int Dh, int Dp) { return d == 64 && Dh <= 128 && Dp <= 128; }
 // Which instantiation serves a map: the fixed-shape kernels for the two-layer map of 128 / 256 / 256, the ones
 // that read their extents otherwise; the ReLU fast path needs polynomial parts that end on 32-column blocks.
 struct PhiKernelChoice { bool gen, relu; int pc; };
@@ -574,30 +576,37 @@ inline void launch_kernel(void (*kernel)(P...), dim3 grid, int threads, size_t s
 inline int tc_launch_window1(int head_dim, int exp_poly, int n_sm, const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
                              __nv_bfloat16* o, const Geo& g, const float* rd, int rd_rows, float scale, int c_mode,
                              const ptx::WaitArgs& wa, float* share, int wait_first, int n_items, int pairs, int n_done, cudaStream_t st);
+template <int E, int D>
 inline bool tc_set_attributes1();
 
-template <bool RELU, int PC, bool GEN, bool N>
-inline bool tc_set_phi_attributes() {
-  const auto smem = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  return cudaFuncSetAttribute(phi_tc<RELU, PC, GEN, N, true>, smem, PhShape<N>::SMEM) == cudaSuccess &&
-         cudaFuncSetAttribute(phi_tc<RELU, PC, GEN, N, false>, smem, PhShape<N>::SMEM) == cudaSuccess &&
-         cudaFuncSetAttribute(readout_tc<RELU, PC, GEN, N, true>, smem, RdShape<N>::SMEM) == cudaSuccess &&
-         cudaFuncSetAttribute(readout_tc<RELU, PC, GEN, N, false>, smem, RdShape<N>::SMEM) == cudaSuccess;
+// Shared-memory limits of the kernels a context may launch, and of no others: the first such call for a kernel loads it.
+template <typename K>
+inline bool tc_set_smem(K kernel, int bytes) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess; }
+template <int E>
+inline bool tc_set_window_attributes(int d) {
+  return d == 64 ? tc_set_smem(window_tc<E, 64>, WinShape<64>::SMEM) && tc_set_attributes1<E, 64>()
+                 : tc_set_smem(window_tc<E, 128>, WinShape<128>::SMEM) && tc_set_attributes1<E, 128>();
 }
-inline int tc_set_attributes() {
-  bool ok = tc_set_attributes1() &&
-            cudaFuncSetAttribute(window_tc<0, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, WinShape<128>::SMEM) == cudaSuccess &&
-            cudaFuncSetAttribute(window_tc<1, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, WinShape<128>::SMEM) == cudaSuccess &&
-            cudaFuncSetAttribute(window_tc<2, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, WinShape<128>::SMEM) == cudaSuccess &&
-            cudaFuncSetAttribute(window_tc<3, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, WinShape<128>::SMEM) == cudaSuccess &&
-            cudaFuncSetAttribute(window_tc<0, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, WinShape<64>::SMEM) == cudaSuccess &&
-            cudaFuncSetAttribute(window_tc<1, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, WinShape<64>::SMEM) == cudaSuccess &&
-            cudaFuncSetAttribute(window_tc<2, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, WinShape<64>::SMEM) == cudaSuccess &&
-            cudaFuncSetAttribute(window_tc<3, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, WinShape<64>::SMEM) == cudaSuccess &&
-            tc_set_phi_attributes<true, 2, false, false>() && tc_set_phi_attributes<true, 0, false, false>() &&
-            tc_set_phi_attributes<false, 0, false, false>() && tc_set_phi_attributes<true, 0, true, false>() &&
-            tc_set_phi_attributes<false, 0, true, false>() && tc_set_phi_attributes<true, 0, true, true>() &&
-            tc_set_phi_attributes<false, 0, true, true>();
+template <bool STATE, bool RELU, int PC, bool GEN, bool N>
+inline bool tc_set_phi_attributes() {
+  if constexpr (STATE) return tc_set_smem(phi_tc<RELU, PC, GEN, N, true>, PhShape<N>::SMEM) && tc_set_smem(phi_tc<RELU, PC, GEN, N, false>, PhShape<N>::SMEM);
+  else return tc_set_smem(readout_tc<RELU, PC, GEN, N, true>, RdShape<N>::SMEM) && tc_set_smem(readout_tc<RELU, PC, GEN, N, false>, RdShape<N>::SMEM);
+}
+template <bool STATE>
+inline bool tc_set_phi_attributes(bool narrow, const PhiKernelChoice& ch) {
+  if (narrow) return ch.relu ? tc_set_phi_attributes<STATE, true, 0, true, true>() : tc_set_phi_attributes<STATE, false, 0, true, true>();
+  if (ch.gen) return ch.relu ? tc_set_phi_attributes<STATE, true, 0, true, false>() : tc_set_phi_attributes<STATE, false, 0, true, false>();
+  if (ch.pc == 2) return tc_set_phi_attributes<STATE, true, 2, false, false>();
+  return ch.relu ? tc_set_phi_attributes<STATE, true, 0, false, false>() : tc_set_phi_attributes<STATE, false, 0, false, false>();
+}
+inline int tc_set_attributes(const TcWorkspace* w, int Dh, int Dp, int P, int n_mid, int act_hidden, int act_out) {
+  const int d = w->head_dim;
+  bool ok = w->exp_poly == 0 ? tc_set_window_attributes<0>(d) : w->exp_poly == 2 ? tc_set_window_attributes<2>(d)
+            : w->exp_poly == 3 ? tc_set_window_attributes<3>(d) : tc_set_window_attributes<1>(d);
+  if (w->phi_ok) {
+    const PhiKernelChoice ch = tc_phi_choice(d, Dh, Dp, P, n_mid, act_hidden, act_out);
+    ok = ok && tc_set_phi_attributes<true>(tc_state_narrow(d, Dh, Dp, n_mid), ch) && tc_set_phi_attributes<false>(tc_readout_narrow(d, Dh, Dp), ch);
+  }
   return ok ? REHYAT_OK : REHYAT_ERR_CUDA;
 }
 
@@ -743,7 +752,7 @@ inline int tc_launch_readout(const TcWorkspace* w, const void* q, const rehyat_p
   a.P = P; a.act_hidden = act_hidden; a.act_out = act_out;
   a.d = d; a.Dh = Dh; a.Dp = Dp; a.n_mid = n_mid;
   a.state = state; a.rd = rd; a.rd_rows = rd_rows; a.wa = wa;
-  const bool narrow = d == 64 && Dh <= 128 && Dp <= 128;
+  const bool narrow = tc_readout_narrow(d, Dh, Dp);
   a.rd_walk = rd_walk(g, w->n_sm * (narrow ? 2 : 1));               // one CTA per SM, two of the narrow form
   if (a.rd_walk.per == 0) return REHYAT_OK;
   const int ctas = (a.rd_walk.per_bh * g.BH + a.rd_walk.per - 1) / a.rd_walk.per;

@@ -377,15 +377,7 @@ inline int tc_launch_window1(int head_dim, int exp_poly, int n_sm, const CUtenso
   return cudaGetLastError() == cudaSuccess ? REHYAT_OK : REHYAT_ERR_CUDA;
 }
 
-inline bool tc_set_attributes1() {
-  return cudaFuncSetAttribute(window_tc1<0, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, WinShape<128>::SMEM1) == cudaSuccess &&
-         cudaFuncSetAttribute(window_tc1<1, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, WinShape<128>::SMEM1) == cudaSuccess &&
-         cudaFuncSetAttribute(window_tc1<2, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, WinShape<128>::SMEM1) == cudaSuccess &&
-         cudaFuncSetAttribute(window_tc1<3, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, WinShape<128>::SMEM1) == cudaSuccess &&
-         cudaFuncSetAttribute(window_tc1<0, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, WinShape<64>::SMEM1) == cudaSuccess &&
-         cudaFuncSetAttribute(window_tc1<1, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, WinShape<64>::SMEM1) == cudaSuccess &&
-         cudaFuncSetAttribute(window_tc1<2, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, WinShape<64>::SMEM1) == cudaSuccess &&
-         cudaFuncSetAttribute(window_tc1<3, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, WinShape<64>::SMEM1) == cudaSuccess;
-}
+template <int E, int D>
+inline bool tc_set_attributes1() { return tc_set_smem(window_tc1<E, D>, WinShape<D>::SMEM1); }
 
 }  // namespace rehyat
